@@ -191,7 +191,7 @@ def _csr_rows(g, n, n0, mean):
     return row_ptr, (key % n0).int(), torch.randn(key.numel(), device="cuda", generator=g).abs_()
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
     d, S, B = _dims(case), case["subnets"], case["batch"]
     g = torch.Generator(device="cuda").manual_seed(seed)
     W, b = [], []
@@ -206,6 +206,12 @@ def prepare(case, seed):
         X = torch.randn(n, d[0], device="cuda", generator=g)
         X = X.to(torch.bfloat16) if case["x"] == "bf16" else X
     y = torch.randint(d[-1], (n,), device="cuda", generator=g, dtype=torch.int32)
+    return W, b, X, y
+
+
+def prepare(case, seed):
+    d, S, B = _dims(case), case["subnets"], case["batch"]
+    W, b, X, y = _inputs(case, seed)
     ctx = api.Ist(d, S, api.IST_BF16 if case["precision"] == "bf16" else api.IST_FP32, B,
                   input_is_csr=case["x"] == "csr",
                   partition_rule=api.IST_PART_IID if case["rule"] == "iid" else api.IST_PART_BALANCED)
@@ -233,3 +239,139 @@ def run(state):
         grads.append(dx)
     ctx.reassemble()
     return {"loss": losses, "dx": grads, "W": ctx.W, "b": ctx.b}
+
+
+# ---- the same in 64 bits, with torch alone ------------------------------------------------------
+
+def _splitmix64(state, count):
+    """Outputs 1..count of SplitMix64 (Steele, Lea, Flood 2014) from `state`, as int64 bit patterns."""
+    def signed(v):
+        v &= 2 ** 64 - 1
+        return v - 2 ** 64 if v >= 2 ** 63 else v
+
+    def shifted(v, k):                                 # logical shift right
+        return (v >> k) & (2 ** (64 - k) - 1)
+
+    z = torch.arange(1, count + 1, device="cuda") * signed(0x9E3779B97F4A7C15) + signed(state)
+    z = (z ^ shifted(z, 30)) * signed(0xBF58476D1CE4E5B9)
+    z = (z ^ shifted(z, 27)) * signed(0x94D049BB133111EB)
+    return z ^ shifted(z, 31)
+
+
+def _groups(case, round_seed):
+    """Per hidden layer the S index sets of the partition that `round_seed` draws."""
+    S, out = case["subnets"], []
+    for l, n in enumerate(_dims(case)[1:-1], 1):
+        key = _splitmix64(int(_splitmix64(round_seed, l)[-1]), n)
+        if case["rule"] == "iid":                      # floor(key * S / 2^64) of the unsigned key
+            high, low = (key >> 32) & 0xFFFFFFFF, key & 0xFFFFFFFF
+            which = (high * S + ((low * S) >> 32)) >> 32
+        else:                                          # equal shares of the unsigned order
+            which = torch.empty(n, dtype=torch.int64, device="cuda")
+            sizes = torch.tensor([n // S + (s < n % S) for s in range(S)], device="cuda")
+            order = torch.sort(key ^ -2 ** 63, stable=True).indices
+            which[order] = torch.repeat_interleave(torch.arange(S, device="cuda"), sizes)
+        out.append([torch.nonzero(which == s).flatten() for s in range(S)])
+    return out
+
+
+class _Rows:
+    """Rows r0 .. r0 + n - 1 of the inputs: products with a first-layer matrix and its gradient."""
+
+    def __init__(self, X, r0, n):
+        if isinstance(X, tuple):
+            row_ptr, col, val = X
+            lo, hi = int(row_ptr[r0]), int(row_ptr[r0 + n])
+            counts = (row_ptr[r0 + 1:r0 + n + 1] - row_ptr[r0:r0 + n]).long()
+            row = torch.repeat_interleave(torch.arange(n, device="cuda"), counts)
+            self.csr, self.n = (row, col[lo:hi].long(), val[lo:hi].double()[:, None]), n
+        else:
+            self.csr, self.x = None, X[r0:r0 + n].double()
+
+    def times(self, W):
+        if self.csr is None:
+            return self.x @ W
+        row, col, val = self.csr
+        return torch.zeros(self.n, W.shape[1], dtype=W.dtype, device="cuda").index_add_(0, row, W[col] * val)
+
+    def descend(self, W, delta, lr):
+        if self.csr is None:
+            W.addmm_(self.x.T, delta, alpha=-lr)
+        else:
+            row, col, val = self.csr
+            W.index_add_(0, col, delta[row] * val, alpha=-lr)
+
+
+def _step(case, W, b, x, y):
+    """One SGD step of one subnet (W, b are changed): the mean loss and d(loss)/d(x) where it is asked for."""
+    t, B, a, unit, scale, z = len(W), case["batch"], [], [], [], None
+    for l in range(t):
+        z = (x.times(W[0]) if l == 0 else a[-1] @ W[l]) + b[l]
+        if l + 1 < t:
+            if case["norm"]:
+                centred = z - z.mean(0)
+                scale.append(torch.rsqrt((centred ** 2).mean(0) + 1e-5))
+                z = centred * scale[-1]
+                unit.append(z)
+            a.append(z.clamp_min(0))
+    at = torch.arange(B, device="cuda")
+    logp = torch.log_softmax(z, 1)
+    loss = -logp[at, y].mean()
+    delta = torch.exp(logp)
+    delta[at, y] -= 1
+    delta /= B
+    lr, dx = case["lr"], None
+    for l in range(t - 1, -1, -1):
+        below = delta @ W[l].T if l > 0 or case["call"] == "trunk" else None
+        b[l] -= lr * delta.sum(0)
+        if l == 0:
+            dx = below
+            x.descend(W[0], delta, lr)
+            break
+        W[l].addmm_(a[l - 1].T, delta, alpha=-lr)
+        delta = below * (a[l - 1] > 0)
+        if case["norm"]:
+            zh = unit[l - 1]
+            delta = scale[l - 1] * (delta - delta.mean(0) - zh * (delta * zh).mean(0))
+    return loss, dx
+
+
+def exact(case, seed):
+    W, b, X, y = _inputs(case, seed)
+    y, S, B, K = y.long(), case["subnets"], case["batch"], case["steps"]
+    if case["call"] == "eval":
+        loss, hits = 0.0, 0
+        for r0 in range(0, case["rows"], B):
+            n = min(B, case["rows"] - r0)
+            z = _Rows(X, r0, n).times(W[0].double()) + b[0]
+            for Wl, bl in zip(W[1:], b[1:]):
+                z = z.clamp_min(0) @ Wl.double() + bl
+            labels = y[r0:r0 + n]
+            loss = loss - torch.log_softmax(z, 1)[torch.arange(n, device="cuda"), labels].sum()
+            hits = hits + (z.argmax(1) == labels).sum()
+        return (loss / case["rows"]).reshape(1), hits.reshape(1)
+    t, groups = len(W), _groups(case, seed * 7919 + 1)
+    W, b = [w.double() for w in W], [v.double() for v in b]
+    out_bias = torch.zeros_like(b[-1])
+    losses = torch.empty(S, K, dtype=torch.float64, device="cuda")
+    grads = [torch.empty(S * B, _dims(case)[0], dtype=torch.float64, device="cuda") for _ in range(K)] \
+        if case["call"] == "trunk" else None
+    for s in range(S):
+        rows = [slice(None)] + [g[s][:, None] for g in groups[:-1]] + [groups[-1][s]]
+        cols = [g[s] for g in groups] + [slice(None)]
+        Ws = [W[l][rows[l], cols[l]].clone() for l in range(t)]
+        bs = [b[l][cols[l]].clone() for l in range(t)]
+        for k in range(K):                             # rows [S][K][B] of a round, [K][S][B] with a trunk
+            r0 = (k * S + s) * B if grads is not None else (s * K + k) * B
+            losses[s, k], dx = _step(case, Ws, bs, _Rows(X, r0, B), y[r0:r0 + B])
+            if grads is not None:
+                grads[k][s * B:(s + 1) * B] = dx
+        for l in range(t):
+            W[l][rows[l], cols[l]] = Ws[l]
+            if l + 1 < t:
+                b[l][cols[l]] = bs[l]
+        out_bias += bs[-1] / S
+    b[-1] = out_bias
+    if grads is None:
+        return {"loss": losses, "W": W, "b": b}
+    return {"loss": [losses[:, k:k + 1] for k in range(K)], "dx": grads, "W": W, "b": b}
