@@ -1,0 +1,608 @@
+// Grouped fp32 GEMM on the 5th-generation tensor cores: the fp32 path of the local steps (forward,
+// backward and SGD update of all S subnets; paper Sec. 2.1 "Training Subnets", App. A Eq. (2) on
+// the slices), their input gradients, and the full-width evaluation pass.
+//
+//   C[g](m, n) = sum_k A[g](m, k) * B[g](n, k)
+//
+// Every fp32 operand is the exact sum of three bf16 numbers (8 + 8 + 8 significant bits):
+// x = h + m + l with h = bf16(x), m = bf16(x - h), l = x - h - m.  A product of two of them is then
+// nine bf16 products, of which the six of weight 2^-16 and above are formed:
+//   a b = ah bh + (ah bm + am bh) + (ah bl + am bm + al bh) + O(2^-26 |a b|),
+// and the three left out are below the rounding of a single fp32 multiplication (2^-24).
+// The tensor core's own accumulation is not relied on over long sums: 32 values of k are
+// accumulated in tensor memory (the small products first, so that only the last two
+// instructions act on a sum of full size), and the 32-deep sums are then added up in fp32
+// registers with round-to-nearest.
+//
+// A CTA computes a 128 x BN tile (PAIR = 2: two CTAs of a cluster a 256 x BN one, each with its own
+// 128 rows of A and half of B) in steps of 32 k values.
+//   warps 0..7   load fp32 operands with plain vector loads (any base, any stride: rows of the full
+//                network need not be 16-byte aligned), one or two steps ahead of their use, and
+//                split them into the three bf16 planes in shared memory (128-byte swizzle, two
+//                slots of 32 k values)
+//   warps 8..15  move finished 32-deep sums from tensor memory into registers, adding up
+//   one thread   issues the MMAs.  It is held up for as long as they take to start (60 cycles each,
+//                128 on a 256-column tile), so on narrow tiles, where adding up is quick, it has a
+//                warp of its own; on 256-column tiles, where such a warp would cost the
+//                other sixteen a quarter of their registers, it sits in warp 8
+// Three barriers per slot / accumulator connect them:
+//   full[b]   every loading warp has written its part of slot b
+//   done[b]   the MMAs on slot b are complete: accumulator b can be read, slot b rewritten
+//   taken[b]  every adding warp has read accumulator b: the MMAs after next may overwrite it
+//
+// A product with few tiles is cut along k over the CTAs of a cluster (up to eight); each leaves
+// its sums in shared memory and the cluster adds them up in rank order, every CTA finishing its
+// share of the tile's rows.
+//
+// Values that have no such decomposition (infinities, NaN, and magnitudes that round to infinity
+// in bf16) turn the products they enter into NaN.  The epilogue computes every result that is not
+// finite again as a chain of fp32 multiply-adds, so that the outcome is the one of fp32 arithmetic.
+//
+// What bounds it: pairs, the tensor pipe (12 MMAs per step and 256 x 256 tile, about 1540 cycles) at the
+// clock the power limit leaves: 512 x 16384 x 16384 in 1.18 ms = 234 TFLOP/s of fp32 products,
+// 1.40 PFLOP/s of bf16 ones (the same product on the CUDA cores, 128 x 128 tiles: 6.5 ms).  Single
+// CTAs, the chain wait - split - barrier - MMA of a step, about 0.95 us (256 x 1024 x 1024 of
+// four groups 164 -> 27 us, 1024 x 1024 x 256 of four groups 96 -> 25 us).  Error of a K-term sum
+// against 64 bits, relative 2-norm, before -> now: K = 64 1.0e-7 -> 6e-8, 1024 4.1e-7 -> 1.2e-7,
+// 16384 1.6e-6 -> 4.1e-7.
+//
+// Every wait is bounded, see tc_ptx.cuh.
+#include <algorithm>
+#include <cfloat>
+#include <mutex>
+
+#include "kernels.h"
+#include "tc_ptx.cuh"
+
+namespace ist {
+namespace {
+
+constexpr int BM = 128;
+constexpr int KH = 32;                  // k values of a step
+constexpr int kLoadWarps = 8, kAddWarps = 8, kThreads = 32 * (kLoadWarps + kAddWarps);   // those of finish()
+// narrow tiles: a warp of its own issues the MMAs (with the three beside it that fill up its
+// register-allotment group)
+constexpr int threads_of(int bn) { return bn == 256 ? kThreads : kThreads + 128; }
+constexpr int kMaxProblems = 4;
+
+struct F32Problem {
+  int M, N, K, G;
+  int m_tiles, n_tiles, tile_end;       // tiles tile_end(previous) .. tile_end - 1 of the launch
+  int epi, vec;                         // vec bits: 1 A, 2 B loads, 4 output accesses may be 16-byte vectors
+  const float* A; long long a_st, a_sg; // row stride (K-major) or k stride (MN-major), group stride
+  const float* B; long long b_st, b_sg;
+  const float* bias; long long bias_sg;
+  float* out; long long out_ld, out_sg;
+  const float* mask; long long mask_ld, mask_sg;
+};
+
+struct F32Args {
+  int n_problems;
+  int ksplit;                           // CTAs of a cluster that share a tile's k range
+  float lr;
+  DeviceStatus* status;
+  F32Problem p[kMaxProblems];
+};
+
+__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+// Two floats into their three bf16 parts, packed pairwise.
+__device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+  h = cvt_bf16x2(x, y);
+  const float xr = x - __uint_as_float(h << 16), yr = y - __uint_as_float(h & 0xffff0000u);
+  m = cvt_bf16x2(xr, yr);
+  l = cvt_bf16x2(xr - __uint_as_float(m << 16), yr - __uint_as_float(m & 0xffff0000u));
+}
+__device__ __forceinline__ void add2(uint64_t& acc, uint32_t lo, uint32_t hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(v));
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+// One operand's share of a loading thread: UNITS groups of eight consecutive floats of a step.
+//   K-major (rows contiguous along k): a warp takes 8 rows x 32 k, lane -> row (l / 4) % 2 * 4 + l / 8,
+//     eight k from l % 4 * 8, unit i 64 rows further; the two rows of eight lanes differ by 4, so that
+//     their swizzled 16-byte stores meet eight different bank groups.
+//   MN-major (contiguous along m or n): a warp takes 4 k x 64 columns, unit i 64 columns further.
+template <int MN, int UNITS>
+struct Operand {
+  const float* p;
+  long long unit_step, half_step;
+  int rows;          // K-major: rows left from this thread's first one; MN-major: columns left
+  int kofs;          // first k of this thread inside a step
+  uint32_t off0;     // offset inside the operand's plane, slot 0
+  bool vec;
+  __device__ __forceinline__ void init(const float* base, long long st, int row0, int extent, int k0, int tid, bool v) {
+    const int warp = tid >> 5, lane = tid & 31;
+    vec = v;
+    if (MN) {
+      const int k = warp * 4 + (lane >> 3), col = (lane & 7) * 8;
+      kofs = k;
+      p = base + (long long)(k0 + k) * st + row0 + col;
+      unit_step = 64;
+      half_step = KH * st;
+      rows = extent - row0 - col;
+      off0 = (uint32_t)(k * 128 + (((lane & 7) ^ (k & 7)) << 4));
+    } else {
+      const int r8 = ((lane >> 2) & 1) * 4 + (lane >> 3), r = warp * 8 + r8, u = lane & 3;
+      kofs = u * 8;
+      p = base + (long long)(row0 + r) * st + k0 + u * 8;
+      unit_step = 64 * st;
+      half_step = KH;
+      rows = extent - row0 - r;
+      off0 = (uint32_t)(r * 128 + ((u ^ r8) << 4));
+    }
+  }
+  // slot 1 holds k values 32..63 of the 64-deep swizzled rows
+  __device__ __forceinline__ uint32_t off(int slot) const { return MN ? off0 + slot * 4096u : off0 ^ (slot * 64u); }
+  // krem: k values left from the first one of the step
+  __device__ __forceinline__ void fetch(float (&v)[UNITS][8], int krem) {
+#pragma unroll
+    for (int i = 0; i < UNITS; ++i) {
+      const float* q = p + i * unit_step;
+      const int n = MN ? (kofs < krem ? rows - 64 * i : 0) : (64 * i < rows ? krem - kofs : 0);
+      if (vec && n >= 8) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(q)), b = __ldg(reinterpret_cast<const float4*>(q) + 1);
+        v[i][0] = a.x; v[i][1] = a.y; v[i][2] = a.z; v[i][3] = a.w;
+        v[i][4] = b.x; v[i][5] = b.y; v[i][6] = b.z; v[i][7] = b.w;
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[i][e] = e < n ? __ldg(q + e) : 0.f;
+      }
+    }
+    p += half_step;
+  }
+  template <uint32_t PLANE>
+  __device__ __forceinline__ void store(const float (&v)[UNITS][8], uint8_t* plane0, int slot) const {
+#pragma unroll
+    for (int i = 0; i < UNITS; ++i) {
+      uint4 h, m, l;
+      split2(v[i][0], v[i][1], h.x, m.x, l.x);
+      split2(v[i][2], v[i][3], h.y, m.y, l.y);
+      split2(v[i][4], v[i][5], h.z, m.z, l.z);
+      split2(v[i][6], v[i][7], h.w, m.w, l.w);
+      uint8_t* d = plane0 + off(slot) + i * 8192;
+      *reinterpret_cast<uint4*>(d) = h;
+      *reinterpret_cast<uint4*>(d + PLANE) = m;
+      *reinterpret_cast<uint4*>(d + 2 * PLANE) = l;
+    }
+  }
+};
+
+// The result at (m, n) as a chain of multiply-adds (see the file's comment on non-finite values).
+template <int A_MN, int B_MN>
+__device__ __forceinline__ float fma_chain(const F32Problem& pr, int g, int m, int n) {
+  const float* A = pr.A + (long long)g * pr.a_sg + (A_MN ? m : m * pr.a_st);
+  const float* B = pr.B + (long long)g * pr.b_sg + (B_MN ? n : n * pr.b_st);
+  const long long as = A_MN ? pr.a_st : 1, bs = B_MN ? pr.b_st : 1;
+  float acc = 0.f;
+#pragma unroll 1
+  for (int k = 0; k < pr.K && acc == acc; ++k) acc = fmaf(__ldg(A + k * as), __ldg(B + k * bs), acc);
+  return acc;
+}
+
+template <int BN, int PAIR>
+constexpr uint32_t ring_bytes() { return 3u * (BM + BN / PAIR) * 128u; }
+template <int BN, int PAIR>
+constexpr uint32_t smem_bytes() {
+  const uint32_t tile = BM * (BN + 4) * 4;
+  return (ring_bytes<BN, PAIR>() > tile ? ring_bytes<BN, PAIR>() : tile) + 1024;
+}
+
+// Closing part of a tile, run by all threads: the finished sums lie in shared memory, row by row;
+// apply the epilogue to this CTA's share of the rows and write the result.
+template <int A_MN, int B_MN, int BN, int PAIR>
+__device__ __forceinline__ void finish(const F32Args& a, const F32Problem& pr, int g, int m0, int n0, int rank, int cluster,
+                                       const float* tile_s, int tid) {
+  constexpr int PITCH = BN + 4, Q = BN / 4;             // Q 4-column pieces of a row
+  const int share = PAIR == 1 ? BM / cluster : BM;      // rows this CTA finishes
+  const int r_lo = PAIR == 1 ? rank * share : 0;
+  const int live = min(share, pr.M - m0 - r_lo);        // those inside the result
+  const uint32_t tile_u = smem_u32(tile_s);
+#pragma unroll 2
+  for (int e = tid; e < live * Q; e += kThreads) {
+    const int r = r_lo + e / Q, c4 = (e % Q) * 4, m = m0 + r, n = n0 + c4;
+    if (n >= pr.N) continue;
+    float v[4];
+    if (PAIR == 1 && cluster > 1) {
+      const uint32_t mine = tile_u + (uint32_t)(r * PITCH + c4) * 4;
+      v[0] = v[1] = v[2] = v[3] = 0.f;
+      for (int s = 0; s < cluster; ++s) {               // in rank order: a fixed sum
+        uint32_t addr;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(mine), "r"(s));
+        const float4 t = ld_cluster4(addr);
+        v[0] += t.x; v[1] += t.y; v[2] += t.z; v[3] += t.w;
+      }
+    } else {
+      const float4 t = *reinterpret_cast<const float4*>(tile_s + r * PITCH + c4);
+      v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    }
+    const int cnt = min(4, pr.N - n);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (!(fabsf(v[u]) <= FLT_MAX) && u < cnt) v[u] = fma_chain<A_MN, B_MN>(pr, g, m, n + u);
+    float* out = pr.out + (long long)g * pr.out_sg + (long long)m * pr.out_ld + n;
+    const bool wide = (pr.vec & 4) && cnt == 4;
+    float x[4] = {0.f, 0.f, 0.f, 0.f};                  // the epilogue's other input: bias, mask or the old weight
+    const float* src = pr.epi == EPI_SGD ? out
+                       : pr.epi == EPI_RELU_MASK ? pr.mask + (long long)g * pr.mask_sg + (long long)m * pr.mask_ld + n
+                       : pr.bias                 ? pr.bias + (long long)g * pr.bias_sg + n : nullptr;
+    if (src) {
+      if (wide) {
+        const float4 t = *reinterpret_cast<const float4*>(src);
+        x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (u < cnt) x[u] = src[u];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (pr.epi == EPI_SGD) v[u] = x[u] - a.lr * v[u];
+      else if (pr.epi == EPI_RELU_MASK) v[u] = x[u] > 0.f ? v[u] : 0.f;
+      else {
+        v[u] += x[u];
+        if (pr.epi == EPI_BIAS_RELU) v[u] = fmaxf(v[u], 0.f);
+      }
+    }
+    if (wide) {
+      *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < cnt) out[u] = v[u];
+    }
+  }
+}
+
+template <int A_MN, int B_MN, int BN, int PAIR>
+__global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __grid_constant__ F32Args a) {
+  constexpr int BNL = BN / PAIR;                       // rows of B this CTA loads
+  constexpr uint32_t A_BYTES = BM * 128, PLANE = A_BYTES + BNL * 128;
+  constexpr int UA = BM / 64, UB = BNL / 64;
+  constexpr int NACC = BN / 2;                         // sums per adding thread
+  constexpr int PITCH = BN + 4;                        // floats per row of the finished tile in shared memory
+  constexpr int DEPTH = BN == 256 ? 1 : 2;             // steps whose operands are on their way to registers
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  float* tile_s = reinterpret_cast<float*>(smem);
+  __shared__ uint64_t full[2], done[2], taken[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int cluster = PAIR == 2 ? 2 : a.ksplit;
+  const int rank = cluster > 1 ? (int)cluster_ctarank() : 0;
+  if (tid == 0) {
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&full[b], PAIR * kLoadWarps);
+      mbar_init(&done[b], 1);
+      mbar_init(&taken[b], PAIR * kAddWarps);
+    }
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  if (warp == 0) {
+    if (PAIR == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(2 * BN) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(2 * BN) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (PAIR == 2) cluster_sync_all();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  volatile int* abortp = &abort_flag;
+
+  // which tile, and which part of its k range
+  int pi = 0, tile = (int)blockIdx.x / cluster;
+  while (tile >= a.p[pi].tile_end) ++pi;
+  const F32Problem& pr = a.p[pi];
+  tile -= pi ? a.p[pi - 1].tile_end : 0;
+  const int mt = tile % pr.m_tiles, rest = tile / pr.m_tiles, nt = rest % pr.n_tiles, g = rest / pr.n_tiles;
+  const int m0 = mt * (BM * PAIR) + (PAIR == 2 ? rank * BM : 0);   // this CTA's rows of A and of the result
+  const int n0 = nt * BN;                                          // first column of the tile
+  int step0 = 0, steps = (pr.K + KH - 1) / KH;
+  if (PAIR == 1 && cluster > 1) {
+    const int per = (steps + cluster - 1) / cluster;
+    step0 = min(rank * per, steps);
+    steps = min(per, steps - step0);
+  }
+
+  pdl_wait();       // everything above touched this CTA's own memory only, see common.cuh
+  pdl_trigger();
+
+  // After the last MMA: sums into shared memory, tensor memory back, results out.  Both roles
+  // come here by their own copy of the code, so that each keeps its own register allotment.
+  auto close = [&](const uint64_t* acc) {
+    tc_fence_before();
+    __syncthreads();
+    if (PAIR == 2) cluster_sync_all();   // the peer's MMAs have read this CTA's shared memory
+    const bool bad = *abortp != 0;
+    if (acc) {
+      float* row = tile_s + ((warp & 3) * 32 + lane) * PITCH + ((warp - kLoadWarps) >> 2) * NACC;
+#pragma unroll
+      for (int c = 0; c < NACC / 4; ++c)
+        *reinterpret_cast<ulonglong2*>(row + 4 * c) = make_ulonglong2(acc[2 * c], acc[2 * c + 1]);
+    } else if (warp == 0) {
+      __syncwarp();
+      if (PAIR == 2)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
+      else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
+    }
+    if (PAIR == 1 && cluster > 1) cluster_sync_all(); else __syncthreads();
+    if (!bad && warp < kLoadWarps + kAddWarps) finish<A_MN, B_MN, BN, PAIR>(a, pr, g, m0, n0, rank, cluster, tile_s, tid);
+    if (PAIR == 1 && cluster > 1) cluster_sync_all();   // the others have read this CTA's sums
+  };
+
+  // Descriptors of slot 0, plane 0; the others lie a constant further (an address in 16-byte
+  // units, below 2^14).  Built afresh for every MMA they took 60 cycles each, more than the
+  // tensor core's work on a 64-column tile.
+  constexpr uint32_t idesc = make_idesc(A_MN, B_MN, BN, BM * PAIR);
+  const uint64_t ad0 = A_MN ? make_desc(smem_u32(smem), 8192, 1024) : make_desc(smem_u32(smem), 16, 1024);
+  const uint64_t bd0 = B_MN ? make_desc(smem_u32(smem) + A_BYTES, 8192, 1024) : make_desc(smem_u32(smem) + A_BYTES, 16, 1024);
+  auto issue = [&](int i) -> bool {                          // the MMAs of step i
+    const int b = i & 1;
+    if (!mbar_wait(&full[b], (i >> 1) & 1, abortp, a.status, 21)) return false;
+    if (i >= 2 && !mbar_wait(&taken[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 23)) return false;
+    tc_fence_after();
+    constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};   // low x high first, high x high last
+    const uint64_t ad = ad0 + (b ? (A_MN ? 4096 : 64) >> 4 : 0), bd = bd0 + (b ? (B_MN ? 4096 : 64) >> 4 : 0);
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+#pragma unroll
+      for (int k = 0; k < KH / 16; ++k) {
+        const uint64_t da = ad + ((pa[c] * PLANE + k * (A_MN ? 2048 : 32)) >> 4);
+        const uint64_t db = bd + ((pb[c] * PLANE + k * (B_MN ? 2048 : 32)) >> 4);
+        if (PAIR == 2) tc_mma_pair(tmem + b * BN, da, db, idesc, (c | k) != 0);
+        else tc_mma(tmem + b * BN, da, db, idesc, (c | k) != 0);
+      }
+    if (PAIR == 2) tc_commit_pair(&done[b]); else tc_commit(&done[b]);
+    return true;
+  };
+
+  if (warp < kLoadWarps) {
+    // ---------------------------------------------------------------- load and split
+    // registers at launch: 512 threads x 128, or 640 x 96
+    if (BN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    Operand<A_MN, UA> oa;
+    Operand<B_MN, UB> ob;
+    oa.init(pr.A + (long long)g * pr.a_sg, pr.a_st, m0, pr.M, step0 * KH, tid, pr.vec & 1);
+    ob.init(pr.B + (long long)g * pr.b_sg, pr.b_st, n0 + (PAIR == 2 ? rank * BNL : 0), pr.N, step0 * KH, tid, pr.vec & 2);
+    float va[DEPTH][UA][8], vb[DEPTH][UB][8];
+    int krem = pr.K - step0 * KH;        // k values left from the next step to request
+#pragma unroll
+    for (int d = 0; d < DEPTH; ++d) {
+      if (d < steps) {
+        oa.fetch(va[d], krem);
+        ob.fetch(vb[d], krem);
+      }
+      krem -= KH;
+    }
+    bool ok = true;
+    auto step = [&](int i, float (&xa)[UA][8], float (&xb)[UB][8]) {
+      const int b = i & 1;
+      if (i >= 2) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&done[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 22));
+        if (!ok) return;
+      }
+      oa.template store<PLANE>(xa, smem, b);
+      ob.template store<PLANE>(xb, smem + A_BYTES, b);
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        // release at CTA scope: the bytes lie in this CTA's shared memory and the proxy fence
+        // has ordered them (cluster scope would wait for the loads in flight as well)
+        if (PAIR == 2) mbar_arrive_cluster<false>(map_to_cta(&full[b], 0));
+        else mbar_arrive(&full[b]);
+      }
+      if (i + DEPTH < steps) {
+        oa.fetch(xa, krem);
+        ob.fetch(xb, krem);
+        krem -= KH;
+      }
+    };
+    for (int i = 0; i < steps && ok; i += DEPTH) {
+#pragma unroll
+      for (int d = 0; d < DEPTH; ++d)
+        if (i + d < steps && ok) step(i + d, va[d], vb[d]);
+    }
+    close(nullptr);
+  } else if (BN == 256 || warp < kLoadWarps + kAddWarps) {
+    // ---------------------------------------------------------------- add up
+    if (BN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    const bool issuer = BN == 256 && warp == kLoadWarps && lane == 0 && rank == 0;
+    constexpr int W = BN == 256 ? 16 : 32;             // columns per tensor-memory load
+    uint64_t acc[NACC / 2];
+#pragma unroll
+    for (int i = 0; i < NACC / 2; ++i) acc[i] = 0;
+    const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(((warp - kLoadWarps) >> 2) * NACC);
+    if (issuer && steps > 0) issue(0);
+    __syncwarp();
+    for (int i = 0; i < steps; ++i) {
+      const int b = i & 1;
+      if (issuer && i + 1 < steps) issue(i + 1);
+      __syncwarp();
+      if (!__all_sync(0xffffffffu, mbar_wait(&done[b], (i >> 1) & 1, abortp, a.status, 20))) break;
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < NACC; c += W) {
+        uint32_t v[W];
+        if (W == 32) tc_ld32(t_row + (uint32_t)(b * BN + c), v);
+        else tc_ld16(t_row + (uint32_t)(b * BN + c), v);
+#pragma unroll
+        for (int e = 0; e < W / 2; ++e) add2(acc[c / 2 + e], v[2 * e], v[2 * e + 1]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR == 2) mbar_arrive_cluster<false>(map_to_cta(&taken[b], 0));
+        else mbar_arrive(&taken[b]);
+      }
+    }
+    close(acc);
+  } else {
+    // ---------------------------------------------------------------- issue the MMAs of a narrow tile
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
+    if (warp == kLoadWarps + kAddWarps && lane == 0)
+      for (int i = 0; i < steps; ++i)
+        if (!issue(i)) break;
+    __syncwarp();
+    close(nullptr);
+  }
+}
+
+// ---- host side ---------------------------------------------------------------------------------
+
+template <int A_MN, int B_MN, int BN, int PAIR>
+bool launch(const Launch& L, const F32Args& t, int cluster) {
+  auto kern = gemm_f32_kernel<A_MN, B_MN, BN, PAIR>;
+  constexpr int smem = (int)smem_bytes<BN, PAIR>();
+  static bool ready = false;
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    ready = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+  });
+  if (!ready) return false;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(t.p[t.n_problems - 1].tile_end * cluster));
+  cfg.blockDim = dim3(threads_of(BN));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = L.stream;
+  cudaLaunchAttribute attrs[2];
+  int n = 0;
+  attrs[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attrs[n++].val.programmaticStreamSerializationAllowed = 1;
+  if (cluster > 1) {
+    attrs[n].id = cudaLaunchAttributeClusterDimension;
+    attrs[n].val.clusterDim.x = (unsigned)cluster;
+    attrs[n].val.clusterDim.y = 1;
+    attrs[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attrs;
+  cfg.numAttrs = n;
+  if (cudaLaunchKernelEx(&cfg, kern, t) != cudaSuccess) return false;
+  L.count();
+  return true;
+}
+
+template <int A_MN, int B_MN>
+bool launch_bn(const Launch& L, const F32Args& t, int bn, int pair, int cluster) {
+  if (pair == 2) return launch<A_MN, B_MN, 256, 2>(L, t, 2);
+  if (bn == 128) return launch<A_MN, B_MN, 128, 1>(L, t, cluster);
+  return launch<A_MN, B_MN, 64, 1>(L, t, cluster);
+}
+
+// Tile shape and k split of a launch, and its estimated time in microseconds: as many rounds of
+// tiles as the SMs need, each a fixed part (start, first operands, epilogue) and so much per
+// 32-deep step.  Constants fitted to 12 products of 64 x 64 x 32 to 512 x 16384 x 3072 (measured
+// 5.3 to 244 us, estimates within 25 %); 64-column tiles pay off only where 128-column ones leave
+// SMs idle or the product is narrow, pairs from about 64 tiles of 256 x 256 on.
+struct Shape { int bn, pair, cluster; double us; };
+Shape pick_shape(const GemmArgs<float>* ga, int n) {
+  const int sms = 148;
+  Shape best{64, 1, 1, 1e300};
+  auto consider = [&](int bn, int pair, int cluster, double step_us, double fix_us) {
+    int64_t tiles = 0, steps = 0;
+    for (int i = 0; i < n; ++i) {
+      tiles += ceil_div(ga[i].M, BM * pair) * ceil_div(ga[i].N, bn) * ga[i].G;
+      steps = std::max<int64_t>(steps, ceil_div(ga[i].K, KH));
+    }
+    if (cluster > 1 && (steps < 2 * cluster || tiles * cluster > sms)) return;
+    const int64_t rounds = ceil_div(tiles * pair, sms);
+    const double us = rounds * (fix_us + step_us * ceil_div(steps, cluster)) + (cluster > 1 ? 0.5 + 0.2 * cluster : 0.0);
+    if (us < best.us) best = Shape{bn, pair, cluster, us};
+  };
+  for (int cl = 1; cl <= 8; cl *= 2) {
+    consider(64, 1, cl, 0.95, 4.0);
+    consider(128, 1, cl, 1.2, 5.0);
+  }
+  consider(256, 2, 1, 1.15, 13.0);
+  return best;
+}
+
+// Whether the CUDA-core kernel for short contractions is the quicker one: always up to 16 k values
+// (half a step here; 256 x 1024 x 16 of four groups 6.1 against 7.6 us), else by its time as
+// measured, 3 us and (1.4 + 0.1 K) us per 1024 tiles of 32 x 32 (64 x 64 x 64 of four groups 3.5
+// against 6.2 us, 512 x 4096 x 64 19 against 12 us).
+bool short_wins(const GemmArgs<float>& a, double us) {
+  if (a.K > 64) return false;
+  const double tiles = (double)ceil_div(a.M, 32) * ceil_div(a.N, 32) * a.G;
+  return a.K <= 16 || 3.0 + (1.4 + 0.1 * a.K) * tiles / 1024 < us;
+}
+
+}  // namespace
+
+bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, DeviceStatus* st) {
+  if (n < 1 || n > kMaxProblems) return false;
+  auto a_is_mn = [](const GemmArgs<float>& a) { return a.a_sm == 1 && a.a_sk != 1; };
+  auto b_is_mn = [](const GemmArgs<float>& a) { return a.b_sn == 1 && a.b_sk != 1; };
+  const bool a_mn = a_is_mn(ga[0]), b_mn = b_is_mn(ga[0]);
+  for (int i = 0; i < n; ++i) {
+    const GemmArgs<float>& a = ga[i];
+    if (a.M < 1 || a.N < 1 || a.K < 1 || a.G < 1 || a.lr != ga[0].lr) return false;
+    if (a_is_mn(a) != a_mn || b_is_mn(a) != b_mn) return false;
+    if ((!a_mn && a.a_sk != 1) || (!b_mn && a.b_sk != 1)) return false;
+  }
+  Shape sh = pick_shape(ga, n);
+  if (n == 1 && short_wins(ga[0], sh.us) && gemm_short(L, ga[0])) return true;
+#ifdef F32_PROBE
+  if (getenv("FBN")) { sh.bn = atoi(getenv("FBN")); sh.pair = sh.bn == 256 ? 2 : 1; sh.cluster = atoi(getenv("FCL")); }
+#endif
+  F32Args t{};
+  t.n_problems = n;
+  t.ksplit = sh.cluster;
+  t.lr = ga[0].lr;
+  t.status = st;
+  int64_t end = 0;
+  for (int i = 0; i < n; ++i) {
+    const GemmArgs<float>& a = ga[i];
+    F32Problem& p = t.p[i];
+    p.M = a.M; p.N = a.N; p.K = a.K; p.G = a.G;
+    const int64_t mt = ceil_div(a.M, BM * sh.pair), nt = ceil_div(a.N, sh.bn);
+    p.m_tiles = (int)mt;
+    p.n_tiles = (int)nt;
+    end += mt * nt * a.G;
+    if (end * 8 > 0x7fffffffll) return false;
+    p.tile_end = (int)end;
+    p.epi = a.epi;
+    p.A = a.A; p.a_st = a_mn ? a.a_sk : a.a_sm; p.a_sg = a.a_sg;
+    p.B = a.B; p.b_st = b_mn ? a.b_sk : a.b_sn; p.b_sg = a.b_sg;
+    const bool f32_out = a.epi == EPI_SGD || a.epi == EPI_BIAS_F32;
+    p.bias = (a.epi == EPI_BIAS_RELU || a.epi == EPI_BIAS_F32) ? a.bias : nullptr; p.bias_sg = a.bias_sg;
+    p.out = f32_out ? a.outf : a.out;
+    p.out_ld = f32_out ? a.outf_ld : a.out_ld;
+    p.out_sg = f32_out ? a.outf_sg : a.out_sg;
+    p.mask = a.mask; p.mask_ld = a.mask_ld; p.mask_sg = a.mask_sg;
+    auto vec = [](const void* q, int64_t ld, int64_t sg) { return ((uintptr_t)q & 15) == 0 && ld % 4 == 0 && sg % 4 == 0; };
+    if (vec(p.A, p.a_st, p.a_sg)) p.vec |= 1;
+    if (vec(p.B, p.b_st, p.b_sg)) p.vec |= 2;
+    if (vec(p.out, p.out_ld, p.out_sg) && (!p.bias || vec(p.bias, 0, p.bias_sg)) &&
+        (a.epi != EPI_RELU_MASK || vec(p.mask, p.mask_ld, p.mask_sg)))
+      p.vec |= 4;
+  }
+  if (a_mn && b_mn) return launch_bn<1, 1>(L, t, sh.bn, sh.pair, sh.cluster);
+  if (!a_mn && b_mn) return launch_bn<0, 1>(L, t, sh.bn, sh.pair, sh.cluster);
+  if (!a_mn) return launch_bn<0, 0>(L, t, sh.bn, sh.pair, sh.cluster);
+  return false;
+}
+
+}  // namespace ist

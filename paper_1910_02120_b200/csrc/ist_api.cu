@@ -365,21 +365,19 @@ ist_status check_input(ist_ctx* c, const ist_input* X, const int32_t* y, bool tr
 }
 
 // ---- grouped GEMM dispatch ------------------------------------------------------------------
-// fp32 operands run on the CUDA cores, bf16 operands on the tensor cores.
-bool gemm(ist_ctx* c, const GemmArgs<float>& a) {
-  gemm_simt<float>(c->launch(), a);
-  return true;
-}
+// fp32 operands are split into bf16 parts inside the kernel (or, short contractions, multiplied on the
+// CUDA cores), bf16 operands go to the tensor cores as they are.
+bool gemm(ist_ctx* c, const GemmArgs<float>& a) { return gemm_f32(c->launch(), &a, 1, c->status()); }
 bool gemm(ist_ctx* c, const GemmArgs<bf16>& a) { return gemm_tc(c->launch(), a, c->status()); }
 
-// Several products of one kind in as few launches as possible.  fp32 operands: one CUDA-core
-// launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
+// Several products of one kind in as few launches as possible.  fp32 operands: one launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
 // with `chained`, every problem reads the output of the one before it and the launch orders
 // their tiles through the row-block counters of `region` (one set per problem, indexed by
 // `layer0 + i`; `totals` are the context's running sums for that region).
 bool gemm_list(ist_ctx* c, const std::vector<GemmArgs<float>>& v, bool, Region, std::vector<unsigned>*, int,
                const LossReduce* = nullptr) {
-  for (auto& g : v) gemm_simt<float>(c->launch(), g);
+  for (auto& g : v)
+    if (!gemm(c, g)) return false;
   return true;
 }
 // Whether every launch a weight-update list is cut into can sum the deltas for the bias update.
@@ -1000,6 +998,7 @@ namespace {
 // normalisation mode, the stored statistics (measure = false) or statistics taken over these
 // very rows, which are then stored (measure = true).  Returns the buffer holding layer
 // `last`'s output (row stride N_last).
+// Null: a product cannot be launched.
 const float* full_forward(ist_ctx* c, const ist_input* X, int64_t r0, int rows, int last, bool measure) {
   Launch L = c->launch();
   float* buf[2] = {c->plan.ev_a.at<float>(c->ws), c->plan.ev_b.at<float>(c->ws)};
@@ -1022,7 +1021,7 @@ const float* full_forward(ist_ctx* c, const ist_input* X, int64_t r0, int rows, 
       g.bias = c->b[l - 1];
       if (hidden && !c->norm) { g.epi = EPI_BIAS_RELU; g.out = o; g.out_ld = c->N[l]; }
       else { g.epi = EPI_BIAS_F32; g.outf = o; g.outf_ld = c->N[l]; }
-      gemm_simt<float>(L, g);
+      if (!gemm(c, g)) return nullptr;
     }
     if (hidden && c->norm) {
       if (measure)
@@ -1059,6 +1058,7 @@ extern "C" ist_status ist_eval(ist_ctx* c, const ist_input* X, const int32_t* y_
   for (int64_t r0 = 0; r0 < n; r0 += c->max_batch) {
     const int rows = (int)std::min<int64_t>(c->max_batch, n - r0);
     const float* logits = full_forward(c, X, r0, rows, c->t, false);
+    if (!logits) return fail(c, IST_ERR_UNSUPPORTED, "evaluation GEMMs cannot be launched");
     eval_rows(L, logits, c->N[c->t], rows, (int)c->N[c->t], y_dev + r0, loss_sum, correct, c->status());
   }
   eval_finalize(L, loss_sum, correct, n, mean_loss_out_dev, n_correct_out_dev);
@@ -1100,7 +1100,8 @@ extern "C" ist_status ist_calibrate(ist_ctx* c, const ist_input* X, int64_t n) {
   if (X->kind == IST_X_DENSE_BF16) return fail(c, IST_ERR_UNSUPPORTED, "ist_calibrate takes fp32 or CSR rows");
   {
     Scope sc(c, IST_K_EVAL);
-    full_forward(c, X, 0, (int)n, c->t - 1, true);
+    if (c->t > 1 && !full_forward(c, X, 0, (int)n, c->t - 1, true))
+      return fail(c, IST_ERR_UNSUPPORTED, "calibration GEMMs cannot be launched");
   }
   IST_CUDA(c, cudaGetLastError());
   c->calibrated = true;

@@ -110,7 +110,10 @@ struct GemmArgs {
   float* label_logit;
   float inv_rows;
 };
-template <typename T> void gemm_simt(const Launch& L, const GemmArgs<T>& a);
+// fp32 operands: on the tensor cores, one to four products with the same operand layouts as tiles of
+// one launch, or on the CUDA cores for short contractions (K <= 64).  false: the shape is not taken.
+bool gemm_f32(const Launch& L, const GemmArgs<float>* a, int n, DeviceStatus* st);
+bool gemm_short(const Launch& L, const GemmArgs<float>& a);
 // Tensor-core path (tcgen05 + TMA) for bf16 operands.  Returns false if the shape cannot be
 // described to TMA (misaligned strides) or the operand layouts do not fit an epilogue.
 bool gemm_tc(const Launch& L, const GemmArgs<bf16>& a, DeviceStatus* st);
