@@ -361,6 +361,98 @@ __global__ void eval_rows_kernel(const float* __restrict__ logits, int64_t ld, i
   }
 }
 
+// The same for rows of many classes: a cluster of CTAs per row, each with a range of the columns, one
+// pass with a running (max, sum) pair and 16-byte loads, four of them in flight per thread; the
+// ranges are merged in rank order through distributed shared memory.  Two passes of 4-byte loads by
+// one block per row held too few bytes in flight for the 2.7 MB rows of 670,091 classes (256 rows:
+// 2.46 ms; now 0.21 ms).
+constexpr int kEvalThreads = 512, kEvalCols = 65536;   // columns of a CTA, at most
+struct EvalPart { float m, s; int arg; };
+// Folds b into a; ties go to the lower index.  An empty part carries (-inf, 0).
+__device__ __forceinline__ void eval_fold(EvalPart& a, const EvalPart& b) {
+  const float m = fmaxf(a.m, b.m), ref = m == -INFINITY ? 0.f : m;
+  a.s = a.s * expf(a.m - ref) + b.s * expf(b.m - ref);
+  if (b.m > a.m || (b.m == a.m && b.arg < a.arg)) a.arg = b.arg;
+  a.m = m;
+}
+__global__ void __launch_bounds__(kEvalThreads) eval_rows_wide_kernel(const float* __restrict__ logits, int64_t ld, int Nt,
+                                                                      const int32_t* __restrict__ y, double* loss_sum,
+                                                                      long long* correct, DeviceStatus* st) {
+  __shared__ EvalPart sh[kEvalThreads / 32];
+  pdl_wait();
+  pdl_trigger();
+  const int row = blockIdx.y, rank = blockIdx.x, ranks = gridDim.x, tid = threadIdx.x;
+  const float* z = logits + (int64_t)row * ld;
+  const int per = (int)(((int64_t)Nt + ranks - 1) / ranks);
+  const int c0 = min(rank * per, Nt), c1 = min(c0 + per, Nt);
+  EvalPart p{-INFINITY, 0.f, 0x7fffffff};
+  auto take = [&](const float* v, const int* at, int cnt) {
+    float m = p.m;
+#pragma unroll
+    for (int i = 0; i < cnt; ++i)
+      if (v[i] > m) { m = v[i]; p.arg = at[i]; }
+    const float ref = m == -INFINITY ? 0.f : m;
+    if (m > p.m) p.s *= expf(p.m - ref);
+    p.m = m;
+#pragma unroll
+    for (int i = 0; i < cnt; ++i) p.s += expf(v[i] - ref);
+  };
+  // columns before the first 16-byte boundary and behind the last one by themselves
+  const int head = min((int)((4 - ((reinterpret_cast<uintptr_t>(z + c0) >> 2) & 3)) & 3), c1 - c0);
+  const int quads = (c1 - c0 - head) / 4;
+  if (tid < head) { const int n = c0 + tid; take(z + n, &n, 1); }
+  const float4* zq = reinterpret_cast<const float4*>(z + c0 + head);
+  for (int q0 = tid; q0 < quads; q0 += 4 * kEvalThreads) {
+    float v[16];
+    int at[16];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = q0 + u * kEvalThreads;
+      const float4 t = q < quads ? __ldg(zq + q) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      v[4 * u] = t.x; v[4 * u + 1] = t.y; v[4 * u + 2] = t.z; v[4 * u + 3] = t.w;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) at[4 * u + i] = c0 + head + 4 * q + i;
+    }
+    take(v, at, 16);
+  }
+  const int tail = c0 + head + 4 * quads + tid;
+  if (tail < c1) take(z + tail, &tail, 1);
+  for (int o = 16; o; o >>= 1) {
+    EvalPart q{__shfl_xor_sync(0xffffffffu, p.m, o), __shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.arg, o)};
+    eval_fold(p, q);
+  }
+  if ((tid & 31) == 0) sh[tid >> 5] = p;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < kEvalThreads / 32; ++w) eval_fold(p, sh[w]);
+    sh[0] = p;
+  }
+  if (ranks > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  if (rank == 0 && tid == 0) {
+    for (int r = 1; r < ranks; ++r) {
+      uint32_t addr, w[3];
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"((uint32_t)__cvta_generic_to_shared(&sh[0])), "r"(r));
+#pragma unroll
+      for (int i = 0; i < 3; ++i) asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(w[i]) : "r"(addr + 4 * i) : "memory");
+      eval_fold(p, EvalPart{__uint_as_float(w[0]), __uint_as_float(w[1]), (int)w[2]});
+    }
+    int label = y[row];
+    if (label < 0 || label >= Nt) {
+      report(st, -5, SITE_LABEL, row);
+      label = 0;
+    }
+    atomicAdd(loss_sum, (double)(logf(p.s) + p.m - z[label]));
+    if (p.arg == label) atomicAdd((unsigned long long*)correct, 1ull);
+  }
+  if (ranks > 1) {                                     // rank 0 has read the others' shared memory
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
 __global__ void eval_finalize_kernel(const double* loss_sum, const long long* correct, int64_t n,
                                      float* mean_loss_out, int64_t* correct_out) {
   *mean_loss_out = (float)(*loss_sum / (double)n);
@@ -476,8 +568,27 @@ template void stage_rows<bf16>(const Launch&, const float*, int64_t, int64_t, in
 
 void eval_rows(const Launch& L, const float* logits, int64_t ld, int rows, int Nt, const int32_t* y,
                double* loss_sum, long long* correct, DeviceStatus* st) {
-  eval_rows_kernel<<<rows, row_threads(Nt), 0, L.stream>>>(logits, ld, rows, Nt, y, loss_sum, correct,
-                                                           st);
+  // From 4096 columns on a block's threads have a handful of 16-byte loads each.  As many CTAs per
+  // row as keep the SMs supplied with two blocks each, at most the eight of a portable cluster.
+  if (Nt >= 4096 && rows <= 65535) {
+    int ranks = 1;
+    while (ranks < 8 && ((int64_t)Nt / ranks > kEvalCols || ((int64_t)rows * ranks < 296 && Nt / ranks >= 8192))) ranks *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ranks, (unsigned)rows);
+    cfg.blockDim = dim3(kEvalThreads);
+    cfg.stream = L.stream;
+    cudaLaunchAttribute attrs[2];
+    attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[0].val.programmaticStreamSerializationAllowed = 1;
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = (unsigned)ranks;
+    attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
+    cfg.attrs = attrs;
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, eval_rows_wide_kernel, logits, ld, Nt, y, loss_sum, correct, st);
+  } else {
+    eval_rows_kernel<<<rows, row_threads(Nt), 0, L.stream>>>(logits, ld, rows, Nt, y, loss_sum, correct, st);
+  }
   L.count();
 }
 
