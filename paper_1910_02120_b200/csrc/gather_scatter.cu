@@ -14,57 +14,64 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kRowsPerCta = 8;
 
-// Packed element (s, i, j), j = blockIdx.x*256 + tid, i in a block of kRowsPerCta rows.
+// Several matrices and bias rows as blocks of one launch: block -> (job, subnet, 8 rows, 256 columns).
+// A network of a few layers took two launches per layer in either direction, most of them shorter
+// than the gap between them (64-512-512-10, S = 4: 38 us to gather, 37 us to scatter; now 8.5 us each).
+constexpr int kMaxJobs = 8;
+struct SliceJobs {
+  int n;
+  SliceJob job[kMaxJobs];
+  int x_blocks[kMaxJobs], y_blocks[kMaxJobs];
+  int end[kMaxJobs];                 // blocks end(previous) .. end - 1 are the job's
+};
+
+// Packed element (s, i, j), j = column block * 256 + tid, i in a block of kRowsPerCta rows.
 // Pad rows / columns (beyond the group's true size) are written as zeros so that padded
 // neurons stay inert through the local steps.
-__global__ void gather_kernel(const float* __restrict__ W, SliceMap m, float* __restrict__ master,
-                              bf16* __restrict__ opw) {
-  int s = m.s_first + blockIdx.z;
-  int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (j >= m.ld) return;
-  int64_t ncols = m.col_idx ? (m.col_off[s + 1] - m.col_off[s]) : m.full_cols;
-  int64_t nrows = m.row_idx ? (m.row_off[s + 1] - m.row_off[s]) : m.full_rows;
+template <bool GATHER>
+__global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ SliceJobs a) {
+  pdl_wait();
+  pdl_trigger();
+  int ji = 0, blk = blockIdx.x;
+  while (blk >= a.end[ji]) ++ji;
+  const SliceJob& J = a.job[ji];
+  const SliceMap& m = J.m;
+  blk -= ji ? a.end[ji - 1] : 0;
+  const int64_t j = (int64_t)(blk % a.x_blocks[ji]) * kThreads + threadIdx.x;
+  blk /= a.x_blocks[ji];
+  const int yb = blk % a.y_blocks[ji], s = m.s_first + blk / a.y_blocks[ji];
+  if (!GATHER && J.mean) {
+    if (j >= m.full_cols) return;
+    const float old = J.W[j];
+    float acc = 0.f;
+    for (int g = 0; g < J.S; ++g) acc += J.master[(int64_t)g * m.ld + j] - old;
+    J.W[j] = old + acc / (float)J.S;
+    return;
+  }
+  const int64_t ncols = m.col_idx ? (m.col_off[s + 1] - m.col_off[s]) : m.full_cols;
+  const int64_t nrows = m.row_idx ? (m.row_off[s + 1] - m.row_off[s]) : m.full_rows;
+  if (j >= (GATHER ? m.ld : ncols)) return;
   int64_t c = -1;
   if (j < ncols) c = m.col_idx ? m.col_idx[m.col_off[s] + j] : j;
-  // row blocks blockIdx.y, blockIdx.y + gridDim.y, ... (the y dimension of a grid stops at 65535)
-  for (int64_t i0 = (int64_t)blockIdx.y * kRowsPerCta; i0 < m.rows_pad; i0 += (int64_t)gridDim.y * kRowsPerCta) {
-    float v[kRowsPerCta];
+  const int64_t i0 = (int64_t)yb * kRowsPerCta;
+  float v[kRowsPerCta];
+  int64_t r[kRowsPerCta];
 #pragma unroll
-    for (int u = 0; u < kRowsPerCta; ++u) {
-      int64_t i = i0 + u;
-      v[u] = 0.f;
-      if (c >= 0 && i < nrows) {
-        int64_t r = m.row_idx ? m.row_idx[m.row_off[s] + i] : i;
-        v[u] = __ldg(W + r * m.full_cols + c);
-      }
-    }
+  for (int u = 0; u < kRowsPerCta; ++u)
+    r[u] = (c >= 0 && i0 + u < nrows) ? (m.row_idx ? m.row_idx[m.row_off[s] + i0 + u] : i0 + u) * m.full_cols + c : -1;
+  const int64_t o0 = ((int64_t)s * m.rows_pad + i0) * m.ld + j;
 #pragma unroll
-    for (int u = 0; u < kRowsPerCta; ++u) {
-      int64_t i = i0 + u;
-      if (i < m.rows_pad) {
-        int64_t o = ((int64_t)s * m.rows_pad + i) * m.ld + j;
-        master[o] = v[u];
-        if (opw) opw[o] = __float2bfloat16_rn(v[u]);
-      }
-    }
-  }
-}
-
-__global__ void scatter_kernel(float* __restrict__ W, SliceMap m, const float* __restrict__ master) {
-  int s = m.s_first + blockIdx.z;
-  int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  int64_t ncols = m.col_idx ? (m.col_off[s + 1] - m.col_off[s]) : m.full_cols;
-  int64_t nrows = m.row_idx ? (m.row_off[s + 1] - m.row_off[s]) : m.full_rows;
-  if (j >= ncols) return;
-  int64_t c = m.col_idx ? m.col_idx[m.col_off[s] + j] : j;
-  for (int64_t i0 = (int64_t)blockIdx.y * kRowsPerCta; i0 < nrows; i0 += (int64_t)gridDim.y * kRowsPerCta) {
+  for (int u = 0; u < kRowsPerCta; ++u)
+    v[u] = r[u] >= 0 ? (GATHER ? __ldg(J.W + r[u]) : J.master[o0 + u * m.ld]) : 0.f;
 #pragma unroll
-    for (int u = 0; u < kRowsPerCta; ++u) {
-      int64_t i = i0 + u;
-      if (i < nrows) {
-        int64_t r = m.row_idx ? m.row_idx[m.row_off[s] + i] : i;
-        W[r * m.full_cols + c] = master[((int64_t)s * m.rows_pad + i) * m.ld + j];
+  for (int u = 0; u < kRowsPerCta; ++u) {
+    if (GATHER) {
+      if (i0 + u < m.rows_pad) {
+        J.master[o0 + u * m.ld] = v[u];
+        if (J.opw) J.opw[o0 + u * m.ld] = __float2bfloat16_rn(v[u]);
       }
+    } else if (r[u] >= 0) {
+      J.W[r[u]] = v[u];
     }
   }
 }
@@ -79,6 +86,8 @@ constexpr int kRowU = 4, kColU = 4;
 template <bool GATHER>
 __global__ void __launch_bounds__(kThreads) rows_kernel(float* __restrict__ W, SliceMap m, float* __restrict__ master,
                                                          bf16* __restrict__ opw) {
+  pdl_wait();
+  pdl_trigger();
   const int s = m.s_first + blockIdx.z;
   const int nrows = m.row_off[s + 1] - m.row_off[s];
   const int32_t* rows = m.row_idx + m.row_off[s];
@@ -131,7 +140,7 @@ bool rows_ok(const SliceMap& m) { return m.row_idx && !m.col_idx && m.full_cols 
 template <bool GATHER>
 void launch_rows(const Launch& L, float* W, const SliceMap& m, int S, float* master, bf16* opw) {
   dim3 grid((unsigned)ceil_div(m.ld, kThreads * kColU), (unsigned)std::min<int64_t>(ceil_div(m.rows_pad, kRowU), 65535), S);
-  rows_kernel<GATHER><<<grid, kThreads, 0, L.stream>>>(W, m, master, opw);
+  launch_pdl(rows_kernel<GATHER>, grid, dim3(kThreads), 0, L.stream, W, m, master, opw);
   L.count();
 }
 
@@ -232,6 +241,8 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* __
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  pdl_wait();
+  pdl_trigger();
   find_runs(m, S, c0, c1, &runs);      // contains the barriers that publish the mbarrier init
   const int total = runs.pre[S];
   for (int e = threadIdx.x; e < total; e += kPermThreads) {
@@ -345,19 +356,10 @@ bool launch_permute_cols(const Launch& L, float* W, const SliceMap& m, int S, fl
   if (y > blocks) y = blocks;
   if (y > 65535) y = 65535;
   dim3 grid((unsigned)chunks, (unsigned)y);
-  permute_cols_kernel<GATHER><<<grid, kPermThreads, smem, L.stream>>>(W, m, S, master, opw, st);
+  if (launch_pdl(permute_cols_kernel<GATHER>, grid, dim3(kPermThreads), smem, L.stream, W, m, S, master, opw, st) != cudaSuccess)
+    return false;
   L.count();
   return true;
-}
-
-__global__ void mean_bias_kernel(float* b, int64_t n, int S, const float* __restrict__ packed,
-                                 int64_t ld) {
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  float old = b[j];
-  float acc = 0.f;
-  for (int s = 0; s < S; ++s) acc += packed[(int64_t)s * ld + j] - old;
-  b[j] = old + acc / (float)S;
 }
 
 __global__ void copy_out_kernel(const float* __restrict__ packed, int64_t ld, int64_t rows,
@@ -370,28 +372,52 @@ __global__ void copy_out_kernel(const float* __restrict__ packed, int64_t ld, in
 
 }  // namespace
 
-void gather_slices(const Launch& L, const float* W, const SliceMap& m, int S, float* master,
-                   bf16* opw, DeviceStatus* st) {
-  if (staged_ok(m, S) && launch_permute_cols<true>(L, const_cast<float*>(W), m, S, master, opw, st)) return;
-  if (rows_ok(m)) return launch_rows<true>(L, const_cast<float*>(W), m, S, master, opw);
-  dim3 grid((unsigned)ceil_div(m.ld, kThreads), (unsigned)std::min<int64_t>(ceil_div(m.rows_pad, kRowsPerCta), 65535), S);
-  gather_kernel<<<grid, kThreads, 0, L.stream>>>(W, m, master, opw);
-  L.count();
+namespace {
+
+// Matrices of this many packed elements or more are moved by the kernel made for their kind (first
+// layer: column permutation, last layer: whole rows); smaller ones by blocks of the shared launch,
+// whose scattered 4-byte accesses L2 still absorbs.  Partition + reassembly of 1024-4096-4096-35,
+// S = 4 (4.2 M elements a layer): 98 us with a launch of its own for the first layer, 86 us without;
+// of 3072-16384-16384-10, S = 8 (50 M): 740 against 1180 us.
+constexpr int64_t kOwnLaunch = 1 << 24;
+
+template <bool GATHER>
+void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
+  SliceJobs a{};
+  int64_t blocks = 0;
+  auto flush = [&] {
+    if (a.n) {
+      launch_pdl(move_kernel<GATHER>, dim3((unsigned)blocks), dim3(kThreads), 0, L.stream, a);
+      L.count();
+    }
+    a.n = 0;
+    blocks = 0;
+  };
+  for (int i = 0; i < n; ++i) {
+    const SliceJob& j = jobs[i];
+    if (!j.mean && j.S * j.m.rows_pad * j.m.ld >= kOwnLaunch) {
+      if (staged_ok(j.m, j.S) && launch_permute_cols<GATHER>(L, j.W, j.m, j.S, j.master, j.opw, st)) continue;
+      if (rows_ok(j.m)) {
+        launch_rows<GATHER>(L, j.W, j.m, j.S, j.master, j.opw);
+        continue;
+      }
+    }
+    const int64_t x = ceil_div(j.mean ? j.m.full_cols : j.m.ld, kThreads), y = j.mean ? 1 : ceil_div(j.m.rows_pad, kRowsPerCta);
+    const int64_t b = x * y * (j.mean ? 1 : j.S);
+    if (a.n == kMaxJobs || blocks + b > 0x7fffffffll) flush();
+    a.job[a.n] = j;
+    a.x_blocks[a.n] = (int)x;
+    a.y_blocks[a.n] = (int)y;
+    blocks += b;
+    a.end[a.n++] = (int)blocks;
+  }
+  flush();
 }
 
-void scatter_slices(const Launch& L, float* W, const SliceMap& m, int S, const float* master,
-                    DeviceStatus* st) {
-  if (staged_ok(m, S) && launch_permute_cols<false>(L, W, m, S, const_cast<float*>(master), nullptr, st)) return;
-  if (rows_ok(m)) return launch_rows<false>(L, W, m, S, const_cast<float*>(master), nullptr);
-  dim3 grid((unsigned)ceil_div(m.ld, kThreads), (unsigned)std::min<int64_t>(ceil_div(m.rows_pad, kRowsPerCta), 65535), S);
-  scatter_kernel<<<grid, kThreads, 0, L.stream>>>(W, m, master);
-  L.count();
-}
+}  // namespace
 
-void scatter_mean_bias(const Launch& L, float* b, int64_t n, int S, const float* packed, int64_t ld) {
-  mean_bias_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, L.stream>>>(b, n, S, packed, ld);
-  L.count();
-}
+void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) { move_all<true>(L, jobs, n, st); }
+void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) { move_all<false>(L, jobs, n, st); }
 
 void copy_out_slice(const Launch& L, const float* packed, int64_t ld, int64_t rows, int64_t cols,
                     float* out) {

@@ -205,10 +205,11 @@ void make_plan(ist_ctx* c) {
   p.master.resize(t + 1); p.bias.resize(t + 1); p.opw.resize(t + 1);
   p.act.resize(t + 1); p.delta.resize(t + 1);
   p.status = p.take(sizeof(DeviceStatus));
-  int64_t maxH = 1, maxN = 0;
-  for (int l = 1; l < t; ++l) maxH = std::max(maxH, c->N[l]);
+  int64_t maxN = 0;
   for (int l = 0; l <= t; ++l) maxN = std::max(maxN, c->N[l]);
-  p.part = p.take(partition_scratch_bytes((int)maxH, S));
+  size_t part_bytes = 0;               // the layers of a draw are partitioned side by side
+  for (int l = 1; l < t; ++l) part_bytes += partition_scratch_bytes((int)c->N[l], S);
+  p.part = p.take(part_bytes);
   for (int l = 1; l < t; ++l) {
     p.idx[l] = p.take(c->N[l] * 4);
     p.off[l] = p.take((S + 1) * 4);
@@ -852,21 +853,30 @@ extern "C" ist_status ist_partition(ist_ctx* c, uint64_t seed) {
                       (unsigned long long)seed, (long long)c->group_count[l][s], l, s, (long long)c->np[l]);
     }
   }
-  for (int l = 1; l < t; ++l) {
+  if (t > 1) {
     Scope sc(c, IST_K_PARTITION);
-    uint64_t layer_seed = splitmix64_next(&round_state);
-    PartitionScratch ps{};
-    partition_scratch_carve(c->plan.part.at<char>(c->ws), (int)c->N[l], S, &ps);
-    const bool ok = c->rule == IST_PART_IID
-                        ? partition_layer_iid(L, layer_seed, (int)c->N[l], S, ps, c->idx(l), c->off(l), c->status())
-                        : partition_layer(L, layer_seed, (int)c->N[l], S, ps, c->idx(l), c->off(l), c->status());
-    if (!ok) return fail(c, IST_ERR_UNSUPPORTED, "S = %d exceeds what the partition kernels support (768)", S);
+    std::vector<PartitionJob> jobs(t - 1);
+    char* scratch = c->plan.part.at<char>(c->ws);
+    for (int l = 1; l < t; ++l) {
+      PartitionJob& j = jobs[l - 1];
+      j.seed = splitmix64_next(&round_state);
+      j.N = (int)c->N[l];
+      scratch += partition_scratch_carve(scratch, j.N, S, &j.sc);
+      j.idx = c->idx(l);
+      j.off = c->off(l);
+    }
+    if (!partition_layers(L, jobs.data(), t - 1, S, c->rule == IST_PART_IID, c->status()))
+      return fail(c, IST_ERR_UNSUPPORTED, "S = %d exceeds what the partition kernels support (768)", S);
   }
-  // only the subnets this context trains are gathered (Sec. 2.3: a site receives its own slices)
-  for (int l = 1; l <= t; ++l) {
+  {
+    // only the subnets this context trains are gathered (Sec. 2.3: a site receives its own slices)
     Scope sc(c, IST_K_GATHER);
-    gather_slices(L, c->W[l - 1], slice_map(c, l, c->sub_first), c->sub_count, c->master(l), c->opw(l), c->status());
-    gather_slices(L, c->b[l - 1], bias_map(c, l, c->sub_first), c->sub_count, c->bias(l), nullptr, c->status());
+    std::vector<SliceJob> jobs;
+    for (int l = 1; l <= t; ++l) {
+      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), c->opw(l), slice_map(c, l, c->sub_first), c->sub_count, 0});
+      jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l, c->sub_first), c->sub_count, 0});
+    }
+    gather_slices(L, jobs.data(), (int)jobs.size(), c->status());
   }
   IST_CUDA(c, cudaGetLastError());
   c->state = ST_PARTITIONED;
@@ -977,14 +987,14 @@ extern "C" ist_status ist_reassemble(ist_ctx* c) {
   if (c->state != ST_PARTITIONED) return fail(c, IST_ERR_STATE, "ist_reassemble needs a partition in place");
   Launch L = c->launch();
   const int t = c->t, S = c->S;
-  for (int l = 1; l <= t; ++l) {
-    Scope sc(c, IST_K_SCATTER);
-    scatter_slices(L, c->W[l - 1], slice_map(c, l), S, c->master(l), c->status());
-    if (l < t) scatter_slices(L, c->b[l - 1], bias_map(c, l), S, c->bias(l), c->status());
-  }
   {
     Scope sc(c, IST_K_SCATTER);
-    scatter_mean_bias(L, c->b[t - 1], c->N[t], S, c->bias(t), c->ld[t]);
+    std::vector<SliceJob> jobs;
+    for (int l = 1; l <= t; ++l) {
+      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), nullptr, slice_map(c, l), S, 0});
+      jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l), S, l == t ? 1 : 0});
+    }
+    scatter_slices(L, jobs.data(), (int)jobs.size(), c->status());
   }
   IST_CUDA(c, cudaGetLastError());
   c->state = ST_BOUND;

@@ -91,8 +91,8 @@ extern "C" ist_status ist_partition_layer_static(uint64_t seed, int hidden_layer
   for (int l = 1; l <= hidden_layer; ++l) layer_seed = splitmix64_next(&state);
 
   Launch L{stream, nullptr};
-  if (!partition_layer(L, layer_seed, N, S, sc, idx_out_dev, off_out_dev, reinterpret_cast<DeviceStatus*>(base)))
-    return IST_ERR_UNSUPPORTED;
+  const PartitionJob job{layer_seed, N, sc, idx_out_dev, off_out_dev};
+  if (!partition_layers(L, &job, 1, S, false, reinterpret_cast<DeviceStatus*>(base))) return IST_ERR_UNSUPPORTED;
   return cudaGetLastError() == cudaSuccess ? IST_OK : IST_ERR_CUDA;
 }
 

@@ -35,6 +35,16 @@ bool partition_layer(const Launch& L, uint64_t layer_seed, int N, int S, const P
 // Independent uniform assignment: group_i = floor(key_i * S / 2^64); same outputs.
 bool partition_layer_iid(const Launch& L, uint64_t layer_seed, int N, int S, const PartitionScratch& sc, int32_t* idx,
                          int32_t* off, DeviceStatus* st);
+// All hidden layers of a draw (small ones together in one launch).  The jobs' scratch must not overlap.
+constexpr int kMaxPartitionJobs = 8;
+struct PartitionJob {
+  uint64_t seed;
+  int N;
+  PartitionScratch sc;
+  int32_t* idx;   // [N]
+  int32_t* off;   // [S + 1]
+};
+bool partition_layers(const Launch& L, const PartitionJob* jobs, int n, int S, bool iid, DeviceStatus* st);
 void partition_iid_counts_host(uint64_t layer_seed, int N, int S, int64_t* counts);
 
 // ---- gather_scatter.cu ------------------------------------------------------------------
@@ -49,14 +59,18 @@ struct SliceMap {
   int64_t rows_pad, ld;          // packed slice: [S][rows_pad][ld]
   int s_first;                   // first subnet a launch covers (it covers S consecutive ones)
 };
-// S = number of subnets moved, starting at m.s_first; master / opw point at subnet 0's slab.
-void gather_slices(const Launch& L, const float* W, const SliceMap& m, int S, float* master,
-                   bf16* opw, DeviceStatus* st);
-void scatter_slices(const Launch& L, float* W, const SliceMap& m, int S, const float* master,
-                    DeviceStatus* st);
-// b[j] += (sum_s (packed[s][j] - b[j])) / S for the output bias.
-void scatter_mean_bias(const Launch& L, float* b, int64_t n, int S, const float* packed,
-                       int64_t ld);
+// One matrix (or bias row) to move.  S = number of subnets, starting at m.s_first; master / opw (may be
+// null) point at subnet 0's slab.
+struct SliceJob {
+  float* W;
+  float* master;
+  bf16* opw;
+  SliceMap m;
+  int S;
+  int mean;      // scatter only: the output bias, b[j] += (sum_s (packed[s][j] - b[j])) / S
+};
+void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
+void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
 // Dense copy-out of a packed slice (ist_get_subnet_params).
 void copy_out_slice(const Launch& L, const float* packed, int64_t ld, int64_t rows, int64_t cols,
                     float* out);
