@@ -173,7 +173,6 @@ bool valid_shape(const int64_t* dims, int n_dims, int S, int precision, int max_
 
 // A narrow output layer (bf16 operands, at most 64 padded classes) is handled specially: its
 // logits GEMM is cut into k slices (more tiles, shorter pipelines) that the softmax kernel sums.
-constexpr int kHeadSplitsMax = 8;
 bool narrow_head(const ist_ctx* c) { return c->precision == IST_BF16 && c->t >= 2 && c->ld[c->t] <= 64; }
 int head_splits(const ist_ctx* c) {
   const int64_t nkb = ceil_div(c->np[c->t - 1], 64);

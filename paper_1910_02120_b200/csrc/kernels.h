@@ -167,6 +167,7 @@ void softmax_xent(const Launch& L, const float* logits, int64_t ld, int64_t sg, 
 template <typename T>
 void splitk_mask_reduce(const Launch& L, const float* part, int ks, int G, int B, int64_t ld, const T* mask,
                         int64_t mask_sg, T* out, int64_t out_sg);
+constexpr int kHeadSplitsMax = 8;   // k slices of a narrow output layer's logits, at most
 // Narrow output layer (Nt <= 64): softmax cross-entropy of logits given as ks partial slabs
 // ([G * ks][B][ld] fp32) plus bias; same outputs as softmax_xent.
 template <typename T>

@@ -71,6 +71,50 @@ __global__ void softmax_xent_kernel(const float* __restrict__ logits, int64_t ld
   if (threadIdx.x == 0) row_loss[(int64_t)g * B + b] = logf(se) + mx - z[label];
 }
 
+// Up to 32 V classes: one warp per row, eight rows per block, the row in registers.  The kernel above
+// reads a row three times and crosses eight block barriers, all latency at these sizes (a local step of
+// 256 rows of four subnets, 35 classes: 2 us less).
+template <typename T, int V>
+__global__ void __launch_bounds__(256) softmax_xent_warp_kernel(const float* __restrict__ logits, int64_t ld, int64_t sg, int B,
+                                                                int Nt, const int32_t* __restrict__ y, int64_t y_sg,
+                                                                T* __restrict__ delta, int64_t ld_d, int64_t sg_d,
+                                                                float* __restrict__ row_loss, DeviceStatus* st) {
+  pdl_wait();
+  pdl_trigger();
+  const int g = blockIdx.y, lane = threadIdx.x & 31, b = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (b >= B) return;
+  const float* zr = logits + (int64_t)g * sg + (int64_t)b * ld;
+  int label = y[(int64_t)g * y_sg + b];
+  float z[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) z[v] = lane + 32 * v < Nt ? zr[lane + 32 * v] : -INFINITY;
+  if (label < 0 || label >= Nt) {
+    if (lane == 0) report(st, -5, SITE_LABEL, (long long)g * B + b);
+    label = 0;
+  }
+  float mx = z[0];
+#pragma unroll
+  for (int v = 1; v < V; ++v) mx = fmaxf(mx, z[v]);
+  mx = warp_max(mx);
+  float se = 0.f, zl = 0.f;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    if (lane + 32 * v == label) zl = z[v];
+    z[v] = lane + 32 * v < Nt ? expf(z[v] - mx) : 0.f;
+    se += z[v];
+  }
+  se = warp_sum(se);
+  zl = __shfl_sync(0xffffffffu, zl, label & 31);
+  const float inv = 1.f / se, invB = 1.f / (float)B;
+  T* d = delta + (int64_t)g * sg_d + (int64_t)b * ld_d;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int n = lane + 32 * v;
+    if (n < ld_d) d[n] = from_float<T>(n < Nt ? (z[v] * inv - (n == label ? 1.f : 0.f)) * invB : 0.f);
+  }
+  if (lane == 0) row_loss[(int64_t)g * B + b] = logf(se) + mx - zl;
+}
+
 // Wide rows (hundreds of thousands of classes): one pass with a running (max, sum) pair per
 // thread and 16-byte loads, then one pass that writes delta.  Row length ld is a multiple of 8.
 template <typename T>
@@ -152,17 +196,21 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(
     if (lane == 0) report(st, -5, SITE_LABEL, (long long)g * B + b);
     label = 0;
   }
-  float z[2];
+  // all slices are requested before the first is added (one after the other they were eight trips to L2)
+  float z[2], slice[2][kHeadSplitsMax];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int n = lane + 32 * h;
-    float v = -INFINITY;
-    if (n < Nt) {
-      v = bias ? bias[(int64_t)g * bias_sg + n] : 0.f;
-      for (int s = 0; s < ks; ++s) v += part[(((int64_t)g * ks + s) * B + b) * ld + n];   // fixed order
-    }
-    z[h] = v;
+    z[h] = n < Nt ? (bias ? bias[(int64_t)g * bias_sg + n] : 0.f) : -INFINITY;
+#pragma unroll
+    for (int s = 0; s < kHeadSplitsMax; ++s)
+      slice[h][s] = (n < Nt && s < ks) ? part[(((int64_t)g * ks + s) * B + b) * ld + n] : 0.f;
   }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int s = 0; s < kHeadSplitsMax; ++s)
+      if (s < ks) z[h] += slice[h][s];   // fixed order
   const float mx = warp_max(fmaxf(z[0], z[1]));
   const float e0 = z[0] == -INFINITY ? 0.f : expf(z[0] - mx), e1 = z[1] == -INFINITY ? 0.f : expf(z[1] - mx);
   const float se = warp_sum(e0 + e1);
@@ -494,7 +542,15 @@ void softmax_xent(const Launch& L, const float* logits, int64_t ld, int64_t sg, 
   if (Nt > 8192 && ld % 4 == 0 && ld_d % 4 == 0)
     launch_pdl(softmax_xent_wide_kernel<T>, dim3(B, G), dim3(512), 0, L.stream, logits, ld, sg, B, Nt, y, y_sg, delta,
                ld_d, sg_d, row_loss, st);
-  else
+  else if (Nt <= 1024) {   // a row fits the registers of a warp
+    const dim3 grid((unsigned)ceil_div(B, 8), G);
+    auto go = [&](auto kernel) {
+      launch_pdl(kernel, grid, dim3(256), 0, L.stream, logits, ld, sg, B, Nt, y, y_sg, delta, ld_d, sg_d, row_loss, st);
+    };
+    if (Nt <= 128) go(softmax_xent_warp_kernel<T, 4>);
+    else if (Nt <= 512) go(softmax_xent_warp_kernel<T, 16>);
+    else go(softmax_xent_warp_kernel<T, 32>);
+  } else
     launch_pdl(softmax_xent_kernel<T>, dim3(B, G), dim3(row_threads(Nt)), 0, L.stream, logits, ld, sg, B, Nt, y, y_sg,
                delta, ld_d, sg_d, row_loss, st);
   L.count();

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 # of a step and of a tile; odd widths: rows without 16-byte alignment; few tiles and a deep sum: k cut
 # over a cluster; the last two: pairs of CTAs.
 SIZES = [(1, 1, 1), (5, 16, 3), (24, 33, 17), (31, 65, 64), (33, 64, 16), (128, 128, 128), (129, 127, 65), (64, 5000, 130),
-         (200, 1001, 777), (640, 2048, 4100), (511, 1029, 8209)]
+         (200, 1001, 777), (40, 64, 512), (40, 64, 513), (9, 64, 1024), (9, 64, 1025), (640, 2048, 4100), (511, 1029, 8209)]
 
 
 @pytest.mark.parametrize("B,n0,n1", SIZES)
