@@ -51,6 +51,7 @@
 #include <cfloat>
 #include <mutex>
 
+#include "bias_block.cuh"
 #include "kernels.h"
 #include "tc_ptx.cuh"
 
@@ -63,7 +64,7 @@ constexpr int kLoadWarps = 8, kAddWarps = 8, kThreads = 32 * (kLoadWarps + kAddW
 // narrow tiles: a warp of its own issues the MMAs (with the three beside it that fill up its
 // register-allotment group)
 constexpr int threads_of(int bn) { return bn == 256 ? kThreads : kThreads + 128; }
-constexpr int kMaxProblems = 4;
+constexpr int kMaxProblems = gemm_f32_max_batch();
 
 struct F32Problem {
   int M, N, K, G;
@@ -82,6 +83,8 @@ struct F32Args {
   float lr;
   DeviceStatus* status;
   F32Problem p[kMaxProblems];
+  int side_ctas, side_blocks;           // CTAs behind those of the tiles, and blocks of bias work they share
+  BiasSgdArgs<float> bias;
 };
 
 __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
@@ -282,6 +285,16 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cluster = PAIR == 2 ? 2 : a.ksplit;
+  const int side = (int)blockIdx.x - a.p[a.n_problems - 1].tile_end * cluster;
+  if (side >= 0) {                                     // bias work (a whole cluster of it)
+    pdl_wait();
+    pdl_trigger();
+    for (int b = side; b < a.side_blocks; b += a.side_ctas) {
+      bias_block(a.bias, b, tid, reinterpret_cast<float(*)[65]>(smem));
+      __syncthreads();
+    }
+    return;
+  }
   const int rank = cluster > 1 ? (int)cluster_ctarank() : 0;
   if (tid == 0) {
     for (int b = 0; b < 2; ++b) {
@@ -483,7 +496,7 @@ bool launch(const Launch& L, const F32Args& t, int cluster) {
   });
   if (!ready) return false;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(t.p[t.n_problems - 1].tile_end * cluster));
+  cfg.gridDim = dim3((unsigned)(t.p[t.n_problems - 1].tile_end * cluster + t.side_ctas));
   cfg.blockDim = dim3(threads_of(BN));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = L.stream;
@@ -543,15 +556,20 @@ Shape pick_shape(const GemmArgs<float>* ga, int n) {
 // (half a step here; 256 x 1024 x 16 of four groups 6.1 against 7.6 us), else by its time as
 // measured, 3 us and (1.4 + 0.1 K) us per 1024 tiles of 32 x 32 (64 x 64 x 64 of four groups 3.5
 // against 6.2 us, 512 x 4096 x 64 19 against 12 us).
-bool short_wins(const GemmArgs<float>& a, double us) {
-  if (a.K > 64) return false;
-  const double tiles = (double)ceil_div(a.M, 32) * ceil_div(a.N, 32) * a.G;
-  return a.K <= 16 || 3.0 + (1.4 + 0.1 * a.K) * tiles / 1024 < us;
+bool short_wins(const GemmArgs<float>* a, int n, double us) {
+  double mine = 3.0;
+  bool half = true;
+  for (int i = 0; i < n; ++i) {
+    if (a[i].K > 64) return false;
+    half &= a[i].K <= 16;
+    mine += (1.4 + 0.1 * a[i].K) * (double)ceil_div(a[i].M, 32) * ceil_div(a[i].N, 32) * a[i].G / 1024;
+  }
+  return half || mine < us;
 }
 
 }  // namespace
 
-bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, DeviceStatus* st) {
+bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, const BiasSgdArgs<float>* bias, DeviceStatus* st) {
   if (n < 1 || n > kMaxProblems) return false;
   auto a_is_mn = [](const GemmArgs<float>& a) { return a.a_sm == 1 && a.a_sk != 1; };
   auto b_is_mn = [](const GemmArgs<float>& a) { return a.b_sn == 1 && a.b_sk != 1; };
@@ -563,7 +581,7 @@ bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, DeviceStatus* s
     if ((!a_mn && a.a_sk != 1) || (!b_mn && a.b_sk != 1)) return false;
   }
   Shape sh = pick_shape(ga, n);
-  if (n == 1 && short_wins(ga[0], sh.us) && gemm_short(L, ga[0])) return true;
+  if (short_wins(ga, n, sh.us) && gemm_short(L, ga, n, bias)) return true;
 #ifdef F32_PROBE
   if (getenv("FBN")) { sh.bn = atoi(getenv("FBN")); sh.pair = sh.bn == 256 ? 2 : 1; sh.cluster = atoi(getenv("FCL")); }
 #endif
@@ -598,6 +616,13 @@ bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, DeviceStatus* s
     if (vec(p.out, p.out_ld, p.out_sg) && (!p.bias || vec(p.bias, 0, p.bias_sg)) &&
         (a.epi != EPI_RELU_MASK || vec(p.mask, p.mask_ld, p.mask_sg)))
       p.vec |= 4;
+  }
+  if (bias) {
+    // one CTA per block of bias work, but no more than a round of them
+    t.bias = *bias;
+    t.side_blocks = bias_blocks(t.bias);
+    const int cl = sh.pair == 2 ? 2 : sh.cluster;
+    t.side_ctas = (int)ceil_div(std::min(t.side_blocks, 148), cl) * cl;
   }
   if (a_mn && b_mn) return launch_bn<1, 1>(L, t, sh.bn, sh.pair, sh.cluster);
   if (!a_mn && b_mn) return launch_bn<0, 1>(L, t, sh.bn, sh.pair, sh.cluster);

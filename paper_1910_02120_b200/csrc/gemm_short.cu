@@ -6,6 +6,7 @@
 // along m / n).  A CTA computes a 32 x 32 tile, 2 x 2 per thread.  Such a launch is bound by latency
 // alone, so the whole contraction is fetched at once: one round trip to memory, one barrier.
 // Sums run over k in ascending order.
+#include "bias_block.cuh"
 #include "kernels.h"
 
 namespace ist {
@@ -37,13 +38,33 @@ __device__ __forceinline__ void epilogue_store(const GemmArgs<float>& a, int g, 
   }
 }
 
+struct ShortArgs {
+  int n;
+  GemmArgs<float> p[gemm_f32_max_batch()];
+  int end[gemm_f32_max_batch()];            // blocks end(previous) .. end - 1 are the product's tiles
+  BiasSgdArgs<float> bias;                  // blocks from end[n - 1] on, see bias_block
+};
+
 template <int KMAX>
-__global__ void __launch_bounds__(kThreads) gemm_short_kernel(GemmArgs<float> a) {
+__global__ void __launch_bounds__(kThreads) gemm_short_kernel(const __grid_constant__ ShortArgs args) {
   __shared__ float As[KMAX][kTile + 2];   // + 2: rows stay 8-byte aligned, transposing stores spread over the banks
   __shared__ float Bs[KMAX][kTile + 2];
-  const int g = blockIdx.z, tid = threadIdx.x;
-  const int n_tiles = (a.N + kTile - 1) / kTile;
-  const int m0 = (int)(blockIdx.x / n_tiles) * kTile, n0 = (int)(blockIdx.x % n_tiles) * kTile;
+  const int tid = threadIdx.x;
+  if ((int)blockIdx.x >= args.end[args.n - 1]) {
+    __shared__ float part[32][65];
+    pdl_wait();
+    pdl_trigger();
+    bias_block(args.bias, blockIdx.x - args.end[args.n - 1], tid, part);
+    return;
+  }
+  int pi = 0;
+  while ((int)blockIdx.x >= args.end[pi]) ++pi;
+  const GemmArgs<float>& a = args.p[pi];
+  int tile = blockIdx.x - (pi ? args.end[pi - 1] : 0);
+  const int n_tiles = (a.N + kTile - 1) / kTile, m_tiles = (a.M + kTile - 1) / kTile;
+  const int n0 = tile % n_tiles * kTile;
+  tile /= n_tiles;
+  const int m0 = tile % m_tiles * kTile, g = tile / m_tiles;
   const float* A = a.A + (int64_t)g * a.a_sg;
   const float* B = a.B + (int64_t)g * a.b_sg;
   const bool a_k = a.a_sk == 1, b_k = a.b_sk == 1;   // consecutive lanes along k or along m / n
@@ -84,13 +105,27 @@ __global__ void __launch_bounds__(kThreads) gemm_short_kernel(GemmArgs<float> a)
 
 }  // namespace
 
-bool gemm_short(const Launch& L, const GemmArgs<float>& a) {
-  if (a.M <= 0 || a.N <= 0 || a.G <= 0 || a.K > 64 || a.G > 65535) return false;
-  const int64_t tiles = ceil_div(a.N, kTile) * ceil_div(a.M, kTile);
-  if (tiles > 0x7fffffffll) return false;
-  const dim3 grid((unsigned)tiles, 1, (unsigned)a.G);
-  const cudaError_t e = a.K <= 32 ? launch_pdl(gemm_short_kernel<32>, grid, dim3(kThreads), 0, L.stream, a)
-                                  : launch_pdl(gemm_short_kernel<64>, grid, dim3(kThreads), 0, L.stream, a);
+bool gemm_short(const Launch& L, const GemmArgs<float>* a, int n, const BiasSgdArgs<float>* bias) {
+  if (n < 1 || n > gemm_f32_max_batch()) return false;
+  ShortArgs t{};
+  t.n = n;
+  int64_t end = 0;
+  bool k32 = true;
+  for (int i = 0; i < n; ++i) {
+    if (a[i].M <= 0 || a[i].N <= 0 || a[i].G <= 0 || a[i].K > 64) return false;
+    k32 &= a[i].K <= 32;
+    end += ceil_div(a[i].N, kTile) * ceil_div(a[i].M, kTile) * a[i].G;
+    if (end > 0x3fffffffll) return false;
+    t.p[i] = a[i];
+    t.end[i] = (int)end;
+  }
+  if (bias) {
+    t.bias = *bias;
+    end += bias_blocks(t.bias);
+  }
+  const dim3 grid((unsigned)end);
+  const cudaError_t e = k32 ? launch_pdl(gemm_short_kernel<32>, grid, dim3(kThreads), 0, L.stream, t)
+                            : launch_pdl(gemm_short_kernel<64>, grid, dim3(kThreads), 0, L.stream, t);
   if (e != cudaSuccess) return false;
   L.count();
   return true;

@@ -367,17 +367,20 @@ ist_status check_input(ist_ctx* c, const ist_input* X, const int32_t* y, bool tr
 // ---- grouped GEMM dispatch ------------------------------------------------------------------
 // fp32 operands are split into bf16 parts inside the kernel (or, short contractions, multiplied on the
 // CUDA cores), bf16 operands go to the tensor cores as they are.
-bool gemm(ist_ctx* c, const GemmArgs<float>& a) { return gemm_f32(c->launch(), &a, 1, c->status()); }
+bool gemm(ist_ctx* c, const GemmArgs<float>& a) { return gemm_f32(c->launch(), &a, 1, nullptr, c->status()); }
 bool gemm(ist_ctx* c, const GemmArgs<bf16>& a) { return gemm_tc(c->launch(), a, c->status()); }
 
-// Several products of one kind in as few launches as possible.  fp32 operands: one launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
+// Several products of one kind in as few launches as possible.  fp32 operands: weight updates, which do not
+// depend on one another, gemm_f32_max_batch() to a launch (the first with the bias work), others one launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
 // with `chained`, every problem reads the output of the one before it and the launch orders
 // their tiles through the row-block counters of `region` (one set per problem, indexed by
 // `layer0 + i`; `totals` are the context's running sums for that region).
 bool gemm_list(ist_ctx* c, const std::vector<GemmArgs<float>>& v, bool, Region, std::vector<unsigned>*, int,
-               const LossReduce* = nullptr) {
-  for (auto& g : v)
-    if (!gemm(c, g)) return false;
+               const LossReduce* = nullptr, const BiasSgdArgs<float>* bias = nullptr) {
+  const size_t cap = v.empty() || v[0].epi != EPI_SGD ? 1 : gemm_f32_max_batch();
+  for (size_t i0 = 0; i0 < v.size(); i0 += cap)
+    if (!gemm_f32(c->launch(), v.data() + i0, (int)std::min(cap, v.size() - i0), i0 == 0 ? bias : nullptr, c->status()))
+      return false;
   return true;
 }
 // Whether every launch a weight-update list is cut into can sum the deltas for the bias update.
@@ -390,7 +393,8 @@ bool update_sums_bias(const std::vector<GemmArgs<bf16>>& v) {
 }
 // `loss` (weight-update lists only): the first launch also reduces the step's mean losses.
 bool gemm_list(ist_ctx* c, const std::vector<GemmArgs<bf16>>& v, bool chained, Region region,
-               std::vector<unsigned>* totals, int layer0, const LossReduce* loss = nullptr) {
+               std::vector<unsigned>* totals, int layer0, const LossReduce* loss = nullptr,
+               const BiasSgdArgs<bf16>* = nullptr) {
   const int cap = gemm_tc_max_batch();
   for (size_t i0 = 0; i0 < v.size(); i0 += cap) {
     const int n = (int)std::min<size_t>(cap, v.size() - i0);
@@ -616,20 +620,20 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
                       X->stride_subnet, delta(t), c->ld[t], Bm * c->ld[t], row_loss, st);
     }
     // ---- backward + SGD, last layer first --------------------------------------------------
-    // db_l = sum_b delta_l, layers l_lo..l_hi; the step's mean losses are reduced by the same launch
+    // db_l = sum_b delta_l, layers l_lo..l_hi (kMaxBiasLayers of them at most); the step's mean losses may be
+    // reduced by the same blocks
+    auto bias_args = [&](int l_hi, int l_lo, bool with_loss) {
+      BiasSgdArgs<T> ba{};
+      ba.G = S; ba.B = B; ba.lr = lr;
+      ba.loss = LossReduce{row_loss, with_loss ? loss_out : nullptr, K, k};
+      for (int l = l_hi; l >= l_lo; --l)
+        ba.layer[ba.n_layers++] = BiasSgdLayer<T>{delta(l), c->ld[l], Bm * c->ld[l], bias_of(l), c->ld[l], (int)c->np[l]};
+      return ba;
+    };
     auto update_biases = [&](int l_hi, int l_lo, bool with_loss = true) {
       Scope sc(c, IST_K_BIAS_SGD);
-      BiasSgdArgs<T> ba{};
-      LossReduce lo{row_loss, with_loss ? loss_out : nullptr, K, k};
-      int n = 0;
-      for (int l = l_hi; l >= l_lo; --l) {
-        ba.layer[n++] = BiasSgdLayer<T>{delta(l), c->ld[l], Bm * c->ld[l], bias_of(l), c->ld[l], (int)c->np[l]};
-        if (n == kMaxBiasLayers || l == l_lo) {
-          bias_sgd<T>(L, ba, n, S, B, lr, lo);
-          lo.loss_out = nullptr;
-          n = 0;
-        }
-      }
+      for (int l = l_hi; l >= l_lo; l -= kMaxBiasLayers, with_loss = false)
+        bias_sgd<T>(L, bias_args(l, std::max(l_lo, l - kMaxBiasLayers + 1), with_loss));
     };
     // Every delta is formed from the weights as they stood at the start of the step, so all of
     // them are computed first; the bias update follows at once, while the deltas it sums are still
@@ -712,14 +716,14 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     // stages it streams anyway when the deltas of a step are too large to be still in L2 and the
     // launch runs on single CTAs (a very wide output layer), from memory otherwise (from L2 as a
     // rule; deltas beyond its size come from DRAM a second time there, as they would for the bias
-    // kernel, but in the shadow of the update).  What is left for the bias kernel is a sparse
-    // first layer's bias and the fp32 path, where it runs first if the deltas fit in L2 and last
-    // otherwise.
+    // kernel, but in the shadow of the update).  With fp32 operands it is blocks behind the tiles of the
+    // weight-update launch.  What is left for the bias kernel is a sparse first layer's bias on the bf16
+    // path, and fp32 networks of more layers than one such launch takes along.
     const bool sparse_first = X->kind == IST_X_CSR && t > 1;
     size_t delta_bytes = 0;
     for (int l = 1; l <= t; ++l) delta_bytes += (size_t)S * B * c->ld[l] * sizeof(T);
     const bool bias_first = delta_bytes <= kL2ResidentBytes;
-    const bool bias_in_gemm = bf;
+    const bool bias_in_gemm = bf, bias_beside = !bf && t <= kMaxBiasLayers;
     const bool from_stages = bias_in_gemm && !bias_first && update_sums_bias(upd);
     if (bias_in_gemm) {
       for (auto& g : upd) {
@@ -728,13 +732,15 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
         g.bias_upd_from_memory = from_stages ? 0 : 1;
       }
       if (sparse_first) update_biases(1, 1, false);
-    } else if (bias_first) {
+    } else if (!bias_beside) {
       update_biases(t, 1);
     }
     {
       Scope sc(c, IST_K_DW_SGD);
       LossReduce lo{row_loss, loss_out, K, k};
-      if (!gemm_list(c, upd, false, Region(), nullptr, 0, (bias_in_gemm && loss_out) ? &lo : nullptr))
+      const BiasSgdArgs<T> beside = bias_beside ? bias_args(t, 1, true) : BiasSgdArgs<T>{};
+      if (!gemm_list(c, upd, false, Region(), nullptr, 0, (bias_in_gemm && loss_out) ? &lo : nullptr,
+                     bias_beside ? &beside : nullptr))
         return fail(c, IST_ERR_UNSUPPORTED, "weight-gradient GEMMs cannot be launched");
     }
     if (X->kind == IST_X_CSR && t > 1) {
@@ -743,7 +749,6 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
                            delta(1), c->ld[1], Bm * c->ld[1], (int)c->np[1], master(1), opw(1),
                            c->ld[1], c->slice_elems(1), lr);
     }
-    if (!bias_in_gemm && !bias_first) update_biases(t, 1);
   }
   IST_CUDA(c, cudaGetLastError());
   return IST_OK;

@@ -124,10 +124,13 @@ struct GemmArgs {
   float* label_logit;
   float inv_rows;
 };
-// fp32 operands: on the tensor cores, one to four products with the same operand layouts as tiles of
-// one launch, or on the CUDA cores for short contractions (K <= 64).  false: the shape is not taken.
-bool gemm_f32(const Launch& L, const GemmArgs<float>* a, int n, DeviceStatus* st);
-bool gemm_short(const Launch& L, const GemmArgs<float>& a);
+// fp32 operands: on the tensor cores, one to gemm_f32_max_batch() products with the same operand layouts as
+// tiles of one launch, or on the CUDA cores for short contractions (K <= 64).  bias (weight updates only,
+// may be null): bias updates done by the same launch.  false: the shape is not taken.
+template <typename T> struct BiasSgdArgs;
+constexpr int gemm_f32_max_batch() { return 4; }
+bool gemm_f32(const Launch& L, const GemmArgs<float>* a, int n, const BiasSgdArgs<float>* bias, DeviceStatus* st);
+bool gemm_short(const Launch& L, const GemmArgs<float>* a, int n, const BiasSgdArgs<float>* bias);
 // Tensor-core path (tcgen05 + TMA) for bf16 operands.  Returns false if the shape cannot be
 // described to TMA (misaligned strides) or the operand layouts do not fit an epilogue.
 bool gemm_tc(const Launch& L, const GemmArgs<bf16>& a, DeviceStatus* st);
@@ -199,11 +202,15 @@ template <typename T> struct BiasSgdLayer {
   int n;
 };
 template <typename T> struct BiasSgdArgs {
+  int n_layers, G, B;
+  float lr;
+  LossReduce loss;
   BiasSgdLayer<T> layer[kMaxBiasLayers];
-  int xstart[kMaxBiasLayers + 1];   // filled in by bias_sgd: first block of each layer
+  int xstart[kMaxBiasLayers + 1];   // filled in by bias_blocks: first block of each layer
 };
-template <typename T>
-void bias_sgd(const Launch& L, const BiasSgdArgs<T>& a, int n_layers, int G, int B, float lr, const LossReduce& loss);
+// Fills in xstart; number of blocks bias_block (bias_block.cuh) is to be called for.
+template <typename T> int bias_blocks(BiasSgdArgs<T>& a);
+template <typename T> void bias_sgd(const Launch& L, const BiasSgdArgs<T>& a);
 // fp32 rows -> T rows with leading dimension ld (pad columns zero), per group row offsets.
 template <typename T>
 void stage_rows(const Launch& L, const float* X, int64_t N0, int64_t group_row_stride, int G, int B,

@@ -2,6 +2,7 @@
 // its gradient, the bias update, input staging, and the evaluation reductions.
 #include <algorithm>
 
+#include "bias_block.cuh"
 #include "kernels.h"
 
 namespace ist {
@@ -228,65 +229,13 @@ __global__ void __launch_bounds__(256) softmax_xent_small_kernel(
   if (lane == 0) row_loss[(int64_t)g * B + b] = logf(se) + mx - zl;
 }
 
-// Bias gradient and update of every layer in one launch: blockIdx.y = group, blockIdx.x runs over
-// the layers' blocks of 64 columns one layer after the other (layer i owns blocks xstart[i] ..
-// xstart[i + 1] - 1).  Thread (cx, ry) sums 8 adjacent columns over rows ry, ry + 32, ...; the 32
-// partial sums of a column are added in a fixed order.  When a loss is wanted the grid has one
-// more column of blocks (one per group) that averages the step's row losses (256 threads, fixed
-// summation order).
-__device__ __forceinline__ void load8(const float* p, float v[8]) {
-  float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-__device__ __forceinline__ void load8(const bf16* p, float v[8]) {
-  uint4 u = *reinterpret_cast<const uint4*>(p);
-  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) { v[2 * i] = __low2float(h[i]); v[2 * i + 1] = __high2float(h[i]); }
-}
-
+// Bias gradient and update of every layer in one launch, blocks as bias_block wants them.
 template <typename T>
-__global__ void __launch_bounds__(256) bias_sgd_kernel(BiasSgdArgs<T> a, int n_layers, int B, float lr, LossReduce lo) {
+__global__ void __launch_bounds__(256) bias_sgd_kernel(BiasSgdArgs<T> a) {
   __shared__ float part[32][65];
   pdl_wait();
   pdl_trigger();
-  if ((int)blockIdx.x == a.xstart[n_layers]) {   // the extra column of blocks
-    const int g = blockIdx.y;
-    float acc = 0.f;
-    for (int b = threadIdx.x; b < B; b += blockDim.x) acc += lo.row_loss[(int64_t)g * B + b];
-    acc = block_sum(acc, &part[0][0]);
-    if (threadIdx.x == 0) lo.loss_out[(int64_t)g * lo.out_stride + lo.k] = acc / (float)B;
-    return;
-  }
-  int li = 0;
-  while (li + 1 < n_layers && (int)blockIdx.x >= a.xstart[li + 1]) ++li;
-  const BiasSgdLayer<T> L = a.layer[li];
-  const int g = blockIdx.y, bx = blockIdx.x - a.xstart[li];
-  const int cx = threadIdx.x & 7, ry = threadIdx.x >> 3;
-  const int c0 = bx * 64 + cx * 8;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (c0 < L.ld) {
-    const T* d = L.delta + (int64_t)g * L.sg + c0;
-#pragma unroll 8
-    for (int b = ry; b < B; b += 32) {
-      float v[8];
-      load8(d + (int64_t)b * L.ld, v);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += v[e];
-    }
-  }
-#pragma unroll
-  for (int e = 0; e < 8; ++e) part[ry][cx * 8 + e] = acc[e];
-  __syncthreads();
-  if (threadIdx.x < 64) {
-    const int col = bx * 64 + threadIdx.x;
-    if (col < L.n) {
-      float s = 0.f;
-#pragma unroll
-      for (int u = 0; u < 32; ++u) s += part[u][threadIdx.x];
-      L.bias[(int64_t)g * L.bias_sg + col] -= lr * s;
-    }
-  }
+  bias_block(a, blockIdx.x, threadIdx.x, part);
 }
 
 // lse[g][b] = log sum_n exp(z[g][b][n]) from per-tile partials (m, s) = (max of z * log2(e),
@@ -599,16 +548,23 @@ void lse_row_loss(const Launch& L, const float* lse, const float* label_logit, i
 }
 
 template <typename T>
-void bias_sgd(const Launch& L, const BiasSgdArgs<T>& a, int n_layers, int G, int B, float lr, const LossReduce& loss) {
+int bias_blocks(BiasSgdArgs<T>& a) {
+  a.xstart[0] = 0;
+  for (int i = 0; i < a.n_layers; ++i) a.xstart[i + 1] = a.xstart[i] + (int)ceil_div(a.layer[i].ld, 64);
+  return (a.xstart[a.n_layers] + (a.loss.loss_out ? 1 : 0)) * a.G;
+}
+template int bias_blocks<float>(BiasSgdArgs<float>&);
+template int bias_blocks<bf16>(BiasSgdArgs<bf16>&);
+
+template <typename T>
+void bias_sgd(const Launch& L, const BiasSgdArgs<T>& a) {
   BiasSgdArgs<T> b = a;
-  b.xstart[0] = 0;
-  for (int i = 0; i < n_layers; ++i) b.xstart[i + 1] = b.xstart[i] + (int)ceil_div(a.layer[i].ld, 64);
-  launch_pdl(bias_sgd_kernel<T>, dim3((unsigned)b.xstart[n_layers] + (loss.loss_out ? 1 : 0), G), dim3(256), 0, L.stream, b,
-             n_layers, B, lr, loss);
+  const int blocks = bias_blocks(b);
+  launch_pdl(bias_sgd_kernel<T>, dim3((unsigned)blocks), dim3(256), 0, L.stream, b);
   L.count();
 }
-template void bias_sgd<float>(const Launch&, const BiasSgdArgs<float>&, int, int, int, float, const LossReduce&);
-template void bias_sgd<bf16>(const Launch&, const BiasSgdArgs<bf16>&, int, int, int, float, const LossReduce&);
+template void bias_sgd<float>(const Launch&, const BiasSgdArgs<float>&);
+template void bias_sgd<bf16>(const Launch&, const BiasSgdArgs<bf16>&);
 
 template <typename T>
 void stage_rows(const Launch& L, const float* X, int64_t N0, int64_t group_row_stride, int G, int B,
