@@ -1139,33 +1139,69 @@ bool gemm_tc_wait_selftest(const Launch& L, DeviceStatus* st, long long limit_cy
   return cudaGetLastError() == cudaSuccess;
 }
 
-// Tile shape.  Pairs of CTAs (256 x 256 tiles) are used when the problem has enough of them to
-// give every SM pair work; otherwise single CTAs with the widest of 256 / 128 / 64 columns that
-// still gives every SM a tile.  The weight-update epilogue keeps a chunk ring in shared memory
-// and stays at 128 columns when it runs on single CTAs.  A batch of problems is judged by the
-// tiles of all of them together and must have one problem that qualifies for pairs by itself
-// (more than 128 rows and columns); the small ones then ride along on the same shape.
+// Tile shape: pairs of CTAs on 256 x 256 tiles, or single CTAs with 256, 128 or 64 columns.  A batch of
+// problems must have one that qualifies for pairs by itself (more than 128 rows and columns) to run on
+// them; the small ones then ride along on the same shape.
+//
+// Forward and delta products: the shape with the smallest sum over the problems (a chain runs them one
+// after the other) of rounds of tiles x (64-deep k blocks x cost of one + a fixed part), in cycles.  A k block
+// costs what its operands take from L2 at about 58 bytes per clock, 48 / 32 / 24 KB for 256 / 128 / 64
+// columns and 32 KB per CTA of a pair.  Against the rule before it, which asked for a tile per SM counted over
+// all problems together: 512-3000-3000-3000-64, S = 3, 300 rows, six steps 692 -> 640 us (64 columns);
+// 1472-1664-6656-37, S = 9, 200 rows 456 -> 442 us; 3072-16384-16384-10, S = 8, 128 rows 2190 -> 2123 us (128
+// columns); 512 rows pairs as before.
+//
+// Weight updates: bound by streaming the masters, 10 bytes per weight, so long as the contraction (the
+// batch) is short, and then small tiles keep more transfers in flight: up to 128 rows 64 columns on single CTAs
+// (120-26586-2688-509, S = 9, 128 rows: 804 -> 733 us against pairs; 3072-16384-16384-10 within 1 %).  Up to
+// 320 rows still where the pairs' tiles hang over the matrices' edges by more than 15 % (the same
+// network at 224 rows 890 -> 845 us; 1024-4096-4096-35, which pairs tile exactly, 477 against 484 us).  Not
+// with an output layer of many thousand classes, whose update streams from DRAM for milliseconds
+// (135909-1024-670091, S = 8, 256 rows: 54.3 ms with 128 columns, 56.8 with 64).
 struct TileChoice { int bn, pair; };
 TileChoice pick_tile(const GemmArgs<bf16>* a, int n, int epi) {
   const int sms = sm_count();
   auto n_store = [&](int i) { return a[i].N_store > 0 ? a[i].N_store : a[i].N; };
+  auto tiles_of = [&](int i, int bm, int bn) {
+    return ceil_div(a[i].M, bm) * ceil_div(n_store(i), bn) * a[i].G * (a[i].k_splits > 1 ? a[i].k_splits : 1);
+  };
   auto tiles = [&](int bm, int bn) {
     int64_t s = 0;
-    for (int i = 0; i < n; ++i)
-      s += ceil_div(a[i].M, bm) * ceil_div(n_store(i), bn) * a[i].G * (a[i].k_splits > 1 ? a[i].k_splits : 1);
+    for (int i = 0; i < n; ++i) s += tiles_of(i, bm, bn);
     return s;
   };
-  bool pair_ok = false, wide = false, mid = false;
+  bool pair_ok = false, wide = false, mid = false, huge = false;
   for (int i = 0; i < n; ++i) {
     pair_ok |= a[i].M > BM && n_store(i) > 128;
     wide |= n_store(i) > 128;
+    huge |= n_store(i) > 8192;
     mid |= n_store(i) > 64;
   }
-  if (pair_ok && 4 * tiles(2 * BM, 256) >= 3 * (sms / 2)) return {256, 2};
-  if (epi == EPI_SGD) return {(mid && tiles(BM, 128) >= sms) ? 128 : 64, 1};
-  if (wide && tiles(BM, 256) >= sms) return {256, 1};
-  if (mid && tiles(BM, 128) >= sms) return {128, 1};
-  return {64, 1};
+  if (epi == EPI_SGD) {
+    const int rows = a[0].K;
+    const bool overhang = (double)tiles(2 * BM, 256) * (2 * BM * 256) > 1.15 * (double)tiles(BM, 64) * (BM * 64);
+    if (pair_ok && !huge && (rows <= 128 || (rows <= 320 && overhang))) return {64, 1};
+    if (pair_ok && 4 * tiles(2 * BM, 256) >= 3 * (sms / 2)) return {256, 2};
+    return {(mid && tiles(BM, 128) >= sms) ? 128 : 64, 1};
+  }
+  TileChoice best{64, 1};
+  int64_t best_cost = INT64_MAX;
+  auto consider = [&](int bn, int pair, int per_block, int fixed) {
+    int64_t cost = 0;
+    for (int i = 0; i < n; ++i) {
+      const int64_t blocks = ceil_div(ceil_div(a[i].K, BK), a[i].k_splits > 1 ? a[i].k_splits : 1);
+      cost += ceil_div(tiles_of(i, BM * pair, bn) * pair, sms) * (blocks * per_block + fixed);
+    }
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = TileChoice{bn, pair};
+    }
+  };
+  if (pair_ok) consider(256, 2, 550, 4500);
+  if (wide) consider(256, 1, 830, 4000);
+  if (mid) consider(128, 1, 550, 3500);
+  consider(64, 1, 414, 3000);
+  return best;
 }
 
 // Partials per row the EPI_LSE_PART epilogue writes: one per 256-column tile and warp group.
