@@ -529,6 +529,34 @@ bool launch_bn(const Launch& L, const F32Args& t, int bn, int pair, int cluster)
 // 32-deep step.  Constants fitted to 12 products of 64 x 64 x 32 to 512 x 16384 x 3072 (measured
 // 5.3 to 244 us, estimates within 25 %); 64-column tiles pay off only where 128-column ones leave
 // SMs idle or the product is narrow, pairs from about 64 tiles of 256 x 256 on.
+// Clusters of two, four and eight CTAs that can run at once (a GPU processing cluster holds a whole
+// number of them): 16 of eight did not all fit and took two rounds (128 x 512 x 784 of two groups, 64
+// columns: 18.5 us in clusters of eight, 11.7 us in clusters of four).
+int clusters_at_once(int cluster) {
+  static int n[4] = {148, 0, 0, 0};
+  static std::once_flag once;
+  std::call_once(once, [] {
+    auto kern = gemm_f32_kernel<0, 1, 128, 1>;           // the larger of the two single-CTA shapes
+    constexpr int smem = (int)smem_bytes<128, 1>();
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return;
+    for (int i = 1; i < 4; ++i) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(128);
+      cfg.blockDim = dim3(threads_of(128));
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute attr{};
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = 1u << i;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int k = 0;
+      if (cudaOccupancyMaxActiveClusters(&k, kern, &cfg) == cudaSuccess) n[i] = k;
+    }
+  });
+  return n[cluster == 1 ? 0 : cluster == 2 ? 1 : cluster == 4 ? 2 : 3];
+}
+
 struct Shape { int bn, pair, cluster; double us; };
 Shape pick_shape(const GemmArgs<float>* ga, int n) {
   const int sms = 148;
@@ -539,7 +567,7 @@ Shape pick_shape(const GemmArgs<float>* ga, int n) {
       tiles += ceil_div(ga[i].M, BM * pair) * ceil_div(ga[i].N, bn) * ga[i].G;
       steps = std::max<int64_t>(steps, ceil_div(ga[i].K, KH));
     }
-    if (cluster > 1 && (steps < 2 * cluster || tiles * cluster > sms)) return;
+    if (cluster > 1 && (steps < 2 * cluster || tiles > clusters_at_once(cluster))) return;
     const int64_t rounds = ceil_div(tiles * pair, sms);
     const double us = rounds * (fix_us + step_us * ceil_div(steps, cluster)) + (cluster > 1 ? 0.5 + 0.2 * cluster : 0.0);
     if (us < best.us) best = Shape{bn, pair, cluster, us};
