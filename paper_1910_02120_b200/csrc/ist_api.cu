@@ -437,8 +437,8 @@ void small_softmax(const Launch& L, const float* part, int ks, int64_t ld, int G
                    float* row_loss, DeviceStatus* st) {
   softmax_xent_small<bf16>(L, part, ks, ld, G, B, Nt, bias, bias_sg, y, y_sg, delta, ld_d, sg_d, row_loss, st);
 }
-// A product written as plain fp32: on the tensor-core path the fp32 epilogue without a bias, on
-// the CUDA-core path (operands and output of the same type) a plain store.
+// A product written as plain fp32: with bf16 operands the fp32 epilogue without a bias, with fp32
+// operands (output of the same type) a plain store.
 void set_plain_fp32_output(GemmArgs<bf16>& g, float* out, int64_t ld, int64_t sg) {
   g.epi = EPI_BIAS_F32; g.bias = nullptr; g.outf = out; g.outf_ld = ld; g.outf_sg = sg;
 }
