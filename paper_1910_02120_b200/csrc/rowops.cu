@@ -297,16 +297,31 @@ __global__ void lse_row_loss_kernel(const float* __restrict__ lse, const float* 
   if (b < B) row_loss[(int64_t)g * B + b] = lse[(int64_t)g * lse_sg + b] - zy[(int64_t)g * lse_sg + b];
 }
 
+// One block per row; a thread rounds four pairs of adjacent columns, their eight 4-byte loads (rows start at
+// any 4-byte boundary) in flight together.  With a thread per element 1200 rows of 1001 took 10.7 us,
+// now 6.7.
 template <typename T>
-__global__ void stage_rows_kernel(const float* __restrict__ X, int64_t N0, int64_t group_row_stride,
-                                  int B, T* __restrict__ out, int64_t ld, int64_t sg) {
+__global__ void __launch_bounds__(128) stage_rows_kernel(const float* __restrict__ X, int64_t N0, int64_t group_row_stride,
+                                                         T* __restrict__ out, int64_t ld, int64_t sg) {
+  struct alignas(2 * sizeof(T)) Pair { T a, b; };
+  constexpr int U = 4;
   pdl_wait();
   pdl_trigger();
-  int g = blockIdx.z, b = blockIdx.y;
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= ld) return;
-  float v = j < N0 ? X[((int64_t)g * group_row_stride + b) * N0 + j] : 0.f;
-  out[(int64_t)g * sg + (int64_t)b * ld + j] = from_float<T>(v);
+  const int b = blockIdx.x, g = blockIdx.y;
+  const float* x = X + ((int64_t)g * group_row_stride + b) * N0;
+  Pair* o = reinterpret_cast<Pair*>(out + (int64_t)g * sg + (int64_t)b * ld);   // ld is even, rows of `out` 16-byte aligned
+  for (int64_t p0 = threadIdx.x; p0 < ld / 2; p0 += U * 128) {
+    float v[U][2];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t c = 2 * (p0 + u * 128);
+      v[u][0] = c < N0 ? __ldg(x + c) : 0.f;
+      v[u][1] = c + 1 < N0 ? __ldg(x + c + 1) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (p0 + u * 128 < ld / 2) o[p0 + u * 128] = Pair{from_float<T>(v[u][0]), from_float<T>(v[u][1])};
+  }
 }
 
 __global__ void eval_rows_kernel(const float* __restrict__ logits, int64_t ld, int rows, int Nt,
@@ -569,8 +584,7 @@ template void bias_sgd<bf16>(const Launch&, const BiasSgdArgs<bf16>&);
 template <typename T>
 void stage_rows(const Launch& L, const float* X, int64_t N0, int64_t group_row_stride, int G, int B,
                 T* out, int64_t ld, int64_t sg) {
-  launch_pdl(stage_rows_kernel<T>, dim3((unsigned)ceil_div(ld, 256), B, G), dim3(256), 0, L.stream, X, N0,
-             group_row_stride, B, out, ld, sg);
+  launch_pdl(stage_rows_kernel<T>, dim3((unsigned)B, (unsigned)G), dim3(128), 0, L.stream, X, N0, group_row_stride, out, ld, sg);
   L.count();
 }
 template void stage_rows<float>(const Launch&, const float*, int64_t, int64_t, int, int, float*,
