@@ -74,7 +74,9 @@ __global__ void softmax_xent_kernel(const float* __restrict__ logits, int64_t ld
 
 // Up to 32 V classes: one warp per row, eight rows per block, the row in registers.  The kernel above
 // reads a row three times and crosses eight block barriers, all latency at these sizes (a local step of
-// 256 rows of four subnets, 35 classes: 2 us less).
+// 256 rows of four subnets, 35 classes: 2 us less).  The exponentials are added in that kernel's order, so
+// that a class count's results do not depend on which of the two takes it: row_threads(Nt) strided
+// partial sums, a butterfly over each 32 of them, then the four warps' sums as (0 + 2) + (1 + 3).
 template <typename T, int V>
 __global__ void __launch_bounds__(256) softmax_xent_warp_kernel(const float* __restrict__ logits, int64_t ld, int64_t sg, int B,
                                                                 int Nt, const int32_t* __restrict__ y, int64_t y_sg,
@@ -97,14 +99,17 @@ __global__ void __launch_bounds__(256) softmax_xent_warp_kernel(const float* __r
 #pragma unroll
   for (int v = 1; v < V; ++v) mx = fmaxf(mx, z[v]);
   mx = warp_max(mx);
-  float se = 0.f, zl = 0.f;
+  constexpr int W = V <= 2 ? 1 : 4;                    // warps of that block
+  float part[W] = {}, zl = 0.f;
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     if (lane + 32 * v == label) zl = z[v];
     z[v] = lane + 32 * v < Nt ? expf(z[v] - mx) : 0.f;
-    se += z[v];
+    part[v % W] += z[v];
   }
-  se = warp_sum(se);
+#pragma unroll
+  for (int w = 0; w < W; ++w) part[w] = warp_sum(part[w]);
+  const float se = W == 1 ? part[0] : (part[0] + part[2 % W]) + (part[1 % W] + part[3 % W]);
   zl = __shfl_sync(0xffffffffu, zl, label & 31);
   const float inv = 1.f / se, invB = 1.f / (float)B;
   T* d = delta + (int64_t)g * sg_d + (int64_t)b * ld_d;
@@ -511,7 +516,8 @@ void softmax_xent(const Launch& L, const float* logits, int64_t ld, int64_t sg, 
     auto go = [&](auto kernel) {
       launch_pdl(kernel, grid, dim3(256), 0, L.stream, logits, ld, sg, B, Nt, y, y_sg, delta, ld_d, sg_d, row_loss, st);
     };
-    if (Nt <= 128) go(softmax_xent_warp_kernel<T, 4>);
+    if (Nt <= 64) go(softmax_xent_warp_kernel<T, 2>);
+    else if (Nt <= 128) go(softmax_xent_warp_kernel<T, 4>);
     else if (Nt <= 512) go(softmax_xent_warp_kernel<T, 16>);
     else go(softmax_xent_warp_kernel<T, 32>);
   } else
