@@ -599,15 +599,17 @@ bool short_wins(const GemmArgs<float>* a, int n, double us) {
 
 bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, const BiasSgdArgs<float>* bias, DeviceStatus* st) {
   if (n < 1 || n > kMaxProblems) return false;
-  auto a_is_mn = [](const GemmArgs<float>& a) { return a.a_sm == 1 && a.a_sk != 1; };
-  auto b_is_mn = [](const GemmArgs<float>& a) { return a.b_sn == 1 && a.b_sk != 1; };
-  const bool a_mn = a_is_mn(ga[0]), b_mn = b_is_mn(ga[0]);
+  // One layout per operand for the whole launch: contiguous along k, or along m / n.  An operand with unit
+  // stride in both directions (a width of one) fits either and goes with the others.
+  bool a_k = true, a_m = true, b_k = true, b_n = true;
   for (int i = 0; i < n; ++i) {
     const GemmArgs<float>& a = ga[i];
     if (a.M < 1 || a.N < 1 || a.K < 1 || a.G < 1 || a.lr != ga[0].lr) return false;
-    if (a_is_mn(a) != a_mn || b_is_mn(a) != b_mn) return false;
-    if ((!a_mn && a.a_sk != 1) || (!b_mn && a.b_sk != 1)) return false;
+    a_k &= a.a_sk == 1; a_m &= a.a_sm == 1;
+    b_k &= a.b_sk == 1; b_n &= a.b_sn == 1;
   }
+  if ((!a_k && !a_m) || (!b_k && !b_n)) return false;
+  const bool a_mn = !a_k, b_mn = !b_k || (a_mn && b_n);
   Shape sh = pick_shape(ga, n);
   if (short_wins(ga, n, sh.us) && gemm_short(L, ga, n, bias)) return true;
 #ifdef F32_PROBE
