@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kCols * kLanes) colnorm_forward_kernel(
 // d_z = (d_zh - mean_b d_zh - zh * mean_b(d_zh * zh)) / sigma.
 template <typename T>
 __global__ void __launch_bounds__(kCols * kLanes) colnorm_backward_kernel(
-    T* __restrict__ delta, int64_t ld, int64_t d_sg, const float* __restrict__ z, int64_t z_sg,
-    const float* __restrict__ mu_in, const float* __restrict__ rstd_in, int64_t stat_sg, int B, int n) {
+    T* __restrict__ delta, int64_t ld, int64_t d_sg, const float* z, int64_t z_sg,
+    const float* mu_in, const float* rstd_in, int64_t stat_sg, int B, int n) {
   __shared__ float sh[kLanes][kCols + 1];
   pdl_wait();
   pdl_trigger();
@@ -223,8 +223,8 @@ __global__ void __launch_bounds__(kVecThreads) colnorm_forward_vec_kernel(
 
 template <typename T>
 __global__ void __launch_bounds__(kVecThreads) colnorm_backward_vec_kernel(
-    T* __restrict__ delta, int64_t ld, int64_t d_sg, const float* __restrict__ z, int64_t z_sg,
-    const float* __restrict__ mu_in, const float* __restrict__ rstd_in, int64_t stat_sg, int B) {
+    T* __restrict__ delta, int64_t ld, int64_t d_sg, const float* z, int64_t z_sg,
+    const float* mu_in, const float* rstd_in, int64_t stat_sg, int B) {
   __shared__ float sh[kVecThreads / 32][kVecCols];
   pdl_wait();
   pdl_trigger();

@@ -37,6 +37,9 @@ __device__ __forceinline__ void report(DeviceStatus* st, int code, int site, lon
 // kernel before it in the stream is still running; it must call pdl_wait() before it touches
 // global memory (that waits until the earlier kernel has completed and its writes are visible).
 // pdl_trigger() lets the kernel after this one be scheduled as this grid's CTAs retire.
+// Such a kernel reads with plain loads only, no __ldg and no `const __restrict__` parameters: the
+// non-coherent path asks for data that is constant for the kernel's whole life, which begins while the
+// earlier kernel may still be writing it, and the compiler may move those loads ahead of the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ 
   const int64_t o0 = ((int64_t)s * m.rows_pad + i0) * m.ld + j;
 #pragma unroll
   for (int u = 0; u < kRowsPerCta; ++u)
-    v[u] = r[u] >= 0 ? (GATHER ? __ldg(J.W + r[u]) : J.master[o0 + u * m.ld]) : 0.f;
+    v[u] = r[u] >= 0 ? (GATHER ? J.W[r[u]] : J.master[o0 + u * m.ld]) : 0.f;
 #pragma unroll
   for (int u = 0; u < kRowsPerCta; ++u) {
     if (GATHER) {
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ 
 constexpr int kRowU = 4, kColU = 4;
 
 template <bool GATHER>
-__global__ void __launch_bounds__(kThreads) rows_kernel(float* __restrict__ W, SliceMap m, float* __restrict__ master,
+__global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, float* master,
                                                          bf16* __restrict__ opw) {
   pdl_wait();
   pdl_trigger();
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* __restrict__ W, S
 #pragma unroll
         for (int c = 0; c < kColU; ++c) {
           const int64_t j = j0 + c * kThreads;
-          v[u][c] = (src[u] >= 0 && j < m.full_cols) ? __ldg(W + src[u] + j) : 0.f;   // pad rows / columns are zeros
+          v[u][c] = (src[u] >= 0 && j < m.full_cols) ? W[src[u] + j] : 0.f;   // pad rows / columns are zeros
         }
 #pragma unroll
       for (int u = 0; u < kRowU; ++u)
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* __restrict__ W, S
 #pragma unroll
         for (int c = 0; c < kColU; ++c) {
           const int64_t j = j0 + c * kThreads;
-          v[u][c] = (src[u] >= 0 && j < m.full_cols) ? __ldg(master + ((int64_t)s * m.rows_pad + i0 + u) * m.ld + j) : 0.f;
+          v[u][c] = (src[u] >= 0 && j < m.full_cols) ? master[((int64_t)s * m.rows_pad + i0 + u) * m.ld + j] : 0.f;
         }
 #pragma unroll
       for (int u = 0; u < kRowU; ++u)
@@ -222,8 +222,8 @@ constexpr long long kPermWaitCycles = 2000000000ll;   // ~1 s
 // this one is permuted).  Scatter: packed values are read into the permuted tile, which leaves
 // through bulk stores.  Requires full_cols % 4 == 0 (16-byte row segments).
 template <bool GATHER>
-__global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* __restrict__ W, SliceMap m, int S,
-                                                                      float* __restrict__ master,
+__global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W, SliceMap m, int S,
+                                                                      float* master,
                                                                       bf16* __restrict__ opw, DeviceStatus* st) {
   extern __shared__ __align__(128) unsigned char perm_smem[];
   float* tile = reinterpret_cast<float*>(perm_smem);                                  // [2][rows][cols]

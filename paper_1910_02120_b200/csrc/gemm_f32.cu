@@ -154,12 +154,12 @@ struct Operand {
       const float* q = p + i * unit_step;
       const int n = MN ? (kofs < krem ? rows - 64 * i : 0) : (64 * i < rows ? krem - kofs : 0);
       if (vec && n >= 8) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(q)), b = __ldg(reinterpret_cast<const float4*>(q) + 1);
+        const float4 a = *reinterpret_cast<const float4*>(q), b = *(reinterpret_cast<const float4*>(q) + 1);
         v[i][0] = a.x; v[i][1] = a.y; v[i][2] = a.z; v[i][3] = a.w;
         v[i][4] = b.x; v[i][5] = b.y; v[i][6] = b.z; v[i][7] = b.w;
       } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[i][e] = e < n ? __ldg(q + e) : 0.f;
+        for (int e = 0; e < 8; ++e) v[i][e] = e < n ? q[e] : 0.f;
       }
     }
     p += half_step;
@@ -189,7 +189,7 @@ __device__ __forceinline__ float fma_chain(const F32Problem& pr, int g, int m, i
   const long long as = A_MN ? pr.a_st : 1, bs = B_MN ? pr.b_st : 1;
   float acc = 0.f;
 #pragma unroll 1
-  for (int k = 0; k < pr.K && acc == acc; ++k) acc = fmaf(__ldg(A + k * as), __ldg(B + k * bs), acc);
+  for (int k = 0; k < pr.K && acc == acc; ++k) acc = fmaf(A[k * as], B[k * bs], acc);
   return acc;
 }
 

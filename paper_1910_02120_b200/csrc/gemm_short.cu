@@ -77,8 +77,8 @@ __global__ void __launch_bounds__(kThreads) gemm_short_kernel(const __grid_const
     const int e = tid + kThreads * u;
     const int ka = a_k ? e % KMAX : e / kTile, ma = m0 + (a_k ? e / KMAX : e % kTile);
     const int kb = b_k ? e % KMAX : e / kTile, nb = n0 + (b_k ? e / KMAX : e % kTile);
-    ra[u] = (ma < a.M && ka < a.K) ? __ldg(A + (int64_t)ma * a.a_sm + (int64_t)ka * a.a_sk) : 0.f;
-    rb[u] = (nb < a.N && kb < a.K) ? __ldg(B + (int64_t)nb * a.b_sn + (int64_t)kb * a.b_sk) : 0.f;
+    ra[u] = (ma < a.M && ka < a.K) ? A[(int64_t)ma * a.a_sm + (int64_t)ka * a.a_sk] : 0.f;
+    rb[u] = (nb < a.N && kb < a.K) ? B[(int64_t)nb * a.b_sn + (int64_t)kb * a.b_sk] : 0.f;
   }
 #pragma unroll
   for (int u = 0; u < NE; ++u) {

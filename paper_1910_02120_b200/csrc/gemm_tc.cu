@@ -184,11 +184,11 @@ template <int TILE_M, int TILE_N>
 __device__ __forceinline__ bool tile_live(const TcProblem& pr, const TileAt& at, int g, int* kb_limit) {
   *kb_limit = 0x7fffffff;
   if (!pr.m_off && !pr.n_off && !pr.k_off) return true;
-  if (pr.n_off && at.nt * TILE_N >= __ldg(pr.n_off + g + 1) - __ldg(pr.n_off + g)) return false;
+  if (pr.n_off && at.nt * TILE_N >= pr.n_off[g + 1] - pr.n_off[g]) return false;
   // a tile that carries its columns' bias update runs even if it lies beyond the group's rows
-  if (pr.m_off && at.mt * TILE_M >= __ldg(pr.m_off + g + 1) - __ldg(pr.m_off + g) && !sums_bias(pr, at))
+  if (pr.m_off && at.mt * TILE_M >= pr.m_off[g + 1] - pr.m_off[g] && !sums_bias(pr, at))
     return false;
-  if (pr.k_off) *kb_limit = max(1, (__ldg(pr.k_off + g + 1) - __ldg(pr.k_off + g) + BK - 1) / BK);
+  if (pr.k_off) *kb_limit = max(1, (pr.k_off[g + 1] - pr.k_off[g] + BK - 1) / BK);
   return true;
 }
 
@@ -512,7 +512,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
           const int n = n0 + c * CH + lane;
-          next_bias[c] = (bias && n < pr.N) ? __ldg(bias + n) : 0.f;
+          next_bias[c] = (bias && n < pr.N) ? bias[n] : 0.f;
         }
       }
       if (EPI == EPI_LSE_PART || EPI == EPI_SOFTMAX_DELTA) {
@@ -523,8 +523,8 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
       }
       if (EPI == EPI_SOFTMAX_DELTA) {
         const int row = at.mt * (BM * PAIR) + rank * BM + r;
-        next_lse = row < pr.M ? __ldg(a.lse + (long long)at.slab * a.lse_sg + row) : 0.f;
-        next_label = row < pr.M ? __ldg(a.labels + (long long)at.slab * a.labels_sg + row) : -1;
+        next_lse = row < pr.M ? a.lse[(long long)at.slab * a.lse_sg + row] : 0.f;
+        next_label = row < pr.M ? a.labels[(long long)at.slab * a.labels_sg + row] : -1;
       }
     };
 #pragma unroll
@@ -635,7 +635,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
             const float* bias = a.p[pi].bias ? a.p[pi].bias + (long long)g * a.p[pi].bias_sg + nc : nullptr;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const float4 bv = (bias && nc + 4 * u < pN) ? __ldg(reinterpret_cast<const float4*>(bias) + u)
+              const float4 bv = (bias && nc + 4 * u < pN) ? *(reinterpret_cast<const float4*>(bias) + u)
                                                           : make_float4(0.f, 0.f, 0.f, 0.f);
               z[4 * u + 0] = __uint_as_float(acc[4 * u + 0]) + bv.x;
               z[4 * u + 1] = __uint_as_float(acc[4 * u + 1]) + bv.y;
@@ -879,7 +879,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     if (rank == 0 && sw == kSumWarps - 1 && a.loss.loss_out) {
       for (int g = unit; g < a.loss_G; g += n_units) {
         float acc = 0.f;
-        for (int b = lane; b < a.loss_B; b += 32) acc += __ldg(a.loss.row_loss + (long long)g * a.loss_B + b);
+        for (int b = lane; b < a.loss_B; b += 32) acc += a.loss.row_loss[(long long)g * a.loss_B + b];
 #pragma unroll
         for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) a.loss.loss_out[(long long)g * a.loss.out_stride + a.loss.k] = acc / (float)a.loss_B;
@@ -901,7 +901,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         for (int r0 = 0; r0 < pr.K; r0 += 16) {              // the contraction of a weight update runs over the batch
           uint32_t v[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = r0 + i < pr.K ? __ldg(dp + (long long)(r0 + i) * ld2) : 0u;
+          for (int i = 0; i < 16; ++i) v[i] = r0 + i < pr.K ? dp[(long long)(r0 + i) * ld2] : 0u;
 #pragma unroll
           for (int i = 0; i < 16; ++i) {                     // rows in ascending order: a fixed sum
             acc0 += __uint_as_float(v[i] << 16);

@@ -42,8 +42,8 @@ __device__ float block_sum(float v, float* sh) {
 // One CTA per row (g, b).  loss_row = log(sum exp(z - max)) + max - z[y];
 // delta = (exp(z - max)/sum - [n == y]) / B.
 template <typename T>
-__global__ void softmax_xent_kernel(const float* __restrict__ logits, int64_t ld, int64_t sg, int B,
-                                    int Nt, const int32_t* __restrict__ y, int64_t y_sg,
+__global__ void softmax_xent_kernel(const float* logits, int64_t ld, int64_t sg, int B,
+                                    int Nt, const int32_t* y, int64_t y_sg,
                                     T* __restrict__ delta, int64_t ld_d, int64_t sg_d,
                                     float* __restrict__ row_loss, DeviceStatus* st) {
   __shared__ float sh[32];
@@ -78,8 +78,8 @@ __global__ void softmax_xent_kernel(const float* __restrict__ logits, int64_t ld
 // that a class count's results do not depend on which of the two takes it: row_threads(Nt) strided
 // partial sums, a butterfly over each 32 of them, then the four warps' sums as (0 + 2) + (1 + 3).
 template <typename T, int V>
-__global__ void __launch_bounds__(256) softmax_xent_warp_kernel(const float* __restrict__ logits, int64_t ld, int64_t sg, int B,
-                                                                int Nt, const int32_t* __restrict__ y, int64_t y_sg,
+__global__ void __launch_bounds__(256) softmax_xent_warp_kernel(const float* logits, int64_t ld, int64_t sg, int B,
+                                                                int Nt, const int32_t* y, int64_t y_sg,
                                                                 T* __restrict__ delta, int64_t ld_d, int64_t sg_d,
                                                                 float* __restrict__ row_loss, DeviceStatus* st) {
   pdl_wait();
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) softmax_xent_warp_kernel(const float* __r
 // thread and 16-byte loads, then one pass that writes delta.  Row length ld is a multiple of 8.
 template <typename T>
 __global__ void __launch_bounds__(512) softmax_xent_wide_kernel(
-    const float* __restrict__ logits, int64_t ld, int64_t sg, int B, int Nt, const int32_t* __restrict__ y,
+    const float* logits, int64_t ld, int64_t sg, int B, int Nt, const int32_t* y,
     int64_t y_sg, T* __restrict__ delta, int64_t ld_d, int64_t sg_d, float* __restrict__ row_loss,
     DeviceStatus* st) {
   __shared__ float sm[16], ss[16];
@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(512) softmax_xent_wide_kernel(
 // they are summed here together with the bias, so the split costs no extra launch.
 template <typename T>
 __global__ void __launch_bounds__(256) softmax_xent_small_kernel(
-    const float* __restrict__ part, int ks, int64_t ld, int B, int Nt, const float* __restrict__ bias,
-    int64_t bias_sg, const int32_t* __restrict__ y, int64_t y_sg, T* __restrict__ delta, int64_t ld_d,
+    const float* part, int ks, int64_t ld, int B, int Nt, const float* bias,
+    int64_t bias_sg, const int32_t* y, int64_t y_sg, T* __restrict__ delta, int64_t ld_d,
     int64_t sg_d, float* __restrict__ row_loss, DeviceStatus* st) {
   pdl_wait();
   pdl_trigger();
@@ -246,9 +246,9 @@ __global__ void __launch_bounds__(256) bias_sgd_kernel(BiasSgdArgs<T> a) {
 // lse[g][b] = log sum_n exp(z[g][b][n]) from per-tile partials (m, s) = (max of z * log2(e),
 // sum of 2^(z * log2(e) - m)).  Block: 32 rows x 32 partial lanes; partials of one index are
 // contiguous over rows.
-__global__ void __launch_bounds__(1024) lse_combine_kernel(const float2* __restrict__ part, int parts, int B,
+__global__ void __launch_bounds__(1024) lse_combine_kernel(const float2* part, int parts, int B,
                                                             int64_t lse_sg, float* __restrict__ lse,
-                                                            const int32_t* __restrict__ y, int64_t y_sg, int Nt,
+                                                            const int32_t* y, int64_t y_sg, int Nt,
                                                             DeviceStatus* st) {
   __shared__ float sm[32][33], ss[32][33];
   pdl_wait();
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(1024) lse_combine_kernel(const float2* __restr
   }
 }
 
-__global__ void lse_row_loss_kernel(const float* __restrict__ lse, const float* __restrict__ zy, int B, int64_t lse_sg,
+__global__ void lse_row_loss_kernel(const float* lse, const float* zy, int B, int64_t lse_sg,
                                     float* __restrict__ row_loss) {
   pdl_wait();
   pdl_trigger();
@@ -306,7 +306,7 @@ __global__ void lse_row_loss_kernel(const float* __restrict__ lse, const float* 
 // any 4-byte boundary) in flight together.  With a thread per element 1200 rows of 1001 took 10.7 us,
 // now 6.7.
 template <typename T>
-__global__ void __launch_bounds__(128) stage_rows_kernel(const float* __restrict__ X, int64_t N0, int64_t group_row_stride,
+__global__ void __launch_bounds__(128) stage_rows_kernel(const float* X, int64_t N0, int64_t group_row_stride,
                                                          T* __restrict__ out, int64_t ld, int64_t sg) {
   struct alignas(2 * sizeof(T)) Pair { T a, b; };
   constexpr int U = 4;
@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(128) stage_rows_kernel(const float* __restrict
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t c = 2 * (p0 + u * 128);
-      v[u][0] = c < N0 ? __ldg(x + c) : 0.f;
-      v[u][1] = c + 1 < N0 ? __ldg(x + c + 1) : 0.f;
+      v[u][0] = c < N0 ? x[c] : 0.f;
+      v[u][1] = c + 1 < N0 ? x[c + 1] : 0.f;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -392,8 +392,8 @@ __device__ __forceinline__ void eval_fold(EvalPart& a, const EvalPart& b) {
   if (b.m > a.m || (b.m == a.m && b.arg < a.arg)) a.arg = b.arg;
   a.m = m;
 }
-__global__ void __launch_bounds__(kEvalThreads) eval_rows_wide_kernel(const float* __restrict__ logits, int64_t ld, int Nt,
-                                                                      const int32_t* __restrict__ y, double* loss_sum,
+__global__ void __launch_bounds__(kEvalThreads) eval_rows_wide_kernel(const float* logits, int64_t ld, int Nt,
+                                                                      const int32_t* y, double* loss_sum,
                                                                       long long* correct, DeviceStatus* st) {
   __shared__ EvalPart sh[kEvalThreads / 32];
   pdl_wait();
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_rows_wide_kernel(const floa
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int q = q0 + u * kEvalThreads;
-      const float4 t = q < quads ? __ldg(zq + q) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      const float4 t = q < quads ? zq[q] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
       v[4 * u] = t.x; v[4 * u + 1] = t.y; v[4 * u + 2] = t.z; v[4 * u + 3] = t.w;
 #pragma unroll
       for (int i = 0; i < 4; ++i) at[4 * u + i] = c0 + head + 4 * q + i;
@@ -477,8 +477,8 @@ __global__ void eval_finalize_kernel(const double* loss_sum, const long long* co
 }
 
 template <typename T>
-__global__ void splitk_mask_reduce_kernel(const float* __restrict__ part, int ks, int B, int64_t ld,
-                                          const T* __restrict__ mask, int64_t mask_sg, T* __restrict__ out,
+__global__ void splitk_mask_reduce_kernel(const float* part, int ks, int B, int64_t ld,
+                                          const T* mask, int64_t mask_sg, T* __restrict__ out,
                                           int64_t out_sg) {
   pdl_wait();
   pdl_trigger();
