@@ -19,16 +19,24 @@
 //   warps 0..7   load fp32 operands with plain vector loads (any base, any stride: rows of the full
 //                network need not be 16-byte aligned), one or two steps ahead of their use, and
 //                split them into the three bf16 planes in shared memory (128-byte swizzle, two
-//                slots of 32 k values)
+//                slots of 32 k values; four in a pair)
 //   warps 8..15  move finished 32-deep sums from tensor memory into registers, adding up
 //   one thread   issues the MMAs.  It is held up for as long as they take to start (60 cycles each,
 //                128 on a 256-column tile), so on narrow tiles, where adding up is quick, it has a
 //                warp of its own; on 256-column tiles, where such a warp would cost the
 //                other sixteen a quarter of their registers, it sits in warp 8
 // Three barriers per slot / accumulator connect them:
-//   full[b]   every loading warp has written its part of slot b
-//   done[b]   the MMAs on slot b are complete: accumulator b can be read, slot b rewritten
+//   full[s]   every loading warp has written its part of slot s
+//   done[s]   the MMAs on slot s are complete: their accumulator can be read, slot s rewritten
 //   taken[b]  every adding warp has read accumulator b: the MMAs after next may overwrite it
+// In a pair the MMAs of one CTA read both CTAs' slots.  That the other CTA's slot is written is passed on by one
+// thread on either side (peer[s]): it waits for its own CTA's loading warps, releases at cluster scope, and
+// is acquired there at cluster scope before it counts towards full[s].  Done two steps ahead by an
+// adding warp, the release (most of a microsecond) is off the chain; with a release by every loading
+// warp instead, which also waits for its loads in flight, 512 x 16384 x 16384 takes 1.3 times as long.
+// Against arrivals of the loading warps without cluster scope, which nothing orders against the MMAs' reads,
+// it costs 3 %.  taken[b] carries no memory, only completed tensor-memory reads, and is a relaxed
+// arrival at cluster scope.
 //
 // A product with few tiles is cut along k over the CTAs of a cluster (up to eight); each leaves
 // its sums in shared memory and the cluster adds them up in rank order, every CTA finishing its
@@ -145,8 +153,8 @@ struct Operand {
       off0 = (uint32_t)(r * 128 + ((u ^ r8) << 4));
     }
   }
-  // slot 1 holds k values 32..63 of the 64-deep swizzled rows
-  __device__ __forceinline__ uint32_t off(int slot) const { return MN ? off0 + slot * 4096u : off0 ^ (slot * 64u); }
+  // odd slots hold k values 32..63 of the 64-deep swizzled rows
+  __device__ __forceinline__ uint32_t off(int slot) const { return MN ? off0 + slot * 4096u : off0 ^ (slot * 64u); }   // slot 0 or 1
   // krem: k values left from the first one of the step
   __device__ __forceinline__ void fetch(float (&v)[UNITS][8], int krem) {
 #pragma unroll
@@ -193,8 +201,11 @@ __device__ __forceinline__ float fma_chain(const F32Problem& pr, int g, int m, i
   return acc;
 }
 
+// Slots of 32 k values (two to a swizzled row of 64): pairs have four, so that the relay's round trip
+// between the CTAs is not waited for (with two: 512 x 16384 x 16384 8 % slower).
+constexpr int slots_of(int pair) { return pair == 2 ? 4 : 2; }
 template <int BN, int PAIR>
-constexpr uint32_t ring_bytes() { return 3u * (BM + BN / PAIR) * 128u; }
+constexpr uint32_t ring_bytes() { return 3u * (BM + BN / PAIR) * 64u * slots_of(PAIR); }
 template <int BN, int PAIR>
 constexpr uint32_t smem_bytes() {
   const uint32_t tile = BM * (BN + 4) * 4;
@@ -276,10 +287,11 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
   constexpr int NACC = BN / 2;                         // sums per adding thread
   constexpr int PITCH = BN + 4;                        // floats per row of the finished tile in shared memory
   constexpr int DEPTH = BN == 256 ? 1 : 2;             // steps whose operands are on their way to registers
+  constexpr int SLOTS = slots_of(PAIR), LG = SLOTS == 4 ? 2 : 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float* tile_s = reinterpret_cast<float*>(smem);
-  __shared__ uint64_t full[2], done[2], taken[2];
+  __shared__ uint64_t full[SLOTS], done[SLOTS], taken[2], peer[SLOTS];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
@@ -297,11 +309,12 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
   }
   const int rank = cluster > 1 ? (int)cluster_ctarank() : 0;
   if (tid == 0) {
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&full[b], PAIR * kLoadWarps);
+    for (int b = 0; b < SLOTS; ++b) {
+      mbar_init(&full[b], kLoadWarps + (PAIR == 2 && rank == 0 ? 1 : 0));
       mbar_init(&done[b], 1);
-      mbar_init(&taken[b], PAIR * kAddWarps);
+      mbar_init(&peer[b], 1);
     }
+    for (int b = 0; b < 2; ++b) mbar_init(&taken[b], PAIR * kAddWarps);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -371,12 +384,13 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
   const uint64_t ad0 = A_MN ? make_desc(smem_u32(smem), 8192, 1024) : make_desc(smem_u32(smem), 16, 1024);
   const uint64_t bd0 = B_MN ? make_desc(smem_u32(smem) + A_BYTES, 8192, 1024) : make_desc(smem_u32(smem) + A_BYTES, 16, 1024);
   auto issue = [&](int i) -> bool {                          // the MMAs of step i
-    const int b = i & 1;
-    if (!mbar_wait(&full[b], (i >> 1) & 1, abortp, a.status, 21)) return false;
-    if (i >= 2 && !mbar_wait(&taken[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 23)) return false;
+    const int b = i & 1, sl = i & (SLOTS - 1);
+    if (!mbar_wait(&full[sl], (i >> LG) & 1, abortp, a.status, 21)) return false;
+    if (i >= 2 && !mbar_wait<PAIR == 2>(&taken[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 23)) return false;
     tc_fence_after();
     constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};   // low x high first, high x high last
-    const uint64_t ad = ad0 + (b ? (A_MN ? 4096 : 64) >> 4 : 0), bd = bd0 + (b ? (B_MN ? 4096 : 64) >> 4 : 0);
+    const uint32_t at = (uint32_t)(sl >> 1) * (3 * PLANE >> 4);
+    const uint64_t ad = ad0 + at + (b ? (A_MN ? 4096 : 64) >> 4 : 0), bd = bd0 + at + (b ? (B_MN ? 4096 : 64) >> 4 : 0);
 #pragma unroll
     for (int c = 0; c < 6; ++c)
 #pragma unroll
@@ -386,8 +400,15 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
         if (PAIR == 2) tc_mma_pair(tmem + b * BN, da, db, idesc, (c | k) != 0);
         else tc_mma(tmem + b * BN, da, db, idesc, (c | k) != 0);
       }
-    if (PAIR == 2) tc_commit_pair(&done[b]); else tc_commit(&done[b]);
+    if (PAIR == 2) tc_commit_pair(&done[sl]); else tc_commit(&done[sl]);
     return true;
+  };
+  // Pairs: passes on that the peer CTA's half of step i lies in its shared memory.
+  auto relay = [&](int i) {
+    if (i >= steps) return;
+    const int sl = i & (SLOTS - 1);
+    if (!mbar_wait<true>(rank ? &full[sl] : &peer[sl], (i >> LG) & 1, abortp, a.status, 24)) return;
+    if (rank) mbar_arrive_cluster<true>(map_to_cta(&peer[sl], 0)); else mbar_arrive(&full[sl]);
   };
 
   if (warp < kLoadWarps) {
@@ -411,21 +432,17 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
     }
     bool ok = true;
     auto step = [&](int i, float (&xa)[UA][8], float (&xb)[UB][8]) {
-      const int b = i & 1;
-      if (i >= 2) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&done[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 22));
+      const int sl = i & (SLOTS - 1);
+      if (i >= SLOTS) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&done[sl], ((i >> LG) & 1) ^ 1, abortp, a.status, 22));
         if (!ok) return;
       }
-      oa.template store<PLANE>(xa, smem, b);
-      ob.template store<PLANE>(xb, smem + A_BYTES, b);
+      uint8_t* slot = smem + (sl >> 1) * (3 * PLANE);
+      oa.template store<PLANE>(xa, slot, sl & 1);
+      ob.template store<PLANE>(xb, slot + A_BYTES, sl & 1);
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) {
-        // release at CTA scope: the bytes lie in this CTA's shared memory and the proxy fence
-        // has ordered them (cluster scope would wait for the loads in flight as well)
-        if (PAIR == 2) mbar_arrive_cluster<false>(map_to_cta(&full[b], 0));
-        else mbar_arrive(&full[b]);
-      }
+      if (lane == 0) mbar_arrive(&full[sl]);
       if (i + DEPTH < steps) {
         oa.fetch(xa, krem);
         ob.fetch(xb, krem);
@@ -443,18 +460,23 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
     if (BN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
     else asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     const bool issuer = BN == 256 && warp == kLoadWarps && lane == 0 && rank == 0;
+    const bool relayer = PAIR == 2 && warp == kLoadWarps + 1 && lane == 0;
+    constexpr int AHEAD = 2;                           // steps ahead of the one being added up, see above
     constexpr int W = BN == 256 ? 16 : 32;             // columns per tensor-memory load
     uint64_t acc[NACC / 2];
 #pragma unroll
     for (int i = 0; i < NACC / 2; ++i) acc[i] = 0;
     const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(((warp - kLoadWarps) >> 2) * NACC);
     if (issuer && steps > 0) issue(0);
+    if (relayer)
+      for (int i = 0; i < AHEAD; ++i) relay(i);
     __syncwarp();
     for (int i = 0; i < steps; ++i) {
       const int b = i & 1;
       if (issuer && i + 1 < steps) issue(i + 1);
+      if (relayer) relay(i + AHEAD);
       __syncwarp();
-      if (!__all_sync(0xffffffffu, mbar_wait(&done[b], (i >> 1) & 1, abortp, a.status, 20))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&done[i & (SLOTS - 1)], (i >> LG) & 1, abortp, a.status, 20))) break;
       tc_fence_after();
 #pragma unroll
       for (int c = 0; c < NACC; c += W) {
@@ -467,7 +489,7 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        if (PAIR == 2) mbar_arrive_cluster<false>(map_to_cta(&taken[b], 0));
+        if (PAIR == 2) mbar_arrive_relaxed_cluster(map_to_cta(&taken[b], 0));
         else mbar_arrive(&taken[b]);
       }
     }

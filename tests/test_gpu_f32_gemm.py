@@ -12,9 +12,11 @@ pytestmark = pytest.mark.gpu
 
 # 16 / 17 k values: the line to the short-contraction kernel; 64 / 65: its end; 31..33 and 127..129: edges
 # of a step and of a tile; odd widths: rows without 16-byte alignment; few tiles and a deep sum: k cut
-# over a cluster; the last two: pairs of CTAs.
+# over a cluster; (640, ...) and (511, ...): pairs of CTAs; the last four: pairs whose update takes 5 to 9 steps
+# through four operand slots.
 SIZES = [(1, 1, 1), (5, 16, 3), (24, 33, 17), (31, 65, 64), (33, 64, 16), (128, 128, 128), (129, 127, 65), (64, 5000, 130),
-         (200, 1001, 777), (40, 64, 512), (40, 64, 513), (9, 64, 1024), (9, 64, 1025), (640, 2048, 4100), (511, 1029, 8209)]
+         (200, 1001, 777), (40, 64, 512), (40, 64, 513), (9, 64, 1024), (9, 64, 1025), (640, 2048, 4100), (511, 1029, 8209),
+         (129, 4100, 4099), (161, 4099, 4100), (225, 4100, 4100), (260, 4099, 4099)]
 
 
 @pytest.mark.parametrize("B,n0,n1", SIZES)
