@@ -43,8 +43,8 @@
 // share of the tile's rows.
 //
 // Values that have no such decomposition (infinities, NaN, and magnitudes that round to infinity
-// in bf16) turn the products they enter into NaN.  The epilogue computes every result that is not
-// finite again as a chain of fp32 multiply-adds, so that the outcome is the one of fp32 arithmetic.
+// in bf16) turn the products they enter into NaN.  Every result that is not finite is computed again
+// as a chain of fp32 multiply-adds, see redo(), so that the outcome is the one of fp32 arithmetic.
 //
 // What bounds it: pairs, the tensor pipe (12 MMAs per step and 256 x 256 tile, about 1540 cycles) at the
 // clock the power limit leaves: 512 x 16384 x 16384 in 1.18 ms = 234 TFLOP/s of fp32 products,
@@ -189,93 +189,197 @@ struct Operand {
   }
 };
 
-// The result at (m, n) as a chain of multiply-adds (see the file's comment on non-finite values).
-template <int A_MN, int B_MN>
-__device__ __forceinline__ float fma_chain(const F32Problem& pr, int g, int m, int n) {
-  const float* A = pr.A + (long long)g * pr.a_sg + (A_MN ? m : m * pr.a_st);
-  const float* B = pr.B + (long long)g * pr.b_sg + (B_MN ? n : n * pr.b_st);
-  const long long as = A_MN ? pr.a_st : 1, bs = B_MN ? pr.b_st : 1;
-  float acc = 0.f;
-#pragma unroll 1
-  for (int k = 0; k < pr.K && acc == acc; ++k) acc = fmaf(A[k * as], B[k * bs], acc);
-  return acc;
-}
-
 // Slots of 32 k values (two to a swizzled row of 64): pairs have four, so that the relay's round trip
 // between the CTAs is not waited for (with two: 512 x 16384 x 16384 8 % slower).
 constexpr int slots_of(int pair) { return pair == 2 ? 4 : 2; }
 template <int BN, int PAIR>
 constexpr uint32_t ring_bytes() { return 3u * (BM + BN / PAIR) * 64u * slots_of(PAIR); }
+// k values, rows and columns of redo(), and its operands in shared memory behind the finished tile
+constexpr int kRedoK = 32, kRedoRows = 128, kRedoCols = 64;
+constexpr int kRedoBytes = kRedoK * (kRedoRows + 4 + kRedoCols + 4) * 4;
 template <int BN, int PAIR>
 constexpr uint32_t smem_bytes() {
-  const uint32_t tile = BM * (BN + 4) * 4;
+  const uint32_t tile = BM * (BN + 4) * 4 + kRedoBytes;
   return (ring_bytes<BN, PAIR>() > tile ? ring_bytes<BN, PAIR>() : tile) + 1024;
 }
 
-// Closing part of a tile, run by all threads: the finished sums lie in shared memory, row by row;
+// Barrier of the kThreads threads that run finish(); returns whether `p` holds in any of them.
+__device__ __forceinline__ bool finish_barrier(bool p) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred q, r;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "barrier.cta.red.or.pred r, 1, %2, q;\n\t"
+      "selp.u32 %0, 1, 0, r;\n\t}"
+      : "=r"(any) : "r"((uint32_t)p), "n"(kThreads) : "memory");
+  return any != 0;
+}
+__device__ __forceinline__ bool is_finite(float v) { return fabsf(v) <= FLT_MAX; }
+
+// Four adjacent results through the epilogue.
+__device__ __forceinline__ void emit(const F32Args& a, const F32Problem& pr, int g, int m, int n, float (&v)[4]) {
+  const int cnt = min(4, pr.N - n);
+  float* out = pr.out + (long long)g * pr.out_sg + (long long)m * pr.out_ld + n;
+  const bool wide = (pr.vec & 4) && cnt == 4;
+  float x[4] = {0.f, 0.f, 0.f, 0.f};                    // the epilogue's other input: bias, mask or the old weight
+  const float* src = pr.epi == EPI_SGD ? out
+                     : pr.epi == EPI_RELU_MASK ? pr.mask + (long long)g * pr.mask_sg + (long long)m * pr.mask_ld + n
+                     : pr.bias                 ? pr.bias + (long long)g * pr.bias_sg + n : nullptr;
+  if (src) {
+    if (wide) {
+      const float4 t = *reinterpret_cast<const float4*>(src);
+      x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < cnt) x[u] = src[u];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (pr.epi == EPI_SGD) v[u] = x[u] - a.lr * v[u];
+    else if (pr.epi == EPI_RELU_MASK) v[u] = x[u] > 0.f ? v[u] : 0.f;
+    else {
+      v[u] += x[u];
+      if (pr.epi == EPI_BIAS_RELU) v[u] = fmaxf(v[u], 0.f);
+    }
+  }
+  if (wide) {
+    *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < cnt) out[u] = v[u];
+  }
+}
+
+// 128 rows x 64 columns from (r0, c0) of the tile once more, as chains of fp32 multiply-adds with k ascending:
+// the results that finish() left behind because a sum of theirs is not finite.  32 k values at a time go
+// through shared memory (`slab`), the next ones on their way; a thread forms 4 x 4 results.  The k loop ends
+// when all of them are NaN.
+// An evaluation of 512 rows on 256-2048-2048-2048 with one hidden neuron at infinity: 0.79 ms (0.13 with
+// finite values, 12.8 with a chain per result and thread); on 1024-8192-8192-100 5.2 ms (0.44).
+template <int A_MN, int B_MN, int PITCH>
+__device__ __forceinline__ void redo(const F32Args& a, const F32Problem& pr, int g, int m0, int n0, int r0, int live, int c0,
+                                     const float* tile_s, float* slab, int tid) {
+  constexpr int PA = kRedoRows + 4, PB = kRedoCols + 4;  // rows stay 16-byte aligned
+  constexpr int NA = kRedoRows * kRedoK / kThreads, NB = kRedoCols * kRedoK / kThreads;
+  float* sa = slab;                                      // [kRedoK][PA]
+  float* sb = slab + kRedoK * PA;                        // [kRedoK][PB]
+  const int ty = tid / 16, tx = tid % 16;                // this thread's rows 4 ty.., columns 4 tx..
+  const float* A = pr.A + (long long)g * pr.a_sg;
+  const float* B = pr.B + (long long)g * pr.b_sg;
+  float acc[4][4];
+  uint32_t need = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      acc[i][j] = 0.f;
+      if (4 * ty + i < live && n0 + c0 + 4 * tx + j < pr.N && !is_finite(tile_s[(r0 + 4 * ty + i) * PITCH + c0 + 4 * tx + j]))
+        need |= 1u << (4 * i + j);
+    }
+  const bool any_here = __any_sync(0xffffffffu, need != 0);   // in this warp's 8 rows
+  float ra[NA], rb[NB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int e = tid + kThreads * u, k = k0 + (A_MN ? e / kRedoRows : e % kRedoK), m = A_MN ? e % kRedoRows : e / kRedoK;
+      const long long row = m0 + r0 + m;
+      ra[u] = m < live && k < pr.K ? A[A_MN ? k * pr.a_st + row : row * pr.a_st + k] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int e = tid + kThreads * u, k = k0 + (B_MN ? e / kRedoCols : e % kRedoK), n = n0 + c0 + (B_MN ? e % kRedoCols : e / kRedoK);
+      rb[u] = n < pr.N && k < pr.K ? B[B_MN ? k * pr.b_st + n : n * pr.b_st + k] : 0.f;
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < pr.K; k0 += kRedoK) {
+    bool alive = false;                                  // a result that is not NaN yet
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) alive |= (need >> (4 * i + j) & 1) && acc[i][j] == acc[i][j];
+    if (!finish_barrier(alive)) break;
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int e = tid + kThreads * u;
+      sa[(A_MN ? e / kRedoRows : e % kRedoK) * PA + (A_MN ? e % kRedoRows : e / kRedoK)] = ra[u];
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int e = tid + kThreads * u;
+      sb[(B_MN ? e / kRedoCols : e % kRedoK) * PB + (B_MN ? e % kRedoCols : e / kRedoK)] = rb[u];
+    }
+    finish_barrier(false);
+    if (k0 + kRedoK < pr.K) fetch(k0 + kRedoK);
+    if (!any_here) continue;
+#pragma unroll 4
+    for (int k = 0; k < kRedoK; ++k) {
+      const float4 x = *reinterpret_cast<const float4*>(sa + k * PA + 4 * ty), y = *reinterpret_cast<const float4*>(sb + k * PB + 4 * tx);
+      const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xs[i], ys[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (!(need >> (4 * i) & 15)) continue;
+    const int r = r0 + 4 * ty + i, c = c0 + 4 * tx;
+    float v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = need >> (4 * i + j) & 1 ? acc[i][j] : tile_s[r * PITCH + c + j];
+    emit(a, pr, g, m0 + r, n0 + c, v);
+  }
+}
+
+// Closing part of a tile, run by kThreads threads: the finished sums lie in shared memory, row by row;
 // apply the epilogue to this CTA's share of the rows and write the result.
 template <int A_MN, int B_MN, int BN, int PAIR>
 __device__ __forceinline__ void finish(const F32Args& a, const F32Problem& pr, int g, int m0, int n0, int rank, int cluster,
-                                       const float* tile_s, int tid) {
+                                       float* tile_s, int tid) {
   constexpr int PITCH = BN + 4, Q = BN / 4;             // Q 4-column pieces of a row
   const int share = PAIR == 1 ? BM / cluster : BM;      // rows this CTA finishes
   const int r_lo = PAIR == 1 ? rank * share : 0;
   const int live = min(share, pr.M - m0 - r_lo);        // those inside the result
   const uint32_t tile_u = smem_u32(tile_s);
+  bool left = false;
 #pragma unroll 2
   for (int e = tid; e < live * Q; e += kThreads) {
     const int r = r_lo + e / Q, c4 = (e % Q) * 4, m = m0 + r, n = n0 + c4;
     if (n >= pr.N) continue;
     float v[4];
+    float4* mine = reinterpret_cast<float4*>(tile_s + r * PITCH + c4);
     if (PAIR == 1 && cluster > 1) {
-      const uint32_t mine = tile_u + (uint32_t)(r * PITCH + c4) * 4;
       v[0] = v[1] = v[2] = v[3] = 0.f;
       for (int s = 0; s < cluster; ++s) {               // in rank order: a fixed sum
         uint32_t addr;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(mine), "r"(s));
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(tile_u + (uint32_t)(r * PITCH + c4) * 4), "r"(s));
         const float4 t = ld_cluster4(addr);
         v[0] += t.x; v[1] += t.y; v[2] += t.z; v[3] += t.w;
       }
     } else {
-      const float4 t = *reinterpret_cast<const float4*>(tile_s + r * PITCH + c4);
+      const float4 t = *mine;
       v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
     }
-    const int cnt = min(4, pr.N - n);
+    bool ok = true;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (!(fabsf(v[u]) <= FLT_MAX) && u < cnt) v[u] = fma_chain<A_MN, B_MN>(pr, g, m, n + u);
-    float* out = pr.out + (long long)g * pr.out_sg + (long long)m * pr.out_ld + n;
-    const bool wide = (pr.vec & 4) && cnt == 4;
-    float x[4] = {0.f, 0.f, 0.f, 0.f};                  // the epilogue's other input: bias, mask or the old weight
-    const float* src = pr.epi == EPI_SGD ? out
-                       : pr.epi == EPI_RELU_MASK ? pr.mask + (long long)g * pr.mask_sg + (long long)m * pr.mask_ld + n
-                       : pr.bias                 ? pr.bias + (long long)g * pr.bias_sg + n : nullptr;
-    if (src) {
-      if (wide) {
-        const float4 t = *reinterpret_cast<const float4*>(src);
-        x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
-      } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (u < cnt) x[u] = src[u];
-      }
+    for (int u = 0; u < 4; ++u) ok &= is_finite(v[u]) || n + u >= pr.N;
+    if (ok) {
+      emit(a, pr, g, m, n, v);
+    } else {                                            // nobody else reads these rows of this CTA's sums
+      *mine = make_float4(v[0], v[1], v[2], v[3]);
+      left = true;
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (pr.epi == EPI_SGD) v[u] = x[u] - a.lr * v[u];
-      else if (pr.epi == EPI_RELU_MASK) v[u] = x[u] > 0.f ? v[u] : 0.f;
-      else {
-        v[u] += x[u];
-        if (pr.epi == EPI_BIAS_RELU) v[u] = fmaxf(v[u], 0.f);
-      }
-    }
-    if (wide) {
-      *reinterpret_cast<float4*>(out) = make_float4(v[0], v[1], v[2], v[3]);
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (u < cnt) out[u] = v[u];
-    }
+  }
+  if (finish_barrier(left)) {
+    float* slab = tile_s + BM * PITCH;
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN && n0 + c0 < pr.N; c0 += kRedoCols)
+      redo<A_MN, B_MN, PITCH>(a, pr, g, m0, n0, r_lo, live, c0, tile_s, slab, tid);
   }
 }
 
