@@ -302,9 +302,9 @@ __global__ void lse_row_loss_kernel(const float* lse, const float* zy, int B, in
   if (b < B) row_loss[(int64_t)g * B + b] = lse[(int64_t)g * lse_sg + b] - zy[(int64_t)g * lse_sg + b];
 }
 
-// One block per row; a thread rounds four pairs of adjacent columns, their eight 4-byte loads (rows start at
-// any 4-byte boundary) in flight together.  With a thread per element 1200 rows of 1001 took 10.7 us,
-// now 6.7.
+// A thread rounds four pairs of adjacent columns, their eight 4-byte loads (rows start at any 4-byte boundary)
+// in flight together.  One block per row, or several (blockIdx.z) where the rows alone are too few to
+// fill the GPU.  With a thread per element 1200 rows of 1001 took 10.7 us, now 6.7.
 template <typename T>
 __global__ void __launch_bounds__(128) stage_rows_kernel(const float* X, int64_t N0, int64_t group_row_stride,
                                                          T* __restrict__ out, int64_t ld, int64_t sg) {
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(128) stage_rows_kernel(const float* X, int64_t
   const int b = blockIdx.x, g = blockIdx.y;
   const float* x = X + ((int64_t)g * group_row_stride + b) * N0;
   Pair* o = reinterpret_cast<Pair*>(out + (int64_t)g * sg + (int64_t)b * ld);   // ld is even, rows of `out` 16-byte aligned
-  for (int64_t p0 = threadIdx.x; p0 < ld / 2; p0 += U * 128) {
+  for (int64_t p0 = blockIdx.z * (U * 128) + threadIdx.x; p0 < ld / 2; p0 += gridDim.z * (U * 128)) {
     float v[U][2];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -590,7 +590,10 @@ template void bias_sgd<bf16>(const Launch&, const BiasSgdArgs<bf16>&);
 template <typename T>
 void stage_rows(const Launch& L, const float* X, int64_t N0, int64_t group_row_stride, int G, int B,
                 T* out, int64_t ld, int64_t sg) {
-  launch_pdl(stage_rows_kernel<T>, dim3((unsigned)B, (unsigned)G), dim3(128), 0, L.stream, X, N0, group_row_stride, out, ld, sg);
+  // sixteen blocks fit on an SM, 2368 on the GPU; a block beyond that, or beyond a row's 1024-column pieces, has nothing to do
+  const int64_t pieces = std::max<int64_t>(1, std::min(ceil_div(ld, 1024), 2368 / ((int64_t)B * G)));
+  launch_pdl(stage_rows_kernel<T>, dim3((unsigned)B, (unsigned)G, (unsigned)pieces), dim3(128), 0, L.stream, X, N0,
+             group_row_stride, out, ld, sg);
   L.count();
 }
 template void stage_rows<float>(const Launch&, const float*, int64_t, int64_t, int, int, float*,
