@@ -376,10 +376,14 @@ namespace {
 
 // Matrices of this many packed elements or more are moved by the kernel made for their kind (first
 // layer: column permutation, last layer: whole rows); smaller ones by blocks of the shared launch,
-// whose scattered 4-byte accesses L2 still absorbs.  Partition + reassembly of 1024-4096-4096-35,
-// S = 4 (4.2 M elements a layer): 98 us with a launch of its own for the first layer, 86 us without;
-// of 3072-16384-16384-10, S = 8 (50 M): 740 against 1180 us.
-constexpr int64_t kOwnLaunch = 1 << 24;
+// whose scattered 4-byte accesses L2 still absorbs.  Partition + reassembly with the large matrix in the shared
+// launch and in one of its own, S = 1 / 16 subnets, bf16 operands, us:
+//   first layer  1024 x 4096   51 / 62   against  55 / 59     last layer  3072 x 1024  44 / 44   against  38 / 39
+//                1536 x 4096   58 / 77            59 / 66                 4096 x 1024  50 / 50            41 / 43
+//                768 x 16384  114 / 144          111 / 121                8192 x 1024  75 / 75            50 / 53
+//   3072 x 16384, S = 8: 1180 against 740                                 5003 x 3000 112 / 114           74 / 76
+// The column permutation has a fixed part of some 10 us, which few subnets do not repay below 12 M.
+constexpr int64_t kOwnColumns = 12 << 20, kOwnRows = 3 << 20;
 
 template <bool GATHER>
 void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
@@ -395,12 +399,12 @@ void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
   };
   for (int i = 0; i < n; ++i) {
     const SliceJob& j = jobs[i];
-    if (!j.mean && j.S * j.m.rows_pad * j.m.ld >= kOwnLaunch) {
-      if (staged_ok(j.m, j.S) && launch_permute_cols<GATHER>(L, j.W, j.m, j.S, j.master, j.opw, st)) continue;
-      if (rows_ok(j.m)) {
-        launch_rows<GATHER>(L, j.W, j.m, j.S, j.master, j.opw);
-        continue;
-      }
+    const int64_t elements = j.mean ? 0 : j.S * j.m.rows_pad * j.m.ld;
+    if (elements >= kOwnColumns && staged_ok(j.m, j.S) && launch_permute_cols<GATHER>(L, j.W, j.m, j.S, j.master, j.opw, st))
+      continue;
+    if (elements >= kOwnRows && rows_ok(j.m)) {
+      launch_rows<GATHER>(L, j.W, j.m, j.S, j.master, j.opw);
+      continue;
     }
     const int64_t x = ceil_div(j.mean ? j.m.full_cols : j.m.ld, kThreads), y = j.mean ? 1 : ceil_div(j.m.rows_pad, kRowsPerCta);
     const int64_t b = x * y * (j.mean ? 1 : j.S);

@@ -1,0 +1,54 @@
+"""Gather and scatter of first- and last-layer matrices around the sizes at which they get a launch of their own:
+values bit for bit, and a rate where the shared launch's scattered 4-byte accesses fall behind."""
+import pytest
+import torch
+
+from oracle import ist_oracle as O
+from paper_1910_02120_b200 import api
+
+pytestmark = pytest.mark.gpu
+
+
+def _context(dims, S, precision=None):
+    g = torch.Generator(device="cuda").manual_seed(S)
+    W = [torch.randn(a, b, device="cuda", generator=g) for a, b in zip(dims, dims[1:])]
+    b = [torch.randn(n, device="cuda", generator=g) for n in dims[1:]]
+    ctx = api.Ist(dims, S, api.IST_FP32 if precision is None else precision, 4)
+    ctx.bind_weights(W, b)
+    return ctx, W, b
+
+
+# packed elements of the first / last layer: just below and above 12 * 2^20 and 3 * 2^20, widths of every alignment
+@pytest.mark.parametrize("dims,S", [([1535, 8192, 8], 4), ([1537, 8192, 8], 4), ([1540, 8189, 8], 3), ([8, 3071, 1024], 1),
+                                    ([8, 3073, 1024], 7), ([8, 3100, 1031], 16), ([8, 5003, 3001], 16)])
+def test_values(dims, S):
+    ctx, W, b = _context(dims, S)
+    before = [w.clone() for w in W + b]
+    ctx.partition(7)
+    parts = O.partition(7, dims, S)
+    for s in {0, S - 1}:
+        cols = torch.as_tensor(O.group(parts, 1, s), device="cuda").long()
+        assert torch.equal(ctx.get_subnet_params(1, s)[0], before[0][:, cols])
+        assert torch.equal(ctx.get_subnet_params(2, s)[0], before[1][cols])
+    for w in W:
+        w.fill_(float("nan"))                       # every entry belongs to a subnet and comes back
+    ctx.reassemble()
+    ctx.sync_status()
+    assert all(torch.equal(p, q) for p, q in zip(W + b, before))
+
+
+@pytest.mark.parametrize("dims,S", [([8, 5003, 3000], 4), ([8, 1000, 15000], 16)])
+def test_whole_rows_are_copied_at_a_fair_rate(dims, S):
+    """15 M weights: 8 bytes each are read and 10 written in the two directions, 270 MB; 5 TB/s and four launches
+    of 5 us each are 74 us."""
+    ctx, W, b = _context(dims, S, api.IST_BF16)
+    best = 1e30
+    for seed in range(8):
+        ctx.profile(True)
+        ctx.partition(seed)
+        ctx.reassemble()
+        took = ctx.profile_read()
+        ctx.profile(False)
+        best = min(best, took["gather"][1] + took["scatter"][1])
+    ctx.sync_status()
+    assert best <= 0.074, best
