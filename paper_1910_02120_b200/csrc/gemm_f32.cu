@@ -4,11 +4,15 @@
 //
 //   C[g](m, n) = sum_k A[g](m, k) * B[g](n, k)
 //
-// Every fp32 operand is the exact sum of three bf16 numbers (8 + 8 + 8 significant bits):
-// x = h + m + l with h = bf16(x), m = bf16(x - h), l = x - h - m.  A product of two of them is then
-// nine bf16 products, of which the six of weight 2^-16 and above are formed:
-//   a b = ah bh + (ah bm + am bh) + (ah bl + am bm + al bh) + O(2^-26 |a b|),
-// and the three left out are below the rounding of a single fp32 multiplication (2^-24).
+// Every fp32 operand is split into three bf16 numbers (8 + 8 + 8 significant bits):
+// x = h + 2^-8 m + 2^-16 l with h = bf16(x), m = bf16(2^8 (x - h)), l = 2^8 (2^8 (x - h) - m).  A
+// product of two of them is then nine bf16 products, of which the six of weight 2^-16 and above are formed:
+//   a b = ah bh + 2^-8 (ah bm + am bh) + 2^-16 (ah bl + am bm + al bh) + O(2^-26 |a b|),
+// and the three left out are below the rounding of a single fp32 multiplication (2^-24).  The weights
+// are applied to the accumulator between the groups, by the MMA's own scaling of it.  With the scaled parts
+// the split is exact down to |x| = 2^-118, where l nears bf16's smallest normal number, and loses less than
+// 1.3e-8 of x from there to fp32's smallest normal number (with parts of their own size it lost bits from 2^-110
+// on and 1.2e-5 at the end; the scaling costs 1024 x 1024 x 256 of four groups some 2 %).
 // The tensor core's own accumulation is not relied on over long sums: 32 values of k are
 // accumulated in tensor memory (the small products first, so that only the last two
 // instructions act on a sum of full size), and the 32-deep sums are then added up in fp32
@@ -100,12 +104,29 @@ __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
+__device__ __forceinline__ uint64_t pack2(uint32_t lo, uint32_t hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
+  return v;
+}
+// (x, y) - (the two bf16 numbers in `part`), times 2^8: both steps are exact.
+__device__ __forceinline__ void rest2(float& x, float& y, uint32_t part) {
+  uint64_t v = pack2(__float_as_uint(x), __float_as_uint(y));
+  const uint64_t p = pack2(part << 16, part & 0xffff0000u), c = pack2(0x43800000u, 0x43800000u);   // 256
+  uint32_t lo, hi;
+  asm("sub.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(p));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(c));
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
+  x = __uint_as_float(lo);
+  y = __uint_as_float(hi);
+}
 // Two floats into their three bf16 parts, packed pairwise.
 __device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
   h = cvt_bf16x2(x, y);
-  const float xr = x - __uint_as_float(h << 16), yr = y - __uint_as_float(h & 0xffff0000u);
-  m = cvt_bf16x2(xr, yr);
-  l = cvt_bf16x2(xr - __uint_as_float(m << 16), yr - __uint_as_float(m & 0xffff0000u));
+  rest2(x, y, h);
+  m = cvt_bf16x2(x, y);
+  rest2(x, y, m);
+  l = cvt_bf16x2(x, y);
 }
 __device__ __forceinline__ void add2(uint64_t& acc, uint32_t lo, uint32_t hi) {
   uint64_t v;
@@ -501,8 +522,13 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
       for (int k = 0; k < KH / 16; ++k) {
         const uint64_t da = ad + ((pa[c] * PLANE + k * (A_MN ? 2048 : 32)) >> 4);
         const uint64_t db = bd + ((pb[c] * PLANE + k * (B_MN ? 2048 : 32)) >> 4);
-        if (PAIR == 2) tc_mma_pair(tmem + b * BN, da, db, idesc, (c | k) != 0);
-        else tc_mma(tmem + b * BN, da, db, idesc, (c | k) != 0);
+        if ((c == 3 || c == 5) && k == 0) {              // from one weight to the next: 2^8
+          if (PAIR == 2) tc_mma_pair<8>(tmem + b * BN, da, db, idesc, 1);
+          else tc_mma<8>(tmem + b * BN, da, db, idesc, 1);
+        } else {
+          if (PAIR == 2) tc_mma_pair(tmem + b * BN, da, db, idesc, (c | k) != 0);
+          else tc_mma(tmem + b * BN, da, db, idesc, (c | k) != 0);
+        }
       }
     if (PAIR == 2) tc_commit_pair(&done[sl]); else tc_commit(&done[sl]);
     return true;
