@@ -51,12 +51,13 @@
 // as a chain of fp32 multiply-adds, see redo(), so that the outcome is the one of fp32 arithmetic.
 //
 // What bounds it: pairs, the tensor pipe (12 MMAs per step and 256 x 256 tile, about 1540 cycles) at the
-// clock the power limit leaves: 512 x 16384 x 16384 in 1.18 ms = 234 TFLOP/s of fp32 products,
-// 1.40 PFLOP/s of bf16 ones (the same product on the CUDA cores, 128 x 128 tiles: 6.5 ms).  Single
+// clock the power limit leaves: 512 x 16384 x 16384 in 1.23 ms = 223 TFLOP/s of fp32 products,
+// 1.34 PFLOP/s of bf16 ones (the same product on the CUDA cores, 128 x 128 tiles: 6.5 ms).  Single
 // CTAs, the chain wait - split - barrier - MMA of a step, about 0.95 us (256 x 1024 x 1024 of
-// four groups 164 -> 27 us, 1024 x 1024 x 256 of four groups 96 -> 25 us).  Error of a K-term sum
+// four groups 164 -> 28 us, 1024 x 1024 x 256 of four groups 96 -> 25 us).  Error of a K-term sum
 // against 64 bits, relative 2-norm, before -> now: K = 64 1.0e-7 -> 6e-8, 1024 4.1e-7 -> 1.2e-7,
-// 16384 1.6e-6 -> 4.1e-7.
+// 16384 1.6e-6 -> 4.1e-7.  The tensor core cuts its sums off instead of rounding them: sums of
+// terms of one sign come out 4.5e-8 too small on average, at any depth (terms of both signs: below 2e-8).
 //
 // Every wait is bounded, see tc_ptx.cuh.
 #include <algorithm>
@@ -676,11 +677,6 @@ bool launch_bn(const Launch& L, const F32Args& t, int bn, int pair, int cluster)
   return launch<A_MN, B_MN, 64, 1>(L, t, cluster);
 }
 
-// Tile shape and k split of a launch, and its estimated time in microseconds: as many rounds of
-// tiles as the SMs need, each a fixed part (start, first operands, epilogue) and so much per
-// 32-deep step.  Constants fitted to 12 products of 64 x 64 x 32 to 512 x 16384 x 3072 (measured
-// 5.3 to 244 us, estimates within 25 %); 64-column tiles pay off only where 128-column ones leave
-// SMs idle or the product is narrow, pairs from about 64 tiles of 256 x 256 on.
 // Clusters of two, four and eight CTAs that can run at once (a GPU processing cluster holds a whole
 // number of them): 16 of eight did not all fit and took two rounds (128 x 512 x 784 of two groups, 64
 // columns: 18.5 us in clusters of eight, 11.7 us in clusters of four).
@@ -709,6 +705,11 @@ int clusters_at_once(int cluster) {
   return n[cluster == 1 ? 0 : cluster == 2 ? 1 : cluster == 4 ? 2 : 3];
 }
 
+// Tile shape and k split of a launch, and its estimated time in microseconds: as many rounds of
+// tiles as the SMs need, each a fixed part (start, first operands, epilogue) and so much per
+// 32-deep step.  Constants fitted to 12 products of 64 x 64 x 32 to 512 x 16384 x 3072 (measured
+// 5.3 to 244 us, estimates within 25 %); 64-column tiles pay off only where 128-column ones leave
+// SMs idle or the product is narrow, pairs from about 64 tiles of 256 x 256 on.
 struct Shape { int bn, pair, cluster; double us; };
 Shape pick_shape(const GemmArgs<float>* ga, int n) {
   const int sms = 148;
@@ -762,11 +763,8 @@ bool gemm_f32(const Launch& L, const GemmArgs<float>* ga, int n, const BiasSgdAr
   }
   if ((!a_k && !a_m) || (!b_k && !b_n)) return false;
   const bool a_mn = !a_k, b_mn = !b_k || (a_mn && b_n);
-  Shape sh = pick_shape(ga, n);
+  const Shape sh = pick_shape(ga, n);
   if (short_wins(ga, n, sh.us) && gemm_short(L, ga, n, bias)) return true;
-#ifdef F32_PROBE
-  if (getenv("FBN")) { sh.bn = atoi(getenv("FBN")); sh.pair = sh.bn == 256 ? 2 : 1; sh.cluster = atoi(getenv("FCL")); }
-#endif
   F32Args t{};
   t.n_problems = n;
   t.ksplit = sh.cluster;

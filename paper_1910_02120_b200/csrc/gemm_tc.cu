@@ -1156,8 +1156,10 @@ bool gemm_tc_wait_selftest(const Launch& L, DeviceStatus* st, long long limit_cy
 // (120-26586-2688-509, S = 9, 128 rows: 804 -> 733 us against pairs; 3072-16384-16384-10 within 1 %).  Up to
 // 320 rows still where the pairs' tiles hang over the matrices' edges by more than 15 % (the same
 // network at 224 rows 890 -> 845 us; 1024-4096-4096-35, which pairs tile exactly, 477 against 484 us).  Not
-// with an output layer of many thousand classes, whose update streams from DRAM for milliseconds
-// (135909-1024-670091, S = 8, 256 rows: 54.3 ms with 128 columns, 56.8 with 64).
+// with a layer of more than 8192 columns, whose update streams from DRAM: an output layer of 670,091
+// classes behind 1024 neurons, S = 8, 256 rows, 54.3 ms with 128 columns and 56.8 with 64; 30,000 classes at 128 rows
+// 851 and 874 us.  Hidden layers of 9000 to 20,000 neurons would gain 1 to 4 % up to 128 rows (512-20000-2048-10,
+// 64 rows: 1298 -> 1281 us) and nothing above.
 struct TileChoice { int bn, pair; };
 TileChoice pick_tile(const GemmArgs<bf16>* a, int n, int epi) {
   const int sms = sm_count();

@@ -371,7 +371,8 @@ bool gemm(ist_ctx* c, const GemmArgs<float>& a) { return gemm_f32(c->launch(), &
 bool gemm(ist_ctx* c, const GemmArgs<bf16>& a) { return gemm_tc(c->launch(), a, c->status()); }
 
 // Several products of one kind in as few launches as possible.  fp32 operands: weight updates, which do not
-// depend on one another, gemm_f32_max_batch() to a launch (the first with the bias work), others one launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
+// depend on one another, gemm_f32_max_batch() to a launch (the first with the bias work), others one
+// launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
 // with `chained`, every problem reads the output of the one before it and the launch orders
 // their tiles through the row-block counters of `region` (one set per problem, indexed by
 // `layer0 + i`; `totals` are the context's running sums for that region).
@@ -718,7 +719,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     // rule; deltas beyond its size come from DRAM a second time there, as they would for the bias
     // kernel, but in the shadow of the update).  With fp32 operands it is blocks behind the tiles of the
     // weight-update launch.  What is left for the bias kernel is a sparse first layer's bias on the bf16
-    // path, and fp32 networks of more layers than one such launch takes along.
+    // path, and fp32 networks of more bias work (see bias_beside) or more layers than such a launch takes along.
     const bool sparse_first = X->kind == IST_X_CSR && t > 1;
     size_t delta_bytes = 0;
     for (int l = 1; l <= t; ++l) delta_bytes += (size_t)S * B * c->ld[l] * sizeof(T);

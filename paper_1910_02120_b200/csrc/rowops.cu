@@ -383,7 +383,7 @@ __global__ void eval_rows_kernel(const float* __restrict__ logits, int64_t ld, i
 // ranges are merged in rank order through distributed shared memory.  Two passes of 4-byte loads by
 // one block per row held too few bytes in flight for the 2.7 MB rows of 670,091 classes (256 rows:
 // 2.46 ms; now 0.21 ms).
-constexpr int kEvalThreads = 512, kEvalCols = 65536;   // columns of a CTA, at most
+constexpr int kEvalThreads = 512, kEvalCols = 65536;   // a row is cut until a CTA has no more columns, or by eight
 struct EvalPart { float m, s; int arg; };
 // Folds b into a; ties go to the lower index.  An empty part carries (-inf, 0).
 __device__ __forceinline__ void eval_fold(EvalPart& a, const EvalPart& b) {
