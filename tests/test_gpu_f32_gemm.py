@@ -5,17 +5,19 @@ kinds of product by themselves: z = X W + b through the loss, d(loss)/dX = delta
 import pytest
 import torch
 
-from paper_1910_02120_b200 import api
+from paper_1910_02120_b200 import api, synth
+from tests import helpers as H
 
 pytestmark = pytest.mark.gpu
 
 
 # 16 / 17 k values: the line to the short-contraction kernel; 64 / 65: its end; 31..33 and 127..129: edges
 # of a step and of a tile; odd widths: rows without 16-byte alignment; few tiles and a deep sum: k cut
-# over a cluster; (640, ...) and (511, ...): pairs of CTAs; the last four: pairs whose update takes 5 to 9 steps
-# through four operand slots.
+# over a cluster; (640, 2048, 4100) and (511, ...): pairs of CTAs in the forward product and the update, (640, 4100,
+# 1029) in the input gradient as well; the last four: pairs whose update takes 5 to 9 steps through four operand slots.
 SIZES = [(1, 1, 1), (5, 16, 3), (24, 33, 17), (31, 65, 64), (33, 64, 16), (128, 128, 128), (129, 127, 65), (64, 5000, 130),
          (200, 1001, 777), (40, 64, 512), (40, 64, 513), (9, 64, 1024), (9, 64, 1025), (640, 2048, 4100), (511, 1029, 8209),
+         (640, 4100, 1029),
          (129, 4100, 4099), (161, 4099, 4100), (225, 4100, 4100), (260, 4099, 4099)]
 
 
@@ -73,3 +75,39 @@ def test_values_without_a_bf16_decomposition():
     loss, _ = ctx.eval(X[2:].contiguous(), y[2:].contiguous(), 1)
     assert abs(loss.item() - torch.log(torch.tensor(float(n1))).item()) <= 1e-5
     ctx.sync_status()
+
+
+# 256 blocks of bias work ride on the update launch, 368 go out as a launch of their own (the line is 296)
+@pytest.mark.parametrize("classes", [700, 1100])
+@pytest.mark.parametrize("B", [20, 70])
+def test_bias_updates_beside_and_before_the_weight_updates(classes, B):
+    w = synth.Workload("bias", (20, 3200, classes), S=16, B=B, K=2, rounds=1, precision="fp32", x_dist="normal", lr=0.5, seed=B)
+    W, b, data = H.make_problem(w)
+    o, _, oloss = H.oracle_round(w, W, b, data, 5)
+    _, gW, gb, _, gloss = H.gpu_round(w, W, b, data, 5)
+    H.assert_close(gloss, oloss, 1e-4, "losses")
+    for l in range(len(W)):
+        H.assert_close(gW[l], o.W[l], 1e-4, f"W_{l + 1}")
+        H.assert_close(gb[l] - b[l], o.b[l] - b[l], 1e-3, f"update of b_{l + 1}")
+
+
+@pytest.mark.parametrize("B,n0,n1", [(64, 512, 64), (1024, 512, 64), (16384, 512, 64), (1024, 4096, 4096)])
+def test_mean_signed_error(B, n0, n1):
+    """Accumulation that cuts off instead of rounding has a sign.  Logits far apart make every row's delta +-1/B in two
+    columns, so the update there is the mean of X's rows and all products are exact: what is seen is the summing.  Sums
+    of positive terms, the worst case, stay within the rounding of one number on average; their spread is that of B / 32
+    additions, each off by a uniform share of 2^-24 of a sum that grows to its end, beside a few roundings."""
+    g = torch.Generator(device="cuda").manual_seed(B)
+    X = torch.rand(B, n0, device="cuda", generator=g) + 0.5
+    W, b = torch.zeros(n0, n1, device="cuda"), torch.zeros(n1, device="cuda")
+    b[0] = 300.0
+    ctx = api.Ist([n0, n1], 1, api.IST_FP32, B)
+    ctx.bind_weights([W], [b])
+    ctx.partition(1)
+    ctx.local_steps(X, torch.ones(B, device="cuda", dtype=torch.int32), -1.0, 1, B)
+    ctx.reassemble()
+    ctx.sync_status()
+    want = X.double().mean(0)
+    for column in (W[:, 0], -W[:, 1]):
+        err = (column.double() - want) / want
+        assert err.mean().abs() <= 2 ** -24 and err.square().mean().sqrt() <= 2 ** -24 * (4 + (B / 32) ** 0.5 / 4)

@@ -12,7 +12,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("rule", ["balanced", "iid"])
 @pytest.mark.parametrize("hidden,S", [((1, 2), 1), ((7, 8, 9), 7), ((1023, 1024, 1025), 3), ((8191, 8193), 5),
-                                      ((16384, 16385, 2049), 16), ((40,) * 11, 4), ((700,), 700)])
+                                      ((16384, 16385, 2049), 16), ((40,) * 11, 4), ((700,), 700),
+                                      # above 2^14 neurons a layer takes the whole-GPU launches; the second draw mixes both routes
+                                      ((16385,), 16), ((16384, 40, 16385, 24), 16)])
 def test_partition_and_reassembly(hidden, S, rule):
     dims = [3, *hidden, 5]
     g = torch.Generator(device="cuda").manual_seed(S)
