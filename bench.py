@@ -83,11 +83,13 @@ def measured_traffic(workload_name: str, kernel_class: str, work_per_launch_now:
     """DRAM bytes per launch of this class from the recorded ncu capture, scaled by the launch's
     algorithmic work in the record's unit (bytes for HBM-bound classes, flop for the contractions;
     the capture may be of a reduced case of the same kernel), or None when there
-    is no capture for this workload and class or the kernel source has changed since."""
+    is no capture for this workload and class or the kernel's sources (one file, or a list of them
+    hashed one after the other) have changed since."""
     import hashlib
     try:
         rec = json.load(open(TRAFFIC_FILE))[workload_name][kernel_class]
-        src = open(os.path.join(CSRC, rec["source"]), "rb").read()
+        files = rec["source"] if isinstance(rec["source"], list) else [rec["source"]]
+        src = b"".join(open(os.path.join(CSRC, f), "rb").read() for f in files)
     except (OSError, KeyError, ValueError):
         return None
     if hashlib.sha256(src).hexdigest() != rec["source_sha256"]:

@@ -90,3 +90,21 @@ def test_recorded_dram_traffic_is_dropped_when_the_kernel_source_changes(tmp_pat
     assert bench.measured_traffic("V", "upd", 200.0) is None
     src.write_text("kernel v2")
     assert bench.measured_traffic("W", "upd", 200.0) is None
+
+
+def test_recorded_dram_traffic_covers_the_headers_it_names(tmp_path, monkeypatch):
+    """A record may name several sources; an edit of any of them voids it.  The tracked records name the header of
+    instruction wrappers beside the kernel."""
+    import hashlib
+    (tmp_path / "k.cu").write_text("kernel")
+    (tmp_path / "k.cuh").write_text("wrappers")
+    rec = {"W": {"upd": {"dram_bytes_per_launch": 110.0, "algorithmic_per_launch": 100.0, "unit": "bytes",
+                         "source": ["k.cu", "k.cuh"], "source_sha256": hashlib.sha256(b"kernelwrappers").hexdigest()}}}
+    tracked = bench.TRAFFIC_FILE
+    (tmp_path / "t.json").write_text(json.dumps(rec))
+    monkeypatch.setattr(bench, "TRAFFIC_FILE", str(tmp_path / "t.json"))
+    monkeypatch.setattr(bench, "CSRC", str(tmp_path))
+    assert bench.measured_traffic("W", "upd", 100.0) == 110.0
+    (tmp_path / "k.cuh").write_text("other wrappers")
+    assert bench.measured_traffic("W", "upd", 100.0) is None
+    assert all("tc_ptx.cuh" in entry["source"] for entry in json.load(open(tracked))["C3-wide-pixels"].values())
