@@ -9,10 +9,11 @@
 // product of two of them is then nine bf16 products, of which the six of weight 2^-16 and above are formed:
 //   a b = ah bh + 2^-8 (ah bm + am bh) + 2^-16 (ah bl + am bm + al bh) + O(2^-26 |a b|),
 // and the three left out are below the rounding of a single fp32 multiplication (2^-24).  The weights
-// are applied to the accumulator between the groups, by the MMA's own scaling of it.  With the scaled parts
-// the split is exact down to |x| = 2^-118, where l nears bf16's smallest normal number, and loses less than
-// 1.3e-8 of x from there to fp32's smallest normal number (with parts of their own size it lost bits from 2^-110
-// on and 1.2e-5 at the end; the scaling costs 1024 x 1024 x 256 of four groups some 2 %).
+// are applied to the accumulator between the groups, by the MMA's own scaling of it.  The split is exact for
+// every normal number: l's last bit, 2^-149 for the smallest of them, is 2^-133 in l, bf16's smallest subnormal
+// number.  (With parts of their own size bits were lost from 2^-110 down: a 100-term sum of products of 2^-126 and 2^126
+// was off by up to 3.9e-4, now by 1.0e-7 as at any other magnitude.  The scaling costs single-CTA products 2 to 5 %,
+// pairs nothing.)
 // The tensor core's own accumulation is not relied on over long sums: 32 values of k are
 // accumulated in tensor memory (the small products first, so that only the last two
 // instructions act on a sum of full size), and the 32-deep sums are then added up in fp32
@@ -110,23 +111,33 @@ __device__ __forceinline__ uint64_t pack2(uint32_t lo, uint32_t hi) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
   return v;
 }
-// (x, y) - (the two bf16 numbers in `part`), times 2^8: both steps are exact.
+// (x, y) - (the two bf16 numbers in `part`), times 2^8: both steps are exact.  PACKED: as two-float
+// instructions, which is what the loading warps of a pair, bound by issue slots, are better off with (512 x 16384 x
+// 16384 1.30 against 1.33 ms); on single CTAs, bound by the chain of a step, they are in the way (300 rows of an
+// evaluation of 1024-4096-4096-35 272 against 255 us).
+template <bool PACKED>
 __device__ __forceinline__ void rest2(float& x, float& y, uint32_t part) {
-  uint64_t v = pack2(__float_as_uint(x), __float_as_uint(y));
-  const uint64_t p = pack2(part << 16, part & 0xffff0000u), c = pack2(0x43800000u, 0x43800000u);   // 256
-  uint32_t lo, hi;
-  asm("sub.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(p));
-  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(c));
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
-  x = __uint_as_float(lo);
-  y = __uint_as_float(hi);
+  if (PACKED) {
+    uint64_t v = pack2(__float_as_uint(x), __float_as_uint(y));
+    const uint64_t p = pack2(part << 16, part & 0xffff0000u), c = pack2(0x43800000u, 0x43800000u);   // 256
+    uint32_t lo, hi;
+    asm("sub.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(p));
+    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(c));
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
+    x = __uint_as_float(lo);
+    y = __uint_as_float(hi);
+  } else {
+    x = (x - __uint_as_float(part << 16)) * 256.f;
+    y = (y - __uint_as_float(part & 0xffff0000u)) * 256.f;
+  }
 }
 // Two floats into their three bf16 parts, packed pairwise.
+template <bool PACKED>
 __device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
   h = cvt_bf16x2(x, y);
-  rest2(x, y, h);
+  rest2<PACKED>(x, y, h);
   m = cvt_bf16x2(x, y);
-  rest2(x, y, m);
+  rest2<PACKED>(x, y, m);
   l = cvt_bf16x2(x, y);
 }
 __device__ __forceinline__ void add2(uint64_t& acc, uint32_t lo, uint32_t hi) {
@@ -194,15 +205,15 @@ struct Operand {
     }
     p += half_step;
   }
-  template <uint32_t PLANE>
+  template <uint32_t PLANE, bool PACKED>
   __device__ __forceinline__ void store(const float (&v)[UNITS][8], uint8_t* plane0, int slot) const {
 #pragma unroll
     for (int i = 0; i < UNITS; ++i) {
       uint4 h, m, l;
-      split2(v[i][0], v[i][1], h.x, m.x, l.x);
-      split2(v[i][2], v[i][3], h.y, m.y, l.y);
-      split2(v[i][4], v[i][5], h.z, m.z, l.z);
-      split2(v[i][6], v[i][7], h.w, m.w, l.w);
+      split2<PACKED>(v[i][0], v[i][1], h.x, m.x, l.x);
+      split2<PACKED>(v[i][2], v[i][3], h.y, m.y, l.y);
+      split2<PACKED>(v[i][4], v[i][5], h.z, m.z, l.z);
+      split2<PACKED>(v[i][6], v[i][7], h.w, m.w, l.w);
       uint8_t* d = plane0 + off(slot) + i * 8192;
       *reinterpret_cast<uint4*>(d) = h;
       *reinterpret_cast<uint4*>(d + PLANE) = m;
@@ -569,8 +580,8 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
         if (!ok) return;
       }
       uint8_t* slot = smem + (sl >> 1) * (3 * PLANE);
-      oa.template store<PLANE>(xa, slot, sl & 1);
-      ob.template store<PLANE>(xb, slot + A_BYTES, sl & 1);
+      oa.template store<PLANE, PAIR == 2>(xa, slot, sl & 1);
+      ob.template store<PLANE, PAIR == 2>(xb, slot + A_BYTES, sl & 1);
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[sl]);

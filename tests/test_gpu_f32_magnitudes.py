@@ -1,6 +1,6 @@
 """fp32 products over fp32's whole range of exponents: scaling one operand by a power of two and the other by its
-inverse changes no bit of the result, as in fp32 arithmetic, down to operands of 2^-118, and less than the
-rounding of a single product down to the smallest normal number."""
+inverse changes no bit of the result, as in fp32 arithmetic; with operands whose low bf16 parts are subnormal numbers,
+no more than the rounding of a single product."""
 import pytest
 import torch
 
