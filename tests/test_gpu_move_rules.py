@@ -39,8 +39,8 @@ def test_values(dims, S):
 
 @pytest.mark.parametrize("dims,S", [([8, 5003, 3000], 4), ([8, 1000, 15000], 16)])
 def test_whole_rows_are_copied_at_a_fair_rate(dims, S):
-    """15 M weights: 8 bytes each are read and 10 written in the two directions, 270 MB; 5 TB/s and four launches
-    of 5 us each are 74 us."""
+    """15 M weights: 8 bytes each are read and 10 written in the two directions, 270 MB; 4 TB/s and four launches
+    of 5 us each are 88 us (62 measured, 99 in the shared launch)."""
     ctx, W, b = _context(dims, S, api.IST_BF16)
     best = 1e30
     for seed in range(8):
@@ -51,4 +51,4 @@ def test_whole_rows_are_copied_at_a_fair_rate(dims, S):
         ctx.profile(False)
         best = min(best, took["gather"][1] + took["scatter"][1])
     ctx.sync_status()
-    assert best <= 0.074, best
+    assert best <= 0.088, best
