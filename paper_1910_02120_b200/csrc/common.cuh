@@ -66,6 +66,26 @@ __host__ __device__ __forceinline__ constexpr int64_t round_up(int64_t a, int64_
   return ceil_div(a, b) * b;
 }
 
+// An fp32 master and the bf16 operand made from it take 32 bits together: the operand is the master rounded to
+// its upper 16 bits, ties away from zero, and beside it lie the lower 16 bits of the master; the operand's last bit and
+// the low half's first say whether the rounding went up, so the master comes back bit for bit.  (With ties to
+// even, two masters would share an operand and a low half.)  A weight update then moves 8 bytes per weight
+// instead of 10.  NaNs become one NaN: their payloads do not fit.
+__device__ __forceinline__ void split_master(float w, uint16_t* hi, uint16_t* lo) {
+  uint32_t u = __float_as_uint(w);
+  if (w != w) u = 0x7fc00000u;
+  *hi = (uint16_t)((u + 0x8000u) >> 16);
+  *lo = (uint16_t)u;
+}
+__device__ __forceinline__ float join_master(uint16_t hi, uint16_t lo) {
+  return __uint_as_float(((uint32_t)hi << 16) + (uint32_t)(int)(int16_t)lo);
+}
+__device__ __forceinline__ uint16_t operand_bits(float w) {
+  uint16_t hi, lo;
+  split_master(w, &hi, &lo);
+  return hi;
+}
+
 __device__ __forceinline__ float to_float(float v) { return v; }
 __device__ __forceinline__ float to_float(bf16 v) { return __bfloat162float(v); }
 template <typename T> __device__ __forceinline__ T from_float(float v);

@@ -2,7 +2,8 @@
 // per-subnet packed buffers (paper Sec. 2.1 "Constructing Subnets": a subnet's weights are the
 // entries whose row and column neurons it owns; "Training Subnets": the trained slices go back
 // to the positions they came from).  Pure data movement:
-// fp32 values are moved bit for bit; the bf16 operand copy is a rounding of the moved value.
+// fp32 values are moved bit for bit; the bf16 operand copy is a rounding of the moved value.  Masters that are kept
+// as operand and low half (split_master) are taken apart and joined on the way.
 #include <algorithm>
 #include <mutex>
 
@@ -11,10 +12,46 @@
 namespace ist {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kRowsPerCta = 8;
+// Packed elements o and o + 1 of a slice (o even): stored and loaded in whichever form the masters are kept in.  Pairs,
+// because a thread that loads 2-byte halves one by one has half the bytes in flight (scatter of
+// 3072-16384-16384-10, S = 8: 518 -> 395 us; 400 with fp32 words).
+__device__ __forceinline__ void put2(float* master, bf16* opw, uint16_t* lo, int64_t o, float v0, float v1) {
+  ushort2 h, l;
+  split_master(v0, &h.x, &l.x);
+  split_master(v1, &h.y, &l.y);
+  if (lo) *reinterpret_cast<ushort2*>(lo + o) = l;
+  else *reinterpret_cast<float2*>(master + o) = make_float2(v0, v1);
+  if (opw) *reinterpret_cast<ushort2*>(opw + o) = h;
+}
+// Loading is two steps, the words as they lie and then the values, so that a kernel has all its loads in flight
+// first: a branch on the form around every load keeps the compiler from that.
+template <bool SPLIT>
+__device__ __forceinline__ uint2 raw2(const float* master, const bf16* opw, const uint16_t* lo, int64_t o) {
+  if (!SPLIT) return *reinterpret_cast<const uint2*>(master + o);
+  return make_uint2(*reinterpret_cast<const uint32_t*>(opw + o), *reinterpret_cast<const uint32_t*>(lo + o));
+}
+template <bool SPLIT>
+__device__ __forceinline__ float2 value2(uint2 p) {
+  if (!SPLIT) return make_float2(__uint_as_float(p.x), __uint_as_float(p.y));
+  return make_float2(join_master((uint16_t)p.x, (uint16_t)p.y), join_master((uint16_t)(p.x >> 16), (uint16_t)(p.y >> 16)));
+}
+// The same for one element, where the positions of neighbours are not known to be a pair.
+__device__ __forceinline__ void put(float* master, bf16* opw, uint16_t* lo, int64_t o, float v) {
+  uint16_t h, l;
+  split_master(v, &h, &l);
+  if (lo) lo[o] = l;
+  else master[o] = v;
+  if (opw) reinterpret_cast<uint16_t*>(opw)[o] = h;
+}
+template <bool SPLIT>
+__device__ __forceinline__ float get(const float* master, const bf16* opw, const uint16_t* lo, int64_t o) {
+  return SPLIT ? join_master(reinterpret_cast<const uint16_t*>(opw)[o], lo[o]) : master[o];
+}
 
-// Several matrices and bias rows as blocks of one launch: block -> (job, subnet, 8 rows, 256 columns).
+constexpr int kThreads = 256;
+constexpr int kRowsPerCta = 4;
+
+// Several matrices and bias rows as blocks of one launch: block -> (job, subnet, 4 rows, 512 columns).
 // A network of a few layers took two launches per layer in either direction, most of them shorter
 // than the gap between them (64-512-512-10, S = 4: 38 us to gather, 37 us to scatter; now 8.5 us each).
 constexpr int kMaxJobs = 8;
@@ -25,11 +62,27 @@ struct SliceJobs {
   int end[kMaxJobs];                 // blocks end(previous) .. end - 1 are the job's
 };
 
-// Packed element (s, i, j), j = column block * 256 + tid, i in a block of kRowsPerCta rows.
+// Packed element (s, i, j), j = column block * 512 + 2 tid (and j + 1), i in a block of kRowsPerCta rows.
 // Pad rows / columns (beyond the group's true size) are written as zeros so that padded
 // neurons stay inert through the local steps.
+// Two rows at a time: with the loads of all rows in flight before the first store, the stores of a large matrix
+// come in bursts that DRAM takes worse (middle layer of 32768 x 32768, S = 8: 1100 -> 1390 us for four rows).
+template <bool SPLIT>
+__device__ __forceinline__ void scatter_rows(const SliceJob& J, int64_t o0, const int64_t* c, const int32_t* rows, int64_t i0,
+                                             int64_t i1) {
+  const int64_t ld = J.m.ld, full = J.m.full_cols;
+#pragma unroll 2
+  for (int64_t i = i0; i < i1; ++i, o0 += ld) {
+    const float2 f = value2<SPLIT>(raw2<SPLIT>(J.master, J.opw, J.lo, o0));
+    float* w = J.W + (rows ? rows[i] : i) * full;
+    w[c[0]] = f.x;
+    if (c[1] >= 0) w[c[1]] = f.y;
+  }
+}
+
 template <bool GATHER>
 __global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ SliceJobs a) {
+  constexpr int R = kRowsPerCta;
   pdl_wait();
   pdl_trigger();
   int ji = 0, blk = blockIdx.x;
@@ -37,61 +90,83 @@ __global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ 
   const SliceJob& J = a.job[ji];
   const SliceMap& m = J.m;
   blk -= ji ? a.end[ji - 1] : 0;
-  const int64_t j = (int64_t)(blk % a.x_blocks[ji]) * kThreads + threadIdx.x;
+  const int64_t j = ((int64_t)(blk % a.x_blocks[ji]) * kThreads + threadIdx.x) * 2;   // columns j and j + 1
   blk /= a.x_blocks[ji];
   const int yb = blk % a.y_blocks[ji], s = m.s_first + blk / a.y_blocks[ji];
   if (!GATHER && J.mean) {
-    if (j >= m.full_cols) return;
-    const float old = J.W[j];
-    float acc = 0.f;
-    for (int g = 0; g < J.S; ++g) acc += J.master[(int64_t)g * m.ld + j] - old;
-    J.W[j] = old + acc / (float)J.S;
+    for (int64_t n = j; n < min(j + 2, m.full_cols); ++n) {
+      const float old = J.W[n];
+      float acc = 0.f;
+      for (int g = 0; g < J.S; ++g) acc += J.master[(int64_t)g * m.ld + n] - old;
+      J.W[n] = old + acc / (float)J.S;
+    }
     return;
   }
   const int64_t ncols = m.col_idx ? (m.col_off[s + 1] - m.col_off[s]) : m.full_cols;
   const int64_t nrows = m.row_idx ? (m.row_off[s + 1] - m.row_off[s]) : m.full_rows;
   if (j >= (GATHER ? m.ld : ncols)) return;
-  int64_t c = -1;
-  if (j < ncols) c = m.col_idx ? m.col_idx[m.col_off[s] + j] : j;
-  const int64_t i0 = (int64_t)yb * kRowsPerCta;
-  float v[kRowsPerCta];
-  int64_t r[kRowsPerCta];
+  int64_t c[2] = {-1, -1};
 #pragma unroll
-  for (int u = 0; u < kRowsPerCta; ++u)
-    r[u] = (c >= 0 && i0 + u < nrows) ? (m.row_idx ? m.row_idx[m.row_off[s] + i0 + u] : i0 + u) * m.full_cols + c : -1;
+  for (int e = 0; e < 2; ++e)
+    if (j + e < ncols) c[e] = m.col_idx ? m.col_idx[m.col_off[s] + j + e] : j + e;
+  const int64_t i0 = (int64_t)yb * R;
   const int64_t o0 = ((int64_t)s * m.rows_pad + i0) * m.ld + j;
-#pragma unroll
-  for (int u = 0; u < kRowsPerCta; ++u)
-    v[u] = r[u] >= 0 ? (GATHER ? J.W[r[u]] : J.master[o0 + u * m.ld]) : 0.f;
-#pragma unroll
-  for (int u = 0; u < kRowsPerCta; ++u) {
-    if (GATHER) {
-      if (i0 + u < m.rows_pad) {
-        J.master[o0 + u * m.ld] = v[u];
-        if (J.opw) J.opw[o0 + u * m.ld] = __float2bfloat16_rn(v[u]);
-      }
-    } else if (r[u] >= 0) {
-      J.W[r[u]] = v[u];
-    }
+  if (!GATHER) {
+    const int64_t i1 = min(i0 + R, nrows);
+    const int32_t* rows = m.row_idx ? m.row_idx + m.row_off[s] : nullptr;
+    if (J.lo) scatter_rows<true>(J, o0, c, rows, i0, i1);
+    else scatter_rows<false>(J, o0, c, rows, i0, i1);
+    return;
   }
+  float v[R][2];
+  int64_t r[R];
+#pragma unroll
+  for (int u = 0; u < R; ++u)
+    r[u] = i0 + u < nrows ? (m.row_idx ? m.row_idx[m.row_off[s] + i0 + u] : i0 + u) * m.full_cols : -1;
+#pragma unroll
+  for (int u = 0; u < R; ++u)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) v[u][e] = r[u] >= 0 && c[e] >= 0 ? J.W[r[u] + c[e]] : 0.f;
+#pragma unroll
+  for (int u = 0; u < R; ++u)
+    if (i0 + u < m.rows_pad) put2(J.master, J.opw, J.lo, o0 + u * m.ld, v[u][0], v[u][1]);
 }
 
 // ---- last layer: whole rows, picked by the previous hidden layer's partition --------------------
 // W_t[G_{t-1}^s, :] keeps every column, so both sides are contiguous along a row and the kernel is a
 // strided row copy.  Rows of the full matrix start at any 4-byte offset (N_t is arbitrary), hence
-// scalar accesses; a thread keeps kRowU x kColU of them in flight (consecutive lanes on
-// consecutive columns), which is what the copy needs to approach the DRAM rate.
+// scalar accesses there, consecutive lanes on consecutive columns; a warp takes spans of 64 columns, of which a lane
+// has columns l and 32 + l on that side and the pair 2 l, 2 l + 1 on the packed side, exchanged by shuffles.  A
+// thread keeps kRowU x kColU values in flight, which is what the copy needs to approach the DRAM rate.
 constexpr int kRowU = 4, kColU = 4;
 
-template <bool GATHER>
-__global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, float* master,
-                                                         bf16* __restrict__ opw) {
+// (columns l, 32 + l) of a span <-> (columns 2 l, 2 l + 1)
+__device__ __forceinline__ void to_pairs(float& a, float& b) {
+  const int lane = threadIdx.x & 31, src = 2 * (lane & 15);
+  const float a0 = __shfl_sync(0xffffffffu, a, src), a1 = __shfl_sync(0xffffffffu, a, src + 1);
+  const float b0 = __shfl_sync(0xffffffffu, b, src), b1 = __shfl_sync(0xffffffffu, b, src + 1);
+  a = lane < 16 ? a0 : b0;
+  b = lane < 16 ? a1 : b1;
+}
+__device__ __forceinline__ void from_pairs(float& a, float& b) {
+  const int lane = threadIdx.x & 31, src = lane >> 1;
+  const float a0 = __shfl_sync(0xffffffffu, a, src), b0 = __shfl_sync(0xffffffffu, b, src);
+  const float a1 = __shfl_sync(0xffffffffu, a, 16 + src), b1 = __shfl_sync(0xffffffffu, b, 16 + src);
+  a = lane & 1 ? b0 : a0;
+  b = lane & 1 ? b1 : a1;
+}
+
+template <bool GATHER, bool SPLIT>
+__global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, float* master, bf16* opw,
+                                                         uint16_t* lo) {
   pdl_wait();
   pdl_trigger();
   const int s = m.s_first + blockIdx.z;
   const int nrows = m.row_off[s + 1] - m.row_off[s];
   const int32_t* rows = m.row_idx + m.row_off[s];
-  const int64_t j0 = (int64_t)blockIdx.x * (kThreads * kColU) + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  // this warp's spans of 64 columns start at j0 + c * kThreads, c = 0, 2, ...
+  const int64_t j0 = (int64_t)blockIdx.x * (kThreads * kColU) + (threadIdx.x >> 5) * 64;
   for (int64_t i0 = (int64_t)blockIdx.y * kRowU; i0 < (GATHER ? m.rows_pad : nrows); i0 += (int64_t)gridDim.y * kRowU) {
     float v[kRowU][kColU];
     int64_t src[kRowU];
@@ -102,34 +177,41 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, fl
       for (int u = 0; u < kRowU; ++u)
 #pragma unroll
         for (int c = 0; c < kColU; ++c) {
-          const int64_t j = j0 + c * kThreads;
+          const int64_t j = j0 + (c & ~1) * kThreads + (c & 1) * 32 + lane;
           v[u][c] = (src[u] >= 0 && j < m.full_cols) ? W[src[u] + j] : 0.f;   // pad rows / columns are zeros
         }
 #pragma unroll
       for (int u = 0; u < kRowU; ++u)
 #pragma unroll
-        for (int c = 0; c < kColU; ++c) {
-          const int64_t j = j0 + c * kThreads;
-          if (i0 + u < m.rows_pad && j < m.ld) {
-            const int64_t o = ((int64_t)s * m.rows_pad + i0 + u) * m.ld + j;
-            master[o] = v[u][c];
-            if (opw) opw[o] = __float2bfloat16_rn(v[u][c]);
-          }
+        for (int c = 0; c < kColU; c += 2) {
+          const int64_t j = j0 + c * kThreads + 2 * lane;
+          to_pairs(v[u][c], v[u][c + 1]);
+          if (i0 + u < m.rows_pad && j < m.ld)
+            put2(master, opw, lo, ((int64_t)s * m.rows_pad + i0 + u) * m.ld + j, v[u][c], v[u][c + 1]);
         }
     } else {
+      uint2 p[kRowU][kColU / 2];
 #pragma unroll
       for (int u = 0; u < kRowU; ++u)
 #pragma unroll
-        for (int c = 0; c < kColU; ++c) {
-          const int64_t j = j0 + c * kThreads;
-          v[u][c] = (src[u] >= 0 && j < m.full_cols) ? master[((int64_t)s * m.rows_pad + i0 + u) * m.ld + j] : 0.f;
+        for (int c = 0; c < kColU; c += 2) {
+          const int64_t j = j0 + c * kThreads + 2 * lane;
+          p[u][c / 2] = (src[u] >= 0 && j < m.full_cols)
+                            ? raw2<SPLIT>(master, opw, lo, ((int64_t)s * m.rows_pad + i0 + u) * m.ld + j) : make_uint2(0, 0);
         }
 #pragma unroll
       for (int u = 0; u < kRowU; ++u)
 #pragma unroll
-        for (int c = 0; c < kColU; ++c) {
-          const int64_t j = j0 + c * kThreads;
-          if (src[u] >= 0 && j < m.full_cols) W[src[u] + j] = v[u][c];
+        for (int c = 0; c < kColU; c += 2) {
+          const float2 f = value2<SPLIT>(p[u][c / 2]);
+          v[u][c] = f.x;
+          v[u][c + 1] = f.y;
+          from_pairs(v[u][c], v[u][c + 1]);
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int64_t j = j0 + c * kThreads + e * 32 + lane;
+            if (src[u] >= 0 && j < m.full_cols) W[src[u] + j] = v[u][c + e];
+          }
         }
     }
   }
@@ -138,9 +220,9 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, fl
 bool rows_ok(const SliceMap& m) { return m.row_idx && !m.col_idx && m.full_cols >= 1024; }
 
 template <bool GATHER>
-void launch_rows(const Launch& L, float* W, const SliceMap& m, int S, float* master, bf16* opw) {
+void launch_rows(const Launch& L, float* W, const SliceMap& m, int S, float* master, bf16* opw, uint16_t* lo) {
   dim3 grid((unsigned)ceil_div(m.ld, kThreads * kColU), (unsigned)std::min<int64_t>(ceil_div(m.rows_pad, kRowU), 65535), S);
-  launch_pdl(rows_kernel<GATHER>, grid, dim3(kThreads), 0, L.stream, W, m, master, opw);
+  launch_pdl(lo ? rows_kernel<GATHER, true> : rows_kernel<GATHER, false>, grid, dim3(kThreads), 0, L.stream, W, m, master, opw, lo);
   L.count();
 }
 
@@ -221,10 +303,10 @@ constexpr long long kPermWaitCycles = 2000000000ll;   // ~1 s
 // Gather: row blocks arrive through double-buffered bulk copies (the next block loads while
 // this one is permuted).  Scatter: packed values are read into the permuted tile, which leaves
 // through bulk stores.  Requires full_cols % 4 == 0 (16-byte row segments).
-template <bool GATHER>
+template <bool GATHER, bool SPLIT>
 __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W, SliceMap m, int S,
-                                                                      float* master,
-                                                                      bf16* __restrict__ opw, DeviceStatus* st) {
+                                                                      float* master, bf16* opw, uint16_t* lo,
+                                                                      DeviceStatus* st) {
   extern __shared__ __align__(128) unsigned char perm_smem[];
   float* tile = reinterpret_cast<float*>(perm_smem);                                  // [2][rows][cols]
   long long* map_off = reinterpret_cast<long long*>(tile + 2 * kStageRows * kStageCols);   // [cols]
@@ -289,9 +371,7 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
 #pragma unroll
         for (int r = 0; r < kStageRows; ++r) {
           if (r < nrows) {
-            const float v = t[r * kStageCols + col];
-            master[o + (long long)r * m.ld] = v;
-            if (opw) opw[o + (long long)r * m.ld] = __float2bfloat16_rn(v);
+            put(master, opw, lo, o + (long long)r * m.ld, t[r * kStageCols + col]);
           }
         }
       }
@@ -301,8 +381,7 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
           const int npad = (int)m.ld - cnt;
           for (int e = threadIdx.x; e < npad * nrows; e += kPermThreads) {
             const long long o = ((long long)s * m.rows_pad + k0 + e / npad) * m.ld + cnt + e % npad;
-            master[o] = 0.f;
-            if (opw) opw[o] = __float2bfloat16_rn(0.f);
+            put(master, opw, lo, o, 0.f);
           }
         }
       }
@@ -311,14 +390,21 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
       // this buffer's previous stores (two iterations ago) must have read it
       if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
       __syncthreads();
-      for (int e = threadIdx.x; e < total; e += kPermThreads) {
-        const int col = map_col[e];
-        const long long o = map_off[e] + k0 * m.ld;
-        float v[kStageRows];
+      for (int e = threadIdx.x; e < total; e += 2 * kPermThreads) {   // two entries' rows in flight
+        const bool two = e + kPermThreads < total;
+        const int col = map_col[e], col2 = two ? map_col[e + kPermThreads] : 0;
+        const long long o = map_off[e] + k0 * m.ld, o2 = two ? map_off[e + kPermThreads] + k0 * m.ld : o;
+        float v[kStageRows], v2[kStageRows];
 #pragma unroll
-        for (int r = 0; r < kStageRows; ++r) v[r] = r < nrows ? master[o + (long long)r * m.ld] : 0.f;
+        for (int r = 0; r < kStageRows; ++r) {
+          v[r] = r < nrows ? get<SPLIT>(master, opw, lo, o + (long long)r * m.ld) : 0.f;
+          v2[r] = r < nrows ? get<SPLIT>(master, opw, lo, o2 + (long long)r * m.ld) : 0.f;
+        }
 #pragma unroll
-        for (int r = 0; r < kStageRows; ++r) t[r * kStageCols + col] = v[r];
+        for (int r = 0; r < kStageRows; ++r) {
+          t[r * kStageCols + col] = v[r];
+          if (two) t[r * kStageCols + col2] = v2[r];
+        }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
@@ -337,14 +423,14 @@ bool staged_ok(const SliceMap& m, int S) {
          m.full_cols >= 256 && m.full_cols % 4 == 0;
 }
 
-template <bool GATHER>
-bool launch_permute_cols(const Launch& L, float* W, const SliceMap& m, int S, float* master, bf16* opw,
+template <bool GATHER, bool SPLIT>
+bool launch_permute_cols(const Launch& L, float* W, const SliceMap& m, int S, float* master, bf16* opw, uint16_t* lo,
                          DeviceStatus* st) {
   constexpr int smem = 2 * kStageRows * kStageCols * (int)sizeof(float) + kStageCols * 8 + kStageCols * 2;
   static std::once_flag once;     // one instance per direction; any host thread may come first
   static bool configured = false;
   std::call_once(once, [] {
-    configured = cudaFuncSetAttribute(permute_cols_kernel<GATHER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    configured = cudaFuncSetAttribute(permute_cols_kernel<GATHER, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       smem) == cudaSuccess;
   });
   if (!configured) return false;
@@ -356,18 +442,36 @@ bool launch_permute_cols(const Launch& L, float* W, const SliceMap& m, int S, fl
   if (y > blocks) y = blocks;
   if (y > 65535) y = 65535;
   dim3 grid((unsigned)chunks, (unsigned)y);
-  if (launch_pdl(permute_cols_kernel<GATHER>, grid, dim3(kPermThreads), smem, L.stream, W, m, S, master, opw, st) != cudaSuccess)
+  if (launch_pdl(permute_cols_kernel<GATHER, SPLIT>, grid, dim3(kPermThreads), smem, L.stream, W, m, S, master, opw, lo, st) != cudaSuccess)
     return false;
   L.count();
   return true;
 }
 
-__global__ void copy_out_kernel(const float* __restrict__ packed, int64_t ld, int64_t rows,
+__global__ void copy_out_kernel(const float* packed, const bf16* opw, const uint16_t* lo, int64_t ld, int64_t rows,
                                 int64_t cols, float* __restrict__ out) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t i = blockIdx.y;
   if (j < cols)
-    for (; i < rows; i += gridDim.y) out[i * cols + j] = packed[i * ld + j];
+    for (; i < rows; i += gridDim.y) out[i * cols + j] = lo ? get<true>(packed, opw, lo, i * ld + j) : get<false>(packed, opw, lo, i * ld + j);
+}
+
+// Masters first .. end - 1 of n become fp32 words in place.  The low halves are the second half of the words, so
+// word i takes the place of low halves 2 i - n and 2 i - n + 1, both at or before i: a launch may cover words as long as
+// they replace only low halves of words before its first.  One block may end the array: it reads all it needs
+// before it writes.
+__global__ void join_masters_kernel(float* master, const bf16* opw, int64_t n, int64_t first, int64_t end) {
+  const uint16_t* lo = reinterpret_cast<const uint16_t*>(master) + n;
+  const uint16_t* hi = reinterpret_cast<const uint16_t*>(opw);
+  if (gridDim.x > 1) {
+    for (int64_t i = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end; i += (int64_t)gridDim.x * blockDim.x)
+      master[i] = join_master(hi[i], lo[i]);
+  } else {
+    const int64_t i = first + threadIdx.x;
+    const float w = i < end ? join_master(hi[i], lo[i]) : 0.f;
+    __syncthreads();
+    if (i < end) master[i] = w;
+  }
 }
 
 }  // namespace
@@ -400,13 +504,13 @@ void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
   for (int i = 0; i < n; ++i) {
     const SliceJob& j = jobs[i];
     const int64_t elements = j.mean ? 0 : j.S * j.m.rows_pad * j.m.ld;
-    if (elements >= kOwnColumns && staged_ok(j.m, j.S) && launch_permute_cols<GATHER>(L, j.W, j.m, j.S, j.master, j.opw, st))
+    if (elements >= kOwnColumns && staged_ok(j.m, j.S) && (j.lo ? launch_permute_cols<GATHER, true> : launch_permute_cols<GATHER, false>)(L, j.W, j.m, j.S, j.master, j.opw, j.lo, st))
       continue;
     if (elements >= kOwnRows && rows_ok(j.m)) {
-      launch_rows<GATHER>(L, j.W, j.m, j.S, j.master, j.opw);
+      launch_rows<GATHER>(L, j.W, j.m, j.S, j.master, j.opw, j.lo);
       continue;
     }
-    const int64_t x = ceil_div(j.mean ? j.m.full_cols : j.m.ld, kThreads), y = j.mean ? 1 : ceil_div(j.m.rows_pad, kRowsPerCta);
+    const int64_t x = ceil_div(j.mean ? j.m.full_cols : j.m.ld, 2 * kThreads), y = j.mean ? 1 : ceil_div(j.m.rows_pad, kRowsPerCta);
     const int64_t b = x * y * (j.mean ? 1 : j.S);
     if (a.n == kMaxJobs || blocks + b > 0x7fffffffll) flush();
     a.job[a.n] = j;
@@ -423,11 +527,24 @@ void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
 void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) { move_all<true>(L, jobs, n, st); }
 void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) { move_all<false>(L, jobs, n, st); }
 
-void copy_out_slice(const Launch& L, const float* packed, int64_t ld, int64_t rows, int64_t cols,
-                    float* out) {
+void copy_out_slice(const Launch& L, const float* packed, const bf16* opw, const uint16_t* lo, int64_t ld, int64_t rows,
+                    int64_t cols, float* out) {
   dim3 grid((unsigned)ceil_div(cols, 256), (unsigned)(rows < 1024 ? rows : 1024));
-  copy_out_kernel<<<grid, 256, 0, L.stream>>>(packed, ld, rows, cols, out);
+  copy_out_kernel<<<grid, 256, 0, L.stream>>>(packed, opw, lo, ld, rows, cols, out);
   L.count();
+}
+
+void join_masters(const Launch& L, float* master, const bf16* opw, int64_t n) {
+  constexpr int kJoin = 1024;
+  int64_t first = 0;
+  while (first < n) {
+    int64_t end = first + (n - first) / 2;     // words below this replace low halves below `first` only
+    if (n - first <= kJoin) end = n;
+    const int64_t blocks = n - first <= kJoin ? 1 : std::max<int64_t>(2, std::min<int64_t>(ceil_div(end - first, kJoin), 4096));
+    join_masters_kernel<<<(unsigned)blocks, kJoin, 0, L.stream>>>(master, opw, n, first, end);
+    L.count();
+    first = end;
+  }
 }
 
 }  // namespace ist

@@ -28,9 +28,11 @@
 // The epilogue has no CTA-wide barrier: slots move between loader, epilogue warps and storer
 // through mbarriers (slot_full -> chunk_done -> slot_empty), so warps work on different chunks
 // at the same time and a slow chunk does not hold the others back.
-// The weight-update epilogue is the HBM-heavy part of a step (10 bytes per weight against
-// 2*B flops): its fp32 master chunks are prefetched through the slot ring while earlier chunks
-// are updated in place in shared memory and stored back.
+// The weight-update epilogue is the HBM-heavy part of a step (8 bytes per weight against
+// 2*B flops): its master chunks, bf16 operand and low half (split_master), are prefetched through the slot ring
+// while earlier chunks are updated in place in shared memory and stored back.  With fp32 masters and an operand
+// copy beside them (10 bytes; kept for contexts that hand out fp32 slices) the launch takes 190 us
+// instead of 155 at 3072-16384-16384-10, S = 8, 512 rows, and 63.8 instead of 55.7 at 1024-8192-8192-100, S = 4.
 //
 // PAIR = 2 runs two CTAs of a cluster as one unit (tcgen05 cta_group::2): the pair computes a
 // 256 x BN tile, each CTA loads its own 128 rows of A and its half (BN/2 rows) of B and keeps its
@@ -71,15 +73,20 @@ namespace {
 constexpr int BM = 128;
 constexpr int BK = 64;                   // 64 bf16 = 128 bytes = one swizzle row
 constexpr int CH = 32;                   // epilogue chunk: 32 output columns
+// Updates of split masters on single CTAs work in chunks twice as wide: both areas then have 128-byte rows and half the
+// hand-offs (update of 1024 x 670,091, S = 8, 256 rows: 2.13 -> 1.73 ms).  On pairs six narrow slots are better than
+// four wide ones (1024-8192-8192-100, S = 4, 512 rows: 55.7 against 58.8 us; 63.8 with fp32 masters).
+constexpr int chunk_cols(int epi, int pair) { return epi == 7 /* EPI_SGD_SPLIT */ && pair == 1 ? 2 * CH : CH; }
 // Warps of a CTA, see the role list above: loader, MMA issuer, the epilogue warps (two groups of
 // four; four groups for the two softmax passes over a very wide output layer, whose epilogues are
 // long chains of dependent instructions and need more warps to hide them), the epilogue input
 // loader, four storers, and two summing warps for weight-update launches (bias gradient).
 constexpr int kSumWarps = 2;
-constexpr bool sums_in_kernel(int epi, int pair) { return epi == 3 /* EPI_SGD */ && pair == 1; }   // sums from the B stages
-constexpr bool has_sum_warps(int epi) { return epi == 3 /* EPI_SGD */; }
+constexpr bool is_update(int epi) { return epi == 3 /* EPI_SGD */ || epi == 7 /* EPI_SGD_SPLIT */; }
+constexpr bool sums_in_kernel(int epi, int pair) { return is_update(epi) && pair == 1; }   // sums from the B stages
+constexpr bool has_sum_warps(int epi) { return is_update(epi); }
 constexpr int epi_warps(int epi) { return (epi == 5 /* EPI_LSE_PART */ || epi == 6 /* EPI_SOFTMAX_DELTA */) ? 16 : 8; }
-constexpr bool has_aux(int epi) { return epi == 2 /* EPI_RELU_MASK */ || epi == 3; }   // EpiTraits::kAux
+constexpr bool has_aux(int epi) { return epi == 2 /* EPI_RELU_MASK */ || is_update(epi); }   // EpiTraits::kAux
 // storers: none where the epilogue stores no chunks (EpiTraits::k32 || k16), two beside sixteen
 // epilogue warps (20 warps leave a thread 96 registers, 22 would leave 80), else four
 constexpr int store_warps(int epi) { return epi == 5 ? 0 : epi == 6 ? 2 : 4; }
@@ -137,7 +144,7 @@ struct TcArgs {
 
 struct TcMaps {
   CUtensorMap a[kMaxProblems], b[kMaxProblems];
-  CUtensorMap c32[kMaxProblems];     // fp32 chunks: logits out, master in/out
+  CUtensorMap c32[kMaxProblems];     // fp32 chunks: logits out, master in/out; EPI_SGD_SPLIT: the masters' low halves
   CUtensorMap c16[kMaxProblems];     // bf16 chunks out: activations, delta, weights
   CUtensorMap aux16[kMaxProblems];   // bf16 chunks in: ReLU mask
 };
@@ -204,12 +211,14 @@ __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.pr
 
 // Chunk staging: a ring of fp32 areas ([128][32] floats, 128-byte swizzle) and / or a ring of
 // bf16 areas ([128][32] bf16, 64-byte swizzle); kAux says whether chunks are loaded before use
-// (the fp32 ring for the SGD update, the bf16 ring for the ReLU mask).
+// (the fp32 ring for the SGD update, the bf16 ring for the ReLU mask).  Where the masters are kept as operand + low
+// half (EPI_SGD_SPLIT) a slot is two areas of 16-bit values, the operands and the low halves, loaded and stored alike.
 template <int EPI> struct EpiTraits;
 template <> struct EpiTraits<EPI_BIAS_RELU> { static constexpr bool k32 = false, k16 = true, kAux = false; };
 template <> struct EpiTraits<EPI_BIAS_F32> { static constexpr bool k32 = true, k16 = false, kAux = false; };
 template <> struct EpiTraits<EPI_RELU_MASK> { static constexpr bool k32 = false, k16 = true, kAux = true; };
 template <> struct EpiTraits<EPI_SGD> { static constexpr bool k32 = true, k16 = true, kAux = true; };
+template <> struct EpiTraits<EPI_SGD_SPLIT> { static constexpr bool k32 = false, k16 = true, kAux = true; };
 template <> struct EpiTraits<EPI_LSE_PART> { static constexpr bool k32 = false, k16 = false, kAux = false; };
 template <> struct EpiTraits<EPI_SOFTMAX_DELTA> { static constexpr bool k32 = false, k16 = true, kAux = false; };
 
@@ -235,6 +244,39 @@ __device__ __forceinline__ void unpack8(uint4 u, float* v) {
   v[4] = __low2float(c); v[5] = __high2float(c); v[6] = __low2float(d); v[7] = __high2float(d);
 }
 
+// Bits of an updated master.  The NaN that arithmetic gives, 0x7fffffff, would round to minus zero: the signed minimum
+// makes it one that stays a NaN and leaves every number as it is.
+__device__ __forceinline__ uint32_t master_bits(float w) { return (uint32_t)min(__float_as_int(w), 0x7fff7fff); }
+// The operands of eight masters (see split_master), as one 16-byte unit.
+__device__ __forceinline__ uint4 pack8_operand(const float* w) {
+  uint32_t h[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) h[e] = master_bits(w[e]) + 0x8000u;
+  return make_uint4(__byte_perm(h[0], h[1], 0x7632), __byte_perm(h[2], h[3], 0x7632), __byte_perm(h[4], h[5], 0x7632),
+                    __byte_perm(h[6], h[7], 0x7632));
+}
+// Eight masters kept as operand and low half: joined, and taken apart again.
+__device__ __forceinline__ void join8(const uint4& h, const uint4& l, float* w) {
+  const uint32_t hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    w[2 * i] = __uint_as_float((hv[i] << 16) + (uint32_t)((int)(lv[i] << 16) >> 16));
+    w[2 * i + 1] = __uint_as_float((hv[i] & 0xffff0000u) + (uint32_t)((int)lv[i] >> 16));
+  }
+}
+__device__ __forceinline__ void split8(const float* w, uint4* h, uint4* l) {
+  uint32_t v[8], hv[4], lv[4];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = master_bits(w[e]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    hv[i] = __byte_perm(v[2 * i] + 0x8000u, v[2 * i + 1] + 0x8000u, 0x7632);
+    lv[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
+  }
+  *h = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+  *l = make_uint4(lv[0], lv[1], lv[2], lv[3]);
+}
+
 // Row r of a chunk slot.  fp32 area: 128-byte rows, 16-byte unit u stored at u ^ (r & 7).
 // bf16 area: 64-byte rows, 16-byte unit u stored at u ^ ((r >> 1) & 3).
 __device__ __forceinline__ float4* f32_unit(uint8_t* area, int r, int u) {
@@ -244,6 +286,10 @@ __device__ __forceinline__ uint4* b16_unit(uint8_t* area, int r, int u) {
   return reinterpret_cast<uint4*>(area + r * 64 + ((u ^ ((r >> 1) & 3)) << 4));
 }
 
+__device__ __forceinline__ uint4* row128_unit(uint8_t* area, int r, int u) {   // 128-byte rows of any type
+  return reinterpret_cast<uint4*>(f32_unit(area, r, u));
+}
+
 template <int A_MN, int B_MN, int BN, int STAGES, int NS, int EPI, int PAIR>
 __global__ void __launch_bounds__(threads_for(EPI, PAIR), 1)
 gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcArgs a) {
@@ -251,14 +297,17 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   constexpr int BNL = BN / PAIR;   // rows of the B tile this CTA loads
   constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BNL * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
   // a slot holds one 128 x 32 chunk: an fp32 area and / or a bf16 area, as the epilogue needs
-  constexpr uint32_t F32_BYTES = ET::k32 ? BM * CH * 4 : 0, B16_BYTES = ET::k16 ? BM * CH * 2 : 0;
-  constexpr uint32_t SLOT_BYTES = F32_BYTES + B16_BYTES;
-  constexpr uint32_t AUX_BYTES = EPI == EPI_SGD ? F32_BYTES : B16_BYTES;
+  constexpr int CW = chunk_cols(EPI, PAIR);
+  constexpr uint32_t F32_BYTES = ET::k32 ? BM * CW * 4 : 0, B16_BYTES = ET::k16 ? BM * CW * 2 : 0;
+  constexpr bool kSplit = EPI == EPI_SGD_SPLIT;
+  constexpr uint32_t LO_BYTES = kSplit ? BM * CW * 2 : 0;          // behind the bf16 area
+  constexpr uint32_t SLOT_BYTES = F32_BYTES + B16_BYTES + LO_BYTES;
+  constexpr uint32_t AUX_BYTES = EPI == EPI_SGD ? F32_BYTES : B16_BYTES + LO_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BN;
-  constexpr int NCH = BN / CH;
+  constexpr int NCH = BN / CW;
   constexpr bool kStore = ET::k32 || ET::k16;   // the epilogue writes chunks through the slot ring
   constexpr bool kSums = sums_in_kernel(EPI, PAIR);   // two more warps sum the deltas for the bias update
-  static_assert(EPI_RELU_MASK == 2 && EPI_SGD == 3 && EPI_LSE_PART == 5 && EPI_SOFTMAX_DELTA == 6 &&
+  static_assert(EPI_RELU_MASK == 2 && EPI_SGD == 3 && EPI_SGD_SPLIT == 7 && EPI_LSE_PART == 5 && EPI_SOFTMAX_DELTA == 6 &&
                     has_aux(EPI) == ET::kAux && (store_warps(EPI) > 0) == kStore,
                 "the role layout functions name epilogues by value");
   constexpr int kEpiWarps = epi_warps(EPI), NG = kEpiWarps / 4;   // epilogue warps; groups of four
@@ -285,7 +334,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     for (int i = 0; i < a.n_problems; ++i) {
       prefetch_map(&maps.a[i]);
       prefetch_map(&maps.b[i]);
-      if (ET::k32 || (EPI == EPI_BIAS_RELU && a.p[i].head_f32)) prefetch_map(&maps.c32[i]);
+      if (ET::k32 || kSplit || (EPI == EPI_BIAS_RELU && a.p[i].head_f32)) prefetch_map(&maps.c32[i]);
       if (ET::k16) prefetch_map(&maps.c16[i]);
       if (EPI == EPI_RELU_MASK) prefetch_map(&maps.aux16[i]);
     }
@@ -511,7 +560,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const float* bias = pr.bias ? pr.bias + (long long)group_of(pr, at.slab) * pr.bias_sg : nullptr;
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-          const int n = n0 + c * CH + lane;
+          const int n = n0 + c * CW + lane;
           next_bias[c] = (bias && n < pr.N) ? bias[n] : 0.f;
         }
       }
@@ -544,7 +593,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
       const int pN = a.p[pi].N, pNt = a.p[pi].n_true, pM = a.p[pi].M, p_ntiles = a.p[pi].n_tiles;
       // a narrow fp32 head works in 16-column chunks: 128 x 16 floats fill the bf16 area of a slot
       const bool head = EPI == EPI_BIAS_RELU && a.p[pi].head_f32;
-      const int cw = head ? CH / 2 : CH, nch = head ? 2 * NCH : NCH;
+      const int cw = head ? CW / 2 : CW, nch = head ? 2 * NCH : NCH;
       const int n0 = at.nt * BN;
       const int g = at.slab;                          // output slab (group, k slice)
       const int b = j & 1;
@@ -596,7 +645,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           if (lane == 0) mbar_arrive(&chunk_done[slot]);
           continue;
         }
-        tc_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c * CH), acc);
+        if (!kSplit) tc_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c * CW), acc);
         if (EPI == EPI_SGD) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) {               // 8 columns per iteration
@@ -614,7 +663,22 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
             w[7] = w1.w - a.lr * __uint_as_float(acc[8 * u + 7]);
             *p0 = make_float4(w[0], w[1], w[2], w[3]);
             *p1 = make_float4(w[4], w[5], w[6], w[7]);
-            *b16_unit(b16, r, u) = pack8(w);
+            *b16_unit(b16, r, u) = pack8_operand(w);
+          }
+        } else if (kSplit) {
+#pragma unroll
+          for (int h = 0; h < CW / CH; ++h) {
+            tc_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c * CW + h * CH), acc);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {             // 8 columns per iteration
+              float w[8];
+              uint4* ph = CW == CH ? b16_unit(b16, r, u) : row128_unit(b16, r, 4 * h + u);
+              uint4* pl = CW == CH ? b16_unit(b16 + B16_BYTES, r, u) : row128_unit(b16 + B16_BYTES, r, 4 * h + u);
+              join8(*ph, *pl, w);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) w[e] -= a.lr * __uint_as_float(acc[8 * u + e]);
+              split8(w, ph, pl);
+            }
           }
         } else if (EPI == EPI_RELU_MASK) {
 #pragma unroll
@@ -763,14 +827,17 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const int n0 = at.nt * BN;
         const int g = at.slab;
         for (int c = 0; c < NCH; ++c, ++cq) {
-          const int nc = n0 + c * CH;
+          const int nc = n0 + c * CW;
           if (nc >= pN) break;
           const int slot = cq % NS;
           ok = mbar_wait(&slot_empty[slot], ((cq / NS) & 1) ^ 1, abortp, a.status, 6);
           if (!ok) break;
           mbar_expect_tx(&slot_full[slot], AUX_BYTES);
           if (EPI == EPI_SGD) tma_load_3d(slots + slot * SLOT_BYTES, &maps.c32[pi], &slot_full[slot], nc, m0, g);
-          else tma_load_3d(slots + slot * SLOT_BYTES + F32_BYTES, &maps.aux16[pi], &slot_full[slot], nc, m0, g);
+          else if (kSplit) {
+            tma_load_3d(slots + slot * SLOT_BYTES, &maps.c16[pi], &slot_full[slot], nc, m0, g);
+            tma_load_3d(slots + slot * SLOT_BYTES + B16_BYTES, &maps.c32[pi], &slot_full[slot], nc, m0, g);
+          } else tma_load_3d(slots + slot * SLOT_BYTES + F32_BYTES, &maps.aux16[pi], &slot_full[slot], nc, m0, g);
         }
       }
       if (!ok) {
@@ -807,7 +874,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const int g = at.slab;
         unsigned stored = 0;                 // chunks of this tile this thread has stored
         const bool head = EPI == EPI_BIAS_RELU && pr.head_f32;
-        const int cw = head ? CH / 2 : CH, nch = head ? 2 * NCH : NCH;
+        const int cw = head ? CW / 2 : CW, nch = head ? 2 * NCH : NCH;
         for (int c = 0; c < nch; ++c, ++cq) {
           const int nc = n0 + c * cw;
           if (nc >= pr.N) break;
@@ -823,10 +890,11 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           } else {
             if (ET::k32) tma_store_3d(&maps.c32[pi], f32, nc, m0, g);
             if (ET::k16) tma_store_3d(&maps.c16[pi], f32 + F32_BYTES, nc, m0, g);
+            if (kSplit) tma_store_3d(&maps.c32[pi], f32 + B16_BYTES, nc, m0, g);
           }
           tma_commit_group();
           ++stored;
-          if (EPI == EPI_SGD && PAIR == 2) {
+          if (is_update(EPI) && PAIR == 2) {
             // The same chunk of this unit's next tile is asked into L2 now, one tile ahead of its
             // load, so that the load finds it there.  The request is issued here, where the
             // thread would wait for its store anyway; issued by the loader it delayed the loads.
@@ -835,9 +903,11 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
             const int nt = tile + n_units;
             if (nt < total_tiles) {
               const TileAt nx = locate(a, nt, pi_next);
-              const int pn = nx.nt * BN + c * CH;
-              if (pn < a.p[pi_next].N)
+              const int pn = nx.nt * BN + c * CW;
+              if (pn < a.p[pi_next].N) {
                 tma_prefetch_l2_3d(&maps.c32[pi_next], pn, nx.mt * (BM * PAIR) + rank * BM, nx.slab);
+                if (kSplit) tma_prefetch_l2_3d(&maps.c16[pi_next], pn, nx.mt * (BM * PAIR) + rank * BM, nx.slab);
+              }
             }
           }
           // once the store has read the slot it can be refilled (by the loader) or rewritten (by
@@ -1078,7 +1148,8 @@ bool make_map(CUtensorMap* out, const void* base, int elem_bytes, long long inne
 template <int A_MN, int B_MN, int BN, int STAGES, int NS, int EPI, int PAIR>
 bool launch(const Launch& L, const TcMaps& m, const TcArgs& t) {
   using ET = EpiTraits<EPI>;
-  constexpr int slot_bytes = (ET::k32 ? BM * CH * 4 : 0) + (ET::k16 ? BM * CH * 2 : 0);
+  constexpr int CW = chunk_cols(EPI, PAIR);
+  constexpr int slot_bytes = BM * CW * ((ET::k32 ? 4 : 0) + (ET::k16 ? 2 : 0) + (EPI == EPI_SGD_SPLIT ? 2 : 0));
   constexpr int smem = STAGES * (BM * BK * 2 + (BN / PAIR) * BK * 2) + NS * slot_bytes + 1024;
   static_assert(smem <= 227 * 1024 - 512, "shared memory budget exceeded");
   auto kern = gemm_tc_kernel<A_MN, B_MN, BN, STAGES, NS, EPI, PAIR>;
@@ -1151,11 +1222,12 @@ bool gemm_tc_wait_selftest(const Launch& L, DeviceStatus* st, long long limit_cy
 // 1472-1664-6656-37, S = 9, 200 rows 456 -> 442 us; 3072-16384-16384-10, S = 8, 128 rows 2190 -> 2123 us (128
 // columns); 512 rows pairs as before.
 //
-// Weight updates: bound by streaming the masters, 10 bytes per weight, so long as the contraction (the
+// Weight updates: bound by streaming the masters, 8 bytes per weight, so long as the contraction (the
 // batch) is short, and then small tiles keep more transfers in flight: up to 128 rows 64 columns on single CTAs
 // (120-26586-2688-509, S = 9, 128 rows: 804 -> 733 us against pairs; 3072-16384-16384-10 within 1 %).  Up to
 // 320 rows still where the pairs' tiles hang over the matrices' edges by more than 15 % (the same
-// network at 224 rows 890 -> 845 us; 1024-4096-4096-35, which pairs tile exactly, 477 against 484 us).  Not
+// network at 224 rows 890 -> 845 us; 1024-4096-4096-35, which pairs tile exactly, 477 against 484 us), with 128 columns
+// where the masters are split (1001-5000-3001-77, S = 6, 200 rows: the launch 32.9 us with 64, 31.3 with 128).  Not
 // with a layer of more than 8192 columns, whose update streams from DRAM: an output layer of 670,091
 // classes behind 1024 neurons, S = 8, 256 rows, 54.3 ms with 128 columns and 56.8 with 64; 30,000 classes at 128 rows
 // 851 and 874 us.  Hidden layers of 9000 to 20,000 neurons would gain 1 to 4 % up to 128 rows (512-20000-2048-10,
@@ -1182,7 +1254,7 @@ TileChoice pick_tile(const GemmArgs<bf16>* a, int n, int epi) {
   if (epi == EPI_SGD) {
     const int rows = a[0].K;
     const bool overhang = (double)tiles(2 * BM, 256) * (2 * BM * 256) > 1.15 * (double)tiles(BM, 64) * (BM * 64);
-    if (pair_ok && !huge && (rows <= 128 || (rows <= 320 && overhang))) return {64, 1};
+    if (pair_ok && !huge && (rows <= 128 || (rows <= 320 && overhang))) return {rows > 128 && a[0].lo ? 128 : 64, 1};
     if (pair_ok && 4 * tiles(2 * BM, 256) >= 3 * (sms / 2)) return {256, 2};
     return {(mid && tiles(BM, 128) >= sms) ? 128 : 64, 1};
   }
@@ -1254,6 +1326,7 @@ bool gemm_tc_batch(const Launch& L, const GemmArgs<bf16>* ga, int n, const GemmC
     const bool ai = a.a_sm == 1 && a.a_sk != 1, bi = a.b_sn == 1 && a.b_sk != 1;
     const bool is_head = head && i == n - 1;
     if ((a.epi != epi && !is_head) || ai != a_mn || bi != b_mn) return false;   // one kernel instance serves the batch
+    if (epi == EPI_SGD && (a.lo != nullptr) != (a0.lo != nullptr)) return false;
     if (!ai && a.a_sk != 1) return false;
     if (!bi && a.b_sk != 1) return false;
     if (n > 1 && a.k_splits > 1 && !is_head) return false;
@@ -1363,8 +1436,13 @@ bool gemm_tc_batch(const Launch& L, const GemmArgs<bf16>* ga, int n, const GemmC
         break;
       case EPI_SGD:
         if (!a_mn || !b_mn || !a.opw) return false;
-        if (!make_map(&m.c32[i], a.outf, 4, n_store, a.M, a.G, a.outf_ld, a.outf_sg, CH, BM, 128)) return false;
-        if (!make_map(&m.c16[i], a.opw, 2, n_store, a.M, a.G, a.outf_ld, a.outf_sg, CH, BM, 64)) return false;
+        {
+          const int cw = a.lo ? chunk_cols(EPI_SGD_SPLIT, pair) : CH;
+          if (a.lo ? !make_map(&m.c32[i], a.lo, 2, n_store, a.M, a.G, a.outf_ld, a.outf_sg, cw, BM, 2 * cw)
+                   : !make_map(&m.c32[i], a.outf, 4, n_store, a.M, a.G, a.outf_ld, a.outf_sg, cw, BM, 4 * cw))
+            return false;
+          if (!make_map(&m.c16[i], a.opw, 2, n_store, a.M, a.G, a.outf_ld, a.outf_sg, cw, BM, 2 * cw)) return false;
+        }
         break;
       default:
         return false;
@@ -1419,6 +1497,11 @@ bool gemm_tc_batch(const Launch& L, const GemmArgs<bf16>* ga, int n, const GemmC
       if (bn == 128) return launch<0, 0, 128, 6, 4, EPI_RELU_MASK, 1>(L, m, t);
       return launch<0, 0, 64, 8, 4, EPI_RELU_MASK, 1>(L, m, t);
     case EPI_SGD:
+      if (a0.lo) {
+        if (pair == 2) return launch<1, 1, 256, 4, 6, EPI_SGD_SPLIT, 2>(L, m, t);
+        if (bn == 128) return launch<1, 1, 128, 4, 2, EPI_SGD_SPLIT, 1>(L, m, t);
+        return launch<1, 1, 64, 6, 2, EPI_SGD_SPLIT, 1>(L, m, t);
+      }
       if (pair == 2) return launch<1, 1, 256, 4, 4, EPI_SGD, 2>(L, m, t);
       if (bn == 128) return launch<1, 1, 128, 4, 4, EPI_SGD, 1>(L, m, t);
       return launch<1, 1, 64, 5, 4, EPI_SGD, 1>(L, m, t);

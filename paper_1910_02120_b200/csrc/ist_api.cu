@@ -72,6 +72,12 @@ struct ist_ctx {
   int rule = IST_PART_BALANCED;
   std::vector<std::vector<int64_t>> group_count;   // [hidden layer][subnet]
 
+  // Masters of layers updated by the tensor-core launches are kept as operand + low half (split_master): the
+  // operand in its own buffer, the low halves in the second half of the layer's master buffer.  A context whose packed
+  // slices have been asked for (ist_packed_layer) holds fp32 words from then on.
+  bool packed_seen = false;
+  bool split(int l) const { return precision == IST_BF16 && !packed_seen && !(csr && l == 1); }
+
   // subnets this context trains in ist_local_steps (all S unless ist_set_subnet_range narrowed it)
   int sub_first = 0, sub_count = 0;
 
@@ -122,6 +128,9 @@ struct ist_ctx {
   bf16* opw(int l) const { return precision == IST_BF16 ? plan.opw[l].at<bf16>(ws) : nullptr; }
   int64_t rows_pad(int l) const { return np[l - 1]; }              // packed rows of layer l
   int64_t slice_elems(int l) const { return np[l - 1] * ld[l]; }   // per subnet
+  uint16_t* lo(int l) const {
+    return split(l) ? reinterpret_cast<uint16_t*>(master(l)) + (int64_t)S * slice_elems(l) : nullptr;
+  }
 };
 
 namespace {
@@ -462,6 +471,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
   auto delta = [&](int l) { return c->plan.delta[l].at<T>(c->ws); };
   auto master = [&](int l) { return c->master(l) + (int64_t)s0 * c->slice_elems(l); };
   auto opw = [&](int l) -> bf16* { return bf ? c->opw(l) + (int64_t)s0 * c->slice_elems(l) : nullptr; };
+  auto lo = [&](int l) -> uint16_t* { return c->split(l) ? c->lo(l) + (int64_t)s0 * c->slice_elems(l) : nullptr; };
   auto bias_of = [&](int l) { return c->bias(l) + (int64_t)s0 * c->ld[l]; };
   auto weights = [&](int l) -> const T* {       // operand copy of layer l's slices
     return bf ? reinterpret_cast<const T*>(opw(l)) : reinterpret_cast<const T*>(master(l));
@@ -708,6 +718,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       g.epi = EPI_SGD;
       g.outf = master(l); g.outf_ld = c->ld[l]; g.outf_sg = c->slice_elems(l);
       g.opw = opw(l);
+      g.lo = lo(l);
       g.lr = lr;
       upd.push_back(g);
     }
@@ -882,8 +893,8 @@ extern "C" ist_status ist_partition(ist_ctx* c, uint64_t seed) {
     Scope sc(c, IST_K_GATHER);
     std::vector<SliceJob> jobs;
     for (int l = 1; l <= t; ++l) {
-      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), c->opw(l), slice_map(c, l, c->sub_first), c->sub_count, 0});
-      jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l, c->sub_first), c->sub_count, 0});
+      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), c->opw(l), slice_map(c, l, c->sub_first), c->sub_count, c->lo(l), 0});
+      jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l, c->sub_first), c->sub_count, nullptr, 0});
     }
     gather_slices(L, jobs.data(), (int)jobs.size(), c->status());
   }
@@ -933,10 +944,12 @@ extern "C" ist_status ist_get_subnet_params(ist_ctx* c, int layer, int s, float*
   auto count = [&](int l) { return group_size(c, l, s); };
   Launch L = c->launch();
   if (W_out_dev)
-    copy_out_slice(L, c->master(layer) + (int64_t)s * c->slice_elems(layer), c->ld[layer],
+    copy_out_slice(L, c->master(layer) + (int64_t)s * c->slice_elems(layer),
+                   c->split(layer) ? c->opw(layer) + (int64_t)s * c->slice_elems(layer) : nullptr,
+                   c->split(layer) ? c->lo(layer) + (int64_t)s * c->slice_elems(layer) : nullptr, c->ld[layer],
                    count(layer - 1), count(layer), W_out_dev);
   if (b_out_dev)
-    copy_out_slice(L, c->bias(layer) + (int64_t)s * c->ld[layer], c->ld[layer], 1, count(layer), b_out_dev);
+    copy_out_slice(L, c->bias(layer) + (int64_t)s * c->ld[layer], nullptr, nullptr, c->ld[layer], 1, count(layer), b_out_dev);
   IST_CUDA(c, cudaGetLastError());
   return IST_OK;
 }
@@ -984,6 +997,15 @@ extern "C" ist_status ist_packed_layer(ist_ctx* c, int layer, void** master_dev,
                                        void** bias_dev, size_t* bias_bytes_per_subnet) {
   if (!c) return IST_ERR_ARG;
   if (layer < 1 || layer > c->t) return fail(c, IST_ERR_ARG, "layer outside 1..t");
+  if (!c->packed_seen) {
+    // the caller reads and writes fp32 slices from here on: those in place are converted now
+    if (c->state == ST_PARTITIONED) {
+      for (int l = 1; l <= c->t; ++l)
+        if (c->split(l)) join_masters(c->launch(), c->master(l), c->opw(l), (int64_t)c->S * c->slice_elems(l));
+      IST_CUDA(c, cudaGetLastError());
+    }
+    c->packed_seen = true;
+  }
   if (master_dev) *master_dev = c->master(layer);
   if (master_bytes_per_subnet) *master_bytes_per_subnet = (size_t)c->slice_elems(layer) * 4;
   if (bias_dev) *bias_dev = c->bias(layer);
@@ -1000,8 +1022,8 @@ extern "C" ist_status ist_reassemble(ist_ctx* c) {
     Scope sc(c, IST_K_SCATTER);
     std::vector<SliceJob> jobs;
     for (int l = 1; l <= t; ++l) {
-      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), nullptr, slice_map(c, l), S, 0});
-      jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l), S, l == t ? 1 : 0});
+      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), c->opw(l), slice_map(c, l), S, c->lo(l), 0});
+      jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l), S, nullptr, l == t ? 1 : 0});
     }
     scatter_slices(L, jobs.data(), (int)jobs.size(), c->status());
   }

@@ -67,13 +67,16 @@ struct SliceJob {
   bf16* opw;
   SliceMap m;
   int S;
+  uint16_t* lo;  // null: master holds fp32 values (and opw, where given, the operands); else the master is (opw, lo), see split_master
   int mean;      // scatter only: the output bias, b[j] += (sum_s (packed[s][j] - b[j])) / S
 };
 void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
 void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
-// Dense copy-out of a packed slice (ist_get_subnet_params).
-void copy_out_slice(const Launch& L, const float* packed, int64_t ld, int64_t rows, int64_t cols,
-                    float* out);
+// Dense copy-out of a packed slice (ist_get_subnet_params); lo as in SliceJob.
+void copy_out_slice(const Launch& L, const float* packed, const bf16* opw, const uint16_t* lo, int64_t ld, int64_t rows,
+                    int64_t cols, float* out);
+// n masters kept as (opw, lo) become fp32 values in place: lo is the second half of the n fp32 words at `master`.
+void join_masters(const Launch& L, float* master, const bf16* opw, int64_t n);
 
 // ---- grouped GEMM -----------------------------------------------------------------------
 // C[g](m, n) = sum_k A[g](m, k) * B[g](n, k), fp32 accumulation, followed by an epilogue.
@@ -86,7 +89,8 @@ enum Epilogue : int {
   // Softmax cross-entropy over a very wide output layer without storing the logits (two passes
   // over the same product):
   EPI_LSE_PART = 5,   // per row and column tile: (max, sum exp(z - max)) of z = C + bias -> lse_part
-  EPI_SOFTMAX_DELTA = 6  // out = T((exp(z - lse[m]) - [n == label[m]]) * inv_rows); z[m][label[m]] -> label_logit
+  EPI_SOFTMAX_DELTA = 6, // out = T((exp(z - lse[m]) - [n == label[m]]) * inv_rows); z[m][label[m]] -> label_logit
+  EPI_SGD_SPLIT = 7   // EPI_SGD with the masters kept as operand + low half (GemmArgs::lo); asked for as EPI_SGD
 };
 
 template <typename T>
@@ -115,6 +119,7 @@ struct GemmArgs {
   float* outf; int64_t outf_ld, outf_sg;
   const T* mask; int64_t mask_ld, mask_sg;
   bf16* opw;
+  uint16_t* lo;   // EPI_SGD: not null: the master is (opw, lo), see split_master, and outf is not used
   float lr;
   // wide softmax head.  lse_part: [G][gemm_tc_lse_parts(N_store)][M] float2 (a few partials per
   // 256-column tile); lse / label_logit: [G][lse_sg]; labels: labels[g * labels_sg + m].
