@@ -86,6 +86,39 @@ __device__ __forceinline__ uint16_t operand_bits(float w) {
   return hi;
 }
 
+// Bits of an updated master.  The NaN that arithmetic gives, 0x7fffffff, would round to minus zero: the signed minimum
+// makes it one that stays a NaN and leaves every number as it is.
+__device__ __forceinline__ uint32_t master_bits(float w) { return (uint32_t)min(__float_as_int(w), 0x7fff7fff); }
+// The operands of eight masters (see split_master), as one 16-byte unit.
+__device__ __forceinline__ uint4 pack8_operand(const float* w) {
+  uint32_t h[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) h[e] = master_bits(w[e]) + 0x8000u;
+  return make_uint4(__byte_perm(h[0], h[1], 0x7632), __byte_perm(h[2], h[3], 0x7632), __byte_perm(h[4], h[5], 0x7632),
+                    __byte_perm(h[6], h[7], 0x7632));
+}
+// Eight masters kept as operand and low half: joined, and taken apart again.
+__device__ __forceinline__ void join8(const uint4& h, const uint4& l, float* w) {
+  const uint32_t hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    w[2 * i] = __uint_as_float((hv[i] << 16) + (uint32_t)((int)(lv[i] << 16) >> 16));
+    w[2 * i + 1] = __uint_as_float((hv[i] & 0xffff0000u) + (uint32_t)((int)lv[i] >> 16));
+  }
+}
+__device__ __forceinline__ void split8(const float* w, uint4* h, uint4* l) {
+  uint32_t v[8], hv[4], lv[4];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = master_bits(w[e]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    hv[i] = __byte_perm(v[2 * i] + 0x8000u, v[2 * i + 1] + 0x8000u, 0x7632);
+    lv[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
+  }
+  *h = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+  *l = make_uint4(lv[0], lv[1], lv[2], lv[3]);
+}
+
 __device__ __forceinline__ float to_float(float v) { return v; }
 __device__ __forceinline__ float to_float(bf16 v) { return __bfloat162float(v); }
 template <typename T> __device__ __forceinline__ T from_float(float v);

@@ -66,6 +66,7 @@
 
 #include "kernels.h"
 #include "tc_ptx.cuh"
+#include "tma_map.h"
 
 namespace ist {
 namespace {
@@ -242,39 +243,6 @@ __device__ __forceinline__ void unpack8(uint4 u, float* v) {
   __nv_bfloat162 c = *reinterpret_cast<__nv_bfloat162*>(&u.z), d = *reinterpret_cast<__nv_bfloat162*>(&u.w);
   v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b);
   v[4] = __low2float(c); v[5] = __high2float(c); v[6] = __low2float(d); v[7] = __high2float(d);
-}
-
-// Bits of an updated master.  The NaN that arithmetic gives, 0x7fffffff, would round to minus zero: the signed minimum
-// makes it one that stays a NaN and leaves every number as it is.
-__device__ __forceinline__ uint32_t master_bits(float w) { return (uint32_t)min(__float_as_int(w), 0x7fff7fff); }
-// The operands of eight masters (see split_master), as one 16-byte unit.
-__device__ __forceinline__ uint4 pack8_operand(const float* w) {
-  uint32_t h[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) h[e] = master_bits(w[e]) + 0x8000u;
-  return make_uint4(__byte_perm(h[0], h[1], 0x7632), __byte_perm(h[2], h[3], 0x7632), __byte_perm(h[4], h[5], 0x7632),
-                    __byte_perm(h[6], h[7], 0x7632));
-}
-// Eight masters kept as operand and low half: joined, and taken apart again.
-__device__ __forceinline__ void join8(const uint4& h, const uint4& l, float* w) {
-  const uint32_t hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    w[2 * i] = __uint_as_float((hv[i] << 16) + (uint32_t)((int)(lv[i] << 16) >> 16));
-    w[2 * i + 1] = __uint_as_float((hv[i] & 0xffff0000u) + (uint32_t)((int)lv[i] >> 16));
-  }
-}
-__device__ __forceinline__ void split8(const float* w, uint4* h, uint4* l) {
-  uint32_t v[8], hv[4], lv[4];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) v[e] = master_bits(w[e]);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    hv[i] = __byte_perm(v[2 * i] + 0x8000u, v[2 * i + 1] + 0x8000u, 0x7632);
-    lv[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
-  }
-  *h = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-  *l = make_uint4(lv[0], lv[1], lv[2], lv[3]);
 }
 
 // Row r of a chunk slot.  fp32 area: 128-byte rows, 16-byte unit u stored at u ^ (r & 7).
@@ -1087,6 +1055,18 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+using MapKey = std::tuple<const void*, long long, long long, long long, long long, long long, int, int, int, int>;
+std::map<MapKey, CUtensorMap>& map_cache() {
+  static std::map<MapKey, CUtensorMap> c;
+  return c;
+}
+std::mutex& map_mutex() {
+  static std::mutex m;
+  return m;
+}
+
+}  // namespace
+
 int sm_count() {
   static int n = 0;
   static std::once_flag once;
@@ -1097,18 +1077,6 @@ int sm_count() {
       n = 148;
   });
   return n;
-}
-
-// Tensor [groups][outer][inner] (inner contiguous, strides in elements) with box
-// {box_inner, box_outer, 1}.  elem_bytes 2 = bf16, 4 = fp32.  swizzle_bytes 128 or 64.
-using MapKey = std::tuple<const void*, long long, long long, long long, long long, long long, int, int, int, int>;
-std::map<MapKey, CUtensorMap>& map_cache() {
-  static std::map<MapKey, CUtensorMap> c;
-  return c;
-}
-std::mutex& map_mutex() {
-  static std::mutex m;
-  return m;
 }
 
 bool make_map(CUtensorMap* out, const void* base, int elem_bytes, long long inner, long long outer,
@@ -1144,6 +1112,8 @@ bool make_map(CUtensorMap* out, const void* base, int elem_bytes, long long inne
   cache[key] = *out;
   return true;
 }
+
+namespace {
 
 template <int A_MN, int B_MN, int BN, int STAGES, int NS, int EPI, int PAIR>
 bool launch(const Launch& L, const TcMaps& m, const TcArgs& t) {

@@ -447,6 +447,11 @@ void small_softmax(const Launch& L, const float* part, int ks, int64_t ld, int G
                    float* row_loss, DeviceStatus* st) {
   softmax_xent_small<bf16>(L, part, ks, ld, G, B, Nt, bias, bias_sg, y, y_sg, delta, ld_d, sg_d, row_loss, st);
 }
+// The one-kernel second pass over a very wide output layer; operands and low halves exist on the bf16 path only.
+bool fused_head_ok(const WideHead&, const float*) { return false; }
+bool fused_head_ok(const WideHead& w, const bf16*) { return w.lo && wide_head_ok(w); }
+void head_buffers(WideHead&, const float*, float*) {}
+void head_buffers(WideHead& w, const bf16* x, bf16* delta) { w.x = x; w.delta = delta; }
 // A product written as plain fp32: with bf16 operands the fp32 epilogue without a bias, with fp32
 // operands (output of the same type) a plain store.
 void set_plain_fp32_output(GemmArgs<bf16>& g, float* out, int64_t ld, int64_t sg) {
@@ -530,6 +535,21 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       colnorm_forward<T>(L, c->zbuf(l), c->ld[l], Bm * c->ld[l], S, B, (int)c->np[l], c->norm_eps, c->nmu(l),
                          c->nrstd(l), c->ld[l], act(l), Bm * c->ld[l]);
     };
+    WideHead wh{};
+    if (wide && t > 1) {
+      wh.S = S; wh.B = B; wh.H = (int)c->np[t - 1]; wh.N = (int)c->N[t];
+      wh.ldx = (int)c->ld[t - 1]; wh.x_sg = Bm * c->ld[t - 1];
+      head_buffers(wh, act(t - 1), delta(t - 1));
+      wh.opw = opw(t); wh.lo = lo(t); wh.ldw = c->ld[t]; wh.w_sg = c->slice_elems(t);
+      wh.bias = bias_of(t);
+      wh.lse = lse; wh.labels = y + row0; wh.label_logit = label_logit; wh.lse_sg = Bm; wh.labels_sg = X->stride_subnet;
+      wh.lse_part = logits;
+      wh.row_loss = row_loss;
+      wh.lr = lr;
+      wh.scratch = reinterpret_cast<float*>(delta(t));   // the deltas themselves are not stored
+      wh.scratch_bytes = (size_t)c->S * Bm * c->ld[t] * sizeof(T);
+    }
+    const bool fused_head = wide && t > 1 && fused_head_ok(wh, (const T*)nullptr);
     // ---- forward ---------------------------------------------------------------------------
     // Hidden layers without standardisation form a chain a_l = relu(a_{l-1} W_l + b_l): they are
     // collected and go out together (tiles of one launch, see gemm_list).
@@ -598,7 +618,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       if (!flush_fwd()) return fail(c, IST_ERR_UNSUPPORTED, "forward GEMMs below layer %d cannot be launched", l);
       {
         Scope sc(c, IST_K_FWD);
-        if (!gemm(c, g)) return fail(c, IST_ERR_UNSUPPORTED, "forward GEMM of layer %d cannot be launched", l);
+        if (l == t && fused_head ? !wide_head_lse(L, wh, st) : !gemm(c, g)) return fail(c, IST_ERR_UNSUPPORTED, "forward GEMM of layer %d cannot be launched", l);
       }
       if (l < t && c->norm) standardise(l);
     }
@@ -606,7 +626,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     // ---- loss and its gradient -------------------------------------------------------------
     {
       Scope sc(c, IST_K_LOSS);
-      if (wide) {
+      if (wide && !fused_head) {
         lse_combine(L, logits, gemm_tc_lse_parts(c->ld[t]), S, B, Bm, lse, y + row0, X->stride_subnet, (int)c->N[t], st);
         GemmArgs<T> g{};             // second pass: the same product, written out as delta_t
         g.M = B; g.N = (int)c->np[t]; g.K = (int)c->np[t - 1]; g.G = S;
@@ -623,6 +643,8 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
         g.inv_rows = 1.f / (float)B;
         if (!gemm(c, g)) return fail(c, IST_ERR_UNSUPPORTED, "softmax pass of the output layer cannot be launched");
         lse_row_loss(L, lse, label_logit, S, B, Bm, row_loss);
+      } else if (wide) {
+        // the rows' log-sum-exps are there; everything else about the layer follows in one pass below
       } else if (head)
         small_softmax(L, logits, head_ks, c->ld[t], S, B, (int)c->N[t], bias_of(t), c->ld[t], y + row0,
                       X->stride_subnet, delta(t), c->ld[t], Bm * c->ld[t], row_loss, st);
@@ -631,6 +653,10 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
                       X->stride_subnet, delta(t), c->ld[t], Bm * c->ld[t], row_loss, st);
     }
     // ---- backward + SGD, last layer first --------------------------------------------------
+    if (fused_head) {
+      Scope sc(c, IST_K_DW_SGD);
+      if (!wide_head_pass(L, wh, st)) return fail(c, IST_ERR_UNSUPPORTED, "the pass over the output layer cannot be launched");
+    }
     // db_l = sum_b delta_l, layers l_lo..l_hi (kMaxBiasLayers of them at most); the step's mean losses may be
     // reduced by the same blocks
     auto bias_args = [&](int l_hi, int l_lo, bool with_loss) {
@@ -659,7 +685,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       return ok;
     };
     for (int l = t; l > 1; --l) {
-      {
+      if (!(fused_head && l == t)) {
         GemmArgs<T> g{};
         g.M = B; g.N = (int)c->np[l - 1]; g.K = (int)c->np[l]; g.G = S;
         g.N_store = (int)c->ld[l - 1];
@@ -707,7 +733,8 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     }
     // the weight updates of the dense layers do not depend on one another: tiles of one launch
     std::vector<GemmArgs<T>> upd;
-    for (int l = t; l >= 1; --l) {
+    const int top = fused_head ? t - 1 : t;   // the highest layer that is still to be updated
+    for (int l = top; l >= 1; --l) {
       if (l == 1 && X->kind == IST_X_CSR && t > 1) continue;
       GemmArgs<T> g{};
       g.M = (int)c->np[l - 1]; g.N = (int)c->np[l]; g.K = B; g.G = S;
@@ -733,7 +760,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     // path, and fp32 networks of more bias work (see bias_beside) or more layers than such a launch takes along.
     const bool sparse_first = X->kind == IST_X_CSR && t > 1;
     size_t delta_bytes = 0;
-    for (int l = 1; l <= t; ++l) delta_bytes += (size_t)S * B * c->ld[l] * sizeof(T);
+    for (int l = 1; l <= top; ++l) delta_bytes += (size_t)S * B * c->ld[l] * sizeof(T);
     const bool bias_first = delta_bytes <= kL2ResidentBytes;
     // beside the tiles while the blocks of bias work (one of them per SM, where the bias kernel has eight) are no
     // more than two rounds: 14552-1608-4530, S = 11, in fp32 with 800 of them: 6 us a step slower beside
@@ -743,11 +770,11 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     const bool from_stages = bias_in_gemm && !bias_first && update_sums_bias(upd);
     if (bias_in_gemm) {
       for (auto& g : upd) {
-        const int l = t - (int)(&g - upd.data());   // upd[i] is layer t - i
+        const int l = top - (int)(&g - upd.data());   // upd[i] is layer top - i
         g.bias_upd = bias_of(l); g.bias_upd_sg = c->ld[l]; g.bias_n = (int)c->np[l];
         g.bias_upd_from_memory = from_stages ? 0 : 1;
       }
-      if (sparse_first) update_biases(1, 1, false);
+      if (sparse_first) update_biases(1, 1, upd.empty());
     } else if (!bias_beside) {
       update_biases(t, 1);
     }

@@ -163,6 +163,27 @@ bool gemm_tc_wait_selftest(const Launch& L, DeviceStatus* st, long long limit_cy
 int gemm_tc_splits(int K, int want);
 int gemm_tc_lse_parts(int64_t n_store);
 
+// ---- wide_head.cu -----------------------------------------------------------------------
+// A very wide output layer behind a narrow hidden layer.  wide_head_lse: the rows' log-sum-exp (labels checked on
+// the way).  wide_head_pass: all that follows it: delta, the input gradient of the layer below, the update of the
+// layer's weights (operand + low half) and bias, the rows' losses.  Two launches each.
+struct WideHead {
+  int S, B, H, N;                  // subnets, rows, width of the layer below, classes
+  const bf16* x; int ldx; long long x_sg;          // activations of the layer below, [S][..][ldx], x_sg apart
+  bf16* delta;                     // delta of the layer below, laid out like x
+  bf16* opw; uint16_t* lo; long long ldw, w_sg;    // [S][H][ldw]
+  float* bias;                     // [S][ldw]
+  float* lse; const int32_t* labels; float* label_logit; long long lse_sg, labels_sg;
+  float* lse_part;                 // scratch of the first pass, as much as gemm_tc_lse_parts asks for
+  float* row_loss;                 // [S][B]
+  float lr;
+  float* scratch; size_t scratch_bytes;            // partial sums of the input gradient
+};
+// Whether the pass takes this shape: at most 128 neurons and 256 rows, scratch for half the SMs at least.
+bool wide_head_ok(const WideHead& w);
+bool wide_head_lse(const Launch& L, const WideHead& w, DeviceStatus* st);
+bool wide_head_pass(const Launch& L, const WideHead& w, DeviceStatus* st);
+
 // ---- rowops.cu --------------------------------------------------------------------------
 // Row-wise softmax cross-entropy of logits [G][B][ld] against labels; writes
 // delta = (softmax - onehot)/B (zero in columns Nt..ld_d) and row_loss [G][B].

@@ -1,0 +1,75 @@
+"""One pass over a very wide output layer (delta, input gradient, update, bias, losses) against the launches it
+stands in for, which a context that hands out fp32 slices still takes: the same operands are multiplied and only the
+order of the fp32 sums differs.  One local step, so that nothing feeds back."""
+import pytest
+import torch
+
+from oracle import ist_oracle as O
+from paper_1910_02120_b200 import api, synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+def _step(dims, S, B, fused, norm=False, csr=False, K=1, lr=0.5):
+    g = torch.Generator(device="cuda").manual_seed(7)
+    W = [torch.randn(a, b, device="cuda", generator=g) * (2.0 / a) ** 0.5 for a, b in zip(dims, dims[1:])]
+    b = [torch.randn(n, device="cuda", generator=g) * 0.1 for n in dims[1:]]
+    rows = S * K * B
+    if csr:
+        col = torch.stack([torch.randperm(dims[0], device="cuda", generator=g)[:5].sort().values for _ in range(rows)]).int()
+        X = (torch.arange(0, 5 * rows + 1, 5, device="cuda", dtype=torch.int32), col.view(-1).contiguous(),
+             torch.randn(5 * rows, device="cuda", generator=g).abs())
+    else:
+        X = torch.randn(rows, dims[0], device="cuda", generator=g).bfloat16()
+    y = torch.randint(dims[-1], (rows,), device="cuda", generator=g, dtype=torch.int32)
+    y[0], y[-1] = 0, dims[-1] - 1
+    ctx = api.Ist(dims, S, api.IST_BF16, B, input_is_csr=csr)
+    ctx.bind_weights([w.clone() for w in W], [v.clone() for v in b])
+    if norm:
+        ctx.enable_normalization(1e-5)
+    if not fused:
+        ctx.packed_layer(1)
+    ctx.profile(True)
+    loss = ctx.round(3, X, y, lr, K, B)
+    ctx.sync_status()
+    return W + b, ctx.W + ctx.b, loss, ctx.profile_read()["loss"][0]   # the separate launches: three of this class
+
+
+# widths of the hidden slice (one and two 64-neuron halves, remainders of 16 and of 8), batches (one and two blocks of 128
+# rows, remainders), classes (remainders of 64 and of 8), subnets that share CTAs and that do not
+@pytest.mark.parametrize("dims,S,B,kind", [
+    ([16, 128, 20008], 1, 256, ""), ([16, 8, 8193], 1, 1, ""), ([32, 300, 9001], 3, 129, ""), ([24, 64, 12000], 1, 128, ""),
+    ([64, 640, 8200], 5, 77, "norm"), ([40, 256, 384, 10007], 3, 200, ""), ([500, 1024, 20011], 8, 256, "csr"),
+    ([300, 96, 65, 8300], 2, 31, "csr"), ([16, 160, 40000], 16, 40, "")])
+def test_against_the_separate_launches(dims, S, B, kind):
+    kw = dict(norm=kind == "norm", csr=kind == "csr")
+    start, got, loss, n_fused = _step(dims, S, B, True, **kw)
+    _, want, loss_ref, n_ref = _step(dims, S, B, False, **kw)
+    assert n_fused == 0 and n_ref == 3
+    # the losses come from the same log-sum-exps and from logits that differ in the order of at most 128 products
+    assert torch.allclose(loss, loss_ref, rtol=1e-6, atol=1e-6)
+    t = len(dims) - 1
+    for i, (p0, p, q) in enumerate(zip(start, got, want)):
+        if kind == "norm" and t <= i < 2 * t - 1:
+            continue                                        # a standardised layer's bias has no gradient but rounding errors
+        upd, ref = (p - p0).double(), (q - p0).double()
+        err = float((upd - ref).norm() / ref.norm().clamp_min(1e-30))
+        # output layer: delta is the same bf16 numbers (a logit on the edge of a rounding aside, 2^-9 of one entry) and
+        # the update is rounded to fp32 weights, 2^-24 of a weight against an update of at least 2^-12 of it; layers
+        # below: their delta is rounded to bf16 from sums in another order, an ulp (2^-8) in a few per cent of entries
+        assert err <= (2e-3 if i in (t - 1, 2 * t - 1) else 1e-2), (i, err)
+
+
+@pytest.mark.parametrize("dims,S,B,K", [((64, 320, 8300), 4, 160, 2), ((48, 100, 96, 9000), 2, 64, 2)])
+def test_against_the_oracle(dims, S, B, K):
+    w = synth.Workload("h", dims, S=S, B=B, K=K, rounds=1, precision="bf16", x_dist="normal", lr=0.1, seed=8)
+    W, b, data = H.make_problem(w, bias_scale=0.1)
+    o, _, oloss = H.oracle_round(w, W, b, data, 5)
+    _, Wg, bg, parts, gl = H.gpu_round(w, W, b, data, seed=5)
+    for l in range(len(W)):
+        H.assert_close(Wg[l], o.W[l], 2e-2, f"W_{l + 1}")
+        H.assert_close(bg[l], o.b[l], 2e-2, f"b_{l + 1}")
+        upd, ref = Wg[l].astype("float64") - W[l], o.W[l] - W[l]
+        assert ((upd - ref) ** 2).sum() ** 0.5 <= 1e-1 * (ref ** 2).sum() ** 0.5
+    assert abs(float(gl.mean()) - float(oloss.mean())) <= 1e-3
