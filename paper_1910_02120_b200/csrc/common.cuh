@@ -67,15 +67,28 @@ __host__ __device__ __forceinline__ constexpr int64_t round_up(int64_t a, int64_
 }
 
 // An fp32 master and the bf16 operand made from it take 32 bits together: the operand is the master rounded to
-// its upper 16 bits, ties away from zero, and beside it lie the lower 16 bits of the master; the operand's last bit and
-// the low half's first say whether the rounding went up, so the master comes back bit for bit.  (With ties to
-// even, two masters would share an operand and a low half.)  A weight update then moves 8 bytes per weight
-// instead of 10.  NaNs become one NaN: their payloads do not fit.
+// its upper 16 bits (to nearest, ties to even), and beside it lie the lower 16 bits of the master; the operand's last bit
+// and the low half's first say whether the rounding went up, so the master comes back.  A weight update then
+// moves 8 bytes per weight instead of 10.  One pattern does not fit: a tie that rounds down would share its code with the
+// tie that rounds up to the same operand, so it is kept as the value one ulp nearer to zero (one master in 2^17, by
+// 2^-24 of it; rounding ties away from zero instead keeps such masters exact but changes their operands by 2^-8, which
+// turns ReLU masks over).  Where a slice goes back, masters that no step has changed are told by
+// their source (unnudged).  NaNs become one NaN: their payloads do not fit.
+__device__ __forceinline__ uint32_t nudged(uint32_t bits) { return bits - ((bits & 0x1ffffu) == 0x8000u ? 1u : 0u); }
 __device__ __forceinline__ void split_master(float w, uint16_t* hi, uint16_t* lo) {
-  uint32_t u = __float_as_uint(w);
-  if (w != w) u = 0x7fc00000u;
+  const uint32_t u = w != w ? 0x7fc00000u : nudged(__float_as_uint(w));
   *hi = (uint16_t)((u + 0x8000u) >> 16);
   *lo = (uint16_t)u;
+}
+// Whether a joined master may be a nudged one.
+__device__ __forceinline__ bool is_nudged(float v) { return (__float_as_uint(v) & 0x1ffffu) == 0x7fffu; }
+// A joined master v that came from *source: the source itself if v is its nudged form.
+__device__ __forceinline__ float unnudged(float v, const float* source) {
+  if (is_nudged(v)) {
+    const float o = *source;
+    if (__float_as_uint(o) == __float_as_uint(v) + 1u) return o;
+  }
+  return v;
 }
 __device__ __forceinline__ float join_master(uint16_t hi, uint16_t lo) {
   return __uint_as_float(((uint32_t)hi << 16) + (uint32_t)(int)(int16_t)lo);
@@ -86,17 +99,6 @@ __device__ __forceinline__ uint16_t operand_bits(float w) {
   return hi;
 }
 
-// Bits of an updated master.  The NaN that arithmetic gives, 0x7fffffff, would round to minus zero: the signed minimum
-// makes it one that stays a NaN and leaves every number as it is.
-__device__ __forceinline__ uint32_t master_bits(float w) { return (uint32_t)min(__float_as_int(w), 0x7fff7fff); }
-// The operands of eight masters (see split_master), as one 16-byte unit.
-__device__ __forceinline__ uint4 pack8_operand(const float* w) {
-  uint32_t h[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) h[e] = master_bits(w[e]) + 0x8000u;
-  return make_uint4(__byte_perm(h[0], h[1], 0x7632), __byte_perm(h[2], h[3], 0x7632), __byte_perm(h[4], h[5], 0x7632),
-                    __byte_perm(h[6], h[7], 0x7632));
-}
 // Eight masters kept as operand and low half: joined, and taken apart again.
 __device__ __forceinline__ void join8(const uint4& h, const uint4& l, float* w) {
   const uint32_t hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
@@ -106,14 +108,16 @@ __device__ __forceinline__ void join8(const uint4& h, const uint4& l, float* w) 
     w[2 * i + 1] = __uint_as_float((hv[i] & 0xffff0000u) + (uint32_t)((int)lv[i] >> 16));
   }
 }
+// The distance of a master from its operand, in ulps of the master, is -2^15 .. 2^15; saturation to 16 bits is the nudge (and
+// turns the NaN that arithmetic gives into one whose operand is a NaN too).
 __device__ __forceinline__ void split8(const float* w, uint4* h, uint4* l) {
-  uint32_t v[8], hv[4], lv[4];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) v[e] = master_bits(w[e]);
+  uint32_t hv[4], lv[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    hv[i] = __byte_perm(v[2 * i] + 0x8000u, v[2 * i + 1] + 0x8000u, 0x7632);
-    lv[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
+    const __nv_bfloat162 o = __floats2bfloat162_rn(w[2 * i], w[2 * i + 1]);
+    hv[i] = *reinterpret_cast<const uint32_t*>(&o);
+    const uint32_t d0 = __float_as_uint(w[2 * i]) - (hv[i] << 16), d1 = __float_as_uint(w[2 * i + 1]) - (hv[i] & 0xffff0000u);
+    asm("cvt.pack.sat.s16.s32 %0, %1, %2;" : "=r"(lv[i]) : "r"(d1), "r"(d0));
   }
   *h = make_uint4(hv[0], hv[1], hv[2], hv[3]);
   *l = make_uint4(lv[0], lv[1], lv[2], lv[3]);

@@ -71,12 +71,27 @@ template <bool SPLIT>
 __device__ __forceinline__ void scatter_rows(const SliceJob& J, int64_t o0, const int64_t* c, const int32_t* rows, int64_t i0,
                                              int64_t i1) {
   const int64_t ld = J.m.ld, full = J.m.full_cols;
-#pragma unroll 2
-  for (int64_t i = i0; i < i1; ++i, o0 += ld) {
-    const float2 f = value2<SPLIT>(raw2<SPLIT>(J.master, J.opw, J.lo, o0));
-    float* w = J.W + (rows ? rows[i] : i) * full;
-    w[c[0]] = f.x;
-    if (c[1] >= 0) w[c[1]] = f.y;
+  for (int64_t i = i0; i < i1; i += 2, o0 += 2 * ld) {
+    const bool two = i + 1 < i1;
+    const uint2 p0 = raw2<SPLIT>(J.master, J.opw, J.lo, o0), p1 = two ? raw2<SPLIT>(J.master, J.opw, J.lo, o0 + ld) : p0;
+    float* w0 = J.W + (rows ? rows[i] : i) * full;
+    float* w1 = J.W + (two ? (rows ? rows[i + 1] : i + 1) * full : 0);
+    float2 f0 = value2<SPLIT>(p0), f1 = value2<SPLIT>(p1);
+    // both rows' loads have been asked for before this branch, which is hardly ever taken
+    if (SPLIT && (is_nudged(f0.x) | is_nudged(f0.y) | is_nudged(f1.x) | is_nudged(f1.y))) {
+      f0.x = unnudged(f0.x, w0 + c[0]);
+      if (c[1] >= 0) f0.y = unnudged(f0.y, w0 + c[1]);
+      if (two) {
+        f1.x = unnudged(f1.x, w1 + c[0]);
+        if (c[1] >= 0) f1.y = unnudged(f1.y, w1 + c[1]);
+      }
+    }
+    w0[c[0]] = f0.x;
+    if (c[1] >= 0) w0[c[1]] = f0.y;
+    if (two) {
+      w1[c[0]] = f1.x;
+      if (c[1] >= 0) w1[c[1]] = f1.y;
+    }
   }
 }
 
@@ -207,12 +222,24 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, fl
           v[u][c] = f.x;
           v[u][c + 1] = f.y;
           from_pairs(v[u][c], v[u][c + 1]);
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int64_t j = j0 + c * kThreads + e * 32 + lane;
-            if (src[u] >= 0 && j < m.full_cols) W[src[u] + j] = v[u][c + e];
-          }
         }
+      bool rare = false;                     // one branch for all of a thread's values, behind all its loads
+#pragma unroll
+      for (int u = 0; u < kRowU; ++u)
+#pragma unroll
+        for (int c = 0; c < kColU; ++c) rare |= SPLIT && is_nudged(v[u][c]);
+      auto at = [&](int c) { return j0 + (c & ~1) * kThreads + (c & 1) * 32 + lane; };
+      if (rare)
+#pragma unroll
+        for (int u = 0; u < kRowU; ++u)
+#pragma unroll
+          for (int c = 0; c < kColU; ++c)
+            if (src[u] >= 0 && at(c) < m.full_cols) v[u][c] = unnudged(v[u][c], W + src[u] + at(c));
+#pragma unroll
+      for (int u = 0; u < kRowU; ++u)
+#pragma unroll
+        for (int c = 0; c < kColU; ++c)
+          if (src[u] >= 0 && at(c) < m.full_cols) W[src[u] + at(c)] = v[u][c];
     }
   }
 }
@@ -400,6 +427,17 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
           v[r] = r < nrows ? get<SPLIT>(master, opw, lo, o + (long long)r * m.ld) : 0.f;
           v2[r] = r < nrows ? get<SPLIT>(master, opw, lo, o2 + (long long)r * m.ld) : 0.f;
         }
+        bool rare = false;                   // one branch for all of them, behind all the loads
+#pragma unroll
+        for (int r = 0; r < kStageRows; ++r) rare |= SPLIT && (is_nudged(v[r]) | is_nudged(v2[r]));
+        if (rare)
+#pragma unroll
+          for (int r = 0; r < kStageRows; ++r) {
+            if (r >= nrows) break;
+            const float* full = W + (k0 + r) * m.full_cols + c0;
+            v[r] = unnudged(v[r], full + col);
+            if (two) v2[r] = unnudged(v2[r], full + col2);
+          }
 #pragma unroll
         for (int r = 0; r < kStageRows; ++r) {
           t[r * kStageCols + col] = v[r];
@@ -448,29 +486,47 @@ bool launch_permute_cols(const Launch& L, float* W, const SliceMap& m, int S, fl
   return true;
 }
 
-__global__ void copy_out_kernel(const float* packed, const bf16* opw, const uint16_t* lo, int64_t ld, int64_t rows,
+// Where packed element (s, i, j) lies in the full matrix; null: it is padding.
+__device__ __forceinline__ const float* source_of(const float* W, const SliceMap& m, int s, int64_t i, int64_t j) {
+  const int64_t nrows = m.row_idx ? m.row_off[s + 1] - m.row_off[s] : m.full_rows;
+  const int64_t ncols = m.col_idx ? m.col_off[s + 1] - m.col_off[s] : m.full_cols;
+  if (i >= nrows || j >= ncols) return nullptr;
+  return W + (m.row_idx ? m.row_idx[m.row_off[s] + i] : i) * m.full_cols + (m.col_idx ? m.col_idx[m.col_off[s] + j] : j);
+}
+
+// packed, opw, lo: subnet s's slab.
+__global__ void copy_out_kernel(const SliceJob job, int s, const float* packed, const bf16* opw, const uint16_t* lo, int64_t rows,
                                 int64_t cols, float* __restrict__ out) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t i = blockIdx.y;
   if (j < cols)
-    for (; i < rows; i += gridDim.y) out[i * cols + j] = lo ? get<true>(packed, opw, lo, i * ld + j) : get<false>(packed, opw, lo, i * ld + j);
+    for (; i < rows; i += gridDim.y) {
+      const int64_t o = i * job.m.ld + j;
+      out[i * cols + j] = lo ? unnudged(get<true>(packed, opw, lo, o), source_of(job.W, job.m, s, i, j)) : packed[o];
+    }
 }
 
 // Masters first .. end - 1 of n become fp32 words in place.  The low halves are the second half of the words, so
 // word i takes the place of low halves 2 i - n and 2 i - n + 1, both at or before i: a launch may cover words as long as
 // they replace only low halves of words before its first.  One block may end the array: it reads all it needs
 // before it writes.
-__global__ void join_masters_kernel(float* master, const bf16* opw, int64_t n, int64_t first, int64_t end) {
-  const uint16_t* lo = reinterpret_cast<const uint16_t*>(master) + n;
-  const uint16_t* hi = reinterpret_cast<const uint16_t*>(opw);
+__device__ __forceinline__ float joined(const SliceJob& job, int64_t n, int64_t i) {
+  const float v = get<true>(job.master, job.opw, reinterpret_cast<const uint16_t*>(job.master) + n, i);
+  if (!is_nudged(v)) return v;
+  // where it came from decides
+  const int64_t slab = job.m.rows_pad * job.m.ld, s = i / slab, e = i - s * slab;
+  const float* src = source_of(job.W, job.m, (int)s, e / job.m.ld, e % job.m.ld);
+  return src ? unnudged(v, src) : v;
+}
+__global__ void join_masters_kernel(const SliceJob job, int64_t n, int64_t first, int64_t end) {
   if (gridDim.x > 1) {
     for (int64_t i = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end; i += (int64_t)gridDim.x * blockDim.x)
-      master[i] = join_master(hi[i], lo[i]);
+      job.master[i] = joined(job, n, i);
   } else {
     const int64_t i = first + threadIdx.x;
-    const float w = i < end ? join_master(hi[i], lo[i]) : 0.f;
+    const float w = i < end ? joined(job, n, i) : 0.f;
     __syncthreads();
-    if (i < end) master[i] = w;
+    if (i < end) job.master[i] = w;
   }
 }
 
@@ -527,21 +583,23 @@ void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
 void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) { move_all<true>(L, jobs, n, st); }
 void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) { move_all<false>(L, jobs, n, st); }
 
-void copy_out_slice(const Launch& L, const float* packed, const bf16* opw, const uint16_t* lo, int64_t ld, int64_t rows,
-                    int64_t cols, float* out) {
+void copy_out_slice(const Launch& L, const SliceJob& j, int s, int64_t rows, int64_t cols, float* out) {
   dim3 grid((unsigned)ceil_div(cols, 256), (unsigned)(rows < 1024 ? rows : 1024));
-  copy_out_kernel<<<grid, 256, 0, L.stream>>>(packed, opw, lo, ld, rows, cols, out);
+  const int64_t slab = (int64_t)s * j.m.rows_pad * j.m.ld;
+  copy_out_kernel<<<grid, 256, 0, L.stream>>>(j, s, j.master + slab, j.opw ? j.opw + slab : nullptr, j.lo ? j.lo + slab : nullptr,
+                                              rows, cols, out);
   L.count();
 }
 
-void join_masters(const Launch& L, float* master, const bf16* opw, int64_t n) {
+void join_masters(const Launch& L, const SliceJob& j) {
   constexpr int kJoin = 1024;
+  const int64_t n = j.S * j.m.rows_pad * j.m.ld;
   int64_t first = 0;
   while (first < n) {
     int64_t end = first + (n - first) / 2;     // words below this replace low halves below `first` only
     if (n - first <= kJoin) end = n;
     const int64_t blocks = n - first <= kJoin ? 1 : std::max<int64_t>(2, std::min<int64_t>(ceil_div(end - first, kJoin), 4096));
-    join_masters_kernel<<<(unsigned)blocks, kJoin, 0, L.stream>>>(master, opw, n, first, end);
+    join_masters_kernel<<<(unsigned)blocks, kJoin, 0, L.stream>>>(j, n, first, end);
     L.count();
     first = end;
   }

@@ -631,7 +631,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
             w[7] = w1.w - a.lr * __uint_as_float(acc[8 * u + 7]);
             *p0 = make_float4(w[0], w[1], w[2], w[3]);
             *p1 = make_float4(w[4], w[5], w[6], w[7]);
-            *b16_unit(b16, r, u) = pack8_operand(w);
+            *b16_unit(b16, r, u) = pack8(w);
           }
         } else if (kSplit) {
 #pragma unroll

@@ -335,6 +335,11 @@ SliceMap slice_map(const ist_ctx* c, int l, int s_first = 0) {
   return m;
 }
 
+// All S slices of layer l.
+SliceJob slice_job(const ist_ctx* c, int l) {
+  return SliceJob{c->W[l - 1], c->master(l), c->opw(l), slice_map(c, l), c->S, c->lo(l), 0};
+}
+
 SliceMap bias_map(const ist_ctx* c, int l, int s_first = 0) {
   SliceMap m{};
   m.s_first = s_first;
@@ -970,13 +975,10 @@ extern "C" ist_status ist_get_subnet_params(ist_ctx* c, int layer, int s, float*
   if (layer < 1 || layer > c->t || s < 0 || s >= c->S) return fail(c, IST_ERR_ARG, "layer or subnet out of range");
   auto count = [&](int l) { return group_size(c, l, s); };
   Launch L = c->launch();
-  if (W_out_dev)
-    copy_out_slice(L, c->master(layer) + (int64_t)s * c->slice_elems(layer),
-                   c->split(layer) ? c->opw(layer) + (int64_t)s * c->slice_elems(layer) : nullptr,
-                   c->split(layer) ? c->lo(layer) + (int64_t)s * c->slice_elems(layer) : nullptr, c->ld[layer],
-                   count(layer - 1), count(layer), W_out_dev);
+  if (W_out_dev) copy_out_slice(L, slice_job(c, layer), s, count(layer - 1), count(layer), W_out_dev);
   if (b_out_dev)
-    copy_out_slice(L, c->bias(layer) + (int64_t)s * c->ld[layer], nullptr, nullptr, c->ld[layer], 1, count(layer), b_out_dev);
+    copy_out_slice(L, SliceJob{c->b[layer - 1], c->bias(layer), nullptr, bias_map(c, layer), c->S, nullptr, 0}, s, 1, count(layer),
+                   b_out_dev);
   IST_CUDA(c, cudaGetLastError());
   return IST_OK;
 }
@@ -1028,7 +1030,7 @@ extern "C" ist_status ist_packed_layer(ist_ctx* c, int layer, void** master_dev,
     // the caller reads and writes fp32 slices from here on: those in place are converted now
     if (c->state == ST_PARTITIONED) {
       for (int l = 1; l <= c->t; ++l)
-        if (c->split(l)) join_masters(c->launch(), c->master(l), c->opw(l), (int64_t)c->S * c->slice_elems(l));
+        if (c->split(l)) join_masters(c->launch(), slice_job(c, l));
       IST_CUDA(c, cudaGetLastError());
     }
     c->packed_seen = true;
@@ -1049,7 +1051,7 @@ extern "C" ist_status ist_reassemble(ist_ctx* c) {
     Scope sc(c, IST_K_SCATTER);
     std::vector<SliceJob> jobs;
     for (int l = 1; l <= t; ++l) {
-      jobs.push_back(SliceJob{c->W[l - 1], c->master(l), c->opw(l), slice_map(c, l), S, c->lo(l), 0});
+      jobs.push_back(slice_job(c, l));
       jobs.push_back(SliceJob{c->b[l - 1], c->bias(l), nullptr, bias_map(c, l), S, nullptr, l == t ? 1 : 0});
     }
     scatter_slices(L, jobs.data(), (int)jobs.size(), c->status());

@@ -72,11 +72,10 @@ struct SliceJob {
 };
 void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
 void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
-// Dense copy-out of a packed slice (ist_get_subnet_params); lo as in SliceJob.
-void copy_out_slice(const Launch& L, const float* packed, const bf16* opw, const uint16_t* lo, int64_t ld, int64_t rows,
-                    int64_t cols, float* out);
-// n masters kept as (opw, lo) become fp32 values in place: lo is the second half of the n fp32 words at `master`.
-void join_masters(const Launch& L, float* master, const bf16* opw, int64_t n);
+// Dense copy-out of subnet s's packed slice (ist_get_subnet_params).
+void copy_out_slice(const Launch& L, const SliceJob& job, int s, int64_t rows, int64_t cols, float* out);
+// Masters kept as (opw, lo) become fp32 words in place, all S slabs; lo is the second half of the words at master.
+void join_masters(const Launch& L, const SliceJob& job);
 
 // ---- grouped GEMM -----------------------------------------------------------------------
 // C[g](m, n) = sum_k A[g](m, k) * B[g](n, k), fp32 accumulation, followed by an epilogue.
