@@ -7,17 +7,17 @@
 //   C[g](m, n) = sum_k A[g](m, k) * B[g](n, k),   fp32 accumulation
 //
 // One CTA per SM walks over 128 x BN output tiles (tile = blockIdx.x + i * gridDim.x).
-//   warp 0 (one lane)  TMA loads of the A / B k-slabs into a ring of STAGES slots
-//   warp 1 (one lane)  tcgen05.mma issue; owns the tensor-memory allocation (2 accumulators,
+//   warp 0             TMA loads of the A / B k-slabs into a ring of STAGES slots
+//   warp 1             tcgen05.mma issue; owns the tensor-memory allocation (2 accumulators,
 //                      so the MMAs of tile i+1 overlap the epilogue of tile i)
 //   then the epilogue warps, groups of four that take the 32-column chunks in turn (two groups;
 //                      four for the softmax passes over a very wide output layer):
 //                      tcgen05.ld (warp w reads lanes 32*(w%4)..+31, one row per thread), apply
 //                      the epilogue, write the chunk into a swizzled shared-memory slot
-//   then one warp (one lane), where the epilogue has input chunks: their TMA loads into the
+//   then one warp, where the epilogue has input chunks: their TMA loads into the
 //                      slots (the fp32 master slice for the SGD update, the ReLU mask for the
 //                      delta GEMM)
-//   then the storers (one lane each; four, two beside sixteen epilogue warps, none where the
+//   then the storers (a warp each; four, two beside sixteen epilogue warps, none where the
 //                      epilogue stores no chunks): TMA stores of finished slots (coalesced,
 //                      clipped at the tensor edge); slot i belongs to storer i % (their number),
 //                      which hands the slot back as soon as its own store has read it, without
@@ -293,7 +293,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: known to be uniform
   const int total_tiles = a.total_tiles;             // tiles of (128 * PAIR) x BN x k slice, all problems
   const int rank = PAIR == 2 ? (int)cluster_ctarank() : 0;
   const int unit = blockIdx.x / PAIR, n_units = gridDim.x / PAIR;   // a unit = a CTA or a pair
@@ -356,7 +356,11 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
 
   if (warp == 0) {
     // ---------------------------------------------------------------- operand loads
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
+      auto wait = [&](uint64_t* bar, uint32_t parity, int where) {
+        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, abortp, a.status, where));
+      };
       int it = 0, pi = 0;
       uint32_t sum_pending = 0, sum_parity = 0;
       bool ok = true;
@@ -377,30 +381,33 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           // A is the output of the problem before this one: wait until every chunk of these rows
           // has been stored (the storers count them), then order the copies below after that
           const unsigned* ctr = pr.wait_ctr + (long long)g * pr.m_tiles + at.mt;
-          const long long t0 = clock64();
-          while ((int)(ld_acquire(ctr) - pr.wait_target) < 0) {
-            if (*abortp) { ok = false; break; }
-            if (clock64() - t0 > kWaitLimitCycles) {
-              *abortp = 1;
-              report(a.status, -6, SITE_TC_PIPE, 8);
-              ok = false;
-              break;
+          if (leader) {
+            const long long t0 = clock64();
+            while ((int)(ld_acquire(ctr) - pr.wait_target) < 0) {
+              if (*abortp) { ok = false; break; }
+              if (clock64() - t0 > kWaitLimitCycles) {
+                *abortp = 1;
+                report(a.status, -6, SITE_TC_PIPE, 8);
+                ok = false;
+                break;
+              }
+              __nanosleep(64);
             }
-            __nanosleep(64);
+            fence_proxy_async_all();
           }
+          ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          fence_proxy_async_all();
         }
         const bool sums = kSums && sums_bias(pr, at);   // the summing warps read this tile's B stages
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int s = it % STAGES;
-          ok = mbar_wait(&empty_bar[s], ((it / STAGES) & 1) ^ 1, abortp, a.status, 1);
+          ok = wait(&empty_bar[s], ((it / STAGES) & 1) ^ 1, 1);
           if (!ok) break;
           if (kSums) {
             // a stage that a summing tile filled last is free once the summing warps have read it
             // too; they signal per stage, so bit s of sum_parity is the phase to wait for next
             if ((sum_pending >> s) & 1u) {
-              ok = mbar_wait(&sum_done[s], (sum_parity >> s) & 1u, abortp, a.status, 12);
+              ok = wait(&sum_done[s], (sum_parity >> s) & 1u, 12);
               if (!ok) break;
               sum_parity ^= 1u << s;
               sum_pending &= ~(1u << s);
@@ -409,7 +416,8 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           }
           uint8_t* sa = smem + s * STAGE_BYTES;
           uint8_t* sb = sa + A_BYTES;
-          if (PAIR == 2) {
+          if (!leader) {
+          } else if (PAIR == 2) {
             // both CTAs' copies complete on the leader's barrier, which expects the bytes of both
             const uint32_t bar = map_to_cta(&full_bar[s], 0);
             if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * STAGE_BYTES);
@@ -444,9 +452,10 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
               tma_load_3d(sb, tmB, &full_bar[s], kb * BK, n0, gb);
             }
           }
+          __syncwarp();
         }
       }
-      if (!ok && rank == 0) {
+      if (!ok && rank == 0 && leader) {
         // let copies already in flight land before the CTA's shared memory goes away (a peer CTA
         // is held by the closing cluster barrier until the leader has got here)
         for (int j = max(0, it - STAGES); j < it; ++j) {
@@ -457,8 +466,22 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issue
-    if (lane == 0 && rank == 0) {
+    // The whole warp goes through the tiles, one elected lane issues (see elect_one), here and in the roles that issue
+    // copies.  With the loops in a branch of one lane an MMA took 80 to 100 cycles to issue, more than it runs on
+    // 64- and 128-column tiles (1024-4096-4096-35, S = 4, 256 rows: forward chain 29.3 -> 25.5 us, delta chain 20.8 -> 18.8,
+    // updates 25.0 -> 22.9; 2048-4096-1024-200, S = 2, 384 rows: forward 47.4 -> 39.8 us).
+    if (rank == 0) {
       constexpr uint32_t idesc = make_idesc(A_MN, B_MN, BN, BM * PAIR);
+      const bool leader = elect_one();
+      auto wait = [&](uint64_t* bar, uint32_t parity, int where) {
+        return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, abortp, a.status, where));
+      };
+      // Descriptors of stage 0; the others lie a constant further (an address in 16-byte units, below 2^14).
+      // K-major: 16 k-elements = 32 bytes inside the swizzle row; 8-row groups 1024 B apart.
+      // MN-major: 16 k-rows = 2048 B; 64-element MN chunks (one TMA box each) 8192 B apart.
+      constexpr uint32_t A_STEP = (A_MN ? 2048 : 32) >> 4, B_STEP = (B_MN ? 2048 : 32) >> 4;
+      const uint64_t a0 = make_desc(smem_u32(smem), A_MN ? BK * 128 : 16, 1024);
+      const uint64_t b0 = make_desc(smem_u32(smem) + A_BYTES, B_MN ? BK * 128 : 16, 1024);
       int it = 0, j = 0, pi = 0, sit = 0;
       bool ok = true;
       for (int tile = unit; tile < total_tiles && ok; tile += n_units) {
@@ -467,7 +490,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         int kb_limit;
         if (!tile_live<BM * PAIR, BN>(pr, at, group_of(pr, at.slab), &kb_limit)) continue;
         const int b = j & 1;
-        ok = mbar_wait(&acc_empty[b], ((j >> 1) & 1) ^ 1, abortp, a.status, 2);
+        ok = wait(&acc_empty[b], ((j >> 1) & 1) ^ 1, 2);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
@@ -477,33 +500,29 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const bool sums = kSums && sums_bias(pr, at);   // the summing warps follow this tile
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int s = it % STAGES;
-          ok = mbar_wait(&full_bar[s], (it / STAGES) & 1, abortp, a.status, 3);
+          ok = wait(&full_bar[s], (it / STAGES) & 1, 3);
           if (!ok) break;
           tc_fence_after();
-          if (kSums && sums) {
-            // tell the summing warps that the stage is full; they have a ring of their own,
-            // stepped once per stage of a summing tile, so that its phases stay in step with
-            // them although they skip the other tiles
-            mbar_arrive(&stage_here[sit % STAGES]);
-            ++sit;
-          }
-          const uint32_t sa = smem_u32(smem + s * STAGE_BYTES), sb = sa + A_BYTES;
+          const uint64_t ad = a0 + (uint64_t)(s * (STAGE_BYTES >> 4)), bd = b0 + (uint64_t)(s * (STAGE_BYTES >> 4));
+          if (leader) {
+            // tell the summing warps that the stage is full; they have a ring of their own, stepped once per
+            // stage of a summing tile, so that its phases stay in step with them although they skip the other tiles
+            if (kSums && sums) mbar_arrive(&stage_here[sit % STAGES]);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            // K-major: 16 k-elements = 32 bytes inside the swizzle row; 8-row groups 1024 B apart.
-            // MN-major: 16 k-rows = 2048 B; 64-element MN chunks (one TMA box each) 8192 B apart.
-            const uint64_t ad = A_MN ? make_desc(sa + k * 2048, BK * 128, 1024) : make_desc(sa + k * 32, 16, 1024);
-            const uint64_t bd = B_MN ? make_desc(sb + k * 2048, BK * 128, 1024) : make_desc(sb + k * 32, 16, 1024);
-            if (PAIR == 2) tc_mma_pair(d_tmem, ad, bd, idesc, ((kb - kb0) | k) != 0);
-            else tc_mma(d_tmem, ad, bd, idesc, ((kb - kb0) | k) != 0);
+            for (int k = 0; k < BK / 16; ++k) {
+              if (PAIR == 2) tc_mma_pair(d_tmem, ad + k * A_STEP, bd + k * B_STEP, idesc, ((kb - kb0) | k) != 0);
+              else tc_mma(d_tmem, ad + k * A_STEP, bd + k * B_STEP, idesc, ((kb - kb0) | k) != 0);
+            }
+            // frees the slot (in both CTAs of a pair) once these MMAs have read it
+            if (PAIR == 2) tc_commit_pair(&empty_bar[s]); else tc_commit(&empty_bar[s]);
           }
-          // frees the slot (in both CTAs of a pair) once these MMAs have read it
-          if (PAIR == 2) tc_commit_pair(&empty_bar[s]); else tc_commit(&empty_bar[s]);
-
+          if (kSums && sums) ++sit;
+          __syncwarp();
         }
-        if (ok) {
+        if (ok && leader) {
           if (PAIR == 2) tc_commit_pair(&acc_full[b]); else tc_commit(&acc_full[b]);
         }
+        __syncwarp();
         ++j;
       }
     }
@@ -781,7 +800,8 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     }
   } else if (ET::kAux && warp == kAuxWarp) {
     // ---------------------------------------------------------------- epilogue input loads
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       int cq = 0, pi = 0;
       bool ok = true;
       for (int tile = unit; tile < total_tiles && ok; tile += n_units) {
@@ -798,8 +818,9 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           const int nc = n0 + c * CW;
           if (nc >= pN) break;
           const int slot = cq % NS;
-          ok = mbar_wait(&slot_empty[slot], ((cq / NS) & 1) ^ 1, abortp, a.status, 6);
+          ok = __all_sync(0xffffffffu, mbar_wait(&slot_empty[slot], ((cq / NS) & 1) ^ 1, abortp, a.status, 6));
           if (!ok) break;
+          if (!leader) continue;
           mbar_expect_tx(&slot_full[slot], AUX_BYTES);
           if (EPI == EPI_SGD) tma_load_3d(slots + slot * SLOT_BYTES, &maps.c32[pi], &slot_full[slot], nc, m0, g);
           else if (kSplit) {
@@ -808,7 +829,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           } else tma_load_3d(slots + slot * SLOT_BYTES + F32_BYTES, &maps.aux16[pi], &slot_full[slot], nc, m0, g);
         }
       }
-      if (!ok) {
+      if (!ok && leader) {
         for (int jq = max(0, cq - NS); jq < cq; ++jq) {
           long long t0 = clock64();
           while (!mbar_try_wait(&slot_full[jq % NS], (jq / NS) & 1) && clock64() - t0 < kWaitLimitCycles) {}
@@ -817,7 +838,8 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     }
   } else if (warp < kStoreWarp0 + kStoreWarps) {
     // ---------------------------------------------------------------- chunk stores
-    if (kStore && lane == 0) {
+    if (kStore) {
+      const bool leader = elect_one();
       const int sj = warp - kStoreWarp0;
       int cq = 0, pi = 0, pi_next = 0;
       bool ok = true;
@@ -829,7 +851,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           if (!tile_live<BM * PAIR, BN>(pr, at, group_of(pr, at.slab), &kb_limit)) {
             // A skipped tile still counts towards its row block, so that the rows' readers wait for
             // the same total whatever the group's extent (they never read behind the extent).
-            if (pr.signal_ctr && sj == 0) {
+            if (pr.signal_ctr && sj == 0 && leader) {
               const int live = min(NCH, (pr.N - at.nt * BN + CH - 1) / CH);
               if (live > 0)
                 red_release_add(pr.signal_ctr + (long long)group_of(pr, at.slab) * pr.m_tiles + at.mt, (unsigned)live);
@@ -850,8 +872,10 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           // a slot always belongs to the same storer, so that storer sees the slot's barrier
           // phases in order (a parity wait cannot tell phase p from phase p + 2)
           if (slot % kStoreWarps != sj) continue;
-          ok = mbar_wait(&chunk_done[slot], (cq / NS) & 1, abortp, a.status, 7);
+          ok = __all_sync(0xffffffffu, mbar_wait(&chunk_done[slot], (cq / NS) & 1, abortp, a.status, 7));
           if (!ok) break;
+          ++stored;
+          if (!leader) continue;
           uint8_t* f32 = slots + slot * SLOT_BYTES;
           if (head) {
             tma_store_3d(&maps.c32[pi], f32 + F32_BYTES, nc, m0, g);
@@ -861,7 +885,6 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
             if (kSplit) tma_store_3d(&maps.c32[pi], f32 + B16_BYTES, nc, m0, g);
           }
           tma_commit_group();
-          ++stored;
           if (is_update(EPI) && PAIR == 2) {
             // The same chunk of this unit's next tile is asked into L2 now, one tile ahead of its
             // load, so that the load finds it there.  The request is issued here, where the
@@ -883,7 +906,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           tma_wait_read<0>();
           mbar_arrive(&slot_empty[slot]);
         }
-        if (ok && pr.signal_ctr && stored) {
+        if (ok && pr.signal_ctr && stored && leader) {
           // a later problem of this launch reads these rows: once this thread's stores of the tile
           // have completed, add them to the row block's count (release: the reader acquires it)
           tma_wait_all();
@@ -891,7 +914,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
           red_release_add(pr.signal_ctr + (long long)group_of(pr, g) * pr.m_tiles + at.mt, stored);
         }
       }
-      tma_wait_all();                // all stores complete before the CTA exits
+      if (leader) tma_wait_all();    // all stores complete before the CTA exits
     }
   }
   if (has_sum_warps(EPI) && warp >= kStoreWarp0 + kStoreWarps) {

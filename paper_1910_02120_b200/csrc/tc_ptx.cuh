@@ -159,6 +159,13 @@ __device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
       ::"r"(smem_u32(bar)), "h"((uint16_t)3)
       : "memory");
 }
+// One lane of a warp that runs converged.  Roles whose whole warp goes through the loops, with one elected lane issuing, keep
+// addresses and descriptors in uniform registers; in a branch of one lane every MMA and copy first moves them there.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
 // SHIFT: the accumulator is divided by 2^SHIFT before the product is added to it.
 template <int SHIFT = 0>
 __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,

@@ -96,11 +96,6 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
 // 16-byte unit u of 128-byte row r, 128-byte swizzled
 __device__ __forceinline__ uint4* unit_at(uint8_t* tile, int r, int u) {
   return reinterpret_cast<uint4*>(tile + r * 128 + ((u ^ (r & 7)) << 4));
