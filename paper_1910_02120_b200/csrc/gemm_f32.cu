@@ -432,7 +432,8 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr bool WHOLE = BN != 256;                    // see issue
+  const int tid = threadIdx.x, warp = WHOLE ? __shfl_sync(0xffffffffu, tid >> 5, 0) : tid >> 5, lane = tid & 31;
   const int cluster = PAIR == 2 ? 2 : a.ksplit;
   const int side = (int)blockIdx.x - a.p[a.n_problems - 1].tile_end * cluster;
   if (side >= 0) {                                     // bias work (a whole cluster of it)
@@ -520,29 +521,36 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
   constexpr uint32_t idesc = make_idesc(A_MN, B_MN, BN, BM * PAIR);
   const uint64_t ad0 = A_MN ? make_desc(smem_u32(smem), 8192, 1024) : make_desc(smem_u32(smem), 16, 1024);
   const uint64_t bd0 = B_MN ? make_desc(smem_u32(smem) + A_BYTES, 8192, 1024) : make_desc(smem_u32(smem) + A_BYTES, 16, 1024);
-  auto issue = [&](int i) -> bool {                          // the MMAs of step i
+  // The MMAs of step i.  Narrow tiles: the warp that has nothing else to do goes through this whole, one elected lane
+  // issues (see elect_one; 784-1024-10, S = 2, 128 rows, ten steps 407 -> 393 us).  256 columns: one lane of an adding warp
+  // does; with the whole warp in it, evaluation of 3072-16384-16384-10 takes 15.2 instead of 14.1 ms.
+  auto issue = [&](int i, bool leader) -> bool {
     const int b = i & 1, sl = i & (SLOTS - 1);
-    if (!mbar_wait(&full[sl], (i >> LG) & 1, abortp, a.status, 21)) return false;
-    if (i >= 2 && !mbar_wait<PAIR == 2>(&taken[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 23)) return false;
+    auto reached = [&](bool ok) { return WHOLE ? (bool)__all_sync(0xffffffffu, ok) : ok; };
+    if (!reached(mbar_wait(&full[sl], (i >> LG) & 1, abortp, a.status, 21))) return false;
+    if (i >= 2 && !reached(mbar_wait<PAIR == 2>(&taken[b], ((i >> 1) & 1) ^ 1, abortp, a.status, 23))) return false;
     tc_fence_after();
     constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};   // low x high first, high x high last
     const uint32_t at = (uint32_t)(sl >> 1) * (3 * PLANE >> 4);
     const uint64_t ad = ad0 + at + (b ? (A_MN ? 4096 : 64) >> 4 : 0), bd = bd0 + at + (b ? (B_MN ? 4096 : 64) >> 4 : 0);
+    if (leader) {
 #pragma unroll
-    for (int c = 0; c < 6; ++c)
+      for (int c = 0; c < 6; ++c)
 #pragma unroll
-      for (int k = 0; k < KH / 16; ++k) {
-        const uint64_t da = ad + ((pa[c] * PLANE + k * (A_MN ? 2048 : 32)) >> 4);
-        const uint64_t db = bd + ((pb[c] * PLANE + k * (B_MN ? 2048 : 32)) >> 4);
-        if ((c == 3 || c == 5) && k == 0) {              // from one weight to the next: 2^8
-          if (PAIR == 2) tc_mma_pair<8>(tmem + b * BN, da, db, idesc, 1);
-          else tc_mma<8>(tmem + b * BN, da, db, idesc, 1);
-        } else {
-          if (PAIR == 2) tc_mma_pair(tmem + b * BN, da, db, idesc, (c | k) != 0);
-          else tc_mma(tmem + b * BN, da, db, idesc, (c | k) != 0);
+        for (int k = 0; k < KH / 16; ++k) {
+          const uint64_t da = ad + ((pa[c] * PLANE + k * (A_MN ? 2048 : 32)) >> 4);
+          const uint64_t db = bd + ((pb[c] * PLANE + k * (B_MN ? 2048 : 32)) >> 4);
+          if ((c == 3 || c == 5) && k == 0) {              // from one weight to the next: 2^8
+            if (PAIR == 2) tc_mma_pair<8>(tmem + b * BN, da, db, idesc, 1);
+            else tc_mma<8>(tmem + b * BN, da, db, idesc, 1);
+          } else {
+            if (PAIR == 2) tc_mma_pair(tmem + b * BN, da, db, idesc, (c | k) != 0);
+            else tc_mma(tmem + b * BN, da, db, idesc, (c | k) != 0);
+          }
         }
-      }
-    if (PAIR == 2) tc_commit_pair(&done[sl]); else tc_commit(&done[sl]);
+      if (PAIR == 2) tc_commit_pair(&done[sl]); else tc_commit(&done[sl]);
+    }
+    if (WHOLE) __syncwarp();
     return true;
   };
   // Pairs: passes on that the peer CTA's half of step i lies in its shared memory.
@@ -609,13 +617,13 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
 #pragma unroll
     for (int i = 0; i < NACC / 2; ++i) acc[i] = 0;
     const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(((warp - kLoadWarps) >> 2) * NACC);
-    if (issuer && steps > 0) issue(0);
+    if (issuer && steps > 0) issue(0, true);
     if (relayer)
       for (int i = 0; i < AHEAD; ++i) relay(i);
     __syncwarp();
     for (int i = 0; i < steps; ++i) {
       const int b = i & 1;
-      if (issuer && i + 1 < steps) issue(i + 1);
+      if (issuer && i + 1 < steps) issue(i + 1, true);
       if (relayer) relay(i + AHEAD);
       __syncwarp();
       if (!__all_sync(0xffffffffu, mbar_wait(&done[i & (SLOTS - 1)], (i >> LG) & 1, abortp, a.status, 20))) break;
@@ -639,9 +647,11 @@ __global__ void __launch_bounds__(threads_of(BN), 1) gemm_f32_kernel(const __gri
   } else {
     // ---------------------------------------------------------------- issue the MMAs of a narrow tile
     asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
-    if (warp == kLoadWarps + kAddWarps && lane == 0)
+    if (warp == kLoadWarps + kAddWarps) {
+      const bool leader = elect_one();
       for (int i = 0; i < steps; ++i)
-        if (!issue(i)) break;
+        if (!issue(i, leader)) break;
+    }
     __syncwarp();
     close(nullptr);
   }
