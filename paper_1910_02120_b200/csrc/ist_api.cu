@@ -554,7 +554,9 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       wh.scratch = reinterpret_cast<float*>(delta(t));   // the deltas themselves are not stored
       wh.scratch_bytes = (size_t)c->S * Bm * c->ld[t] * sizeof(T);
     }
-    const bool fused_head = wide && t > 1 && fused_head_ok(wh, (const T*)nullptr);
+    // Under independent assignment the columns of a(t-1) behind a group's extent are never written: only launches that
+    // are told the extents may read them.
+    const bool fused_head = wide && t > 1 && !ragged && fused_head_ok(wh, (const T*)nullptr);
     // ---- forward ---------------------------------------------------------------------------
     // Hidden layers without standardisation form a chain a_l = relu(a_{l-1} W_l + b_l): they are
     // collected and go out together (tiles of one launch, see gemm_list).
