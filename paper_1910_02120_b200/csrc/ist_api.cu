@@ -457,6 +457,12 @@ bool fused_head_ok(const WideHead&, const float*) { return false; }
 bool fused_head_ok(const WideHead& w, const bf16*) { return w.lo && wide_head_ok(w); }
 void head_buffers(WideHead&, const float*, float*) {}
 void head_buffers(WideHead& w, const bf16* x, bf16* delta) { w.x = x; w.delta = delta; }
+// The fp32 path's narrow output layer in one launch.
+bool f32_head_ok(HeadF32& h, const float* x, const float* W, float* delta, float* delta_out) {
+  h.x = x; h.W = W; h.delta = delta; h.delta_out = delta_out;
+  return head_f32_ok(h);
+}
+bool f32_head_ok(HeadF32&, const bf16*, const bf16*, bf16*, bf16*) { return false; }
 // A product written as plain fp32: with bf16 operands the fp32 epilogue without a bias, with fp32
 // operands (output of the same type) a plain store.
 void set_plain_fp32_output(GemmArgs<bf16>& g, float* out, int64_t ld, int64_t sg) {
@@ -557,6 +563,14 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     // Under independent assignment the columns of a(t-1) behind a group's extent are never written: only launches that
     // are told the extents may read them.
     const bool fused_head = wide && t > 1 && !ragged && fused_head_ok(wh, (const T*)nullptr);
+    HeadF32 fh{};
+    fh.S = S; fh.B = B; fh.H = (int)c->np[t - 1]; fh.N = (int)c->N[t];
+    fh.ldx = c->ld[t - 1]; fh.x_sg = Bm * c->ld[t - 1];
+    fh.bias = bias_of(t); fh.ldw = c->ld[t]; fh.w_sg = c->slice_elems(t);
+    fh.dout_sg = Bm * c->ld[t];
+    fh.labels = y + row0; fh.labels_sg = X->stride_subnet;
+    fh.row_loss = row_loss;
+    const bool f32_head = t > 1 && f32_head_ok(fh, act(t - 1), weights(t), delta(t - 1), delta(t));
     // ---- forward ---------------------------------------------------------------------------
     // Hidden layers without standardisation form a chain a_l = relu(a_{l-1} W_l + b_l): they are
     // collected and go out together (tiles of one launch, see gemm_list).
@@ -569,7 +583,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       fwd_chain.clear();
       return ok;
     };
-    for (int l = 1; l <= t; ++l) {
+    for (int l = 1; l <= (f32_head ? t - 1 : t); ++l) {
       if (l == 1 && X->kind == IST_X_CSR && t > 1) {
         {
           Scope sc(c, IST_K_SPMM);
@@ -633,7 +647,9 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     // ---- loss and its gradient -------------------------------------------------------------
     {
       Scope sc(c, IST_K_LOSS);
-      if (wide && !fused_head) {
+      if (f32_head) {
+        if (!head_f32(L, fh, st)) return fail(c, IST_ERR_UNSUPPORTED, "the launch over the output layer cannot be made");
+      } else if (wide && !fused_head) {
         lse_combine(L, logits, gemm_tc_lse_parts(c->ld[t]), S, B, Bm, lse, y + row0, X->stride_subnet, (int)c->N[t], st);
         GemmArgs<T> g{};             // second pass: the same product, written out as delta_t
         g.M = B; g.N = (int)c->np[t]; g.K = (int)c->np[t - 1]; g.G = S;
@@ -692,7 +708,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       return ok;
     };
     for (int l = t; l > 1; --l) {
-      if (!(fused_head && l == t)) {
+      if (!((fused_head || f32_head) && l == t)) {
         GemmArgs<T> g{};
         g.M = B; g.N = (int)c->np[l - 1]; g.K = (int)c->np[l]; g.G = S;
         g.N_store = (int)c->ld[l - 1];

@@ -183,6 +183,19 @@ bool wide_head_ok(const WideHead& w);
 bool wide_head_lse(const Launch& L, const WideHead& w, DeviceStatus* st);
 bool wide_head_pass(const Launch& L, const WideHead& w, DeviceStatus* st);
 
+// ---- head_f32.cu ------------------------------------------------------------------------
+// A narrow output layer in fp32: logits, softmax cross-entropy, delta_t and delta_{t-1} in one launch.
+struct HeadF32 {
+  int S, B, H, N;                  // subnets, rows, width of the layer below, classes
+  const float* x; float* delta; int64_t ldx, x_sg;                  // activations of the layer below and their delta
+  const float* W; const float* bias; int64_t ldw, w_sg;             // [S][H][ldw], [S][ldw]
+  float* delta_out; int64_t dout_sg;                                // delta_t, rows of ldw
+  const int32_t* labels; int64_t labels_sg;
+  float* row_loss;                                                  // [S][B]
+};
+bool head_f32_ok(const HeadF32& h);
+bool head_f32(const Launch& L, const HeadF32& h, DeviceStatus* st);
+
 // ---- rowops.cu --------------------------------------------------------------------------
 // Row-wise softmax cross-entropy of logits [G][B][ld] against labels; writes
 // delta = (softmax - onehot)/B (zero in columns Nt..ld_d) and row_loss [G][B].
