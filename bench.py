@@ -164,6 +164,17 @@ def work_model(w: synth.Workload, norm=False, data=None):
     }
 
 
+def moved_bytes(w: synth.Workload, wm):
+    """work_model counts an fp32 master and a bf16 copy, 10 bytes per weight gathered or updated.  Masters of dense
+    bf16 layers are kept as operand and low half, 8 bytes: rates are of what is moved."""
+    if w.precision == "bf16":
+        d, S = w.layer_dims, w.S
+        split = wm["packed_elems"] - (d[0] * -(-d[1] // S) * S if w.x_dist == "csr" else 0)
+        wm["bytes"]["gather"] -= 2 * split
+        wm["bytes"]["dw_sgd"] -= 2 * split * w.K
+    return wm
+
+
 # ---------------------------------------------------------------------------------------------
 # clocks
 # ---------------------------------------------------------------------------------------------
@@ -479,7 +490,7 @@ def run_ours(args, w):
         return
 
     pk = peaks()
-    wm = work_model(w, norm=args.norm_eps is not None, data=data if data.is_csr else None)
+    wm = moved_bytes(w, work_model(w, norm=args.norm_eps is not None, data=data if data.is_csr else None))
     if shard:      # this rank ran the local steps of its own subnets only; gather / scatter cover all S
         for k in ("fwd", "dx", "dw_sgd"):
             wm["flops"][k] = wm["flops"][k] * count // w.S
@@ -499,7 +510,7 @@ def run_ours(args, w):
             ent["gbs"] = wm["bytes"][name] / sec / 1e9
         kernels[name] = ent
     # Which roofline bounds each class: x*W and delta*W^T are dense contractions (tensor cores);
-    # a^T*delta with the fused update moves 10 bytes per weight for 2*B flop, so HBM bounds it, like
+    # a^T*delta with the fused update moves 8 bytes per weight for 2*B flop, so HBM bounds it, like
     # gather and scatter.  The fp32 path forms six bf16 products per fp32 one on the tensor cores.
     dominant = max(kernels, key=lambda k: kernels[k]["ms_per_step"])
     dk = kernels[dominant]
@@ -596,7 +607,7 @@ def run_sweep(args):
                 torch.cuda.synchronize(dev)
                 ctx.sync_status()
                 ms = e0.elapsed_time(e1) / reps
-                wm = work_model(w)
+                wm = moved_bytes(w, work_model(w))
                 flops = sum(wm["flops"].values())
                 print(json.dumps({"sweep": "C5", "H": H, "S": S, "K": K, "ms_per_round": ms,
                                   "samples_per_s": w.samples_per_round / (ms * 1e-3),
