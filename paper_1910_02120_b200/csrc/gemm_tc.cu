@@ -1325,7 +1325,7 @@ bool gemm_tc_batch(const Launch& L, const GemmArgs<bf16>* ga, int n, const GemmC
     if (n > 1 && a.k_splits > 1 && !is_head) return false;
   }
   if (n > 1 && epi != EPI_BIAS_RELU && epi != EPI_RELU_MASK && epi != EPI_SGD) return false;
-  if (chain && (epi == EPI_SGD || n < 2 || !chain->counters || !chain->totals)) return false;
+  if (chain && (epi == EPI_SGD || n < 2 || !chain->counters || !chain->sets)) return false;
   TileChoice tc = pick_tile(ga, n, epi);
   if (epi == EPI_LSE_PART || epi == EPI_SOFTMAX_DELTA)   // the partials are laid out per 256-column tile
     tc = TileChoice{256, a0.M > BM ? 2 : 1};
@@ -1446,15 +1446,22 @@ bool gemm_tc_batch(const Launch& L, const GemmArgs<bf16>* ga, int n, const GemmC
   if (chain) {
     // Problem i + 1 reads problem i's output rows: same groups, same rows, hence the same tile rows.
     // Every CTA of a unit stores ceil(N / 32) chunks per (group, tile row) and launch; the running
-    // totals are kept by the caller, who clears counters and totals together.
+    // totals are kept by the caller, who clears counters and totals together.  Pairs count 256 rows in a
+    // counter and two CTAs' chunks: what single CTAs have left in the set is no start for them, nor theirs for single ones.
     for (int i = 0; i + 1 < n; ++i) {
       if (ga[i + 1].M != ga[i].M || ga[i + 1].G != ga[i].G || ga[i + 1].A != ga[i].out) return false;
       unsigned* ctr = chain->counters + (size_t)i * chain->stride;
       if ((size_t)t.p[i].G * t.p[i].m_tiles > chain->stride) return false;
-      chain->totals[i] += (unsigned)(pair * ceil_div(t.p[i].N, CH));
+      ChainSet& set = chain->sets[i];
+      if (set.rows != 0 && set.rows != BM * pair) {
+        if (cudaMemsetAsync(ctr, 0, chain->stride * sizeof(unsigned), L.stream) != cudaSuccess) return false;
+        set.total = 0;
+      }
+      set.rows = BM * pair;
+      set.total += (unsigned)(pair * ceil_div(t.p[i].N, CH));
       t.p[i].signal_ctr = ctr;
       t.p[i + 1].wait_ctr = ctr;
-      t.p[i + 1].wait_target = chain->totals[i];
+      t.p[i + 1].wait_target = set.total;
     }
   }
 

@@ -83,7 +83,7 @@ struct ist_ctx {
 
   // chained launches: running totals of the row-block counters (index = layer), and the batch size
   // and subnet count they were accumulated with (a change clears counters and totals)
-  std::vector<unsigned> fwd_totals, dx_totals;
+  std::vector<ChainSet> fwd_sets, dx_sets;
   int chain_B = -1, chain_S = -1;
   size_t chain_stride() const { return (size_t)S * ceil_div((int64_t)max_batch, 128); }
 
@@ -389,8 +389,8 @@ bool gemm(ist_ctx* c, const GemmArgs<bf16>& a) { return gemm_tc(c->launch(), a, 
 // launch each.  bf16 operands: tiles of one tensor-core launch per gemm_tc_max_batch() problems;
 // with `chained`, every problem reads the output of the one before it and the launch orders
 // their tiles through the row-block counters of `region` (one set per problem, indexed by
-// `layer0 + i`; `totals` are the context's running sums for that region).
-bool gemm_list(ist_ctx* c, const std::vector<GemmArgs<float>>& v, bool, Region, std::vector<unsigned>*, int,
+// `layer0 + i`; `sets` are the context's running sums for that region).
+bool gemm_list(ist_ctx* c, const std::vector<GemmArgs<float>>& v, bool, Region, std::vector<ChainSet>*, int,
                const LossReduce* = nullptr, const BiasSgdArgs<float>* bias = nullptr) {
   const size_t cap = v.empty() || v[0].epi != EPI_SGD ? 1 : gemm_f32_max_batch();
   for (size_t i0 = 0; i0 < v.size(); i0 += cap)
@@ -408,14 +408,14 @@ bool update_sums_bias(const std::vector<GemmArgs<bf16>>& v) {
 }
 // `loss` (weight-update lists only): the first launch also reduces the step's mean losses.
 bool gemm_list(ist_ctx* c, const std::vector<GemmArgs<bf16>>& v, bool chained, Region region,
-               std::vector<unsigned>* totals, int layer0, const LossReduce* loss = nullptr,
+               std::vector<ChainSet>* sets, int layer0, const LossReduce* loss = nullptr,
                const BiasSgdArgs<bf16>* = nullptr) {
   const int cap = gemm_tc_max_batch();
   for (size_t i0 = 0; i0 < v.size(); i0 += cap) {
     const int n = (int)std::min<size_t>(cap, v.size() - i0);
     if (chained && n > 1) {
       GemmChain ch{region.at<unsigned>(c->ws) + (size_t)(layer0 + i0) * c->chain_stride(), c->chain_stride(),
-                   totals->data() + layer0 + i0};
+                   sets->data() + layer0 + i0};
       if (!gemm_tc_batch(c->launch(), v.data() + i0, n, &ch, nullptr, c->status())) return false;
     } else if (!gemm_tc_batch(c->launch(), v.data() + i0, n, nullptr, i0 == 0 ? loss : nullptr, c->status())) {
       return false;
@@ -502,12 +502,12 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
   DeviceStatus* st = c->status();
   Launch L = c->launch();
   if (bf && (c->chain_B != B || c->chain_S != S)) {
-    // the counters' per-launch increments depend on the tile shape, which follows the batch
+    // the counters' places follow from the groups and their rows
     if (c->plan.chain_dx.offset > c->plan.chain_fwd.offset)
       IST_CUDA(c, cudaMemsetAsync(c->plan.chain_fwd.at<char>(c->ws), 0,
                                   2 * (c->plan.chain_dx.offset - c->plan.chain_fwd.offset), c->stream));
-    c->fwd_totals.assign(t + 2, 0u);
-    c->dx_totals.assign(t + 2, 0u);
+    c->fwd_sets.assign(t + 2, ChainSet{});
+    c->dx_sets.assign(t + 2, ChainSet{});
     c->chain_B = B;
     c->chain_S = S;
   }
@@ -579,7 +579,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     auto flush_fwd = [&]() -> bool {
       if (fwd_chain.empty()) return true;
       Scope sc(c, IST_K_FWD);
-      const bool ok = gemm_list(c, fwd_chain, true, c->plan.chain_fwd, &c->fwd_totals, fwd_chain_l0);
+      const bool ok = gemm_list(c, fwd_chain, true, c->plan.chain_fwd, &c->fwd_sets, fwd_chain_l0);
       fwd_chain.clear();
       return ok;
     };
@@ -703,7 +703,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
     auto flush_dx = [&]() -> bool {
       if (dx_chain.empty()) return true;
       Scope sc(c, IST_K_DX);
-      const bool ok = gemm_list(c, dx_chain, true, c->plan.chain_dx, &c->dx_totals, dx_chain_l0);
+      const bool ok = gemm_list(c, dx_chain, true, c->plan.chain_dx, &c->dx_sets, dx_chain_l0);
       dx_chain.clear();
       return ok;
     };

@@ -142,13 +142,19 @@ bool gemm_tc(const Launch& L, const GemmArgs<bf16>& a, DeviceStatus* st);
 // update) as tiles of one launch; at most gemm_tc_max_batch() of them, none k-split.  With a
 // chain, problem i + 1 must read problem i's output (A == out, same M and G) and its tiles wait for
 // the rows they read.  counters: device, [n - 1][stride] unsigned, stride >= G * ceil(M / 128);
-// totals: host, [n - 1], running sums this call advances.  The caller clears counters and totals
-// together (once at start, and whenever the batch's shape changes).  A chain must not be used
+// sets: host, [n - 1], what the counters of each product have been counted to, which this call advances.
+// The caller clears counters and sets together (once at start, and whenever the batch's shape changes).
+// The tile shape is chosen for a whole chain, so the same product may be counted by other rows in a chain
+// of other products: this call clears a set that was last counted so.  A chain must not be used
 // from two streams at once.
+struct ChainSet {
+  unsigned total;   // every counter of the set once the launches so far have run
+  int rows;         // output rows per counter; 0: cleared
+};
 struct GemmChain {
   unsigned* counters;
   size_t stride;
-  unsigned* totals;
+  ChainSet* sets;
 };
 // loss (weight-update launches only, may be null): the step's mean losses are reduced by the launch.
 struct LossReduce;

@@ -98,3 +98,30 @@ def test_unequal_subnets_read_nothing_behind_their_extent():
         err = float((p.double() - q.double()).norm() / (q.double() - p0).norm())
         # the same launches either way: masters of split and of whole words differ by an fp32 ulp in one of 2^17
         assert err <= 1e-4, (i, err)
+
+
+def test_slices_handed_out_between_rounds():
+    """The output layer's own product joins the delta chain once the slices are fp32, and the chain goes from CTA pairs to
+    single CTAs with it (200 rows, 69 neurons per subnet below the classes): the counters of the products that both chains
+    have in common start again."""
+    dims, S, B = [64, 8192, 1024, 1024, 8200], 15, 200
+    g = torch.Generator(device="cuda").manual_seed(4)
+    W = [torch.randn(a, b, device="cuda", generator=g) * (2.0 / a) ** 0.5 for a, b in zip(dims, dims[1:])]
+    b = [torch.zeros(n, device="cuda") for n in dims[1:]]
+    X = torch.randn(S * B, dims[0], device="cuda", generator=g).bfloat16()
+    y = torch.randint(dims[-1], (S * B,), device="cuda", generator=g, dtype=torch.int32)
+    nets = []
+    for first in (False, True):
+        ctx = api.Ist(dims, S, api.IST_BF16, B)
+        ctx.bind_weights([w.clone() for w in W], [v.clone() for v in b])
+        if first:
+            ctx.packed_layer(1)
+        ctx.round(1, X, y, 0.1, 1, B)
+        ctx.packed_layer(1)
+        for seed in (2, 3):
+            ctx.round(seed, X, y, 0.1, 1, B)
+            ctx.sync_status()
+        nets.append(ctx.W + ctx.b)
+    for i, (p0, p, q) in enumerate(zip(W + b, *nets)):
+        err = float((p - q).double().norm() / (q - p0).double().norm())
+        assert err <= 2e-2, (i, err)     # the first of three steps differs as in test_against_the_separate_launches
