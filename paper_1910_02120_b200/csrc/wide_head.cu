@@ -108,7 +108,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
   uint8_t* delta_s = x_s + kXBytes;
   uint8_t* his = delta_s + kDeltaBytes;
   uint8_t* los = his + kHi * kTile;
-  __shared__ uint64_t x_full, hi_full[kHi], hi_empty[kHi], lo_full[kLo], upd_done[2];
+  __shared__ uint64_t x_full, hi_full[kHi], hi_empty[kHi], lo_full[kLo], upd_done[kLo];
   __shared__ uint64_t z_full[2], z_empty[2], d_full[2], d_ready[2], d_empty[2], dw_full[2], dw_empty[2], grp_done, grp_flushed;
   __shared__ __align__(16) float bias_s[kHi][kCols];   // the block's biases travel with its operands
   __shared__ uint32_t tmem_slot;
@@ -122,14 +122,16 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       mbar_init(&hi_full[s], 1);
       mbar_init(&hi_empty[s], 1);
     }
-    for (int s = 0; s < kLo; ++s) mbar_init(&lo_full[s], 1);
+    for (int s = 0; s < kLo; ++s) {
+      mbar_init(&lo_full[s], 1);
+      mbar_init(&upd_done[s], 4);            // one per low-half tile: a block's has no second phase before its own store
+    }
     for (int h = 0; h < 2; ++h) {
       mbar_init(&z_full[h], 1);
       mbar_init(&z_empty[h], 8);
       mbar_init(&d_full[h], 8);
       mbar_init(&d_ready[h], 8 * NH);        // both halves of every other block's delta, for the group that sums it
       mbar_init(&d_empty[h], 1 + 4);         // the products' commit and the four summing warps
-      mbar_init(&upd_done[h], 4);
       mbar_init(&dw_full[h], 1);
       mbar_init(&dw_empty[h], 4);
     }
@@ -203,7 +205,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       bool ok = true;
       int g = g0, blk = b0, gs = g0, bs = b0, i = 0;   // block of the next load, of the next store
       auto store = [&](int j) -> bool {
-        if (!mbar_wait(&upd_done[j & 1], (j >> 1) & 1, abortp, a.status, 214)) return false;
+        if (!mbar_wait(&upd_done[j % kLo], (j / kLo) & 1, abortp, a.status, 214)) return false;
         tma_store_3d(&maps.hi, his + (j % kHi) * kTile, bs * kCols, 0, gs);
         tma_store_3d(&maps.lo, los + (j % kLo) * kTile, bs * kCols, 0, gs);
         tma_commit_group();
@@ -489,7 +491,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       }
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&upd_done[grp]);
+      if (lane == 0) mbar_arrive(&upd_done[i % kLo]);
     }
   }
   tc_fence_before();
