@@ -423,42 +423,50 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
     // ---------------------------------------------------------------- bias and weight updates
     const int grp = (warp - 19) >> 2, q = warp & 3;
     const int r = q * 32 + lane;             // neuron of this thread
-    const uint32_t ones = 0x3f803f80u;
-    const uint32_t delta_base = smem_u32(delta_s);
     bool ok = true;
     for (int i = grp; i < count && ok; i += 2) {
       const int s = i % kHi;
-      // Column sums of delta, 16 columns per warp, on the tensor cores' small form: a row of ones times delta.  Plain loads and
-      // additions took longer than the products, and delta's buffer is held until its sums are taken.
+      // Column sums of delta, 16 columns per warp: a lane adds up eight columns of every sixteenth row (the eight lanes of a
+      // quarter warp read eight rows, every bank once), sixteen lanes then share their sums out.  All in fp32 additions: a row
+      // of ones times delta on the tensor cores, accumulated from 16 rows to the next, was 6e-7 off over 256 rows
+      // where additions in four chains are 0.8e-7 off, and always to the same side.
       ok = __all_sync(0xffffffffu, mbar_wait(&d_ready[grp], (i >> 1) & 1, abortp, a.status, 215));
       if (!ok) break;
-      float sum[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // of 8 columns each: columns 2 (lane % 4), + 1 first
+      f32x2 sum[4] = {pair(0.f, 0.f), pair(0.f, 0.f), pair(0.f, 0.f), pair(0.f, 0.f)};
       for (int h = 0; h < NH; ++h) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {        // 16 rows; lanes 0-15 address those of the first 8 columns, 16-31 of the others
-          const int rr = h * 128 + 16 * j + (lane & 15);
-          uint32_t b[4];
-          asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
-                       : "r"(delta_base + rr * 128 + (((2 * q + (lane >> 4)) ^ (rr & 7)) << 4))
-                       : "memory");
+        for (int j = 0; j < 8; ++j) {
+          const uint4 v = *unit_at(delta_s, h * 128 + 16 * j + (lane & 15), 2 * q + (lane >> 4));
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int e = 0; e < 2; ++e)
-            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %4, %4, %4}, {%5, %6}, {%0, %1, %2, %3};"
-                         : "+f"(sum[e][0]), "+f"(sum[e][1]), "+f"(sum[e][2]), "+f"(sum[e][3])
-                         : "r"(ones), "r"(b[2 * e]), "r"(b[2 * e + 1]));
+          for (int e = 0; e < 4; ++e)
+            sum[e] = add2(sum[e], pair(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)));
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&d_empty[h]);
       }
       {
+        float c[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 t = unpair(sum[e]);
+          c[2 * e] = t.x;
+          c[2 * e + 1] = t.y;
+        }
+#pragma unroll
+        for (int w = 4; w >= 1; w >>= 1) {   // of the columns held, a lane keeps half and gives the other half away
+          const bool up = lane & (2 * w);
+#pragma unroll
+          for (int e = 0; e < w; ++e) {
+            const float mine = up ? c[w + e] : c[e], other = up ? c[e] : c[w + e];
+            c[e] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * w);
+          }
+        }
+        c[0] += __shfl_xor_sync(0xffffffffu, c[0], 1);
         const long long item = it0 + i;
         const int g = (int)(item / a.blocks), blk = (int)(item - (long long)g * a.blocks);
-        const int n = blk * kCols + 16 * q + 2 * (lane & 7);   // every row of the product is the same sum
-        const float s0 = lane & 4 ? sum[1][0] : sum[0][0], s1 = lane & 4 ? sum[1][1] : sum[0][1];
-        float* bp = a.bias + g * a.bias_sg + n;
-        if (lane < 8 && n < a.N) bp[0] = bias_s[s][n - blk * kCols] - a.lr * s0;
-        if (lane < 8 && n + 1 < a.N) bp[1] = bias_s[s][n - blk * kCols + 1] - a.lr * s1;
+        const int col = 16 * q + 8 * (lane >> 4) + ((lane >> 1) & 7), n = blk * kCols + col;
+        if ((lane & 1) == 0 && n < a.N) a.bias[g * a.bias_sg + n] = bias_s[s][col] - a.lr * c[0];
       }
       __syncwarp();
       ok = mbar_wait(&dw_full[grp], (i >> 1) & 1, abortp, a.status, 212) &&
