@@ -40,6 +40,9 @@ constexpr int kThreads = 28 * 32;
 constexpr uint32_t kXChunk = 256 * 128;   // 64 neurons of 256 rows
 constexpr uint32_t kXBytes = 2 * kXChunk, kDeltaBytes = 256 * 128, kTile = 128 * 128;
 constexpr int kSmem = kXBytes + kDeltaBytes + (kHi + kLo) * kTile + 1024;
+// Blocks whose share of dx is summed in tensor memory, at most: 10,240 classes.  Sums there lose precision with their
+// length, and slices of the separate launches have some 10,500.
+constexpr int kDxBlocks = 160;
 constexpr uint32_t kDxCol = 0, kZCol = 256, kDwCol = 384;
 
 struct HeadArgs {
@@ -109,7 +112,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
   uint8_t* his = delta_s + kDeltaBytes;
   uint8_t* los = his + kHi * kTile;
   __shared__ uint64_t x_full, hi_full[kHi], hi_empty[kHi], lo_full[kLo], upd_done[kLo];
-  __shared__ uint64_t z_full[2], z_empty[2], d_full[2], d_ready[2], d_empty[2], dw_full[2], dw_empty[2], grp_done, grp_flushed;
+  __shared__ uint64_t z_full[2], z_empty[2], d_full[2], d_ready[2], d_empty[2], dw_full[2], dw_empty[2], dx_done, dx_flushed, x_free;
   __shared__ __align__(16) float bias_s[kHi][kCols];   // the block's biases travel with its operands
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
@@ -135,8 +138,9 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       mbar_init(&dw_full[h], 1);
       mbar_init(&dw_empty[h], 4);
     }
-    mbar_init(&grp_done, 1);
-    mbar_init(&grp_flushed, 8 * NH);
+    mbar_init(&dx_done, 1);
+    mbar_init(&dx_flushed, 8 * NH);
+    mbar_init(&x_free, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -172,7 +176,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       for (; i < count; ++i) {
         if (i == 0 || blk == 0) {
           // x of the next subnet: once every product that read the last one has completed
-          if (groups > 0) ok = mbar_wait(&grp_done, (groups - 1) & 1, abortp, a.status, 201);
+          if (groups > 0) ok = mbar_wait(&x_free, (groups - 1) & 1, abortp, a.status, 201);
           if (!ok) break;
           mbar_expect_tx(&x_full, kXBytes);
           tma_load_3d(x_s, &maps.x, &x_full, 0, 0, g);
@@ -241,11 +245,12 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
     };
     const int kz = (a.H + 15) / 16;                                // 16-deep steps of x W
     bool ok = true;
-    int blk = b0, groups = 0;
-    bool fresh = true;                                             // first block of a subnet: dx starts from zero
+    int blk = b0;
     // descriptors of the tiles' first steps; the address field counts 16-byte units, so steps are additions
     if (warp == 1) {
       const uint32_t id_z = make_idesc(0, 1, kCols, 128);
+      int groups = 0;
+      bool fresh = true;                                           // first block of a subnet
       const uint64_t x_k = make_desc(smem_u32(x_s), 16, 1024), w0 = make_desc(smem_u32(his), 8192, 1024);
       for (int i = 0; i < count && ok; ++i) {
         if (fresh) ok = wait(&x_full, groups & 1, 205);
@@ -274,9 +279,11 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       const uint32_t id_dw = make_idesc(1, 1, kCols, 128), id_dx = make_idesc(0, 0, kz * 16, 128);
       const uint64_t x_mn = make_desc(smem_u32(x_s), kXChunk, 1024), w0 = make_desc(smem_u32(his), 16, 1024);
       const uint64_t d_k = make_desc(smem_u32(delta_s), 16, 1024), d_mn = make_desc(smem_u32(delta_s), 8192, 1024);
+      int held = 0, parts = 0;                                     // blocks in dx so far; sums handed over
       for (int i = 0; i < count && ok; ++i) {
-        if (fresh && groups > 0) ok = wait(&grp_flushed, (groups - 1) & 1, 206);
+        if (held == 0 && parts > 0) ok = wait(&dx_flushed, (parts - 1) & 1, 206);
         const bool last = i + 1 == count || blk + 1 == a.blocks;   // of this subnet here
+        const bool full = last || held + 1 == kDxBlocks;
         const uint64_t w = w0 + (uint64_t)(((i % kHi) * kTile) >> 4);
         const uint32_t dw = tmem + kDwCol + (i & 1) * kCols;
         ok = ok && wait(&dw_empty[i & 1], ((i >> 1) & 1) ^ 1, 207);
@@ -289,7 +296,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
           if (leader) {
 #pragma unroll
             for (int k = 0; k < kCols / 16; ++k)                   // dx[rows of h] += delta W^T
-              tc_mma(tmem + kDxCol + h * 128, dk + (k * 32 >> 4), w + (k * 32 >> 4), id_dx, !fresh || k != 0);
+              tc_mma(tmem + kDxCol + h * 128, dk + (k * 32 >> 4), w + (k * 32 >> 4), id_dx, (held | k) != 0);
 #pragma unroll
             for (int k = 0; k < 8; ++k)                            // x^T delta over the rows of h
               tc_mma(dw, xm + (k * 2048 >> 4), dm + (k * 2048 >> 4), id_dw, (h | k) != 0);
@@ -300,11 +307,12 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
         if (!ok) break;
         if (leader) {
           tc_commit(&dw_full[i & 1]);
-          if (last) tc_commit(&grp_done);    // z of this block has completed too: delta was made from it
+          if (full) tc_commit(&dx_done);
+          if (last) tc_commit(&x_free);      // z of this block has completed too: delta was made from it
         }
         __syncwarp();
-        fresh = last;
-        if (last) ++groups;
+        held = full ? 0 : held + 1;
+        if (full) ++parts;
         if (++blk == a.blocks) blk = 0;
       }
     }
@@ -316,7 +324,8 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
     constexpr float kLog2e = 1.4426950408889634f;
     const bool live = row < a.B;
     bool ok = h < NH;
-    int g = g0, blk = b0, groups = 0;
+    int g = g0, blk = b0, held = 0, parts = 0;
+    bool more = false;                       // dx of this subnet has been written before
     float row_lse = INFINITY;                // rows beyond the batch: delta is zero
     int label = -1;
     for (int i = 0; i < count && ok; ++i) {
@@ -393,9 +402,11 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
         mbar_arrive(&d_full[h]);
         mbar_arrive(&d_ready[i & 1]);
       }
-      if (i + 1 == count || blk + 1 == a.blocks) {
-        // the subnet's last block here: its share of dx leaves tensor memory
-        ok = __all_sync(0xffffffffu, mbar_wait(&grp_done, groups & 1, abortp, a.status, 211));
+      const bool last = i + 1 == count || blk + 1 == a.blocks;
+      ++held;
+      if (last || held == kDxBlocks) {
+        // the subnet's last block here, or as many as are summed in one piece: their share of dx leaves tensor memory
+        ok = __all_sync(0xffffffffu, mbar_wait(&dx_done, parts & 1, abortp, a.status, 211));
         if (!ok) break;
         tc_fence_after();
         const int part = (int)blockIdx.x - cta_of(items, a.n_cta, (long long)g * a.blocks);
@@ -408,14 +419,23 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
           if (live)
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-              if (32 * c + 4 * u < a.ldx)
-                *reinterpret_cast<uint4*>(out + 32 * c + 4 * u) = make_uint4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+              if (32 * c + 4 * u < a.ldx) {
+                float4* o = reinterpret_cast<float4*>(out + 32 * c + 4 * u);
+                float4 s = more ? *o : make_float4(0.f, 0.f, 0.f, 0.f);
+                s.x += __uint_as_float(v[4 * u]);
+                s.y += __uint_as_float(v[4 * u + 1]);
+                s.z += __uint_as_float(v[4 * u + 2]);
+                s.w += __uint_as_float(v[4 * u + 3]);
+                *o = s;
+              }
           __syncwarp();
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&grp_flushed);
-        ++groups;
+        if (lane == 0) mbar_arrive(&dx_flushed);
+        ++parts;
+        held = 0;
+        more = !last;
       }
       if (++blk == a.blocks) { blk = 0; ++g; }
     }

@@ -151,3 +151,33 @@ def test_bias_sums_are_as_exact_as_additions():
     # the launches it is compared with add 256 rows one after the other, which drops what is below half an ulp of the sum so
     # far: sums in shorter chains come out up to some 2^-23 larger, and not smaller
     assert -5e-8 <= float(off.median()) <= 3e-7, float(off.median())
+
+
+def test_input_gradient_over_many_classes_of_one_cta():
+    """148 subnets of two neurons: a CTA adds up all of a subnet's 65,536 classes.  Weights of one sign, so that nothing
+    cancels; each gradient is rounded to bf16, which errs to both sides: 2^-9 / sqrt(3) of one, 1.2e-5 of the mean of 9472."""
+    dims, S, B = [8, 296, 65536], 148, 32
+    g = torch.Generator(device="cuda").manual_seed(3)
+    W = [torch.ones(8, 296, device="cuda"), (torch.rand(296, 65536, device="cuda", generator=g) + 0.5).bfloat16().float()]
+    b = [torch.zeros(n, device="cuda") for n in dims[1:]]
+    X = (torch.rand(S * B, 8, device="cuda", generator=g) * 0.25).bfloat16()
+    y = torch.full((S * B,), 7, device="cuda", dtype=torch.int32)
+    b[1][7] = 12.0                                           # the label's share of the gradient is small beside the others'
+    W[1][:, 7] = 0.0
+    ctx = api.Ist(dims, S, api.IST_BF16, B)
+    ctx.bind_weights([w.clone() for w in W], [v.clone() for v in b])
+    ctx.partition(3)
+    idx, off = ctx.get_partition(1)
+    dx = torch.empty(S * B, 8, device="cuda")
+    ctx.local_steps(X, y, 0.0, 1, B, dx_out=dx)
+    ctx.sync_status()
+    rel = []
+    for s in range(S):
+        own = idx[off[s]:off[s + 1]].long()
+        a = (X[s * B:(s + 1) * B].double() @ W[0][:, own].double()).clamp_min(0).float().bfloat16().double()
+        p = torch.softmax(a @ W[1][own].double() + b[1].double(), 1)
+        p[:, 7] -= 1
+        want = ((p / B) @ W[1][own].double().T).sum(1)       # W_1 is all ones: every column of dX is the sum of both neurons
+        rel.append(dx[s * B:(s + 1) * B, 0].double() / want - 1)
+    mean = float(torch.cat(rel).mean())
+    assert abs(mean) <= 6e-5, mean
