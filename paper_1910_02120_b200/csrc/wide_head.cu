@@ -730,14 +730,21 @@ wide_lse_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ H
           float m4[4] = {z[0], z[1], z[2], z[3]};
 #pragma unroll
           for (int e = 4; e < 32; ++e) m4[e & 3] = fmaxf(m4[e & 3], z[e]);
-          const float mn = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * kLog2e;   // column nc counts: finite
-          if (sum != 0.f) {
-            const float scale = exp2_fast(ref - mn);
-            sum *= scale;
-            rest *= scale;
+          const float mn = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * kLog2e;
+          if (mn == -INFINITY) {             // a chunk of classes that biases rule out adds nothing, unless there is a NaN in it
+            float any = 0.f;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) any += z[e];
+            cs = any != any ? any : 0.f;
+          } else {
+            if (sum != 0.f) {
+              const float scale = exp2_fast(ref - mn);
+              sum *= scale;
+              rest *= scale;
+            }
+            ref = mn;
+            cs = sum_exp(mn);
           }
-          ref = mn;
-          cs = sum_exp(mn);
         }
         const float t = sum + cs, bb = t - sum;   // what the addition rounds away is kept: hundreds of chunks follow one another
         rest += (sum - (t - bb)) + (cs - bb);

@@ -181,3 +181,67 @@ def test_input_gradient_over_many_classes_of_one_cta():
         rel.append(dx[s * B:(s + 1) * B, 0].double() / want - 1)
     mean = float(torch.cat(rel).mean())
     assert abs(mean) <= 6e-5, mean
+
+
+@pytest.mark.parametrize("kind", ["ruled out first", "ruled out later", "lowest first", "rising", "falling", "steps"])
+def test_extreme_logits(kind):
+    """Biases that rule classes out and logits spread over more than 2^64: losses against 64 bits."""
+    dims, S, B = [16, 64, 12000], 1, 160
+    g = torch.Generator(device="cuda").manual_seed(3)
+    W = [torch.randn(a, b, device="cuda", generator=g) * (1.0 / a) ** 0.5 for a, b in zip(dims, dims[1:])]
+    b = [torch.zeros(n, device="cuda") for n in dims[1:]]
+    n = torch.arange(dims[-1], device="cuda")
+    if kind == "ruled out first":
+        b[1][:1000] = -float("inf")
+    elif kind == "ruled out later":
+        b[1][70:7000] = -float("inf")
+    elif kind == "lowest first":
+        b[1][:300] = torch.finfo(torch.float32).min
+    elif kind == "rising":
+        b[1] += n / 50.0
+    elif kind == "falling":
+        b[1] -= n / 50.0
+    else:
+        b[1] += torch.where(n % 64 < 32, -300.0, 0.0) + torch.where(n > 9000, 200.0, 0.0)
+    y = 8000 + torch.randint(4000, (B,), device="cuda", generator=g, dtype=torch.int32)
+    X = torch.randn(B, dims[0], device="cuda", generator=g).bfloat16()
+    ctx = api.Ist(dims, S, api.IST_BF16, B)
+    ctx.bind_weights([w.clone() for w in W], [v.clone() for v in b])
+    ctx.profile(True)
+    loss = ctx.round(3, X, y, 0.1, 1, B)
+    ctx.sync_status()
+    assert ctx.profile_read()["loss"][0] == 0                # the pass and not the separate launches
+    a = (X.double() @ W[0].bfloat16().double()).clamp_min(0).bfloat16().double()
+    z = a @ W[1].bfloat16().double() + b[1].double()
+    want = float((torch.logsumexp(z, 1) - z[torch.arange(B, device="cuda"), y.long()]).mean())
+    # logits of up to 500 are fp32, 2^-16 off each; the order of fp32 products may move a bf16 activation by 2^-8
+    assert abs(float(loss) - want) <= 1e-3 + 1e-5 * want, (float(loss), want)
+    assert all(bool(torch.isfinite(w).all()) for w in ctx.W)
+    assert torch.equal(torch.isfinite(ctx.b[1]), torch.isfinite(b[1]))
+
+
+def test_a_nan_row_and_a_label_outside_the_classes():
+    dims, S, B = [16, 64, 9000], 1, 40
+    g = torch.Generator(device="cuda").manual_seed(3)
+    W = [torch.randn(a, b, device="cuda", generator=g) * 0.1 for a, b in zip(dims, dims[1:])]
+    b = [torch.zeros(n, device="cuda") for n in dims[1:]]
+    X = torch.randn(B, dims[0], device="cuda", generator=g).bfloat16()
+    y = torch.randint(dims[-1], (B,), device="cuda", generator=g, dtype=torch.int32)
+    for bad in ("row", "label", "weight"):
+        Wd, Xd, yd = [w.clone() for w in W], X.clone(), y.clone()
+        if bad == "row":
+            Xd[3] = float("nan")
+        elif bad == "weight":
+            Wd[1][5, 100] = float("inf")
+        else:
+            yd[7] = dims[-1]
+        ctx = api.Ist(dims, S, api.IST_BF16, B)
+        ctx.bind_weights(Wd, [v.clone() for v in b])
+        loss = ctx.round(3, Xd, yd, 0.1, 1, B)
+        if bad == "label":
+            with pytest.raises(api.IstError):
+                ctx.sync_status()
+        else:
+            ctx.sync_status()
+            # fp32 arithmetic: relu of NaN is zero, an infinite logit makes the row's loss a NaN
+            assert bool(torch.isnan(loss).any()) == (bad == "weight")
