@@ -210,9 +210,8 @@ ist_status ist_local_steps_dx(ist_ctx* ctx, const ist_input* X, const int32_t* y
  * ist_reassemble writes all S slabs back, whoever trained them.
  * On the bf16 path the slices are otherwise kept as bf16 operands and the masters' low halves, which a
  * weight update moves with 8 bytes per weight instead of 10; the first ist_packed_layer call makes them
- * fp32 in place (enqueued on the context's stream) and the context keeps fp32 slices from then on.  The bf16
- * operands are the masters rounded to nearest even either way; of the updated masters, one in 2^17 (a tie of that
- * rounding) is kept one fp32 ulp nearer to zero while the slices are in operand form.
+ * fp32 in place (enqueued on the context's stream) and the context keeps fp32 slices from then on.  The values
+ * are the same either way, bit for bit; only a NaN may come back as another NaN from the operand form.
  * In ist_local_steps the inputs and losses are then addressed by the local subnet index
  * (0 .. count-1): rows start at i * stride_subnet, loss_out_dev holds count * K values.
  * Default range: all S subnets.  Not allowed while a partition is in place.

@@ -66,37 +66,27 @@ __host__ __device__ __forceinline__ constexpr int64_t round_up(int64_t a, int64_
   return ceil_div(a, b) * b;
 }
 
-// An fp32 master and the bf16 operand made from it take 32 bits together: the operand is the master rounded to
-// its upper 16 bits (to nearest, ties to even), and beside it lie the lower 16 bits of the master; the operand's last bit
-// and the low half's first say whether the rounding went up, so the master comes back.  A weight update then
-// moves 8 bytes per weight instead of 10.  One pattern does not fit: a tie that rounds down would share its code with the
-// tie that rounds up to the same operand, so it is kept as the value one ulp nearer to zero (one master in 2^17, by
-// 2^-24 of it; rounding ties away from zero instead keeps such masters exact but changes their operands by 2^-8, which
-// turns ReLU masks over).  Where a slice goes back, masters that no step has changed are told by
-// their source (unnudged).  NaNs become one NaN: their payloads do not fit.
-__device__ __forceinline__ uint32_t nudged(uint32_t bits) { return bits - ((bits & 0x1ffffu) == 0x8000u ? 1u : 0u); }
-__device__ __forceinline__ void split_master(float w, uint16_t* hi, uint16_t* lo) {
-  const uint32_t u = w != w ? 0x7fc00000u : nudged(__float_as_uint(w));
-  *hi = (uint16_t)((u + 0x8000u) >> 16);
-  *lo = (uint16_t)u;
-}
-// Whether a joined master may be a nudged one.
-__device__ __forceinline__ bool is_nudged(float v) { return (__float_as_uint(v) & 0x1ffffu) == 0x7fffu; }
-// A joined master v that came from *source: the source itself if v is its nudged form.
-__device__ __forceinline__ float unnudged(float v, const float* source) {
-  if (is_nudged(v)) {
-    const float o = *source;
-    if (__float_as_uint(o) == __float_as_uint(v) + 1u) return o;
-  }
-  return v;
-}
-__device__ __forceinline__ float join_master(uint16_t hi, uint16_t lo) {
+// An fp32 master and the bf16 operand made from it take 32 bits together: the operand is the master rounded to its
+// upper 16 bits (to nearest, ties to even), and beside it lie the lower 16 bits of the master; the operand's last bit
+// and the low half's first say whether the rounding went up, so the master comes back.  A weight update then moves 8
+// bytes per weight instead of 10.  Only the two ties that round to the same even operand look alike: a bit per master, a
+// sixty-fourth of the traffic, is set for the one that rounded down, and counts only where operand and low half are such a
+// pair's.  Every number comes back bit for bit, and a NaN as a NaN.  (Rounding ties away from zero would need no bit, but
+// changes the operand of one weight in 2^17 by 2^-8, which turns ReLU masks over.)
+__device__ __forceinline__ float join_master(uint16_t hi, uint16_t lo) {   // of two ties, the one that rounded up
   return __uint_as_float(((uint32_t)hi << 16) + (uint32_t)(int)(int16_t)lo);
 }
-__device__ __forceinline__ uint16_t operand_bits(float w) {
-  uint16_t hi, lo;
-  split_master(w, &hi, &lo);
-  return hi;
+__device__ __forceinline__ bool may_be_tie(float joined) { return (__float_as_uint(joined) & 0x1ffffu) == 0x18000u; }
+__device__ __forceinline__ float other_tie(float joined) { return __uint_as_float(__float_as_uint(joined) + 0x10000u); }
+// Tie bits: words of 32 columns, [slab][columns / 32][rows], so that a warp on consecutive rows reads consecutive words.
+// Column 2 i of the 32 has bit 15 - i, column 2 i + 1 bit 31 - i (see split8).
+__host__ __device__ __forceinline__ constexpr int64_t tie_words(int64_t rows, int64_t ld) { return (ld + 31) / 32 * rows; }   // of a slab
+struct TieBit {
+  int64_t word;
+  uint32_t mask;
+};
+__device__ __forceinline__ TieBit tie_bit(int64_t rows, int64_t ld, int64_t slab, int64_t row, int64_t col) {
+  return TieBit{slab * tie_words(rows, ld) + (col >> 5) * rows + row, 1u << (15 - ((int)col & 31) / 2 + ((int)col & 1) * 16)};
 }
 
 // Eight masters kept as operand and low half: joined, and taken apart again.
@@ -104,20 +94,28 @@ __device__ __forceinline__ void join8(const uint4& h, const uint4& l, float* w) 
   const uint32_t hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    w[2 * i] = __uint_as_float((hv[i] << 16) + (uint32_t)((int)(lv[i] << 16) >> 16));
-    w[2 * i + 1] = __uint_as_float((hv[i] & 0xffff0000u) + (uint32_t)((int)lv[i] >> 16));
+    const uint32_t b = lv[i] ^ 0x80008000u;                  // the low half plus 2^15: no sign to extend
+    w[2 * i] = __uint_as_float(__byte_perm(b, hv[i], 0x5410) - 0x8000u);
+    w[2 * i + 1] = __uint_as_float(__byte_perm(b, hv[i], 0x7632) - 0x8000u);
   }
 }
-// The distance of a master from its operand, in ulps of the master, is -2^15 .. 2^15; saturation to 16 bits is the nudge (and
-// turns the NaN that arithmetic gives into one whose operand is a NaN too).
-__device__ __forceinline__ void split8(const float* w, uint4* h, uint4* l) {
+// Operands and low halves of two masters.  Ties that rounded down are where adding half an operand's ulp and cutting gives the
+// odd neighbour of the operand: bit 0 or 16 of *ties.
+__device__ __forceinline__ void split2(float w0, float w1, uint32_t* h, uint32_t* l, uint32_t* ties) {
+  const uint32_t u0 = __float_as_uint(w0), u1 = __float_as_uint(w1);
+  const __nv_bfloat162 o = __floats2bfloat162_rn(w0, w1);
+  *h = *reinterpret_cast<const uint32_t*>(&o);
+  *l = __byte_perm(u0, u1, 0x5410);
+  *ties = (__byte_perm(u0 + 0x8000u, u1 + 0x8000u, 0x7632) ^ *h) & 0x00010001u;
+}
+// The tie bits are shifted in, two a step: sixteen steps make a word.
+__device__ __forceinline__ void split8(const float* w, uint4* h, uint4* l, uint32_t* ties) {
   uint32_t hv[4], lv[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat162 o = __floats2bfloat162_rn(w[2 * i], w[2 * i + 1]);
-    hv[i] = *reinterpret_cast<const uint32_t*>(&o);
-    const uint32_t d0 = __float_as_uint(w[2 * i]) - (hv[i] << 16), d1 = __float_as_uint(w[2 * i + 1]) - (hv[i] & 0xffff0000u);
-    asm("cvt.pack.sat.s16.s32 %0, %1, %2;" : "=r"(lv[i]) : "r"(d1), "r"(d0));
+    uint32_t t;
+    split2(w[2 * i], w[2 * i + 1], &hv[i], &lv[i], &t);
+    *ties = *ties * 2u + t;
   }
   *h = make_uint4(hv[0], hv[1], hv[2], hv[3]);
   *l = make_uint4(lv[0], lv[1], lv[2], lv[3]);

@@ -3,7 +3,7 @@
 // entries whose row and column neurons it owns; "Training Subnets": the trained slices go back
 // to the positions they came from).  Pure data movement:
 // fp32 values are moved bit for bit; the bf16 operand copy is a rounding of the moved value.  Masters that are kept
-// as operand and low half (split_master) are taken apart and joined on the way.
+// as operand and low half (join_master) are taken apart and joined on the way.
 #include <algorithm>
 #include <mutex>
 
@@ -15,13 +15,23 @@ namespace {
 // Packed elements o and o + 1 of a slice (o even): stored and loaded in whichever form the masters are kept in.  Pairs,
 // because a thread that loads 2-byte halves one by one has half the bytes in flight (scatter of
 // 3072-16384-16384-10, S = 8: 518 -> 395 us; 400 with fp32 words).
-__device__ __forceinline__ void put2(float* master, bf16* opw, uint16_t* lo, int64_t o, float v0, float v1) {
-  ushort2 h, l;
-  split_master(v0, &h.x, &l.x);
-  split_master(v1, &h.y, &l.y);
-  if (lo) *reinterpret_cast<ushort2*>(lo + o) = l;
+// Returns whether there is a tie, whose bit keep_tie must write.  Few are: a thread does that behind all its stores, with
+// values read again, so that it costs no registers.
+__device__ __forceinline__ bool put2(float* master, bf16* opw, uint16_t* lo, int64_t o, float v0, float v1) {
+  uint32_t h, l, ties;
+  split2(v0, v1, &h, &l, &ties);
+  if (lo) *reinterpret_cast<uint32_t*>(lo + o) = l;
   else *reinterpret_cast<float2*>(master + o) = make_float2(v0, v1);
-  if (opw) *reinterpret_cast<ushort2*>(opw + o) = h;
+  if (opw) *reinterpret_cast<uint32_t*>(opw + o) = h;
+  return lo && ((l & 0xffffu) == 0x8000u || l >> 16 == 0x8000u);
+}
+__device__ __forceinline__ uint32_t* ties_of(float* master) { return reinterpret_cast<uint32_t*>(master); }   // see SliceJob::lo
+__device__ __forceinline__ void keep_tie(float* master, const SliceMap& m, int64_t s, int64_t i, int64_t j, float v) {
+  const uint32_t u = __float_as_uint(v);
+  if ((u & 0xffffu) != 0x8000u) return;
+  const TieBit t = tie_bit(m.rows_pad, m.ld, s, i, j);
+  if (u & 0x10000u) atomicAnd(ties_of(master) + t.word, ~t.mask);
+  else atomicOr(ties_of(master) + t.word, t.mask);
 }
 // Loading is two steps, the words as they lie and then the values, so that a kernel has all its loads in flight
 // first: a branch on the form around every load keeps the compiler from that.
@@ -36,16 +46,22 @@ __device__ __forceinline__ float2 value2(uint2 p) {
   return make_float2(join_master((uint16_t)p.x, (uint16_t)p.y), join_master((uint16_t)(p.x >> 16), (uint16_t)(p.y >> 16)));
 }
 // The same for one element, where the positions of neighbours are not known to be a pair.
-__device__ __forceinline__ void put(float* master, bf16* opw, uint16_t* lo, int64_t o, float v) {
-  uint16_t h, l;
-  split_master(v, &h, &l);
+__device__ __forceinline__ bool put(float* master, bf16* opw, uint16_t* lo, int64_t o, float v) {
+  const uint16_t l = (uint16_t)__float_as_uint(v);
   if (lo) lo[o] = l;
   else master[o] = v;
-  if (opw) reinterpret_cast<uint16_t*>(opw)[o] = h;
+  if (opw) opw[o] = __float2bfloat16_rn(v);
+  return lo && l == 0x8000;
 }
 template <bool SPLIT>
 __device__ __forceinline__ float get(const float* master, const bf16* opw, const uint16_t* lo, int64_t o) {
   return SPLIT ? join_master(reinterpret_cast<const uint16_t*>(opw)[o], lo[o]) : master[o];
+}
+// Element (s, i, j) of a split slice, whichever of two ties it is.
+__device__ __forceinline__ float settle(float* master, const SliceMap& m, int64_t s, int64_t i, int64_t j, float v) {
+  if (!may_be_tie(v)) return v;
+  const TieBit t = tie_bit(m.rows_pad, m.ld, s, i, j);
+  return ties_of(master)[t.word] & t.mask ? other_tie(v) : v;
 }
 
 constexpr int kThreads = 256;
@@ -68,9 +84,10 @@ struct SliceJobs {
 // Two rows at a time: with the loads of all rows in flight before the first store, the stores of a large matrix
 // come in bursts that DRAM takes worse (middle layer of 32768 x 32768, S = 8: 1100 -> 1390 us for four rows).
 template <bool SPLIT>
-__device__ __forceinline__ void scatter_rows(const SliceJob& J, int64_t o0, const int64_t* c, const int32_t* rows, int64_t i0,
+__device__ __forceinline__ void scatter_rows(const SliceJob& J, int s, int64_t j, const int64_t* c, const int32_t* rows, int64_t i0,
                                              int64_t i1) {
   const int64_t ld = J.m.ld, full = J.m.full_cols;
+  int64_t o0 = ((int64_t)s * J.m.rows_pad + i0) * ld + j;
   for (int64_t i = i0; i < i1; i += 2, o0 += 2 * ld) {
     const bool two = i + 1 < i1;
     const uint2 p0 = raw2<SPLIT>(J.master, J.opw, J.lo, o0), p1 = two ? raw2<SPLIT>(J.master, J.opw, J.lo, o0 + ld) : p0;
@@ -78,13 +95,9 @@ __device__ __forceinline__ void scatter_rows(const SliceJob& J, int64_t o0, cons
     float* w1 = J.W + (two ? (rows ? rows[i + 1] : i + 1) * full : 0);
     float2 f0 = value2<SPLIT>(p0), f1 = value2<SPLIT>(p1);
     // both rows' loads have been asked for before this branch, which is hardly ever taken
-    if (SPLIT && (is_nudged(f0.x) | is_nudged(f0.y) | is_nudged(f1.x) | is_nudged(f1.y))) {
-      f0.x = unnudged(f0.x, w0 + c[0]);
-      if (c[1] >= 0) f0.y = unnudged(f0.y, w0 + c[1]);
-      if (two) {
-        f1.x = unnudged(f1.x, w1 + c[0]);
-        if (c[1] >= 0) f1.y = unnudged(f1.y, w1 + c[1]);
-      }
+    if (SPLIT && (may_be_tie(f0.x) | may_be_tie(f0.y) | may_be_tie(f1.x) | may_be_tie(f1.y))) {
+      f0 = make_float2(settle(J.master, J.m, s, i, j, f0.x), settle(J.master, J.m, s, i, j + 1, f0.y));
+      if (two) f1 = make_float2(settle(J.master, J.m, s, i + 1, j, f1.x), settle(J.master, J.m, s, i + 1, j + 1, f1.y));
     }
     w0[c[0]] = f0.x;
     if (c[1] >= 0) w0[c[1]] = f0.y;
@@ -129,12 +142,13 @@ __global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ 
   if (!GATHER) {
     const int64_t i1 = min(i0 + R, nrows);
     const int32_t* rows = m.row_idx ? m.row_idx + m.row_off[s] : nullptr;
-    if (J.lo) scatter_rows<true>(J, o0, c, rows, i0, i1);
-    else scatter_rows<false>(J, o0, c, rows, i0, i1);
+    if (J.lo) scatter_rows<true>(J, s, j, c, rows, i0, i1);
+    else scatter_rows<false>(J, s, j, c, rows, i0, i1);
     return;
   }
   float v[R][2];
   int64_t r[R];
+  bool tie = false;
 #pragma unroll
   for (int u = 0; u < R; ++u)
     r[u] = i0 + u < nrows ? (m.row_idx ? m.row_idx[m.row_off[s] + i0 + u] : i0 + u) * m.full_cols : -1;
@@ -144,7 +158,14 @@ __global__ void __launch_bounds__(kThreads) move_kernel(const __grid_constant__ 
     for (int e = 0; e < 2; ++e) v[u][e] = r[u] >= 0 && c[e] >= 0 ? J.W[r[u] + c[e]] : 0.f;
 #pragma unroll
   for (int u = 0; u < R; ++u)
-    if (i0 + u < m.rows_pad) put2(J.master, J.opw, J.lo, o0 + u * m.ld, v[u][0], v[u][1]);
+    if (i0 + u < m.rows_pad) tie |= put2(J.master, J.opw, J.lo, o0 + u * m.ld, v[u][0], v[u][1]);
+  if (tie)
+#pragma unroll 1
+    for (int64_t i = i0; i < min(i0 + R, nrows); ++i) {
+      const float* w = J.W + (m.row_idx ? m.row_idx[m.row_off[s] + i] : i) * m.full_cols;
+      keep_tie(J.master, m, s, i, j, w[c[0]]);               // c[0] >= 0: padding holds no tie
+      if (c[1] >= 0) keep_tie(J.master, m, s, i, j + 1, w[c[1]]);
+    }
 }
 
 // ---- last layer: whole rows, picked by the previous hidden layer's partition --------------------
@@ -185,6 +206,7 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, fl
   for (int64_t i0 = (int64_t)blockIdx.y * kRowU; i0 < (GATHER ? m.rows_pad : nrows); i0 += (int64_t)gridDim.y * kRowU) {
     float v[kRowU][kColU];
     int64_t src[kRowU];
+    bool tie = false;
 #pragma unroll
     for (int u = 0; u < kRowU; ++u) src[u] = (i0 + u < nrows) ? (int64_t)rows[i0 + u] * m.full_cols : -1;
     if (GATHER) {
@@ -202,8 +224,15 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, fl
           const int64_t j = j0 + c * kThreads + 2 * lane;
           to_pairs(v[u][c], v[u][c + 1]);
           if (i0 + u < m.rows_pad && j < m.ld)
-            put2(master, opw, lo, ((int64_t)s * m.rows_pad + i0 + u) * m.ld + j, v[u][c], v[u][c + 1]);
+            tie |= put2(master, opw, lo, ((int64_t)s * m.rows_pad + i0 + u) * m.ld + j, v[u][c], v[u][c + 1]);
         }
+      if (tie)
+#pragma unroll 1
+        for (int e = 0; e < kRowU * kColU; ++e) {
+          const int64_t i = i0 + e / kColU, j = j0 + (e % kColU & ~1) * kThreads + 2 * lane + (e & 1);
+          if (i < nrows && j < m.full_cols) keep_tie(master, m, s, i, j, W[(int64_t)rows[i] * m.full_cols + j]);
+        }
+      __syncwarp();
     } else {
       uint2 p[kRowU][kColU / 2];
 #pragma unroll
@@ -223,23 +252,24 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(float* W, SliceMap m, fl
           v[u][c + 1] = f.y;
           from_pairs(v[u][c], v[u][c + 1]);
         }
-      bool rare = false;                     // one branch for all of a thread's values, behind all its loads
 #pragma unroll
       for (int u = 0; u < kRowU; ++u)
 #pragma unroll
-        for (int c = 0; c < kColU; ++c) rare |= SPLIT && is_nudged(v[u][c]);
-      auto at = [&](int c) { return j0 + (c & ~1) * kThreads + (c & 1) * 32 + lane; };
-      if (rare)
-#pragma unroll
-        for (int u = 0; u < kRowU; ++u)
-#pragma unroll
-          for (int c = 0; c < kColU; ++c)
-            if (src[u] >= 0 && at(c) < m.full_cols) v[u][c] = unnudged(v[u][c], W + src[u] + at(c));
-#pragma unroll
-      for (int u = 0; u < kRowU; ++u)
-#pragma unroll
-        for (int c = 0; c < kColU; ++c)
-          if (src[u] >= 0 && at(c) < m.full_cols) W[src[u] + at(c)] = v[u][c];
+        for (int c = 0; c < kColU; ++c) {
+          const int64_t j = j0 + (c & ~1) * kThreads + (c & 1) * 32 + lane;
+          tie |= SPLIT && may_be_tie(v[u][c]);
+          if (src[u] >= 0 && j < m.full_cols) W[src[u] + j] = v[u][c];
+        }
+      // ties are looked at again, each by the lane that stored it
+      if (tie)
+#pragma unroll 1
+        for (int e = 0; e < kRowU * kColU; ++e) {
+          const int64_t i = i0 + e / kColU, j = j0 + (e % kColU & ~1) * kThreads + (e & 1) * 32 + lane;
+          if (i >= nrows || j >= m.full_cols) continue;
+          float* w = W + (int64_t)rows[i] * m.full_cols + j;
+          *w = settle(master, m, s, i, j, *w);
+        }
+      __syncwarp();
     }
   }
 }
@@ -395,12 +425,16 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
       for (int e = threadIdx.x; e < total; e += kPermThreads) {
         const int col = map_col[e];
         const long long o = map_off[e] + k0 * m.ld;
+        bool tie = false;
 #pragma unroll
-        for (int r = 0; r < kStageRows; ++r) {
-          if (r < nrows) {
-            put(master, opw, lo, o + (long long)r * m.ld, t[r * kStageCols + col]);
+        for (int r = 0; r < kStageRows; ++r)
+          if (r < nrows) tie |= put(master, opw, lo, o + (long long)r * m.ld, t[r * kStageCols + col]);
+        if (tie)
+#pragma unroll 1
+          for (int r = 0; r < nrows; ++r) {
+            const int64_t e0 = map_off[e];                     // of row 0: slab and column
+            keep_tie(master, m, e0 / (m.rows_pad * m.ld), k0 + r, e0 % m.ld, t[r * kStageCols + col]);
           }
-        }
       }
       if (blockIdx.x == 0) {   // pad columns [|G^s|, ld) of these rows are zero
         for (int s = m.s_first; s < m.s_first + S; ++s) {
@@ -422,27 +456,26 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
         const int col = map_col[e], col2 = two ? map_col[e + kPermThreads] : 0;
         const long long o = map_off[e] + k0 * m.ld, o2 = two ? map_off[e + kPermThreads] + k0 * m.ld : o;
         float v[kStageRows], v2[kStageRows];
+        bool tie = false;
 #pragma unroll
         for (int r = 0; r < kStageRows; ++r) {
           v[r] = r < nrows ? get<SPLIT>(master, opw, lo, o + (long long)r * m.ld) : 0.f;
           v2[r] = r < nrows ? get<SPLIT>(master, opw, lo, o2 + (long long)r * m.ld) : 0.f;
         }
-        bool rare = false;                   // one branch for all of them, behind all the loads
-#pragma unroll
-        for (int r = 0; r < kStageRows; ++r) rare |= SPLIT && (is_nudged(v[r]) | is_nudged(v2[r]));
-        if (rare)
-#pragma unroll
-          for (int r = 0; r < kStageRows; ++r) {
-            if (r >= nrows) break;
-            const float* full = W + (k0 + r) * m.full_cols + c0;
-            v[r] = unnudged(v[r], full + col);
-            if (two) v2[r] = unnudged(v2[r], full + col2);
-          }
 #pragma unroll
         for (int r = 0; r < kStageRows; ++r) {
+          tie |= SPLIT && (may_be_tie(v[r]) | may_be_tie(v2[r]));
           t[r * kStageCols + col] = v[r];
           if (two) t[r * kStageCols + col2] = v2[r];
         }
+        if (tie)
+#pragma unroll 1
+          for (int r = 0; r < 2 * nrows; ++r) {
+            if (r >= nrows && !two) break;
+            float* v_at = t + r % nrows * kStageCols + (r < nrows ? col : col2);
+            const int64_t e0 = map_off[r < nrows ? e : e + kPermThreads];
+            *v_at = settle(master, m, e0 / (m.rows_pad * m.ld), k0 + r % nrows, e0 % m.ld, *v_at);
+          }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
@@ -486,47 +519,43 @@ bool launch_permute_cols(const Launch& L, float* W, const SliceMap& m, int S, fl
   return true;
 }
 
-// Where packed element (s, i, j) lies in the full matrix; null: it is padding.
-__device__ __forceinline__ const float* source_of(const float* W, const SliceMap& m, int s, int64_t i, int64_t j) {
-  const int64_t nrows = m.row_idx ? m.row_off[s + 1] - m.row_off[s] : m.full_rows;
-  const int64_t ncols = m.col_idx ? m.col_off[s + 1] - m.col_off[s] : m.full_cols;
-  if (i >= nrows || j >= ncols) return nullptr;
-  return W + (m.row_idx ? m.row_idx[m.row_off[s] + i] : i) * m.full_cols + (m.col_idx ? m.col_idx[m.col_off[s] + j] : j);
-}
-
-// packed, opw, lo: subnet s's slab.
-__global__ void copy_out_kernel(const SliceJob job, int s, const float* packed, const bf16* opw, const uint16_t* lo, int64_t rows,
-                                int64_t cols, float* __restrict__ out) {
+__global__ void copy_out_kernel(const SliceJob job, int s, int64_t rows, int64_t cols, float* __restrict__ out) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t i = blockIdx.y;
   if (j < cols)
     for (; i < rows; i += gridDim.y) {
-      const int64_t o = i * job.m.ld + j;
-      out[i * cols + j] = lo ? unnudged(get<true>(packed, opw, lo, o), source_of(job.W, job.m, s, i, j)) : packed[o];
+      const int64_t o = ((int64_t)s * job.m.rows_pad + i) * job.m.ld + j;
+      out[i * cols + j] = job.lo ? settle(job.master, job.m, s, i, j, get<true>(job.master, job.opw, job.lo, o)) : job.master[o];
     }
 }
 
 // Masters first .. end - 1 of n become fp32 words in place.  The low halves are the second half of the words, so
 // word i takes the place of low halves 2 i - n and 2 i - n + 1, both at or before i: a launch may cover words as long as
 // they replace only low halves of words before its first.  One block may end the array: it reads all it needs
-// before it writes.
-__device__ __forceinline__ float joined(const SliceJob& job, int64_t n, int64_t i) {
-  const float v = get<true>(job.master, job.opw, reinterpret_cast<const uint16_t*>(job.master) + n, i);
-  if (!is_nudged(v)) return v;
-  // where it came from decides
-  const int64_t slab = job.m.rows_pad * job.m.ld, s = i / slab, e = i - s * slab;
-  const float* src = source_of(job.W, job.m, (int)s, e / job.m.ld, e % job.m.ld);
-  return src ? unnudged(v, src) : v;
+// before it writes.  The first words replace the tie bits, so ties that rounded down get the operand that rounding up would
+// give them before, which joins to their value, and their operands are put right here.
+__global__ void write_out_ties_kernel(const SliceJob job, int64_t n) {
+  uint16_t* hi = reinterpret_cast<uint16_t*>(job.opw);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    if (job.lo[i] != 0x8000 || (hi[i] & 1)) continue;
+    const TieBit t = tie_bit(job.m.rows_pad, job.m.ld, i / (job.m.rows_pad * job.m.ld), i / job.m.ld % job.m.rows_pad, i % job.m.ld);
+    if (ties_of(job.master)[t.word] & t.mask) hi[i] += 1;
+  }
 }
-__global__ void join_masters_kernel(const SliceJob job, int64_t n, int64_t first, int64_t end) {
+__device__ __forceinline__ void join_one(const SliceJob& job, int64_t i, float w) {
+  const bf16 operand = __float2bfloat16_rn(w);
+  if (__bfloat16_as_ushort(job.opw[i]) != __bfloat16_as_ushort(operand)) job.opw[i] = operand;
+  job.master[i] = w;
+}
+__global__ void join_masters_kernel(const SliceJob job, int64_t first, int64_t end) {
   if (gridDim.x > 1) {
     for (int64_t i = first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end; i += (int64_t)gridDim.x * blockDim.x)
-      job.master[i] = joined(job, n, i);
+      join_one(job, i, get<true>(job.master, job.opw, job.lo, i));
   } else {
     const int64_t i = first + threadIdx.x;
-    const float w = i < end ? joined(job, n, i) : 0.f;
+    const float w = i < end ? get<true>(job.master, job.opw, job.lo, i) : 0.f;
     __syncthreads();
-    if (i < end) job.master[i] = w;
+    if (i < end) join_one(job, i, w);
   }
 }
 
@@ -585,21 +614,21 @@ void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* 
 
 void copy_out_slice(const Launch& L, const SliceJob& j, int s, int64_t rows, int64_t cols, float* out) {
   dim3 grid((unsigned)ceil_div(cols, 256), (unsigned)(rows < 1024 ? rows : 1024));
-  const int64_t slab = (int64_t)s * j.m.rows_pad * j.m.ld;
-  copy_out_kernel<<<grid, 256, 0, L.stream>>>(j, s, j.master + slab, j.opw ? j.opw + slab : nullptr, j.lo ? j.lo + slab : nullptr,
-                                              rows, cols, out);
+  copy_out_kernel<<<grid, 256, 0, L.stream>>>(j, s, rows, cols, out);
   L.count();
 }
 
 void join_masters(const Launch& L, const SliceJob& j) {
   constexpr int kJoin = 1024;
   const int64_t n = j.S * j.m.rows_pad * j.m.ld;
+  write_out_ties_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, kJoin), 4096), kJoin, 0, L.stream>>>(j, n);
+  L.count();
   int64_t first = 0;
   while (first < n) {
     int64_t end = first + (n - first) / 2;     // words below this replace low halves below `first` only
     if (n - first <= kJoin) end = n;
     const int64_t blocks = n - first <= kJoin ? 1 : std::max<int64_t>(2, std::min<int64_t>(ceil_div(end - first, kJoin), 4096));
-    join_masters_kernel<<<(unsigned)blocks, kJoin, 0, L.stream>>>(j, n, first, end);
+    join_masters_kernel<<<(unsigned)blocks, kJoin, 0, L.stream>>>(j, first, end);
     L.count();
     first = end;
   }

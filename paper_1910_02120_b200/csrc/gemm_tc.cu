@@ -29,7 +29,7 @@
 // through mbarriers (slot_full -> chunk_done -> slot_empty), so warps work on different chunks
 // at the same time and a slow chunk does not hold the others back.
 // The weight-update epilogue is the HBM-heavy part of a step (8 bytes per weight against
-// 2*B flops): its master chunks, bf16 operand and low half (split_master), are prefetched through the slot ring
+// 2*B flops): its master chunks, bf16 operand and low half (join_master), are prefetched through the slot ring
 // while earlier chunks are updated in place in shared memory and stored back.  With fp32 masters and an operand
 // copy beside them (10 bytes; kept for contexts that hand out fp32 slices) the launch takes 190 us
 // instead of 155 at 3072-16384-16384-10, S = 8, 512 rows, and 63.8 instead of 55.7 at 1024-8192-8192-100, S = 4.
@@ -123,6 +123,7 @@ struct TcProblem {
   // has reached wait_target; a storer adds the chunks it has stored for (g, mt) to signal_ctr
   const unsigned* wait_ctr; unsigned wait_target;
   unsigned* signal_ctr;
+  uint32_t* ties; long long ties_sg;   // EPI_SGD_SPLIT: the masters' tie bits (tie_bit), ties_sg words per group
 };
 
 struct TcArgs {
@@ -592,6 +593,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
 #pragma unroll
       for (int c = 0; c < NCH; ++c) bias_reg[c] = next_bias[c];
       const int row = at.mt * (BM * PAIR) + rank * BM + r;   // this thread's row of the output
+      uint32_t next_ties[CW / CH];
       float run_sum = 0.f;                            // EPI_LSE_PART: over this warp group's chunks of the tile
       // softmax pass: log-sum-exp in the log2 domain, with the division by the batch size folded in
       const float row_lse = EPI == EPI_SOFTMAX_DELTA ? next_lse * kLog2e - log2f(a.inv_rows) : 0.f;
@@ -613,6 +615,15 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const int slot = cq % NS;
         uint8_t* f32 = slots + slot * SLOT_BYTES;
         uint8_t* b16 = f32 + F32_BYTES;
+        // tie bits: asked for one chunk of this warp ahead, within a tile
+        auto tie_word = [&](int n) { return a.p[pi].ties + g * a.p[pi].ties_sg + (long long)(n / CH) * pM + row; };
+        uint32_t tie_bits[CW / CH];
+#pragma unroll
+        for (int h = 0; h < CW / CH && kSplit; ++h) {
+          auto bits = [&](int n) { return row < pM && n < pN ? __ldcg(tie_word(n)) : 0u; };
+          tie_bits[h] = c >= NG ? next_ties[h] : bits(nc + h * CH);
+          next_ties[h] = c + NG < NCH ? bits(nc + NG * CW + h * CH) : 0u;
+        }
         // the slot is ready: loaded (input chunk) or drained by the store of an earlier chunk
         if (kStore) {
           if (ET::kAux) ok = mbar_wait(&slot_full[slot], (cq / NS) & 1, abortp, a.status, 5);
@@ -655,17 +666,13 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         } else if (kSplit) {
 #pragma unroll
           for (int h = 0; h < CW / CH; ++h) {
-            tc_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c * CW + h * CH), acc);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {             // 8 columns per iteration
-              float w[8];
-              uint4* ph = CW == CH ? b16_unit(b16, r, u) : row128_unit(b16, r, 4 * h + u);
-              uint4* pl = CW == CH ? b16_unit(b16 + B16_BYTES, r, u) : row128_unit(b16 + B16_BYTES, r, 4 * h + u);
-              join8(*ph, *pl, w);
-#pragma unroll
-              for (int e = 0; e < 8; ++e) w[e] -= a.lr * __uint_as_float(acc[8 * u + e]);
-              split8(w, ph, pl);
-            }
+            auto at = [&](uint8_t* area, int u) { return CW == CH ? b16_unit(area, r, u) : row128_unit(area, r, 4 * h + u); };
+            const uint32_t was = tie_bits[h];
+            const uint32_t now = update_split32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c * CW + h * CH), a.lr,
+                                                [&](int u) { return at(b16, u); }, [&](int u) { return at(b16 + B16_BYTES, u); }, was,
+                                                [] {});
+            if (was | now)
+              if (row < pM && nc + h * CH < pN) *tie_word(nc + h * CH) = now;
           }
         } else if (EPI == EPI_RELU_MASK) {
 #pragma unroll
@@ -1428,7 +1435,8 @@ bool gemm_tc_batch(const Launch& L, const GemmArgs<bf16>* ga, int n, const GemmC
         if (!make_map(&m.aux16[i], a.mask, 2, n_store, a.M, a.G, a.mask_ld, a.mask_sg, CH, BM, 64)) return false;
         break;
       case EPI_SGD:
-        if (!a_mn || !b_mn || !a.opw) return false;
+        if (!a_mn || !b_mn || !a.opw || (a.lo && !a.ties)) return false;
+        p.ties = a.ties; p.ties_sg = tie_words(a.M, a.outf_ld);
         {
           const int cw = a.lo ? chunk_cols(EPI_SGD_SPLIT, pair) : CH;
           if (a.lo ? !make_map(&m.c32[i], a.lo, 2, n_store, a.M, a.G, a.outf_ld, a.outf_sg, cw, BM, 2 * cw)

@@ -72,9 +72,9 @@ struct ist_ctx {
   int rule = IST_PART_BALANCED;
   std::vector<std::vector<int64_t>> group_count;   // [hidden layer][subnet]
 
-  // Masters of layers updated by the tensor-core launches are kept as operand + low half (split_master): the
-  // operand in its own buffer, the low halves in the second half of the layer's master buffer.  A context whose packed
-  // slices have been asked for (ist_packed_layer) holds fp32 words from then on.
+  // Masters of layers updated by the tensor-core launches are kept as operand + low half (join_master): the
+  // operand in its own buffer, the low halves in the second half of the layer's master buffer and the tie bits in the first.
+  // A context whose packed slices have been asked for (ist_packed_layer) holds fp32 words from then on.
   bool packed_seen = false;
   bool split(int l) const { return precision == IST_BF16 && !packed_seen && !(csr && l == 1); }
 
@@ -488,6 +488,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
   auto master = [&](int l) { return c->master(l) + (int64_t)s0 * c->slice_elems(l); };
   auto opw = [&](int l) -> bf16* { return bf ? c->opw(l) + (int64_t)s0 * c->slice_elems(l) : nullptr; };
   auto lo = [&](int l) -> uint16_t* { return c->split(l) ? c->lo(l) + (int64_t)s0 * c->slice_elems(l) : nullptr; };
+  auto ties = [&](int l) { return reinterpret_cast<uint32_t*>(c->master(l)) + s0 * tie_words(c->rows_pad(l), c->ld[l]); };
   auto bias_of = [&](int l) { return c->bias(l) + (int64_t)s0 * c->ld[l]; };
   auto weights = [&](int l) -> const T* {       // operand copy of layer l's slices
     return bf ? reinterpret_cast<const T*>(opw(l)) : reinterpret_cast<const T*>(master(l));
@@ -551,7 +552,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       wh.S = S; wh.B = B; wh.H = (int)c->np[t - 1]; wh.N = (int)c->N[t];
       wh.ldx = (int)c->ld[t - 1]; wh.x_sg = Bm * c->ld[t - 1];
       head_buffers(wh, act(t - 1), delta(t - 1));
-      wh.opw = opw(t); wh.lo = lo(t); wh.ldw = c->ld[t]; wh.w_sg = c->slice_elems(t);
+      wh.opw = opw(t); wh.lo = lo(t); wh.ties = ties(t); wh.ldw = c->ld[t]; wh.w_sg = c->slice_elems(t);
       wh.bias = bias_of(t);
       wh.lse = lse; wh.labels = y + row0; wh.label_logit = label_logit; wh.lse_sg = Bm; wh.labels_sg = X->stride_subnet;
       wh.lse_part = logits;
@@ -768,7 +769,7 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       g.epi = EPI_SGD;
       g.outf = master(l); g.outf_ld = c->ld[l]; g.outf_sg = c->slice_elems(l);
       g.opw = opw(l);
-      g.lo = lo(l);
+      g.lo = lo(l); g.ties = ties(l);
       g.lr = lr;
       upd.push_back(g);
     }

@@ -67,14 +67,15 @@ struct SliceJob {
   bf16* opw;
   SliceMap m;
   int S;
-  uint16_t* lo;  // null: master holds fp32 values (and opw, where given, the operands); else the master is (opw, lo), see split_master
+  uint16_t* lo;  // null: master holds fp32 values (and opw, where given, the operands); else the master is (opw, lo), see
+                 // join_master: lo is the second half of the words at master, and the tie bits lie in the first
   int mean;      // scatter only: the output bias, b[j] += (sum_s (packed[s][j] - b[j])) / S
 };
 void gather_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
 void scatter_slices(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st);
 // Dense copy-out of subnet s's packed slice (ist_get_subnet_params).
 void copy_out_slice(const Launch& L, const SliceJob& job, int s, int64_t rows, int64_t cols, float* out);
-// Masters kept as (opw, lo) become fp32 words in place, all S slabs; lo is the second half of the words at master.
+// Masters kept as (opw, lo) become fp32 words in place, all S slabs.
 void join_masters(const Launch& L, const SliceJob& job);
 
 // ---- grouped GEMM -----------------------------------------------------------------------
@@ -118,7 +119,8 @@ struct GemmArgs {
   float* outf; int64_t outf_ld, outf_sg;
   const T* mask; int64_t mask_ld, mask_sg;
   bf16* opw;
-  uint16_t* lo;   // EPI_SGD: not null: the master is (opw, lo), see split_master, and outf is not used
+  uint16_t* lo;   // EPI_SGD: not null: the master is (opw, lo, ties), see join_master, and outf is not used
+  uint32_t* ties;
   float lr;
   // wide softmax head.  lse_part: [G][gemm_tc_lse_parts(N_store)][M] float2 (a few partials per
   // 256-column tile); lse / label_logit: [G][lse_sg]; labels: labels[g * labels_sg + m].
@@ -176,7 +178,7 @@ struct WideHead {
   int S, B, H, N;                  // subnets, rows, width of the layer below, classes
   const bf16* x; int ldx; long long x_sg;          // activations of the layer below, [S][..][ldx], x_sg apart
   bf16* delta;                     // delta of the layer below, laid out like x
-  bf16* opw; uint16_t* lo; long long ldw, w_sg;    // [S][H][ldw]
+  bf16* opw; uint16_t* lo; uint32_t* ties; long long ldw, w_sg;   // [S][H][ldw]; ties: see tie_bit
   float* bias;                     // [S][ldw]
   float* lse; const int32_t* labels; float* label_logit; long long lse_sg, labels_sg;
   float* lse_part;                 // scratch of the first pass, as much as gemm_tc_lse_parts asks for

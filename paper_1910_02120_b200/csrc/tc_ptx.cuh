@@ -228,6 +228,34 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 32 columns of a row of masters (operand, low half, tie bits: see join_master) in shared memory become w - lr * gradient, the
+// gradient in tensor memory; hi(u), lo(u): 16-byte unit u of their operands and low halves.  Takes the columns' tie
+// bits and returns the new ones; read() is called once tensor memory has been read.  A tie that rounded down (one row of 32 in
+// 4096 holds one) first gets the odd operand that rounding up would give it: that joins to its value.
+template <typename Hi, typename Lo, typename Read>
+__device__ __forceinline__ uint32_t update_split32(uint32_t gradient, float lr, const Hi& hi, const Lo& lo, uint32_t ties,
+                                                   const Read& read) {
+  for (; ties; ties &= ties - 1) {
+    const int b = __ffs(ties) - 1, col = 2 * (15 - (b & 15)) + (b >> 4);
+    uint16_t* h = reinterpret_cast<uint16_t*>(hi(col >> 3)) + (col & 7);
+    if (reinterpret_cast<uint16_t*>(lo(col >> 3))[col & 7] == 0x8000 && !(*h & 1)) *h += 1;
+  }
+  __syncwarp();
+  uint32_t acc[32];
+  tc_ld32(gradient, acc);
+  read();
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    uint4 *ph = hi(u), *pl = lo(u);
+    float w[8];
+    join8(*ph, *pl, w);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] -= lr * __uint_as_float(acc[8 * u + e]);
+    split8(w, ph, pl, &ties);
+  }
+  return ties;
+}
+
 // Shared-memory matrix descriptor for a 128-byte-swizzled tile.
 //   bits  0..13 start address >> 4      bits 16..29 leading byte offset >> 4
 //   bits 32..45 stride byte offset >> 4 bits 46..47 descriptor version (1)

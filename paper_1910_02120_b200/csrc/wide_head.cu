@@ -5,7 +5,7 @@
 //   dx += delta W^T                                (tensor memory, one partial sum per CTA and subnet)
 //   W -= lr x^T delta,  b -= lr sum_b delta        (the weights as they stood before the step are read first)
 //
-// What bounds it: the weights, 4 bytes per weight (operand and low half, see split_master) in and out.  As separate launches
+// What bounds it: the weights, 4 bytes per weight (operand and low half, see join_master) in and out.  As separate launches
 // the deltas of 670,091 classes (2.7 GB per step at 256 rows and S = 8) were written once and read twice beside
 // them and the operands were read three times.  135909-1024-670091, S = 8, 256 rows, per step: softmax and delta 1.10 ms,
 // dx 0.72, update 1.73; in this pass 1.43, 0.6 of the copy rate on its 5.5 GB.  What is left is the chain of a block's
@@ -54,6 +54,7 @@ struct HeadArgs {
   float lr, inv_rows;
   const float* lse; const int32_t* labels; float* label_logit; long long lse_sg, labels_sg;
   float* bias; long long bias_sg;
+  uint32_t* ties;                        // the masters' tie bits, see tie_bit
   float* dx_part;                        // [S][partials][B][ldx]
   float2* lse_part;                      // first pass: [S][partials][B] (reference exponent, sum)
   DeviceStatus* status;
@@ -444,8 +445,15 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
     const int grp = (warp - 19) >> 2, q = warp & 3;
     const int r = q * 32 + lane;             // neuron of this thread
     bool ok = true;
+    const int chunks = (a.ldw + 31) / 32;
+    auto has_ties = [&](int blk, int c) { return r < a.H && 2 * blk + c < chunks; };
+    auto tie_word = [&](int g, int blk, int c) { return a.ties + ((long long)g * chunks + 2 * blk + c) * a.H + r; };
     for (int i = grp; i < count && ok; i += 2) {
       const int s = i % kHi;
+      const int g = (int)((it0 + i) / a.blocks), blk = (int)(it0 + i - (long long)g * a.blocks);
+      // tie bits: asked for here, the waits below take longer
+      const uint32_t ties0 = has_ties(blk, 0) ? __ldcg(tie_word(g, blk, 0)) : 0u;
+      const uint32_t ties1 = has_ties(blk, 1) ? __ldcg(tie_word(g, blk, 1)) : 0u;
       // Column sums of delta, 16 columns per warp: a lane adds up eight columns of every sixteenth row (the eight lanes of a
       // quarter warp read eight rows, every bank once), sixteen lanes then share their sums out.  All in fp32 additions: a row
       // of ones times delta on the tensor cores, accumulated from 16 rows to the next, was 6e-7 off over 256 rows
@@ -483,8 +491,6 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
           }
         }
         c[0] += __shfl_xor_sync(0xffffffffu, c[0], 1);
-        const long long item = it0 + i;
-        const int g = (int)(item / a.blocks), blk = (int)(item - (long long)g * a.blocks);
         const int col = 16 * q + 8 * (lane >> 4) + ((lane >> 1) & 7), n = blk * kCols + col;
         if ((lane & 1) == 0 && n < a.N) a.bias[g * a.bias_sg + n] = bias_s[s][col] - a.lr * c[0];
       }
@@ -499,23 +505,17 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       uint8_t* lo = los + (i % kLo) * kTile;
 #pragma unroll 1
       for (int c = 0; c < 2; ++c) {
-        uint32_t acc[32];
-        tc_ld32(tmem + kDwCol + grp * kCols + c * 32 + ((uint32_t)(q * 32) << 16), acc);
-        if (c == 1) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&dw_empty[grp]);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          uint4* ph = unit_at(hi, r, 4 * c + u);
-          uint4* pl = unit_at(lo, r, 4 * c + u);
-          float w[8];
-          join8(*ph, *pl, w);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) w[e] -= a.lr * __uint_as_float(acc[8 * u + e]);
-          split8(w, ph, pl);
-        }
+        const uint32_t was = c ? ties1 : ties0;
+        const uint32_t now = update_split32(tmem + kDwCol + grp * kCols + c * 32 + ((uint32_t)(q * 32) << 16), a.lr,
+                                            [&](int u) { return unit_at(hi, r, 4 * c + u); },
+                                            [&](int u) { return unit_at(lo, r, 4 * c + u); }, was, [&] {
+                                              if (c == 0) return;
+                                              tc_fence_before();
+                                              __syncwarp();
+                                              if (lane == 0) mbar_arrive(&dw_empty[grp]);
+                                            });
+        if (was | now)
+          if (has_ties(blk, c)) *tie_word(g, blk, c) = now;
       }
       fence_async_smem();
       __syncwarp();
@@ -870,6 +870,7 @@ bool common_args(const WideHead& w, int cols, DeviceStatus* st, HeadArgs* a, Hea
   a->lr = w.lr; a->inv_rows = 1.f / (float)w.B;
   a->lse = w.lse; a->lse_sg = w.lse_sg; a->labels = w.labels; a->labels_sg = w.labels_sg; a->label_logit = w.label_logit;
   a->bias = w.bias; a->bias_sg = w.ldw;
+  a->ties = w.ties;
   a->status = st;
   return make_map(&m->x, w.x, 2, w.H, w.B, w.S, w.ldx, w.x_sg, 64, 256, 128) &&
          make_map(&m->hi, w.opw, 2, w.N, w.H, w.S, w.ldw, w.w_sg, 64, 128, 128) &&
