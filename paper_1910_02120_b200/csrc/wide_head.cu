@@ -462,16 +462,18 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       if (!ok) break;
       f32x2 sum[4] = {pair(0.f, 0.f), pair(0.f, 0.f), pair(0.f, 0.f), pair(0.f, 0.f)};
       for (int h = 0; h < NH; ++h) {
+        uint4 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = *unit_at(delta_s, h * 128 + 16 * j + (lane & 15), 2 * q + (lane >> 4));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&d_empty[h]);   // these rows are in registers
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const uint4 v = *unit_at(delta_s, h * 128 + 16 * j + (lane & 15), 2 * q + (lane >> 4));
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+          const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
 #pragma unroll
           for (int e = 0; e < 4; ++e)
             sum[e] = add2(sum[e], pair(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)));
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&d_empty[h]);
       }
       {
         float c[8];
