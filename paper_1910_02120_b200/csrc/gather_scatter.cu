@@ -410,6 +410,7 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
     const int64_t k0 = rb * kStageRows;
     const int nrows = (int)min((long long)kStageRows, (long long)(m.full_rows - k0));
     float* t = tile + buf * kStageRows * kStageCols;
+    bool tie = false;                        // among this thread's values: they are gone through once more
     if (GATHER) {
       // the other buffer was last read in the previous iteration, which ended with a barrier
       if (threadIdx.x == 0 && rb + gridDim.y < n_blocks) issue_load(rb + gridDim.y, buf ^ 1);
@@ -425,17 +426,19 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
       for (int e = threadIdx.x; e < total; e += kPermThreads) {
         const int col = map_col[e];
         const long long o = map_off[e] + k0 * m.ld;
-        bool tie = false;
 #pragma unroll
         for (int r = 0; r < kStageRows; ++r)
           if (r < nrows) tie |= put(master, opw, lo, o + (long long)r * m.ld, t[r * kStageCols + col]);
-        if (tie)
-#pragma unroll 1
-          for (int r = 0; r < nrows; ++r) {
-            const int64_t e0 = map_off[e];                     // of row 0: slab and column
-            keep_tie(master, m, e0 / (m.rows_pad * m.ld), k0 + r, e0 % m.ld, t[r * kStageCols + col]);
-          }
       }
+      if (tie)
+#pragma unroll 1
+        for (int e = threadIdx.x; e < total; e += kPermThreads) {
+          const int64_t e0 = map_off[e];                       // of row 0: slab and column
+          for (int r = 0; r < nrows; ++r) {
+            const float v = t[r * kStageCols + map_col[e]];
+            if ((uint16_t)__float_as_uint(v) == 0x8000) keep_tie(master, m, e0 / (m.rows_pad * m.ld), k0 + r, e0 % m.ld, v);
+          }
+        }
       if (blockIdx.x == 0) {   // pad columns [|G^s|, ld) of these rows are zero
         for (int s = m.s_first; s < m.s_first + S; ++s) {
           const int cnt = m.col_off[s + 1] - m.col_off[s];
@@ -456,7 +459,6 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
         const int col = map_col[e], col2 = two ? map_col[e + kPermThreads] : 0;
         const long long o = map_off[e] + k0 * m.ld, o2 = two ? map_off[e + kPermThreads] + k0 * m.ld : o;
         float v[kStageRows], v2[kStageRows];
-        bool tie = false;
 #pragma unroll
         for (int r = 0; r < kStageRows; ++r) {
           v[r] = r < nrows ? get<SPLIT>(master, opw, lo, o + (long long)r * m.ld) : 0.f;
@@ -468,15 +470,16 @@ __global__ void __launch_bounds__(kPermThreads, 1) permute_cols_kernel(float* W,
           t[r * kStageCols + col] = v[r];
           if (two) t[r * kStageCols + col2] = v2[r];
         }
-        if (tie)
-#pragma unroll 1
-          for (int r = 0; r < 2 * nrows; ++r) {
-            if (r >= nrows && !two) break;
-            float* v_at = t + r % nrows * kStageCols + (r < nrows ? col : col2);
-            const int64_t e0 = map_off[r < nrows ? e : e + kPermThreads];
-            *v_at = settle(master, m, e0 / (m.rows_pad * m.ld), k0 + r % nrows, e0 % m.ld, *v_at);
-          }
       }
+      if (tie)
+#pragma unroll 1
+        for (int e = threadIdx.x; e < total; e += kPermThreads) {
+          const int64_t e0 = map_off[e];
+          for (int r = 0; r < nrows; ++r) {
+            float* v = t + r * kStageCols + map_col[e];
+            if (may_be_tie(*v)) *v = settle(master, m, e0 / (m.rows_pad * m.ld), k0 + r, e0 % m.ld, *v);
+          }
+        }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
       if (threadIdx.x == 0) {

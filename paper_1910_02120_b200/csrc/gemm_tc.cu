@@ -540,10 +540,20 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     float next_lse = 0.f;
     int next_label = -1;
     TileAt at_next{};                                 // the tile the last prefetch located: the next one to work on
-    auto prefetch_tile_inputs = [&](int tile) {
+    // EPI_SGD_SPLIT: tie bits of this thread's row, of its warp's first chunk of the next tile and of its next in this tile
+    uint32_t first_ties[CW / CH], next_ties[CW / CH];
+    auto tie_word = [&](const TcProblem& pr, int g, int row, int n) { return pr.ties + g * pr.ties_sg + (long long)(n / CH) * pr.M + row; };
+    auto ask_ties = [&](uint32_t* bits, const TcProblem& pr, const TileAt& at, int c) {
+      const int n = at.nt * BN + c * CW, row = at.mt * (BM * PAIR) + rank * BM + r;
+#pragma unroll
+      for (int h = 0; h < CW / CH; ++h)
+        bits[h] = c < NCH && n + h * CH < pr.N && row < pr.M ? __ldcg(tie_word(pr, at.slab, row, n + h * CH)) : 0u;
+    };
+    auto prefetch_tile_inputs = [&](int tile, int cq0) {   // cq0: chunks before the tile's first
       const TileAt at = at_next = locate(a, tile, pi_next);
       const TcProblem& pr = a.p[pi_next];
       const int n0 = at.nt * BN;
+      if (kSplit) ask_ties(first_ties, pr, at, (wg - cq0) & (NG - 1));
       if (EPI == EPI_BIAS_RELU || EPI == EPI_BIAS_F32) {
         const float* bias = pr.bias ? pr.bias + (long long)group_of(pr, at.slab) * pr.bias_sg : nullptr;
 #pragma unroll
@@ -566,7 +576,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
     };
 #pragma unroll
     for (int c = 0; c < NCH; ++c) next_bias[c] = 0.f;
-    if (unit < total_tiles) prefetch_tile_inputs(unit);
+    if (unit < total_tiles) prefetch_tile_inputs(unit, 0);
     for (int tile = unit; tile < total_tiles && ok; tile += n_units) {
       const TileAt at = at_next;                      // located when its inputs were requested
       pi = at.pi;
@@ -574,7 +584,7 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         int kb_limit;
         if (!tile_live<BM * PAIR, BN>(a.p[pi], at, group_of(a.p[pi], at.slab), &kb_limit)) {
           // the inputs requested for this tile are dropped; ask for the next tile's
-          if (tile + n_units < total_tiles) prefetch_tile_inputs(tile + n_units);
+          if (tile + n_units < total_tiles) prefetch_tile_inputs(tile + n_units, cq);
           continue;
         }
       }
@@ -593,12 +603,13 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
 #pragma unroll
       for (int c = 0; c < NCH; ++c) bias_reg[c] = next_bias[c];
       const int row = at.mt * (BM * PAIR) + rank * BM + r;   // this thread's row of the output
-      uint32_t next_ties[CW / CH];
       float run_sum = 0.f;                            // EPI_LSE_PART: over this warp group's chunks of the tile
       // softmax pass: log-sum-exp in the log2 domain, with the division by the batch size folded in
       const float row_lse = EPI == EPI_SOFTMAX_DELTA ? next_lse * kLog2e - log2f(a.inv_rows) : 0.f;
       const int row_label = next_label;
-      if (tile + n_units < total_tiles) prefetch_tile_inputs(tile + n_units);
+#pragma unroll
+      for (int h = 0; h < CW / CH; ++h) next_ties[h] = first_ties[h];
+      if (tile + n_units < total_tiles) prefetch_tile_inputs(tile + n_units, cq + min(nch, (pN - n0 + cw - 1) / cw));
       // warp-uniform outcome: the tensor-memory loads below need the whole warp
       ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (j >> 1) & 1, abortp, a.status, 4));
       if (!ok) break;
@@ -615,14 +626,11 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
         const int slot = cq % NS;
         uint8_t* f32 = slots + slot * SLOT_BYTES;
         uint8_t* b16 = f32 + F32_BYTES;
-        // tie bits: asked for one chunk of this warp ahead, within a tile
-        auto tie_word = [&](int n) { return a.p[pi].ties + g * a.p[pi].ties_sg + (long long)(n / CH) * pM + row; };
         uint32_t tie_bits[CW / CH];
+        if (kSplit) {
 #pragma unroll
-        for (int h = 0; h < CW / CH && kSplit; ++h) {
-          auto bits = [&](int n) { return row < pM && n < pN ? __ldcg(tie_word(n)) : 0u; };
-          tie_bits[h] = c >= NG ? next_ties[h] : bits(nc + h * CH);
-          next_ties[h] = c + NG < NCH ? bits(nc + NG * CW + h * CH) : 0u;
+          for (int h = 0; h < CW / CH; ++h) tie_bits[h] = next_ties[h];
+          if (NCH > NG) ask_ties(next_ties, a.p[pi], at, c + NG);
         }
         // the slot is ready: loaded (input chunk) or drained by the store of an earlier chunk
         if (kStore) {
@@ -664,15 +672,15 @@ gemm_tc_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcAr
             *b16_unit(b16, r, u) = pack8(w);
           }
         } else if (kSplit) {
-#pragma unroll
+#pragma unroll 1
           for (int h = 0; h < CW / CH; ++h) {
-            auto at = [&](uint8_t* area, int u) { return CW == CH ? b16_unit(area, r, u) : row128_unit(area, r, 4 * h + u); };
-            const uint32_t was = tie_bits[h];
+            auto unit_of = [&](uint8_t* area, int u) { return CW == CH ? b16_unit(area, r, u) : row128_unit(area, r, 4 * h + u); };
+            const uint32_t was = h ? tie_bits[CW / CH - 1] : tie_bits[0];
             const uint32_t now = update_split32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c * CW + h * CH), a.lr,
-                                                [&](int u) { return at(b16, u); }, [&](int u) { return at(b16 + B16_BYTES, u); }, was,
-                                                [] {});
+                                                [&](int u) { return unit_of(b16, u); },
+                                                [&](int u) { return unit_of(b16 + B16_BYTES, u); }, was, [] {});
             if (was | now)
-              if (row < pM && nc + h * CH < pN) *tie_word(nc + h * CH) = now;
+              if (row < pM && nc + h * CH < pN) *tie_word(a.p[pi], g, row, nc + h * CH) = now;
           }
         } else if (EPI == EPI_RELU_MASK) {
 #pragma unroll

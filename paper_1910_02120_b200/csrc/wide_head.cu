@@ -419,16 +419,21 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
           tc_ld32(tmem + kDxCol + h * 128 + c * 32 + lane_base, v);
           if (live)
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-              if (32 * c + 4 * u < a.ldx) {
-                float4* o = reinterpret_cast<float4*>(out + 32 * c + 4 * u);
-                float4 s = more ? *o : make_float4(0.f, 0.f, 0.f, 0.f);
-                s.x += __uint_as_float(v[4 * u]);
-                s.y += __uint_as_float(v[4 * u + 1]);
-                s.z += __uint_as_float(v[4 * u + 2]);
-                s.w += __uint_as_float(v[4 * u + 3]);
-                *o = s;
+            for (int u0 = 0; u0 < 8; u0 += 4) {      // four loads in flight
+              float4 s[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                s[u] = more && 32 * c + 4 * (u0 + u) < a.ldx ? *reinterpret_cast<const float4*>(out + 32 * c + 4 * (u0 + u))
+                                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const uint32_t* d = v + 4 * (u0 + u);
+                if (32 * c + 4 * (u0 + u) < a.ldx)
+                  *reinterpret_cast<float4*>(out + 32 * c + 4 * (u0 + u)) =
+                      make_float4(s[u].x + __uint_as_float(d[0]), s[u].y + __uint_as_float(d[1]), s[u].z + __uint_as_float(d[2]),
+                                  s[u].w + __uint_as_float(d[3]));
               }
+            }
           __syncwarp();
         }
         tc_fence_before();
@@ -460,7 +465,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       // where additions in four chains are 0.8e-7 off, and always to the same side.
       ok = __all_sync(0xffffffffu, mbar_wait(&d_ready[grp], (i >> 1) & 1, abortp, a.status, 215));
       if (!ok) break;
-      f32x2 sum[4] = {pair(0.f, 0.f), pair(0.f, 0.f), pair(0.f, 0.f), pair(0.f, 0.f)};
+      float c[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       for (int h = 0; h < NH; ++h) {
         uint4 v[8];
 #pragma unroll
@@ -472,17 +477,11 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
           const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
 #pragma unroll
           for (int e = 0; e < 4; ++e)
-            sum[e] = add2(sum[e], pair(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)));
+            asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
+                : "+f"(c[2 * e]), "+f"(c[2 * e + 1]) : "r"(w[e]));
         }
       }
       {
-        float c[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 t = unpair(sum[e]);
-          c[2 * e] = t.x;
-          c[2 * e + 1] = t.y;
-        }
 #pragma unroll
         for (int w = 4; w >= 1; w >>= 1) {   // of the columns held, a lane keeps half and gives the other half away
           const bool up = lane & (2 * w);
