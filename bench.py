@@ -164,14 +164,25 @@ def work_model(w: synth.Workload, norm=False, data=None):
     }
 
 
-def moved_bytes(w: synth.Workload, wm):
+def moved_bytes(w: synth.Workload, wm, shard=False):
     """work_model counts an fp32 master and a bf16 copy, 10 bytes per weight gathered or updated.  Masters of dense
-    bf16 layers are kept as operand and low half, 8 bytes: rates are of what is moved."""
-    if w.precision == "bf16":
+    bf16 layers are kept as operand and low half, 8 bytes: rates are of what is moved.  Contexts that exchange fp32
+    slices (shard) keep the other form."""
+    if w.precision == "bf16" and not shard:
         d, S = w.layer_dims, w.S
         split = wm["packed_elems"] - (d[0] * -(-d[1] // S) * S if w.x_dist == "csr" else 0)
         wm["bytes"]["gather"] -= 2 * split
         wm["bytes"]["dw_sgd"] -= 2 * split * w.K
+    return wm
+
+
+def fused_head_work(w: synth.Workload, wm, prof):
+    """A very wide output layer whose delta, input gradient and update are one launch has no loss launches of its own, and its
+    time is the update class's: so is the work of its input gradient."""
+    if w.precision == "bf16" and len(w.layer_dims) > 2 and prof["loss"][0] == 0:
+        dx = 2 * w.B * w.S * -(-w.layer_dims[-2] // w.S) * w.layer_dims[-1] * w.K
+        wm["flops"]["dx"] -= dx
+        wm["flops"]["dw_sgd"] += dx
     return wm
 
 
@@ -490,7 +501,8 @@ def run_ours(args, w):
         return
 
     pk = peaks()
-    wm = moved_bytes(w, work_model(w, norm=args.norm_eps is not None, data=data if data.is_csr else None))
+    wm = moved_bytes(w, work_model(w, norm=args.norm_eps is not None, data=data if data.is_csr else None), shard)
+    wm = fused_head_work(w, wm, prof)
     if shard:      # this rank ran the local steps of its own subnets only; gather / scatter cover all S
         for k in ("fwd", "dx", "dw_sgd"):
             wm["flops"][k] = wm["flops"][k] * count // w.S

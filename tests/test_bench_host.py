@@ -107,4 +107,18 @@ def test_recorded_dram_traffic_covers_the_headers_it_names(tmp_path, monkeypatch
     assert bench.measured_traffic("W", "upd", 100.0) == 110.0
     (tmp_path / "k.cuh").write_text("other wrappers")
     assert bench.measured_traffic("W", "upd", 100.0) is None
-    assert all("tc_ptx.cuh" in entry["source"] for entry in json.load(open(tracked))["C3-wide-pixels"].values())
+    for entry in json.load(open(tracked))["C3-wide-pixels"].values():
+        assert {"gemm_tc.cu", "tc_ptx.cuh", "common.cuh"} <= set(entry["source"])   # the update's arithmetic is in the last
+
+
+def test_moved_bytes_and_the_fused_output_layer():
+    import bench
+    from paper_1910_02120_b200 import synth
+    w = synth.Workload("m", (64, 128, 9000), S=2, B=16, K=3, rounds=1, precision="bf16", x_dist="normal")
+    packed = 64 * 128 + 128 * 9000
+    plain, shard = (bench.moved_bytes(w, bench.work_model(w), s) for s in (False, True))
+    assert plain["bytes"]["dw_sgd"] == 8 * packed * 3 and shard["bytes"]["dw_sgd"] == 10 * packed * 3
+    separate = bench.fused_head_work(w, bench.work_model(w), {"loss": (3, 0.1)})
+    fused = bench.fused_head_work(w, bench.work_model(w), {"loss": (0, 0.0)})
+    assert separate["flops"] == bench.work_model(w)["flops"]
+    assert fused["flops"]["dx"] == 0 and sum(fused["flops"].values()) == sum(separate["flops"].values())
