@@ -97,3 +97,32 @@ def test_subnet_range_is_checked():
     with pytest.raises(api.IstError):
         ctx.set_subnet_range(0, 4)                     # not while a partition is in place
     ctx.reassemble()
+
+
+def test_later_rounds_of_half_contexts_equal_a_full_context():
+    """From its first exchange on a sharded context keeps fp32 slices, a full one operands and low halves."""
+    import torch
+    dims, S, B, K = (256, 2048, 2048, 16), 8, 512, 8
+    w = synth.Workload("sh", dims, S=S, B=B, K=K, rounds=1, precision="bf16", x_dist="normal", lr=0.02, seed=31)
+    W, b, data = H.make_problem(w, bias_scale=0.1)
+    X, y = H.gpu_inputs(w, data)
+    ref, Wr, br = H.gpu_context(w, W, b)
+    half = S // 2
+    rows = half * K * B
+    parts = [H.gpu_context(w, W, b) for _ in range(2)]
+    for r, (ctx, _, _) in enumerate(parts):
+        ctx.set_subnet_range(r * half, half)
+    for seed in (5, 6, 7):
+        ref.round(seed, X, y, w.lr, K, B)
+        for r, (ctx, _, _) in enumerate(parts):
+            ctx.partition(seed)
+            ctx.local_steps(X[r * rows:(r + 1) * rows], y[r * rows:(r + 1) * rows], w.lr, K, B)
+        for l in range(1, len(dims)):
+            (m0, b0), (m1, b1) = parts[0][0].packed_layer(l), parts[1][0].packed_layer(l)
+            m0[half:], b0[half:] = m1[half:], b1[half:]
+            m1[:half], b1[:half] = m0[:half], b0[:half]
+        for ctx, Wd, bd in parts:
+            ctx.reassemble()
+            ctx.sync_status()
+            for p, q in zip(Wd + bd, Wr + br):
+                assert torch.equal(p, q)
