@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "tc_ptx.cuh"
 
 namespace ist {
 namespace {
@@ -342,10 +343,6 @@ __device__ __forceinline__ bool bar_try_wait(uint64_t* bar, uint32_t parity) {
       : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ void bulk_load(void* dst_smem, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_addr(dst_smem)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
-}
 __device__ __forceinline__ void bulk_store(void* dst, const void* src_smem, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
                ::"l"(dst), "r"(smem_addr(src_smem)), "r"(bytes) : "memory");
@@ -592,8 +589,10 @@ void move_all(const Launch& L, const SliceJob* jobs, int n, DeviceStatus* st) {
   for (int i = 0; i < n; ++i) {
     const SliceJob& j = jobs[i];
     const int64_t elements = j.mean ? 0 : j.S * j.m.rows_pad * j.m.ld;
-    if (elements >= kOwnColumns && staged_ok(j.m, j.S) && (j.lo ? launch_permute_cols<GATHER, true> : launch_permute_cols<GATHER, false>)(L, j.W, j.m, j.S, j.master, j.opw, j.lo, st))
-      continue;
+    if (elements >= kOwnColumns && staged_ok(j.m, j.S)) {
+      const auto launch = j.lo ? launch_permute_cols<GATHER, true> : launch_permute_cols<GATHER, false>;
+      if (launch(L, j.W, j.m, j.S, j.master, j.opw, j.lo, st)) continue;
+    }
     if (elements >= kOwnRows && rows_ok(j.m)) {
       launch_rows<GATHER>(L, j.W, j.m, j.S, j.master, j.opw, j.lo);
       continue;

@@ -30,9 +30,10 @@
 // at the same time and a slow chunk does not hold the others back.
 // The weight-update epilogue is the HBM-heavy part of a step (8 bytes per weight against
 // 2*B flops): its master chunks, bf16 operand and low half (join_master), are prefetched through the slot ring
-// while earlier chunks are updated in place in shared memory and stored back.  With fp32 masters and an operand
-// copy beside them (10 bytes; kept for contexts that hand out fp32 slices) the launch takes 190 us
-// instead of 155 at 3072-16384-16384-10, S = 8, 512 rows, and 63.8 instead of 55.7 at 1024-8192-8192-100, S = 4.
+// while earlier chunks are updated in place in shared memory and stored back; a tie bit per master comes by plain loads, a
+// chunk ahead.  With fp32 masters and an operand copy beside them (10 bytes; kept for contexts that hand out
+// fp32 slices) the launch takes 190 us instead of 157 at 3072-16384-16384-10, S = 8, 512 rows, and 63.8 instead of 57.6 at
+// 1024-8192-8192-100, S = 4.
 //
 // PAIR = 2 runs two CTAs of a cluster as one unit (tcgen05 cta_group::2): the pair computes a
 // 256 x BN tile, each CTA loads its own 128 rows of A and its half (BN/2 rows) of B and keeps its
@@ -76,7 +77,7 @@ constexpr int BK = 64;                   // 64 bf16 = 128 bytes = one swizzle ro
 constexpr int CH = 32;                   // epilogue chunk: 32 output columns
 // Updates of split masters on single CTAs work in chunks twice as wide: both areas then have 128-byte rows and half the
 // hand-offs (update of 1024 x 670,091, S = 8, 256 rows: 2.13 -> 1.73 ms).  On pairs six narrow slots are better than
-// four wide ones (1024-8192-8192-100, S = 4, 512 rows: 55.7 against 58.8 us; 63.8 with fp32 masters).
+// four wide ones (1024-8192-8192-100, S = 4, 512 rows: 55.7 against 58.8 us without tie bits).
 constexpr int chunk_cols(int epi, int pair) { return epi == 7 /* EPI_SGD_SPLIT */ && pair == 1 ? 2 * CH : CH; }
 // Warps of a CTA, see the role list above: loader, MMA issuer, the epilogue warps (two groups of
 // four; four groups for the two softmax passes over a very wide output layer, whose epilogues are
@@ -224,11 +225,6 @@ template <> struct EpiTraits<EPI_SGD_SPLIT> { static constexpr bool k32 = false,
 template <> struct EpiTraits<EPI_LSE_PART> { static constexpr bool k32 = false, k16 = false, kAux = false; };
 template <> struct EpiTraits<EPI_SOFTMAX_DELTA> { static constexpr bool k32 = false, k16 = true, kAux = false; };
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ uint4 pack8(const float* v) {
   __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
   __nv_bfloat162 c = __floats2bfloat162_rn(v[4], v[5]), d = __floats2bfloat162_rn(v[6], v[7]);
@@ -1235,7 +1231,7 @@ bool gemm_tc_wait_selftest(const Launch& L, DeviceStatus* st, long long limit_cy
 // (120-26586-2688-509, S = 9, 128 rows: 804 -> 733 us against pairs; 3072-16384-16384-10 within 1 %).  Up to
 // 320 rows still where the pairs' tiles hang over the matrices' edges by more than 15 % (the same
 // network at 224 rows 890 -> 845 us; 1024-4096-4096-35, which pairs tile exactly, 477 against 484 us), with 128 columns
-// where the masters are split (1001-5000-3001-77, S = 6, 200 rows: the launch 32.9 us with 64, 31.3 with 128).  Not
+// where the masters are split (1001-5000-3001-77, S = 6, 200 rows: the launch 32.9 us with 64, 31.3 with 128, without tie bits).  Not
 // with a layer of more than 8192 columns, whose update streams from DRAM: an output layer of 670,091
 // classes behind 1024 neurons, S = 8, 256 rows, 54.3 ms with 128 columns and 56.8 with 64; 30,000 classes at 128 rows
 // 851 and 874 us.  Hidden layers of 9000 to 20,000 neurons would gain 1 to 4 % up to 128 rows (512-20000-2048-10,

@@ -640,7 +640,8 @@ ist_status run_local_steps(ist_ctx* c, const ist_input* X, const int32_t* y, flo
       if (!flush_fwd()) return fail(c, IST_ERR_UNSUPPORTED, "forward GEMMs below layer %d cannot be launched", l);
       {
         Scope sc(c, IST_K_FWD);
-        if (l == t && fused_head ? !wide_head_lse(L, wh, st) : !gemm(c, g)) return fail(c, IST_ERR_UNSUPPORTED, "forward GEMM of layer %d cannot be launched", l);
+        const bool launched = l == t && fused_head ? wide_head_lse(L, wh, st) : gemm(c, g);
+        if (!launched) return fail(c, IST_ERR_UNSUPPORTED, "forward GEMM of layer %d cannot be launched", l);
       }
       if (l < t && c->norm) standardise(l);
     }

@@ -256,6 +256,16 @@ __device__ __forceinline__ uint32_t update_split32(uint32_t gradient, float lr, 
   return ties;
 }
 
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
 // Shared-memory matrix descriptor for a 128-byte-swizzled tile.
 //   bits  0..13 start address >> 4      bits 16..29 leading byte offset >> 4
 //   bits 32..45 stride byte offset >> 4 bits 46..47 descriptor version (1)

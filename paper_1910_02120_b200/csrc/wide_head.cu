@@ -2,14 +2,15 @@
 // slice W_t[G^s, :]), everything that follows the rows' log-sum-exp in one kernel.  Per block of 64 classes:
 //
 //   z = x W + b,  delta = (softmax - onehot) / B   (bf16, stays in shared memory)
-//   dx += delta W^T                                (tensor memory, one partial sum per CTA and subnet)
+//   dx += delta W^T                                (tensor memory, 160 blocks at most; one partial sum per CTA and subnet)
 //   W -= lr x^T delta,  b -= lr sum_b delta        (the weights as they stood before the step are read first)
 //
 // What bounds it: the weights, 4 bytes per weight (operand and low half, see join_master) in and out.  As separate launches
 // the deltas of 670,091 classes (2.7 GB per step at 256 rows and S = 8) were written once and read twice beside
 // them and the operands were read three times.  135909-1024-670091, S = 8, 256 rows, per step: softmax and delta 1.10 ms,
-// dx 0.72, update 1.73; in this pass 1.43, 0.6 of the copy rate on its 5.5 GB.  What is left is the chain of a block's
-// hand-offs (z, delta, products, update, store: some 15,000 cycles from load to reload, with five blocks in flight).
+// dx 0.72, update 1.73; in this pass 1.77, 0.47 of the copy rate on its 5.5 GB (1.50 with three shortcuts that lost precision:
+// bias sums on mma.sync, dx of all of a CTA's classes in one sum, no tie bits).  What is left is the chain of a block's
+// hand-offs (z, delta, products, bias sums, update, store: some 18,000 cycles from load to reload, five blocks in flight).
 //
 // Layout.  The subnet's x (256 rows x 128 neurons, 64 KB) stays in shared memory; a block's operands and low halves are
 // [neuron][64 classes] tiles of 128-byte rows, five and three of them in flight; delta is [row][64 classes].  All three are
@@ -19,8 +20,9 @@
 // the tensor pipe per block, against 2900 for its 64 KB of DRAM traffic.
 //
 // Warps: 0 copies; 1-2 MMA issue; 3-18 z -> delta, eight per 128 rows, 32 columns of one row per thread (with eight
-// warps and 64 columns the chain z -> delta was the longest: 1.49 ms against 1.43); 19-26 column sums of delta (bias) and
-// weight updates, two groups of four that take turns; 27 stores and loads of the low halves.  All hand-offs are mbarriers, every wait is bounded, no CTA waits for another.
+// warps and 64 columns the chain z -> delta was the longest: by 0.06 ms); 19-26 column sums of delta (bias) and weight
+// updates, two groups of four that take turns; 27 stores and loads of the low halves.  All hand-offs are mbarriers, every wait
+// is bounded, no CTA waits for another.
 #include <cuda.h>
 
 #include <algorithm>
@@ -90,15 +92,6 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
-}
-__device__ __forceinline__ float exp2_fast(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 // 16-byte unit u of 128-byte row r, 128-byte swizzled
 __device__ __forceinline__ uint4* unit_at(uint8_t* tile, int r, int u) {
@@ -364,8 +357,8 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
         uint32_t p[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const __nv_bfloat162 v = __floats2bfloat162_rn(exp2_fast(fmaf(z[2 * e], kLog2e, -row_lse)),
-                                                         exp2_fast(fmaf(z[2 * e + 1], kLog2e, -row_lse)));
+          const __nv_bfloat162 v = __floats2bfloat162_rn(ex2_approx(fmaf(z[2 * e], kLog2e, -row_lse)),
+                                                         ex2_approx(fmaf(z[2 * e + 1], kLog2e, -row_lse)));
           p[e] = *reinterpret_cast<const uint32_t*>(&v);
         }
         o[u] = make_uint4(p[0], p[1], p[2], p[3]);
@@ -393,7 +386,7 @@ wide_head_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ 
       for (int u = 0; u < 4; ++u) *unit_at(delta_s, row, 4 * part32 + u) = o[u];
       if (lat >= 0 && lat < 32) {
         reinterpret_cast<bf16*>(unit_at(delta_s, row, 4 * part32 + (lat >> 3)))[lat & 7] =
-            __float2bfloat16_rn(exp2_fast(fmaf(zl, kLog2e, -row_lse)) - a.inv_rows);
+            __float2bfloat16_rn(ex2_approx(fmaf(zl, kLog2e, -row_lse)) - a.inv_rows);
         a.label_logit[g * a.lse_sg + row] = zl;
       }
       __syncwarp();
@@ -717,8 +710,8 @@ wide_lse_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ H
 #pragma unroll
           for (int e = 0; e < 32; e += 4) {
             const float2 x0 = unpair(fma2(pair(z[e], z[e + 1]), l2, nr)), x1 = unpair(fma2(pair(z[e + 2], z[e + 3]), l2, nr));
-            s0 = add2(s0, pair(exp2_fast(x0.x), exp2_fast(x0.y)));
-            s1 = add2(s1, pair(exp2_fast(x1.x), exp2_fast(x1.y)));
+            s0 = add2(s0, pair(ex2_approx(x0.x), ex2_approx(x0.y)));
+            s1 = add2(s1, pair(ex2_approx(x1.x), ex2_approx(x1.y)));
           }
           const float2 t = unpair(add2(s0, s1));
           return t.x + t.y;
@@ -739,7 +732,7 @@ wide_lse_kernel(const __grid_constant__ HeadMaps maps, const __grid_constant__ H
             cs = any != any ? any : 0.f;
           } else {
             if (sum != 0.f) {
-              const float scale = exp2_fast(ref - mn);
+              const float scale = ex2_approx(ref - mn);
               sum *= scale;
               rest *= scale;
             }
